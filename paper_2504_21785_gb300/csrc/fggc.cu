@@ -10,8 +10,9 @@
 // s = r - a0 and likewise b0, t for P (eq. 3.6-3.7, FP64).  The true LSA
 // coefficients c~_k(s,t) = conj(A~^+ f~(s,t))_k come from
 //   FP64: f~ of eq. 3.23 in FP64 and A~^+ applied through its eigen factors;
-//   FP32: a Chebyshev surrogate of c~(s,t) built on the host in long double
-//         from the same factors (truncation error below 1e-9), evaluated in FP32.
+//   FP32: a polynomial surrogate of c~(s,t), one per orbit of mirrored
+//         neighbours, built on the host in long double from the same factors
+//         and evaluated in FP32 (build_lsa, coeff_dim32).
 // The shift back of eq. 3.13 and the node phase of the on-grid packet are
 // folded into one phase per coefficient: G(x; a dq, b dp) =
 // g(x - a dq) e^{i b dp x/eps} e^{-i cq cp a b}, and with r = a0 + s,
@@ -741,10 +742,13 @@ Common base_common(const fgr_ctx *ctx) {
     const Lsa &L = ctx->lsa;
     Common c{};
     c.n1 = L.n1;
+    const bool fp32 = ctx->opt.precision == FGR_FP32;
     for (int k = 0; k < L.n1; ++k) {
-        c.dq[k] = L.dq[k];
-        c.dp[k] = L.dp[k];
+        const int kk = fp32 ? L.order[k] : k;
+        c.dq[k] = L.dq[kk];
+        c.dp[k] = L.dp[kk];
     }
+    c.v3 = L.v3;
     c.dqv = M.dq;
     c.dpv = M.dp;
     c.inv_dq = 1.0 / M.dq;
@@ -1119,12 +1123,7 @@ fgr_status enqueue_fggc(fgr_ctx *ctx, const PacketsDev &pk, const FggcBox &box, 
     } else {
         Params32 P{};
         P.c = c;
-        for (int k = 0; k < kMaxN1; ++k)
-            for (int i = 0; i < kCheb; ++i)
-                for (int jj = 0; jj < kCheb; ++jj) {
-                    P.cre[(k * kCheb + i) * kCheb + jj] = L.cheb_re[k][i][jj];
-                    P.cim[(k * kCheb + i) * kCheb + jj] = L.cheb_im[k][i][jj];
-                }
+        memcpy(P.poly, L.poly, sizeof(P.poly));
         fgr_status r;
         if (binned) {
             bin_buffers_at(b.bin, pk.m, bl.box, &bl.buf);
@@ -1375,12 +1374,7 @@ fgr_status enqueue_fggc_batch(int n, const FggcRequest *req, cudaStream_t st) {
             base = b64.get();
         } else {
             b32.reset(new ScatterBatch32());
-            for (int k = 0; k < kMaxN1; ++k)
-                for (int i = 0; i < kCheb; ++i)
-                    for (int jj = 0; jj < kCheb; ++jj) {
-                        b32->cre[(k * kCheb + i) * kCheb + jj] = L.cheb_re[k][i][jj];
-                        b32->cim[(k * kCheb + i) * kCheb + jj] = L.cheb_im[k][i][jj];
-                    }
+            memcpy(b32->poly, L.poly, sizeof(b32->poly));
             base = b32.get();
         }
         base->n = nl;
@@ -1672,10 +1666,13 @@ extern "C" fgr_status fgr_reconstruct_fggc_noalloc(fgr_ctx *ctx, const fgr_packe
 
     Common c{};
     c.n1 = L.n1;
+    const bool fp32 = ctx->opt.precision == FGR_FP32;
     for (int k = 0; k < L.n1; ++k) {
-        c.dq[k] = L.dq[k];
-        c.dp[k] = L.dp[k];
+        const int kk = fp32 ? L.order[k] : k;
+        c.dq[k] = L.dq[kk];
+        c.dp[k] = L.dp[kk];
     }
+    c.v3 = L.v3;
     c.dqv = M.dq;
     c.dpv = M.dp;
     c.inv_dq = 1.0 / M.dq;
@@ -1748,12 +1745,7 @@ extern "C" fgr_status fgr_reconstruct_fggc_noalloc(fgr_ctx *ctx, const fgr_packe
     } else {
         Params32 P{};
         P.c = c;
-        for (int k = 0; k < kMaxN1; ++k)
-            for (int i = 0; i < kCheb; ++i)
-                for (int jj = 0; jj < kCheb; ++jj) {
-                    P.cre[(k * kCheb + i) * kCheb + jj] = L.cheb_re[k][i][jj];
-                    P.cim[(k * kCheb + i) * kCheb + jj] = L.cheb_im[k][i][jj];
-                }
+        memcpy(P.poly, L.poly, sizeof(P.poly));
         rc = launch_coeff_scatter(1, L.n1, st, PacketsDev{m, pk->q, pk->p, pk->s, pk->a}, nullptr, &P, W, flags);
         if (rc != FGR_OK) return rc;
     }

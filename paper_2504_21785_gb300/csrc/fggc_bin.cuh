@@ -158,59 +158,6 @@ __global__ void __launch_bounds__(256) clear_flagged_rows_kernel(float4 *__restr
     }
 }
 
-// coeff_dim32 with the neighbours evaluated one after the other into
-// out[k * stride] (fewer live registers than the unrolled form).
-template <int N1>
-__device__ __forceinline__ void coeff_dim32_rolled(const Params32 &P, double Q, double Pm, int &a0, int &b0,
-                                                   float2 *out, int stride) {
-    const Common &c = P.c;
-    a0 = floor_div_int(Q, c.dqv, c.inv_dq);
-    b0 = floor_div_int(Pm, c.dpv, c.inv_dp);
-    const double fa = (double)a0, fb = (double)b0;
-    const double r = Q * c.inv_dq, rp = Pm * c.inv_dp;
-    const float xs = fmaf(2.f, (float)(r - fa), -1.f), xt = fmaf(2.f, (float)(rp - fb), -1.f);
-    float Ts[kCheb], Tt[kCheb];
-    Ts[0] = 1.f;
-    Ts[1] = xs;
-    Tt[0] = 1.f;
-    Tt[1] = xt;
-#pragma unroll
-    for (int i = 2; i < kCheb; ++i) {
-        Ts[i] = 2.f * xs * Ts[i - 1] - Ts[i - 2];
-        Tt[i] = 2.f * xt * Tt[i - 1] - Tt[i - 2];
-    }
-    double t0 = -c.cc * (r * fb);
-    t0 -= rint(t0);
-    double t1 = -c.cc * fa;
-    t1 -= rint(t1);
-    const float t0f = (float)t0, t1f = (float)t1, ccf = (float)c.cc;
-#pragma unroll 1
-    for (int k = 0; k < N1; ++k) {
-        float sr = 0.f, si = 0.f;
-        const float *Cr = P.cre + k * kCheb * kCheb, *Ci = P.cim + k * kCheb * kCheb;
-#pragma unroll
-        for (int i = 0; i < kCheb; ++i) {
-            float ur = 0.f, ui = 0.f;
-#pragma unroll
-            for (int jj = 0; jj < kCheb; ++jj) {
-                if (i + jj <= cheb_total<N1>()) {
-                    ur = fmaf(Cr[i * kCheb + jj], Tt[jj], ur);
-                    ui = fmaf(Ci[i * kCheb + jj], Tt[jj], ui);
-                }
-            }
-            sr = fmaf(Ts[i], ur, sr);
-            si = fmaf(Ts[i], ui, si);
-        }
-        float tk = t0f + (float)c.dp[k] * t1f - ccf * (float)(c.dq[k] * c.dp[k]);
-        tk -= rint_fast(tk);
-        float sn, cs;
-        sincospif(2.f * tk, &sn, &cs);
-        float vr, vi;
-        cmul(sr, si, cs, sn, vr, vi);
-        out[k * stride] = make_float2(vr, vi);
-    }
-}
-
 // Target cells of one window (node cells of the inner plane).
 constexpr int kWinCells = 1024;
 
@@ -321,33 +268,39 @@ __global__ void __launch_bounds__(kBinT, kBinCtasPerSm) binned_scatter_kernel(
             rowoff[tid] = idx;
             if (in) atomicOr(&s_rows, 1ull << tid);
         }
-        float wr = 0.f, wi = 0.f;
         int ra = 0, rb = 0;  // inner anchor relative to the node box (set by the last dimension)
         float2 *cj = coef + tid * CS;
         if (valid) {
             const int64_t j = sorted[item.y + tid];
-            double ts = s[j] * c.inv_2pi_eps;
-            ts -= rint(ts);
-            float sn, cs;
-            sincospif(2.f * (float)ts, &sn, &cs);
-            cmul((float)(a[j] * c.pref), (float)(a[m + j] * c.pref), cs, sn, wr, wi);
+            const double ar = a[j], ai = a[m + j], sj = s[j];
+            double rB = 0.0;
+            float xy = 0.f;
             // one dimension at a time (one copy of the evaluation) into this
-            // thread's coefficient block
+            // thread's coefficient block; the weight goes with the last
+            // dimension's coefficients, once per packet rather than once per
+            // entry and accumulation pass
 #pragma unroll 1
             for (int l = 0; l < D; ++l) {
                 int a0, b0;
-                coeff_dim32_rolled<N1>(P, q[l * m + j], p[l * m + j], a0, b0, cj + l * N1, 1);
+                float X, Y, zr, zi, yr = 1.f, yi = 0.f;
+                dim_setup32(c, q[l * m + j], p[l * m + j], a0, b0, X, Y, zr, zi, rB, xy);
+                if (l == D - 1) packet_weight32(c, sj, ar, ai, rB, xy, yr, yi);
                 ra = a0 - c.amin[D - 1];
                 rb = b0 - c.bmin[D - 1];
-            }
-            // the weight goes with the last dimension's coefficients, once per
-            // packet rather than once per entry and accumulation pass
 #pragma unroll
-            for (int k = 0; k < N1; ++k) {
-                float2 &v = cj[(D - 1) * N1 + k];
-                float er, ei;
-                cmul(wr, wi, v.x, v.y, er, ei);
-                v = make_float2(er, ei);
+                for (int o = 0; o < N1 / 4; ++o) {
+                    float er[4], ei[4], vr, vi, hr[2], hi[2];
+                    orbit_coeffs<N1>(P.poly + o * kOrbitTable, X, Y, er, ei);
+                    orbit_phase<N1>(c, o, zr, zi, vr, vi);
+                    cmul(yr, yi, vr, vi, hr[0], hi[0]);
+                    cmul(yr, yi, vr, -vi, hr[1], hi[1]);
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) {
+                        float2 t;
+                        cmul(er[g], ei[g], hr[g & 1], hi[g & 1], t.x, t.y);
+                        cj[l * N1 + 4 * o + g] = t;
+                    }
+                }
             }
             atomicMin(&s_box[0], ra + bb.dqmin);
             atomicMax(&s_box[1], ra + bb.dqmax);

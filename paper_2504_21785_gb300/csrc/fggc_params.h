@@ -8,7 +8,8 @@ namespace fgr {
 
 struct Common {
     int n1;
-    int dq[kMaxN1], dp[kMaxN1];
+    int dq[kMaxN1], dp[kMaxN1];      // shifts (FP32: in orbit order, Lsa::order)
+    int v3;                          // FP32: orbits with |v| = 3/2 (Lsa::v3)
     double dqv, dpv;                 // mesh steps
     double inv_dq, inv_dp;
     double cq2_4, cp2_4, half_cqcp;  // eq. 3.23 constants
@@ -27,7 +28,7 @@ struct Params64 {
 
 struct Params32 {
     Common c;
-    float cre[kMaxN1 * kCheb * kCheb], cim[kMaxN1 * kCheb * kCheb];
+    float poly[kSurTable];  // coefficient surrogate (Lsa::poly)
 };
 
 // Node box of one FGGC reconstruction and the sizes of its buffers.
@@ -126,7 +127,7 @@ struct ScatterBatch64 : ScatterBatchBase {
     double vr[kMaxN1 * kMaxN1], vi[kMaxN1 * kMaxN1], inv_lam[kMaxN1];
 };
 struct ScatterBatch32 : ScatterBatchBase {
-    float cre[kMaxN1 * kCheb * kCheb], cim[kMaxN1 * kCheb * kCheb];
+    float poly[kSurTable];
 };
 
 // One request of a batched FGGC call: its context, planned box and buffers,

@@ -14,22 +14,25 @@ namespace fgr {
 constexpr int kMaxDim = 3;
 constexpr int kMaxN1 = 16;  // 1-D neighbours per packet: nq * np <= 16
 
-// Eigen-factored eps-free Gram matrix of eq. 3.22 (paper convention).
-// The Gram A~ is Hermitian PSD: A~ = V diag(lam) V^H, A~^+ = V diag(inv_lam) V^H.
-// Degree of the FP32 coefficient surrogate per variable: its truncation error
-// (3e-10 for Q4P2 at 10, 4e-13 at 12) lies far below the FP32 rounding of its
-// stored coefficients and of its evaluation.
+// FP32 coefficient surrogate: Chebyshev degree per variable and total degree.
+// The terms T_i T_j with i + j <= surrogate_total and i, j < kCheb are kept for
+// n1 <= 8 (Q2P2, Q4P2, Q2P4); their dropped coefficients sum to 1.1e-8 (Q4P2)
+// and 1.1e-11 (Q2P2) of the largest one, under the FP32 rounding of the
+// evaluation (2e-8 rms measured); n1 = 16 (Q4P4) keeps every i, j < kCheb.
 constexpr int kCheb = 10;
-// Terms T_i(s) T_j(t) the FP32 kernels evaluate: i + j <= cheb_total<n1>().
-// For n1 <= 8 (Q2P2, Q4P2) the triangle i + j <= 11 keeps 72 of the 100 terms
-// and the dropped coefficients sum to below 1e-8 of the largest one (Q4P2
-// 8.4e-9, Q2P2 7e-12), under the FP32 rounding of the evaluation; n1 = 16
-// (Q4P4) keeps the whole table.
 template <int N1>
-__host__ __device__ constexpr int cheb_total() {
+__host__ __device__ constexpr int surrogate_total() {
     return N1 <= 8 ? 11 : 2 * (kCheb - 1);
 }
+// Even (or odd) powers per variable in one parity part of the surrogate.
+constexpr int kPow = kCheb / 2;
+// Floats of the surrogate of one orbit of four mirrored neighbours:
+// [re, im][parity part ee, oe, eo, oo][power of X^2][power of Y^2].
+constexpr int kOrbitTable = 2 * 4 * kPow * kPow;
+constexpr int kSurTable = kMaxN1 / 4 * kOrbitTable;
 
+// Eigen-factored eps-free Gram matrix of eq. 3.22 (paper convention).
+// The Gram A~ is Hermitian PSD: A~ = V diag(lam) V^H, A~^+ = V diag(inv_lam) V^H.
 struct Lsa {
     int nq = 4, np = 2, n1 = 8, rank = 0;
     double cq = 0.5, cp = 0.0;
@@ -38,10 +41,13 @@ struct Lsa {
     double inv_lam[kMaxN1] = {};           // 1/lam above the cut-off, else 0
     double vr[kMaxN1 * kMaxN1] = {};       // V[j][i]: component j of eigenvector i
     double vi[kMaxN1 * kMaxN1] = {};
-    // Chebyshev surrogate of the true coefficients c~_k(s,t) = conj(A~^+ f~(s,t))_k
-    // on [0,1]^2: c~_k ~= sum_{i,j<kCheb} cheb[k][i][j] T_i(2s-1) T_j(2t-1).
-    float cheb_re[kMaxN1][kCheb][kCheb] = {};
-    float cheb_im[kMaxN1][kCheb][kCheb] = {};
+    // Neighbours in orbit order: orbit o holds, at 4 o + g, the mirror images
+    // (u, v), (u, -v), (-u, v), (-u, -v) of one shift, (u, v) = (dq - 1/2, dp - 1/2)
+    // with u, v < 0 for g = 0 (FP32 kernels number their neighbours this way).
+    int order[kMaxN1] = {};
+    int v3 = 0;  // bit o: orbit o has |v| = 3/2 (else 1/2)
+    // Surrogate of the first neighbour of every orbit (see build_lsa).
+    float poly[kSurTable] = {};
 };
 
 // Builds Lsa (host, long double Jacobi).  Returns false on bad input.
