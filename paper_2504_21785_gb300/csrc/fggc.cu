@@ -901,7 +901,9 @@ bool make_bin_box(const FggcBox &box, int d, BinBox *bb) {
 
 namespace {
 inline size_t align256(size_t n) { return (n + 255) & ~size_t(255); }
-inline int64_t bin_max_items(int64_t m) { return m / 16 + m / 256 + 1; }
+// A binned cell holds n >= kBinMinCount packets and gives ceil(n / 256) items,
+// at most n / kBinMinCount.
+inline int64_t bin_max_items(int64_t m) { return m / kBinMinCount + 1; }
 }  // namespace
 
 size_t bin_buffer_bytes(int64_t m, const BinBox &bb) {

@@ -152,3 +152,11 @@ def test_rows_left_from_an_earlier_call_are_not_read():
     assert _gpu.rel_l2(got[tuple(pts)], ref) <= 1e-5
     alone = _gpu.reconstruct("fggc", other, grid, eps, opt)
     assert _gpu.rel_l2(got, alone) <= 1e-6
+
+
+def test_every_cell_at_the_smallest_binned_size():
+    """600 cells of 8 packets: one item each, the most items that a packet count can give."""
+    eps = 1 / 64
+    cells = [((a, b), (a2, 3)) for a in range(-5, 5) for b in range(-6, 6) for a2 in range(-2, 3)]
+    pk, mesh = clustered(11, 3, eps, cells, [8] * len(cells), (-0.6, 0.6), (-0.5, 0.5))
+    _check(pk, mesh, _grid([33, 30, 27]), eps, npts=200)
