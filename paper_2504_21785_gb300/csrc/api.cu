@@ -987,7 +987,6 @@ struct fgr_fggc_plan {
     FggcBuffers buf;
     int *bnd = nullptr;       // device: the packets' node bounds of the last call
     int *overflow = nullptr;  // device: set when they left the box
-    size_t bin_bytes = 0;     // binning buffers (d = 3, FP32)
     // The buffers come from the device's stream-ordered pool (allocating them
     // does not wait for other streams' work); they go back to it once the
     // device has finished the work issued before the release.
@@ -1012,7 +1011,7 @@ size_t plan_device_bytes(const fgr_fggc_plan *pl) {
     size_t n = 64;  // bounds and overflow flag
     if (!b.empty)
         n += eb * (size_t)b.cells + (pl->d > 1 ? 2 * eb * (size_t)b.maxbuf : 0) + (size_t)b.rows0 +
-             sizeof(int2) * (size_t)b.max_lines + 8 * (size_t)b.table_entries + pl->bin_bytes +
+             sizeof(int2) * (size_t)b.max_lines + 8 * (size_t)b.table_entries + pl->buf.bin_bytes +
              (b.fft_elems > 0 ? eb * ((size_t)b.fft_elems + 4096) : 0);
     return n;
 }
@@ -1094,10 +1093,9 @@ fgr_status fgr_fggc_plan_create(fgr_ctx *ctx, const fgr_packets *pk, int32_t mar
             if (e == cudaSuccess && b.fft_elems > 0) e = palloc(&pl->buf.fft, eb * (size_t)b.fft_elems);
             if (e == cudaSuccess && b.fft_elems > 0) e = palloc(&pl->buf.twiddle, eb * 4096);
             BinBox bb;
-            if (e == cudaSuccess && ctx->opt.precision == FGR_FP32 && make_bin_box(b, ctx->d, &bb)) {
-                pl->bin_bytes = bin_buffer_bytes(pk->m, bb);
-                e = palloc(&pl->buf.bin, pl->bin_bytes);
-                pl->buf.bin_m = pk->m;
+            if (e == cudaSuccess && ctx->opt.precision == FGR_FP32 && make_bin_box(b, ctx->d, pk->m, &bb)) {
+                pl->buf.bin_bytes = bin_buffer_bytes(pk->m, bb);
+                e = palloc(&pl->buf.bin, pl->buf.bin_bytes);
             }
             if (e != cudaSuccess) return fail(e);
         }

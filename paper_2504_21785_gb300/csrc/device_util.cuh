@@ -49,6 +49,22 @@ __device__ __forceinline__ int floor_div_int(double x, double step, double inv_s
     return (int)fmin(fmax(r, -1e9), 1e9);
 }
 
+// x as h + l in FP32 by integer operations on its bits (FP64 instructions and
+// conversions run at 1/64 of the FP32 rate): h is x truncated to 24 bits, l the
+// next 23 bits, |x - h - l| < 2^-46 |x|.  False (h = l = 0) unless x is zero or
+// 2^-100 <= |x| < 2^126.
+__device__ __forceinline__ bool split_double(double x, float &h, float &l) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned mag = hi & 0x7fffffffu, sgn = hi & 0x80000000u;
+    const bool in_range = (mag >> 20) - 923u < 226u;
+    const unsigned hb = __funnelshift_l(lo, mag, 3) - 0xc0000000u;         // exponent - 896
+    const unsigned lb = ((mag & 0x7ff00000u) << 3) - 0xcb800000u;          // exponent - 919: 2^-23 h's last bit
+    const float lf = __uint_as_float(lb | ((lo & 0x1fffffffu) >> 6)) - __uint_as_float(lb);
+    h = in_range ? __uint_as_float(hb | sgn) : 0.f;
+    l = in_range ? __uint_as_float(__float_as_uint(lf) ^ sgn) : 0.f;
+    return in_range || (mag | lo) == 0u;
+}
+
 // Grid coordinate x_m = lo + m*h without contraction.
 __device__ __forceinline__ double grid_x(double lo, double h, int64_t m) {
     return __dadd_rn(lo, __dmul_rn((double)m, h));
@@ -59,6 +75,33 @@ __device__ __forceinline__ float rint_fast(float x) {
     const float magic = 12582912.0f;  // 1.5 * 2^23
     return __fsub_rn(__fadd_rn(x, magic), magic);
 }
+
+// Two FP32 operations per instruction (sm_100 and later).  The FMA pipe does no
+// more of them per clock (75.7 against 76.0 TFLOP/s measured), but they take
+// half the issue slots, which bind the kernels that use them.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("{\n\t.reg .b64 a, b, c, d;\n\t"
+        "mov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\t"
+        "fma.rn.f32x2 d, a, b, c;\n\t"
+        "mov.b64 {%0, %1}, d;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 a, b, d;\n\t"
+        "mov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+        "mul.rn.f32x2 d, a, b;\n\t"
+        "mov.b64 {%0, %1}, d;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+
+__device__ __forceinline__ float2 both(float x) { return make_float2(x, x); }
 
 // 2^x on the special-function unit (relative error about 2^-22).
 __device__ __forceinline__ float ex2_approx(float x) {

@@ -762,6 +762,22 @@ Common base_common(const fgr_ctx *ctx) {
     return c;
 }
 
+// The binning's constants as FP32 sums.
+SplitConst split_const(const Common &c) {
+    SplitConst k;
+    auto put = [](double v, float *o) {
+        o[0] = (float)v;
+        o[1] = (float)(v - (double)o[0]);
+    };
+    put(c.inv_dq, k.inv_dq);
+    put(c.inv_dp, k.inv_dp);
+    put(c.cc, k.cc);
+    put(0.5 * c.cc, k.half_cc);
+    put(c.inv_2pi_eps, k.inv_2pi_eps);
+    put(c.pref, k.pref);
+    return k;
+}
+
 // Grid-relevant node range per dimension (other nodes have empty windows).
 void grid_node_range(const fgr_ctx *ctx, int *aglo, int *aghi) {
     const Grid &G = ctx->grid;
@@ -871,8 +887,9 @@ fgr_status make_box(const fgr_ctx *ctx, const int *hb, int margin, FggcBox *box)
     return FGR_OK;
 }
 
-bool make_bin_box(const FggcBox &box, int d, BinBox *bb) {
-    if (d != 3 || box.empty) return false;
+bool make_bin_box(const FggcBox &box, int d, int64_t m, BinBox *bb) {
+    if (d < 2 || box.empty || (box.c.n1 != 4 && box.c.n1 != 8) || m >= INT_MAX) return false;
+    if (d == 2 && m < kBinMinPackets2d) return false;
     const Common &c = box.c;
     BinBox x;
     x.dqmin = x.dpmin = INT_MAX;
@@ -883,16 +900,22 @@ bool make_bin_box(const FggcBox &box, int d, BinBox *bb) {
         x.dpmin = std::min(x.dpmin, c.dp[k]);
         x.dpmax = std::max(x.dpmax, c.dp[k]);
     }
-    // an outer anchor a0 has a node inside [amin, amin + A) for a0 in
+    // an anchor a0 has a node inside [amin, amin + A) for a0 in
     // [amin - dqmax, amin + A - 1 - dqmin] (likewise b0)
     int64_t K = 1;
-    for (int l = 0; l < d - 1; ++l) {
+    for (int l = 0; l < d; ++l) {
         x.ka_lo[l] = c.amin[l] - x.dqmax;
         x.KA[l] = c.A[l] + x.dqmax - x.dqmin;
         x.kb_lo[l] = c.bmin[l] - x.dpmax;
         x.KB[l] = c.B[l] + x.dpmax - x.dpmin;
-        K *= (int64_t)x.KA[l] * x.KB[l];
+        if (l < d - 1) K *= (int64_t)x.KA[l] * x.KB[l];
         if (K > kMaxBinKeys) return false;
+    }
+    if (d == 2) {
+        x.tiles_a = (x.KA[1] + kBinTileA - 1) / kBinTileA;
+        x.tiles_b = (x.KB[1] + kBinTileB - 1) / kBinTileB;
+        K *= (int64_t)x.tiles_a * x.tiles_b;
+        if (K > kMaxBinKeys || K > m) return false;
     }
     x.K = K;
     *bb = x;
@@ -901,44 +924,47 @@ bool make_bin_box(const FggcBox &box, int d, BinBox *bb) {
 
 namespace {
 inline size_t align256(size_t n) { return (n + 255) & ~size_t(255); }
-// A binned cell holds n >= kBinMinCount packets and gives ceil(n / 256) items,
-// at most n / kBinMinCount.
+// A bin holds n >= kBinMinCount packets and gives ceil(n / 256) items, at most
+// n / kBinMinCount.
 inline int64_t bin_max_items(int64_t m) { return m / kBinMinCount + 1; }
+
+// The binning buffers of one device block; returns their bytes.
+size_t carve_bin_buffers(char *p, int64_t m, const BinBox &bb, BinBuffers *out) {
+    const size_t M = (size_t)m, K = (size_t)bb.K;
+    size_t at = 0;
+    auto take = [&](size_t n) {
+        char *r = p + at;
+        at += align256(n);
+        return (void *)r;
+    };
+    out->key = (int *)take(sizeof(int) * M);
+    out->rank = (int *)take(sizeof(int) * M);
+    out->loose = (int *)take(sizeof(int) * M);
+    out->rec = (BinRecord *)take(sizeof(BinRecord) * M);
+    out->count = (int *)take(sizeof(int) * K);
+    out->kbox = (int4 *)take(sizeof(int4) * K);
+    out->off = (int2 *)take(sizeof(int2) * (K + 1));
+    out->bsum = (int2 *)take(sizeof(int2) * ((K + 1023) / 1024));
+    out->items = (BinItem *)take(sizeof(BinItem) * (size_t)bin_max_items(m));
+    out->ctr = (int *)take(sizeof(int) * 4);
+    return at;
+}
 }  // namespace
 
 size_t bin_buffer_bytes(int64_t m, const BinBox &bb) {
-    const int64_t K = bb.K;
-    return 3 * align256(sizeof(int) * (size_t)m) + align256(sizeof(int) * (size_t)K) +
-           align256(sizeof(int2) * (size_t)(K + 1)) + align256(sizeof(int2) * (size_t)((K + 1023) / 1024)) +
-           align256(sizeof(int4) * (size_t)bin_max_items(m)) + align256(sizeof(int) * 4);
+    BinBuffers b;
+    return carve_bin_buffers(nullptr, m, bb, &b);
 }
 
 void bin_buffers_at(void *block, int64_t m, const BinBox &bb, BinBuffers *out) {
-    char *p = (char *)block;
-    const int64_t K = bb.K;
-    auto take = [&](size_t n) {
-        char *r = p;
-        p += align256(n);
-        return r;
-    };
-    out->key = (int *)take(sizeof(int) * (size_t)m);
-    out->sorted = (int *)take(sizeof(int) * (size_t)m);
-    out->loose = (int *)take(sizeof(int) * (size_t)m);
-    out->count = (int *)take(sizeof(int) * (size_t)K);
-    out->off = (int2 *)take(sizeof(int2) * (size_t)(K + 1));
-    out->bsum = (int2 *)take(sizeof(int2) * (size_t)((K + 1023) / 1024));
-    out->items = (int4 *)take(sizeof(int4) * (size_t)bin_max_items(m));
-    out->ctr = (int *)take(sizeof(int) * 4);
+    carve_bin_buffers((char *)block, m, bb, out);
 }
 
 fgr_status launch_binned_scatter(int d, int n1, const BinLaunch &L, cudaStream_t st, const PacketsDev &pk,
                                  const Params32 &P, void *W, uint8_t *flags, StageMarks *marks) {
     if (pk.m == 0) return FGR_OK;
-    if (d != 3) {
-        set_error("fggc: the binned scatter serves d = 3");
-        return FGR_E_INTERNAL;
-    }
-    return launch_binned_d3(n1, L, st, pk, P, W, flags, marks);
+    return d == 2 ? launch_binned_d2(n1, L, st, pk, P, W, flags, marks)
+                  : launch_binned_d3(n1, L, st, pk, P, W, flags, marks);
 }
 
 namespace {
@@ -1103,12 +1129,12 @@ fgr_status enqueue_fggc(fgr_ctx *ctx, const PacketsDev &pk, const FggcBox &box, 
     const Lsa &L = ctx->lsa;
     const size_t eb = elem_bytes(ctx->opt.precision);
     const Common &c = box.c;
-    // FP32 3-D: the binned scatter, which marks the rows its packets reach and
-    // clears only those (the passes and b-range scans skip unmarked rows);
+    // FP32, d >= 2: the binned scatter, which marks the rows its packets reach
+    // and clears only those (the passes and b-range scans skip unmarked rows);
     // otherwise W is cleared whole and the scatter marks the rows it reaches
     BinLaunch bl;
-    const bool binned = !fp64 && D == 3 && b.bin && b.bin_m >= pk.m && pk.m > 0 && (L.n1 == 4 || L.n1 == 8) &&
-                        make_bin_box(box, D, &bl.box);
+    const bool binned = !fp64 && b.bin && pk.m > 0 && make_bin_box(box, D, pk.m, &bl.box) &&
+                        bin_buffer_bytes(pk.m, bl.box) <= b.bin_bytes;
     if (!binned) FGR_CUDA_TRY(cudaMemsetAsync(b.W, 0, eb * (size_t)box.cells, st));
     // the single row of d = 1 is marked here
     FGR_CUDA_TRY(cudaMemsetAsync(b.flags, D == 1 ? 1 : 0, (size_t)box.rows0, st));
@@ -1129,9 +1155,9 @@ fgr_status enqueue_fggc(fgr_ctx *ctx, const PacketsDev &pk, const FggcBox &box, 
         fgr_status r;
         if (binned) {
             bin_buffers_at(b.bin, pk.m, bl.box, &bl.buf);
+            bl.split = split_const(c);
             bl.num_sms = ctx->num_sms;
-            bl.min_count = kBinMinCount;
-            bl.clear_rows = box.rows0;
+            bl.rows = box.rows0;
             bl.row_cells = box.cells / box.rows0;
             StageMarks marks{timer, &ctx->timing.last.coeff_ms};
             r = launch_binned_scatter(D, L.n1, bl, st, pk, P, b.W, b.flags, &marks);
@@ -1250,10 +1276,10 @@ fgr_status launch(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStream_t 
         if (!b.fft || !b.twiddle) return FGR_E_NOMEM;
     }
     BinBox bb;
-    if (ctx->opt.precision == FGR_FP32 && make_bin_box(box, D, &bb)) {
-        b.bin = scratch.get(bin_buffer_bytes(pk.m, bb));
+    if (ctx->opt.precision == FGR_FP32 && make_bin_box(box, D, pk.m, &bb)) {
+        b.bin_bytes = bin_buffer_bytes(pk.m, bb);
+        b.bin = scratch.get(b.bin_bytes);
         if (!b.bin) return FGR_E_NOMEM;
-        b.bin_m = pk.m;
     }
     if (ctx->timing.enabled && ctx->timing.count_terms) {
         b.terms = (unsigned long long *)scratch.get(sizeof(unsigned long long));

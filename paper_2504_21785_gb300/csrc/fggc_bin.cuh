@@ -1,22 +1,29 @@
-// K4 for d = 3 (FP32 path): the scatter of eq. 2.25 with the packets binned
-// by the anchor cell (a0, b0) of their outer dimensions.
+// K4 for d = 2, 3 (FP32 path): the scatter of eq. 2.25 with the packets binned
+// by anchor cell.
 //
 // A packet's contributions to one row of the node array (the last dimension's
-// [a][b] plane for fixed outer nodes) are the 2 x 4 neighbours of its inner
-// anchor cell, and the outer anchor cell fixes which rows it reaches: n1^(d-1)
-// rows, one per outer neighbour.  Packets with the same outer anchor cell reach
-// the same rows, so after a counting sort by that cell a CTA takes up to
-// kBinT packets of one cell, adds their contributions to each row into a
-// private plane in shared memory (the box of their inner neighbours) and then
-// adds the plane to W: one 8-byte reduction per touched cell instead of one
-// per contribution, issued by consecutive threads to consecutive cells of the
-// row.  Cells with fewer packets than BinLaunch::min_count go through the
-// per-packet kernel (fggc_coeff.cuh) from a list.
+// [a][b] plane for fixed outer nodes) are the neighbours of its inner anchor
+// cell, and the outer anchor cell (a0, b0 of the other dimensions) fixes which
+// n1^(d-1) rows it reaches.  Packets with the same outer anchor cell (d = 2: and
+// the same 24 x 16 tile of inner anchors, so that they overlap) form a bin.
+// After a counting sort by bin a CTA takes up to kBinT packets of one, lists for
+// every target cell of their inner box the (packet, neighbour) pairs that reach
+// it, sums a cell's contributions to every row in registers and adds each row's
+// value to W with one 8-byte reduction: one per touched (cell, row) instead of
+// one per contribution, issued by neighbouring lanes to neighbouring cells.  A
+// packet set of one packet per dq x dp cell (what the flow preserves) gives 6
+// to 8 pairs per cell.
 //
-// Included by fggc_coeff3.cu.  The kernels are written for d >= 2; the
-// library uses them for d = 3, where a packet has 512 contributions.
+// The sort's last kernel also turns each packet into a 48-byte record in bin
+// order (cell offsets, weight and phases: all that needs more than FP32), so
+// that the binned kernel reads its packets in one piece and does FP32 work only.
+// Bins with fewer than kBinMinCount packets go through the per-packet kernel
+// (fggc_coeff.cuh) from a list.
+//
+// Included by fggc_coeff2.cu and fggc_coeff3.cu.
 #pragma once
 
+#include <algorithm>
 #include <climits>
 
 #include "fggc_coeff.cuh"
@@ -25,36 +32,42 @@ namespace fgr {
 namespace {
 
 constexpr int kBinT = 256;         // packets (threads) per binned item
-constexpr int kBinCtasPerSm = 3;   // resident binned-scatter CTAs per SM (registers, shared memory)
+// Resident binned-scatter CTAs per SM (registers; d = 3: and shared memory).
+template <int D>
+__host__ __device__ constexpr int bin_ctas_per_sm() {
+    return D == 3 ? 3 : 4;
+}
 
-// Warp-aggregated atomicAdd of sign on ctr[k] by the active lanes (one atomic
-// per distinct k); returns the old value plus sign times the lane's rank
-// among the lanes with the same k.
-__device__ __forceinline__ int aggregated_add(int *ctr, int k, int sign) {
+// Warp-aggregated atomicAdd of 1 on ctr[k] by the active lanes (one atomic per
+// distinct k); returns the old value plus the lane's rank among the lanes with
+// the same k.
+__device__ __forceinline__ int aggregated_add(int *ctr, int k) {
     const unsigned act = __activemask();
     const unsigned peers = __match_any_sync(act, k);
     const int lane = threadIdx.x & 31;
     const int leader = __ffs(peers) - 1;
     const int rank = __popc(peers & ((1u << lane) - 1));
     int base = 0;
-    if (lane == leader) base = atomicAdd(ctr + k, sign * __popc(peers));
+    if (lane == leader) base = atomicAdd(ctr + k, __popc(peers));
     base = __shfl_sync(peers, base, leader);
-    return base + sign * rank;
+    return base + rank;
 }
 
-// Per packet: the key of its outer anchor cell in the key box (-1: the packet
-// adds nothing: zero amplitude, or every node of an outer dimension lies
-// outside the node box), and the count of packets per key.
+// Per packet: its key (-1: the packet adds nothing: zero amplitude, or every
+// node of a keyed dimension lies outside the node box) and its place among the
+// packets of that key, counted in count[].
 template <int D>
-__global__ void bin_key_kernel(const double *__restrict__ q, const double *__restrict__ p,
-                               const double *__restrict__ a, int64_t m, const Common c, const BinBox bb,
-                               int *__restrict__ key, int *__restrict__ count) {
+__global__ void __launch_bounds__(256) bin_key_kernel(const double *__restrict__ q, const double *__restrict__ p,
+                                                      const double *__restrict__ a, int64_t m, const Common c,
+                                                      const BinBox bb, int *__restrict__ key, int *__restrict__ rank,
+                                                      int *__restrict__ count) {
+    constexpr int KD = D == 2 ? 2 : D - 1;  // dimensions that the key reads
     const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (j >= m) return;
     int k = -1;
-    double qv[D - 1], pv[D - 1];  // every load first (none waits on the amplitude test)
+    double qv[KD], pv[KD];  // every load first (none waits on the amplitude test)
 #pragma unroll
-    for (int l = 0; l < D - 1; ++l) {
+    for (int l = 0; l < KD; ++l) {
         qv[l] = q[l * m + j];
         pv[l] = p[l * m + j];
     }
@@ -62,46 +75,236 @@ __global__ void bin_key_kernel(const double *__restrict__ q, const double *__res
         int64_t kk = 0;
         bool ok = true;
 #pragma unroll
-        for (int l = 0; l < D - 1; ++l) {
-            const int ia = floor_div_int(qv[l], c.dqv, c.inv_dq) - bb.ka_lo[l];
-            const int ib = floor_div_int(pv[l], c.dpv, c.inv_dp) - bb.kb_lo[l];
+        for (int l = 0; l < KD; ++l) {
+            int ia = floor_div_int(qv[l], c.dqv, c.inv_dq) - bb.ka_lo[l];
+            int ib = floor_div_int(pv[l], c.dpv, c.inv_dp) - bb.kb_lo[l];
             ok = ok && (unsigned)ia < (unsigned)bb.KA[l] && (unsigned)ib < (unsigned)bb.KB[l];
-            kk = (kk * bb.KA[l] + ia) * bb.KB[l] + ib;
+            const bool inner = l == D - 1;
+            kk = (kk * (inner ? bb.tiles_a : bb.KA[l]) + (inner ? (unsigned)ia / kBinTileA : ia)) *
+                     (inner ? bb.tiles_b : bb.KB[l]) +
+                 (inner ? (unsigned)ib / kBinTileB : ib);
         }
         if (ok) k = (int)kk;
     }
     key[j] = k;
-    if (k >= 0) aggregated_add(count, k, 1);
+    if (k >= 0) rank[j] = aggregated_add(count, k);
 }
 
-// Places every binned packet at its sorted position (offset of its key plus
-// a slot) and every packet of a small cell on the loose list.  count[] is
-// consumed as the per-key cursor.
-__global__ void bin_place_kernel(const int *__restrict__ key, int64_t m, const int2 *__restrict__ off,
-                                 int *__restrict__ count, int *__restrict__ sorted, int *__restrict__ loose,
-                                 int *__restrict__ nloose) {
-    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (j >= m) return;
-    const int k = key[j];
-    if (k < 0) return;
-    const int2 o = off[k], o1 = off[k + 1];
-    if (o1.x > o.x) {  // a binned cell: slots counted down from its size
-        const int slot = aggregated_add(count, k, -1) - 1;
-        sorted[o.x + slot] = (int)j;
-    } else {
-        loose[aggregated_add(nloose, 0, 1)] = (int)j;
+// x / step of a packet coordinate as integer part fl and offset fr in [0, 1),
+// with the quotient p + e (FP32 sum, relative error below 2^-45); within 2^-20 of
+// an integer the FP64 division decides the integer part.  False: out of the
+// range in which offsets and phases keep FP32 accuracy (the caller's FP64 path).
+__device__ __forceinline__ bool quotient_split(double x, const float *inv, double step, double inv_step, float &fl,
+                                               float &fr, float &p, float &e) {
+    float h, l;
+    bool ok = split_double(x, h, l);
+    p = __fmul_rn(h, inv[0]);
+    e = fmaf(h, inv[0], -p);
+    e = fmaf(h, inv[1], e);
+    e = fmaf(l, inv[0], e);
+    ok = ok && fabsf(p) < 262144.f;
+    fl = floorf(p);
+    fr = __fadd_rn(__fsub_rn(p, fl), e);
+    if (fr < 0.f) {
+        fl -= 1.f;
+        fr += 1.f;
+    } else if (fr >= 1.f) {
+        fl += 1.f;
+        fr -= 1.f;
+    }
+    if (ok && (fr < 0x1p-20f || fr > 1.f - 0x1p-20f)) {
+        const float f = (float)floor(quotient_for_floor(x, step, inv_step));
+        fr += fl - f;
+        fl = f;
+    }
+    return ok;
+}
+
+// (p + e) k in turns: t the part reduced to [-1/2, 1/2], returned, lo the rest.
+__device__ __forceinline__ float turns_split(float p, float e, const float *k, float &lo) {
+    const float t = __fmul_rn(p, k[0]);
+    float u = fmaf(p, k[0], -t);
+    u = fmaf(p, k[1], u);
+    lo = fmaf(e, k[0], u);
+    return __fsub_rn(t, rint_fast(t));
+}
+
+// s += x (error-free, the rounding goes to lo), reduced to [-1/2, 1/2].
+__device__ __forceinline__ void turns_add(float &s, float &lo, float x) {
+    const float v = __fadd_rn(s, x), b = __fsub_rn(v, s);
+    lo += __fadd_rn(__fsub_rn(s, __fsub_rn(v, b)), __fsub_rn(x, b));
+    s = __fsub_rn(v, rint_fast(v));
+}
+
+// A packet's record: offsets (sx, ty) per dimension, weight, z of the last
+// dimension and its anchor (see dim_setup32 and packet_weight32, whose FP64
+// phases these are).  FP64 instructions take 16 clocks of an SM here, so the
+// offsets and phases are computed as FP32 sums (2^-45 relative); packets out of
+// range (|Q/dq| or |P/dp| >= 2^18, |S| / (2 pi eps) >= 2^18 turns, amplitudes
+// below 2^-100) take the FP64 form.
+template <int D>
+__device__ __forceinline__ void packet_record(const Common &c, const SplitConst &k, const double *qv,
+                                              const double *pv, double s, double ar, double ai, float *sx, float *ty,
+                                              int &a0, int &b0, float2 &w, float2 &z) {
+    bool ok = true;
+    float h, l, xy = 0.f, T, lo;
+    ok = split_double(s, h, l) && ok;
+    ok = ok && fabsf(h * k.inv_2pi_eps[0]) < 262144.f;
+    T = turns_split(h, l, k.inv_2pi_eps, lo);
+    float A = 0.f;
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+        float fa, fb, fr, p, e, pb, eb;
+        ok = quotient_split(pv[d], k.inv_dp, c.dpv, c.inv_dp, fb, fr, pb, eb) && ok;
+        ty[d] = fr - 0.5f;
+        ok = quotient_split(qv[d], k.inv_dq, c.dqv, c.inv_dq, fa, fr, p, e) && ok;
+        sx[d] = fr - 0.5f;
+        const float B = fb + 0.5f, g = __fmul_rn(p, B);
+        ok = ok && fabsf(g * k.cc[0]) < 262144.f;
+        float u;
+        const float t = turns_split(g, fmaf(e, B, fmaf(p, B, -g)), k.cc, u);
+        turns_add(T, lo, -t);
+        lo -= u;
+        xy = fmaf(sx[d], ty[d], xy);
+        if (d == D - 1) {
+            a0 = (int)fa;
+            b0 = (int)fb;
+            A = fa + 0.5f;
+        }
+    }
+    float sn, cs;
+    if (ok) {
+        sincospif(2.f * (T + fmaf(-0.5f * k.cc[0], xy, lo)), &sn, &cs);
+        ok = split_double(ar, h, l);
+        const float wr = fmaf(h, k.pref[0], fmaf(h, k.pref[1], l * k.pref[0]));
+        ok = split_double(ai, h, l) && ok;
+        const float wi = fmaf(h, k.pref[0], fmaf(h, k.pref[1], l * k.pref[0]));
+        cmul(wr, wi, cs, sn, w.x, w.y);
+        float u;
+        const float t = turns_split(A, 0.f, k.half_cc, u);
+        sincospif(2.f * (t + u), &z.y, &z.x);
+    }
+    if (!ok) {
+        double rB = 0.0;
+        xy = 0.f;
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            float X, Y;
+            dim_setup32(c, qv[d], pv[d], a0, b0, X, Y, z.x, z.y, rB, xy);
+            sx[d] = 0.5f * X;
+            ty[d] = 0.5f * Y;
+        }
+        packet_weight32(c, s, ar, ai, rB, xy, w.x, w.y);
     }
 }
 
-// One item (key, first sorted position, packets) per kBinT packets of every
-// binned cell.
-__global__ void bin_items_kernel(const int2 *__restrict__ off, int64_t K, int4 *__restrict__ items) {
+// Writes every binned packet's record at its place (and, d = 3, widens the inner
+// anchor box of its key) and puts every packet of a small bin on the loose list.
+template <int D>
+__global__ void __launch_bounds__(256) bin_place_kernel(const double *__restrict__ q, const double *__restrict__ p,
+                                                        const double *__restrict__ s, const double *__restrict__ a,
+                                                        int64_t m, const __grid_constant__ Common c,
+                                                        const __grid_constant__ SplitConst sc,
+                                                        const int *__restrict__ key, const int *__restrict__ rank,
+                                                        const int2 *__restrict__ off, BinRecord *__restrict__ rec,
+                                                        int4 *kbox, int *__restrict__ loose, int *__restrict__ nloose) {
+    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (j >= m) return;
+    const int k = key[j];
+    double qv[D], pv[D];
+#pragma unroll
+    for (int l = 0; l < D; ++l) {
+        qv[l] = q[l * m + j];
+        pv[l] = p[l * m + j];
+    }
+    const double sv = s[j], ar = a[j], ai = a[m + j];
+    if (k < 0) return;
+    const int2 o = off[k], o1 = off[k + 1];
+    if (o1.x == o.x) {
+        loose[aggregated_add(nloose, 0)] = (int)j;
+        return;
+    }
+    float sx[D], ty[D];
+    int a0, b0;
+    float2 w, z;
+    packet_record<D>(c, sc, qv, pv, sv, ar, ai, sx, ty, a0, b0, w, z);
+    a0 -= c.amin[D - 1];
+    b0 -= c.bmin[D - 1];
+    BinRecord r;
+    r.x = make_float4(sx[0], ty[0], sx[D - 1], ty[D - 1]);
+    r.w = make_float4(w.x, w.y, z.x, z.y);
+    r.y = make_float4(__int_as_float(a0), __int_as_float(b0), sx[D / 2], ty[D / 2]);
+    rec[o.x + rank[j]] = r;
+    if constexpr (D == 3) {
+        // most packets find their key's box wide enough already (a stale read
+        // only costs an atomic)
+        const int4 b = __ldcg(kbox + k);
+        int *kb = reinterpret_cast<int *>(kbox + k);
+        if (a0 < b.x) atomicMin(kb, a0);
+        if (-a0 < b.y) atomicMin(kb + 1, -a0);
+        if (b0 < b.z) atomicMin(kb + 2, b0);
+        if (-b0 < b.w) atomicMin(kb + 3, -b0);
+    }
+}
+
+// Outer anchors of a key (and the tile index of its inner anchors).
+template <int D>
+__device__ __forceinline__ void key_anchors(const BinBox &bb, unsigned k, int *oa, int *ob, int &ta, int &tb) {
+    tb = 0;
+    ta = 0;
+    if (D == 2) {
+        tb = (int)(k % (unsigned)bb.tiles_b);
+        k /= (unsigned)bb.tiles_b;
+        ta = (int)(k % (unsigned)bb.tiles_a);
+        k /= (unsigned)bb.tiles_a;
+    }
+#pragma unroll
+    for (int l = D - 2; l >= 0; --l) {
+        ob[l] = (int)(k % (unsigned)bb.KB[l]) + bb.kb_lo[l];
+        k /= (unsigned)bb.KB[l];
+        oa[l] = (int)(k % (unsigned)bb.KA[l]) + bb.ka_lo[l];
+        k /= (unsigned)bb.KA[l];
+    }
+}
+
+// One item per kBinT packets of every bin.
+template <int D>
+__global__ void bin_items_kernel(const int2 *__restrict__ off, const int4 *__restrict__ kbox, const Common c,
+                                 const BinBox bb, BinItem *__restrict__ items) {
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (k >= K) return;
+    if (k >= bb.K) return;
     const int2 o = off[k], o1 = off[k + 1];
     const int n = o1.x - o.x;
-    for (int t = 0; t < o1.y - o.y; ++t)
-        items[o.y + t] = make_int4((int)k, o.x + t * kBinT, min(kBinT, n - t * kBinT), 0);
+    if (n == 0) return;
+    int oa[D - 1], ob[D - 1], ta, tb;
+    key_anchors<D>(bb, (unsigned)k, oa, ob, ta, tb);
+    int4 an;  // inner anchors: first and last a, first and last b (relative to the node box)
+    if constexpr (D == 3) {
+        const int4 b = kbox[k];
+        an = make_int4(b.x, -b.y, b.z, -b.w);
+    } else {
+        an.x = bb.ka_lo[1] - c.amin[1] + ta * kBinTileA;
+        an.y = bb.ka_lo[1] - c.amin[1] + min(bb.KA[1], (ta + 1) * kBinTileA) - 1;
+        an.z = bb.kb_lo[1] - c.bmin[1] + tb * kBinTileB;
+        an.w = bb.kb_lo[1] - c.bmin[1] + min(bb.KB[1], (tb + 1) * kBinTileB) - 1;
+    }
+    BinItem it;
+    const bool inside = an.x + bb.dqmin >= 0 && an.y + bb.dqmax < c.A[D - 1] && an.z + bb.dpmin >= 0 &&
+                        an.w + bb.dpmax < c.B[D - 1];
+    it.box = make_int4(max(0, an.x + bb.dqmin), min(c.A[D - 1] - 1, an.y + bb.dqmax), max(0, an.z + bb.dpmin),
+                       min(c.B[D - 1] - 1, an.w + bb.dpmax));
+    float z[4] = {1.f, 0.f, 1.f, 0.f};
+#pragma unroll
+    for (int l = 0; l < D - 1; ++l) {
+        double t = 0.5 * c.cc * ((double)oa[l] + 0.5);
+        t -= rint(t);
+        sincospif(2.f * (float)t, &z[2 * l + 1], &z[2 * l]);
+    }
+    it.z = make_float4(z[0], z[1], z[2], z[3]);
+    for (int t = 0; t < o1.y - o.y; ++t) {
+        it.at = make_int4((int)k, o.x + t * kBinT, min(kBinT, n - t * kBinT), inside ? 1 : 0);
+        items[o.y + t] = it;
+    }
 }
 
 // Before the scatter: marks every row of W that the packets of an occupied key
@@ -113,15 +316,8 @@ __global__ void bin_mark_rows_kernel(const int *__restrict__ count, const Common
                                      uint8_t *__restrict__ row_flag) {
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k >= bb.K || count[k] == 0) return;
-    int oa[D - 1], ob[D - 1];
-    int64_t kk = k;
-#pragma unroll
-    for (int l = D - 2; l >= 0; --l) {
-        ob[l] = (int)(kk % bb.KB[l]) + bb.kb_lo[l];
-        kk /= bb.KB[l];
-        oa[l] = (int)(kk % bb.KA[l]) + bb.ka_lo[l];
-        kk /= bb.KA[l];
-    }
+    int oa[D - 1], ob[D - 1], ta, tb;
+    key_anchors<D>(bb, (unsigned)k, oa, ob, ta, tb);
     for (int k0 = 0; k0 < c.n1; ++k0) {
         const int ia0 = oa[0] + c.dq[k0] - c.amin[0], ib0 = ob[0] + c.dp[k0] - c.bmin[0];
         if ((unsigned)ia0 >= (unsigned)c.A[0] || (unsigned)ib0 >= (unsigned)c.B[0]) continue;
@@ -139,7 +335,8 @@ __global__ void bin_mark_rows_kernel(const int *__restrict__ count, const Common
 }
 
 // Zeroes the flagged rows of W (row_f4 16-byte words each): a warp reads the
-// flags of 32 consecutive rows at once and clears the flagged ones together.
+// flags of 32 consecutive rows at once and clears its part (blockIdx.y of
+// gridDim.y) of the flagged ones together.
 __global__ void __launch_bounds__(256) clear_flagged_rows_kernel(float4 *__restrict__ W,
                                                                  const uint8_t *__restrict__ row_flag,
                                                                  int64_t rows, int64_t row_f4) {
@@ -149,11 +346,13 @@ __global__ void __launch_bounds__(256) clear_flagged_rows_kernel(float4 *__restr
          base += nwarps * 32) {
         const bool f = base + lane < rows && row_flag[base + lane] != 0;
         unsigned set = __ballot_sync(0xffffffffu, f);
+        const int64_t part = (row_f4 + gridDim.y - 1) / gridDim.y, i0 = blockIdx.y * part;
+        const int64_t i1 = min(row_f4, i0 + part);
         while (set) {
             const int r = __ffs(set) - 1;
             set &= set - 1;
             float4 *p = W + (base + r) * row_f4;
-            for (int64_t i = lane; i < row_f4; i += 32) p[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int64_t i = i0 + lane; i < i1; i += 32) p[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
     }
 }
@@ -172,322 +371,315 @@ __host__ __device__ constexpr int coef_stride() {
 template <int D, int N1>
 __host__ __device__ constexpr int binned_smem_bytes() {
     return kBinT * coef_stride<D, N1>() * 8  // coefficients [packet][dimension][neighbour] (float2)
-           + 2 * kWinCells * 4     // per-cell entry start and cursor (int)
+           + kWinCells * 4         // entries per cell (int)
+           + kWinCells * 4         // per cell: first entry, end of its entries (16 bits each)
            + kWinCells * 4         // active cells (packed line, column)
            + (D == 3 ? N1 * N1 : N1) * 8  // W offsets of the rows (int64)
            + kBinT * N1 * 2;       // entries (packet << 4 | neighbour), uint16
 }
 
-__device__ __forceinline__ int2 block_exclusive_scan(int2 v, int2 *total);
-
 // Binned coefficient + scatter: persistent CTAs take items from *work.  All
 // packets of an item share the outer anchor cell, so they reach the same
 // n1^(d-1) rows, and a target cell of the inner plane receives, in every row,
-// sum over its entries (packet j, inner neighbour k) of
+// the sum over its entries (packet j, inner neighbour k) of
 //   w_j c_{d-1,j}[k] * c_{0,j}[k0] (* c_{1,j}[k1]).
 // Per item (and window of whole inner q-node lines of the target box) the CTA
-// lists every target cell's entries (a CSR built once); then each thread takes
-// a cell (and a pass over part of the k0 values), accumulates those rows of it
-// in registers as a sum of outer products over its entries, and adds each row's
-// value to W with one 8-byte reduction (consecutive threads: consecutive cells
-// of the row).  No floating-point atomics in shared memory.
+// lists every target cell's entries (a CSR built once); then NP lanes per cell
+// accumulate its rows in registers as a sum of outer products over its entries
+// and add each row's value to W with one 8-byte reduction.  No floating-point
+// atomics in shared memory.
+// Bound by the shared-memory pipe and the barriers between the phases of an item
+// (2-D workload: 53 % of the pipe's wavefronts, issue 52 %).  3-D workload
+// (16.8M packets): 7.45 -> 5.73 ms with the FP64 part and the packet gathers in
+// the sort (whose last kernel grew from 0.09 to 0.76 ms), 2-D (4.2M): 1.02 ms
+// per packet -> 0.50 ms.
 template <int D, int N1>
-__global__ void __launch_bounds__(kBinT, kBinCtasPerSm) binned_scatter_kernel(
-    const double *__restrict__ q, const double *__restrict__ p, const double *__restrict__ s,
-    const double *__restrict__ a, int64_t m, const __grid_constant__ Params32 P, const BinBox bb,
-    const int *__restrict__ sorted, const int4 *__restrict__ items, const int2 *__restrict__ off_end,
-    int *__restrict__ work, float2 *__restrict__ W, uint8_t *__restrict__ row_flag) {
-    constexpr int NR = D == 3 ? N1 * N1 : N1;    // rows reached by one outer anchor cell
-    constexpr int NA = (D == 3 && N1 == 8) ? 2 : N1;  // k0 values per accumulation pass
-    constexpr int NK1 = D == 3 ? N1 : 1;         // k1 values
-    constexpr int kPer = kWinCells / kBinT;      // target cells per thread in the CSR build
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+__global__ void __launch_bounds__(kBinT, bin_ctas_per_sm<D>()) binned_scatter_kernel(
+    const __grid_constant__ Params32 P, const __grid_constant__ BinBox bb, const BinRecord *__restrict__ rec,
+    const BinItem *__restrict__ items, const int2 *__restrict__ off_end, int *__restrict__ work,
+    float2 *__restrict__ W) {
+    constexpr int NR = D == 3 ? N1 * N1 : N1;       // rows reached by one outer anchor cell
+    constexpr int NP = D == 3 && N1 == 8 ? 4 : 1;   // lanes per target cell
+    constexpr int NA = N1 / NP;                     // k0 values per lane
+    constexpr int NK1 = D == 3 ? N1 : 2;            // k1 values (d = 2: none)
+    constexpr int kSub = 32 / NP;                   // target cells per warp
+    constexpr int kPer = kWinCells / kBinT;         // target cells per thread in the CSR build
     constexpr int CS = coef_stride<D, N1>();
-    // [kBinT][CS]: per packet [D][N1] coefficients (the last dimension's
-    // multiplied by the packet's weight w) and padding
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    // [kBinT][CS] per packet: pairs of neighbours as (re, re', im, im') for the
+    // outer dimensions (the operands of the packed multiply-adds), (re, im) times
+    // the packet's weight for the last; padding
     float2 *coef = reinterpret_cast<float2 *>(smem_raw);
-    int *cstart = reinterpret_cast<int *>(coef + kBinT * CS);        // [kWinCells]
-    int *cend = cstart + kWinCells;                                  // [kWinCells]
-    unsigned *act = reinterpret_cast<unsigned *>(cend + kWinCells);  // [kWinCells]
-    int64_t *rowoff = reinterpret_cast<int64_t *>(act + kWinCells);  // [NR]
+    int *cnt = reinterpret_cast<int *>(coef + kBinT * CS);             // [kWinCells], zero between windows
+    unsigned *span = reinterpret_cast<unsigned *>(cnt + kWinCells);    // [kWinCells]
+    unsigned *act = span + kWinCells;                                  // [kWinCells]
+    int64_t *rowoff = reinterpret_cast<int64_t *>(act + kWinCells);    // [NR]
     unsigned short *ent = reinterpret_cast<unsigned short *>(rowoff + NR);  // [kBinT * N1]
-    __shared__ int s_item, s_box[4], s_nact;
-    __shared__ int4 s_desc;
-    __shared__ unsigned long long s_rows;  // bit r: row r lies in the node box
+    __shared__ __align__(16) BinItem s_item[2];
+    __shared__ unsigned s_rows[2];  // bit r: row r lies in the node box
+    __shared__ int2 s_sum[kBinT / 32];
     const Common &c = P.c;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int nitems = off_end->y;
-    // thread 0 fetches the next item (index and descriptor) while the CTA
-    // works on the current one
-    int next = 0;
-    int4 next_desc = make_int4(0, 0, 0, 0);
+    // thread 0 fetches the next item (asynchronous copies into shared memory)
+    // while the CTA works on the current one
+    auto fetch = [&](BinItem *to, int i) {
+        if (i < nitems) {
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(to);
+#pragma unroll
+            for (int o = 0; o < (int)sizeof(BinItem); o += 16)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + o),
+                             "l"(reinterpret_cast<const char *>(items + i) + o)
+                             : "memory");
+        } else {
+            to->at = make_int4(0, 0, 0, 0);
+        }
+    };
+    auto fetched = [] { asm volatile("cp.async.wait_all;" ::: "memory"); };
     if (tid == 0) {
-        next = atomicAdd(work, 1);
-        if (next < nitems) next_desc = items[next];
+        fetch(&s_item[0], atomicAdd(work, 1));
+        fetched();
     }
-    for (;;) {
-        __syncthreads();  // the previous item's shared data are no longer read
-        if (tid == 0) {
-            s_item = next;
-            s_desc = next_desc;
-            s_box[0] = s_box[2] = INT_MAX;
-            s_box[1] = s_box[3] = INT_MIN;
-            s_rows = 0ull;
-        }
-        __syncthreads();
-        const int it = s_item;
-        if (it >= nitems) break;
-        const int4 item = s_desc;
-        if (tid == 0) {
-            next = atomicAdd(work, 1);
-            if (next < nitems) next_desc = items[next];
-        }
-        const bool valid = tid < item.z;
-        // the rows of the item's outer anchor cell: W offsets, flags, in-box bits
-        if (tid < NR) {
-            int oa[D - 1], ob[D - 1];
-            int kk = item.x;
-#pragma unroll
-            for (int l = D - 2; l >= 0; --l) {
-                ob[l] = kk % bb.KB[l] + bb.kb_lo[l];
-                kk /= bb.KB[l];
-                oa[l] = kk % bb.KA[l] + bb.ka_lo[l];
-                kk /= bb.KA[l];
-            }
-            const int k0 = D == 3 ? tid / N1 : tid, k1 = D == 3 ? tid % N1 : 0;
-            const int ia0 = oa[0] + c.dq[k0] - c.amin[0], ib0 = ob[0] + c.dp[k0] - c.bmin[0];
-            bool in = (unsigned)ia0 < (unsigned)c.A[0] && (unsigned)ib0 < (unsigned)c.B[0];
-            int64_t idx = (int64_t)ia0 * c.sa[0] + (int64_t)ib0 * c.sb[0];
-            int64_t row = (int64_t)ia0 * c.ra[0] + (int64_t)ib0 * c.rb[0];
-            if constexpr (D == 3) {
-                const int ia1 = oa[1] + c.dq[k1] - c.amin[1], ib1 = ob[1] + c.dp[k1] - c.bmin[1];
-                in = in && (unsigned)ia1 < (unsigned)c.A[1] && (unsigned)ib1 < (unsigned)c.B[1];
-                idx += (int64_t)ia1 * c.sa[1] + (int64_t)ib1 * c.sb[1];
-                row += (int64_t)ia1 * c.ra[1] + (int64_t)ib1 * c.rb[1];
-            }
-            rowoff[tid] = idx;
-            if (in) atomicOr(&s_rows, 1ull << tid);
-        }
-        int ra = 0, rb = 0;  // inner anchor relative to the node box (set by the last dimension)
+    if (tid < 2) s_rows[tid] = 0u;
+    for (int e = tid; e < kWinCells; e += kBinT) cnt[e] = 0;
+    for (int buf = 0;; buf ^= 1) {
+        __syncthreads();  // the item is there; the previous one's shared data are no longer read
+        const int4 at = s_item[buf].at, box = s_item[buf].box;
+        if (at.z == 0) break;
+        int next = 0;
+        if (tid == 0) next = atomicAdd(work, 1);
+        const bool valid = tid < at.z;
+        const int ta0 = box.x, tb0 = box.z, TA = box.y - ta0 + 1, TB = box.w - tb0 + 1;
+        const int WH = TA > 0 && TB > 0 ? kWinCells / TB : 0;  // inner q-node lines per window
         float2 *cj = coef + tid * CS;
-        if (valid) {
-            const int64_t j = sorted[item.y + tid];
-            const double ar = a[j], ai = a[m + j], sj = s[j];
-            double rB = 0.0;
-            float xy = 0.f;
-            // one dimension at a time (one copy of the evaluation) into this
-            // thread's coefficient block; the weight goes with the last
-            // dimension's coefficients, once per packet rather than once per
-            // entry and accumulation pass
-#pragma unroll 1
-            for (int l = 0; l < D; ++l) {
-                int a0, b0;
-                float X, Y, zr, zi, yr = 1.f, yi = 0.f;
-                dim_setup32(c, q[l * m + j], p[l * m + j], a0, b0, X, Y, zr, zi, rB, xy);
-                if (l == D - 1) packet_weight32(c, sj, ar, ai, rB, xy, yr, yi);
-                ra = a0 - c.amin[D - 1];
-                rb = b0 - c.bmin[D - 1];
+        int ra = 0, rb = 0;  // inner anchor relative to the node box
+        // the packet's target cells in the window of lines [wa, wa + wn), without
+        // tests when the whole box is one window inside the node box
+        const bool plain = at.w != 0 && TA <= WH;
+        auto each_entry = [&](int wa, int wn, auto f) {
+            if (plain) {
+                const int e = (ra - ta0) * TB + rb - tb0;
 #pragma unroll
-                for (int o = 0; o < N1 / 4; ++o) {
-                    float er[4], ei[4], vr, vi, hr[2], hi[2];
-                    orbit_coeffs<N1>(P.poly + o * kOrbitTable, X, Y, er, ei);
-                    orbit_phase<N1>(c, o, zr, zi, vr, vi);
-                    cmul(yr, yi, vr, vi, hr[0], hi[0]);
-                    cmul(yr, yi, vr, -vi, hr[1], hi[1]);
-#pragma unroll
-                    for (int g = 0; g < 4; ++g) {
-                        float2 t;
-                        cmul(er[g], ei[g], hr[g & 1], hi[g & 1], t.x, t.y);
-                        cj[l * N1 + 4 * o + g] = t;
-                    }
-                }
-            }
-            atomicMin(&s_box[0], ra + bb.dqmin);
-            atomicMax(&s_box[1], ra + bb.dqmax);
-            atomicMin(&s_box[2], rb + bb.dpmin);
-            atomicMax(&s_box[3], rb + bb.dpmax);
-        }
-        __syncthreads();
-        const unsigned long long rows_in = s_rows;
-        if (tid < NR && ((rows_in >> tid) & 1ull)) {
-            // first-pass rows that receive contributions
-            const int k0 = D == 3 ? tid / N1 : tid, k1 = D == 3 ? tid % N1 : 0;
-            int kk = item.x;
-            int oa[D - 1], ob[D - 1];
-#pragma unroll
-            for (int l = D - 2; l >= 0; --l) {
-                ob[l] = kk % bb.KB[l] + bb.kb_lo[l];
-                kk /= bb.KB[l];
-                oa[l] = kk % bb.KA[l] + bb.ka_lo[l];
-                kk /= bb.KA[l];
-            }
-            int64_t row = (int64_t)(oa[0] + c.dq[k0] - c.amin[0]) * c.ra[0] +
-                          (int64_t)(ob[0] + c.dp[k0] - c.bmin[0]) * c.rb[0];
-            if constexpr (D == 3)
-                row += (int64_t)(oa[1] + c.dq[k1] - c.amin[1]) * c.ra[1] +
-                       (int64_t)(ob[1] + c.dp[k1] - c.bmin[1]) * c.rb[1];
-            row_flag[row] = 1;
-        }
-        const int ta0 = max(0, s_box[0]), ta1 = min(c.A[D - 1] - 1, s_box[1]);
-        const int tb0 = max(0, s_box[2]), tb1 = min(c.B[D - 1] - 1, s_box[3]);
-        const int TA = ta1 - ta0 + 1, TB = tb1 - tb0 + 1;
-        if (TA <= 0 || TB <= 0 || rows_in == 0ull) continue;  // nothing lands in the node box
-        const int WH = kWinCells / TB;  // inner q-node lines per window
-        if (WH == 0) {
-            // a b-range wider than a window: one reduction per contribution
-            if (valid) {
-                float cr[N1], ci[N1];
-#pragma unroll
-                for (int k = 0; k < N1; ++k) {
-                    const float2 v = cj[(D - 1) * N1 + k];
-                    cr[k] = v.x;
-                    ci[k] = v.y;
-                }
-#pragma unroll 1
-                for (int r = 0; r < NR; ++r) {
-                    if (!((rows_in >> r) & 1ull)) continue;
-                    const int k0 = D == 3 ? r / N1 : r, k1 = D == 3 ? r % N1 : 0;
-                    const float2 c0 = cj[k0];  // w is in cr, ci
-                    float pr = c0.x, pi = c0.y;
-                    if constexpr (D == 3) {
-                        const float2 c1 = cj[N1 + k1];
-                        cmul(pr, pi, c1.x, c1.y, pr, pi);
-                    }
-                    emit_row<D - 1, N1>(W, c, ra + c.amin[D - 1], rb + c.bmin[D - 1], cr, ci, rowoff[r], pr, pi);
-                }
-            }
-            continue;
-        }
-        const int nwin = (TA + WH - 1) / WH;
-#pragma unroll 1
-        for (int w = 0; w < nwin; ++w) {
-            const int wa = w * WH, wn = min(WH, TA - wa), cells = wn * TB;
-            // --- entries of this window: count, scan, fill ---------------------
-            __syncthreads();  // the previous window's lists are no longer read
-            for (int e = tid; e < cells; e += kBinT) cend[e] = 0;
-            __syncthreads();
-            if (valid) {
+                for (int k = 0; k < N1; ++k) f(k, e + c.dq[k] * TB + c.dp[k]);
+            } else {
 #pragma unroll
                 for (int k = 0; k < N1; ++k) {
                     const int ia = ra + c.dq[k] - ta0 - wa, ib = rb + c.dp[k] - tb0;
-                    if ((unsigned)ia < (unsigned)wn && (unsigned)ib < (unsigned)TB) atomicAdd(&cend[ia * TB + ib], 1);
+                    if ((unsigned)ia < (unsigned)wn && (unsigned)ib < (unsigned)TB) f(k, ia * TB + ib);
                 }
             }
-            __syncthreads();
+        };
+        if (valid) {
+            const BinRecord *r = rec + at.y + tid;
+            const float4 x = r->x, w = r->w, y = r->y, z = s_item[buf].z;
+            ra = __float_as_int(y.x);
+            rb = __float_as_int(y.y);
+            if (WH > 0) each_entry(0, min(WH, TA), [&](int, int e) { atomicAdd(&cnt[e], 1); });
+            // one dimension at a time (one copy of the evaluation: two would keep
+            // its constants in registers)
+#pragma unroll 1
+            for (int l = 0; l < D; ++l) {
+                const bool last = l == D - 1;
+                float *cl = reinterpret_cast<float *>(cj + l * N1);
+                coeff_dim32<N1>(P, 2.f * (last ? x.z : l == 0 ? x.x : y.z), 2.f * (last ? x.w : l == 0 ? x.y : y.w),
+                                last ? w.z : l == 0 ? z.x : z.z, last ? w.w : l == 0 ? z.y : z.w,
+                                last ? w.x : 1.f, last ? w.y : 0.f, [&](int k, float re, float im) {
+                                    const int b = 4 * (k >> 1) + (k & 1);
+                                    cl[last ? 2 * k : b] = re;
+                                    cl[last ? 2 * k + 1 : b + 2] = im;
+                                });
+            }
+        }
+        // the rows of the item's outer anchor cell: W offsets and in-box bits
+        if (tid < (NR + 31) / 32 * 32) {
+            bool in = tid < NR;
+            if (in) {
+                int oa[D - 1], ob[D - 1], ta, tb;
+                key_anchors<D>(bb, (unsigned)at.x, oa, ob, ta, tb);
+                const int k0 = D == 3 ? tid / N1 : tid, k1 = D == 3 ? tid % N1 : 0;
+                const int ia0 = oa[0] + c.dq[k0] - c.amin[0], ib0 = ob[0] + c.dp[k0] - c.bmin[0];
+                in = (unsigned)ia0 < (unsigned)c.A[0] && (unsigned)ib0 < (unsigned)c.B[0];
+                int64_t idx = (int64_t)ia0 * c.sa[0] + (int64_t)ib0 * c.sb[0];
+                if constexpr (D == 3) {
+                    const int ia1 = oa[1] + c.dq[k1] - c.amin[1], ib1 = ob[1] + c.dp[k1] - c.bmin[1];
+                    in = in && (unsigned)ia1 < (unsigned)c.A[1] && (unsigned)ib1 < (unsigned)c.B[1];
+                    idx += (int64_t)ia1 * c.sa[1] + (int64_t)ib1 * c.sb[1];
+                }
+                rowoff[tid] = idx;
+            }
+            const unsigned bits = __ballot_sync(0xffffffffu, in);
+            if (lane == 0) s_rows[wid] = bits;
+        }
+        __syncthreads();
+        if (tid == 0) fetch(&s_item[buf ^ 1], next);
+        const unsigned long long rows_in = s_rows[0] | (unsigned long long)s_rows[1] << 32;
+        if (TA > 0 && TB > 0 && WH == 0 && valid) {
+            // a b-range wider than a window: one reduction per contribution
+            float cr[N1], ci[N1];
+#pragma unroll
+            for (int k = 0; k < N1; ++k) {
+                const float2 v = cj[(D - 1) * N1 + k];
+                cr[k] = v.x;
+                ci[k] = v.y;
+            }
+#pragma unroll 1
+            for (int r = 0; r < NR; ++r) {
+                if (!((rows_in >> r) & 1ull)) continue;
+                const int k0 = D == 3 ? r / N1 : r, k1 = D == 3 ? r % N1 : 0;
+                const float *c0 = reinterpret_cast<const float *>(cj) + 4 * (k0 >> 1) + (k0 & 1);
+                float pr = c0[0], pi = c0[2];  // the weight is in cr, ci
+                if constexpr (D == 3) {
+                    const float *c1 = reinterpret_cast<const float *>(cj + N1) + 4 * (k1 >> 1) + (k1 & 1);
+                    float tr, ti;
+                    cmul(pr, pi, c1[0], c1[2], tr, ti);
+                    pr = tr;
+                    pi = ti;
+                }
+                emit_row<D - 1, N1>(W, c, ra + c.amin[D - 1], rb + c.bmin[D - 1], cr, ci, rowoff[r], pr, pi);
+            }
+        }
+        const int nwin = WH > 0 && rows_in != 0ull ? (TA + WH - 1) / WH : 0;
+        if (nwin == 0 && WH > 0)  // nothing lands in the node box: drop the counts
+            for (int e = tid; e < kWinCells; e += kBinT) cnt[e] = 0;
+#pragma unroll 1
+        for (int w = 0; w < nwin; ++w) {
+            const int wa = w * WH, wn = min(WH, TA - wa), cells = wn * TB;
+            if (w > 0) {
+                __syncthreads();  // the previous window's lists are no longer read
+                if (valid) each_entry(wa, wn, [&](int, int e) { atomicAdd(&cnt[e], 1); });
+                __syncthreads();
+            }
+            // --- entry starts and the ordered list of non-empty cells by one block
+            // scan over the counts (thread t: cells [t kPer, (t + 1) kPer)) --------
+            int nact;
             {
-                // thread t owns cells [t kPer, (t + 1) kPer): entry starts and the
-                // ordered list of non-empty cells by one block scan
-                int cnt[kPer];
+                int n[kPer];
                 int2 loc = make_int2(0, 0);
+                const int4 v = *reinterpret_cast<const int4 *>(cnt + tid * kPer);
+                static_assert(kPer == 4, "one 16-byte load of counts per thread");
+                n[0] = v.x;
+                n[1] = v.y;
+                n[2] = v.z;
+                n[3] = v.w;
+                *reinterpret_cast<int4 *>(cnt + tid * kPer) = make_int4(0, 0, 0, 0);
 #pragma unroll
                 for (int i = 0; i < kPer; ++i) {
-                    const int e = tid * kPer + i;
-                    cnt[i] = e < cells ? cend[e] : 0;
-                    loc.x += cnt[i];
-                    loc.y += cnt[i] > 0;
+                    loc.x += n[i];
+                    loc.y += n[i] > 0;
                 }
-                int2 tot;
-                int2 base = block_exclusive_scan(loc, &tot);
+                int2 inc = loc;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int ux = __shfl_up_sync(0xffffffffu, inc.x, o), uy = __shfl_up_sync(0xffffffffu, inc.y, o);
+                    if (lane >= o) {
+                        inc.x += ux;
+                        inc.y += uy;
+                    }
+                }
+                if (lane == 31) s_sum[wid] = inc;
+                __syncthreads();
+                int2 base = make_int2(inc.x - loc.x, inc.y - loc.y);
+                nact = 0;
+#pragma unroll
+                for (int i = 0; i < kBinT / 32; ++i) {
+                    const int2 v2 = s_sum[i];
+                    if (i < wid) {
+                        base.x += v2.x;
+                        base.y += v2.y;
+                    }
+                    nact += v2.y;
+                }
 #pragma unroll
                 for (int i = 0; i < kPer; ++i) {
                     const int e = tid * kPer + i;
                     if (e < cells) {
-                        cstart[e] = base.x;
-                        cend[e] = base.x;  // cursor of the fill below
-                        if (cnt[i] > 0) {
+                        span[e] = (unsigned)base.x * 0x10001u;  // first entry, cursor of the fill below
+                        if (n[i] > 0) {
                             const int ia = e / TB, ib = e - ia * TB;
                             act[base.y++] = ((unsigned)ia << 16) | (unsigned)ib;
                         }
-                        base.x += cnt[i];
-                    }
-                }
-                if (tid == 0) s_nact = tot.y;
-            }
-            __syncthreads();
-            if (valid) {
-#pragma unroll
-                for (int k = 0; k < N1; ++k) {
-                    const int ia = ra + c.dq[k] - ta0 - wa, ib = rb + c.dp[k] - tb0;
-                    if ((unsigned)ia < (unsigned)wn && (unsigned)ib < (unsigned)TB) {
-                        const int pos = atomicAdd(&cend[ia * TB + ib], 1);
-                        ent[pos] = (unsigned short)((tid << 4) | k);
+                        base.x += n[i];
                     }
                 }
             }
             __syncthreads();
-            const int nact = s_nact;
+            if (valid)
+                each_entry(wa, wn, [&](int k, int e) {
+                    ent[atomicAdd(&span[e], 0x10000u) >> 16] = (unsigned short)((tid << 4) | k);
+                });
+            __syncthreads();
             // --- cells: rows in registers, then one reduction per row ----------
-            // work unit = (pass kp over NA values of k0, cell); consecutive
-            // threads take consecutive cells of one pass (coalesced reductions)
-            constexpr int NP = N1 / NA;
-            for (int u0 = tid; u0 < nact * NP; u0 += kBinT) {
-                const int kp = u0 / nact, i = u0 - kp * nact;
+            // A warp takes kSub consecutive cells; its NP lanes per cell share out
+            // the k0 values, so they walk the same entries and a warp waits for
+            // the longest of kSub lists instead of 32.
+            const int kp = lane % NP;
+            for (int g0 = wid * kSub; g0 < nact; g0 += kBinT / 32 * kSub) {
+                const int i = g0 + lane / NP;
+                if (i >= nact) continue;
                 const unsigned cell = act[i];
                 const int ia = (int)(cell >> 16), ib = (int)(cell & 0xffffu);
-                const int e = ia * TB + ib;
-                const int x0 = cstart[e], x1 = cend[e];
+                const unsigned sp = span[ia * TB + ib];
+                const int x0 = (int)(sp & 0xffffu), x1 = (int)(sp >> 16);
                 float2 *Wc = W + (int64_t)(ta0 + wa + ia) * c.sa[D - 1] + tb0 + ib;
-                float accr[NA][NK1], acci[NA][NK1];
+                // pairs of k1 (d = 3) or of k0 (d = 2)
+                constexpr int NU = D == 3 ? NA : 1, NV = D == 3 ? NK1 / 2 : NA / 2;
+                float2 accr[NU][NV], acci[NU][NV];
 #pragma unroll
-                for (int u = 0; u < NA; ++u)
+                for (int u = 0; u < NU; ++u)
 #pragma unroll
-                    for (int v = 0; v < NK1; ++v) accr[u][v] = acci[u][v] = 0.f;
-                for (int x = x0; x < x1; ++x) {
-                    const int en = ent[x], jj = en >> 4, kk = en & 15;
+                    for (int v = 0; v < NV; ++v) accr[u][v] = acci[u][v] = both(0.f);
+                for (int xe = x0; xe < x1; ++xe) {
+                    const int en = ent[xe], jj = en >> 4, kk = en & 15;
                     const float2 ev = coef[jj * CS + (D - 1) * N1 + kk];  // w c_{d-1}[k]
-                    // the packet's coefficients, 16-byte loads (two neighbours each)
                     const float4 *cp4 = reinterpret_cast<const float4 *>(coef + jj * CS);
-                    float2 c0v[NA];
-#pragma unroll
-                    for (int u = 0; u < NA; u += 2) {
-                        const float4 t = cp4[(kp * NA + u) / 2];
-                        c0v[u] = make_float2(t.x, t.y);
-                        c0v[u + 1] = make_float2(t.z, t.w);
-                    }
-                    float2 c1v[NK1];
+                    float2 tr[NA / 2], ti[NA / 2];  // pairs of k0 (d = 3)
                     if constexpr (D == 3) {
 #pragma unroll
-                        for (int v = 0; v < NK1; v += 2) {
-                            const float4 t = cp4[(N1 + v) / 2];
-                            c1v[v] = make_float2(t.x, t.y);
-                            c1v[v + 1] = make_float2(t.z, t.w);
+                        for (int u = 0; u < NA / 2; ++u) {
+                            const float4 t = cp4[kp * (NA / 2) + u];
+                            const float2 re = make_float2(t.x, t.y), im = make_float2(t.z, t.w);
+                            tr[u] = fma2(both(ev.x), re, mul2(both(-ev.y), im));
+                            ti[u] = fma2(both(ev.x), im, mul2(both(ev.y), re));
                         }
                     }
 #pragma unroll
-                    for (int u = 0; u < NA; ++u) {
-                        float tr, ti;
-                        cmul(ev.x, ev.y, c0v[u].x, c0v[u].y, tr, ti);
-                        if constexpr (D == 3) {
+                    for (int v = 0; v < NV; ++v) {
+                        const float4 t = cp4[D == 3 ? N1 / 2 + v : v];
+                        const float2 re = make_float2(t.x, t.y), im = make_float2(t.z, t.w);
 #pragma unroll
-                            for (int v = 0; v < NK1; ++v) {
-                                accr[u][v] = fmaf(tr, c1v[v].x, fmaf(-ti, c1v[v].y, accr[u][v]));
-                                acci[u][v] = fmaf(tr, c1v[v].y, fmaf(ti, c1v[v].x, acci[u][v]));
+                        for (int u = 0; u < NU; ++u) {
+                            float ur = ev.x, ui = ev.y;
+                            if constexpr (D == 3) {
+                                ur = u & 1 ? tr[u / 2].y : tr[u / 2].x;
+                                ui = u & 1 ? ti[u / 2].y : ti[u / 2].x;
                             }
-                        } else {
-                            accr[u][0] += tr;
-                            acci[u][0] += ti;
+                            accr[u][v] = fma2(both(ur), re, fma2(both(-ui), im, accr[u][v]));
+                            acci[u][v] = fma2(both(ur), im, fma2(both(ui), re, acci[u][v]));
                         }
                     }
                 }
 #pragma unroll
-                for (int u = 0; u < NA; ++u)
+                for (int u = 0; u < NU; ++u)
 #pragma unroll
-                    for (int v = 0; v < NK1; ++v) {
-                        const int r = (kp * NA + u) * NK1 + v;
-                        if ((rows_in >> r) & 1ull) atomicAdd(Wc + rowoff[r], make_float2(accr[u][v], acci[u][v]));
+                    for (int v = 0; v < 2 * NV; ++v) {
+                        const int r = D == 3 ? (kp * NA + u) * NK1 + v : v;
+                        const float2 ar = accr[u][v / 2], ai = acci[u][v / 2];
+                        if ((rows_in >> r) & 1ull)
+                            atomicAdd(Wc + rowoff[r], v & 1 ? make_float2(ar.y, ai.y) : make_float2(ar.x, ai.x));
                     }
             }
         }
+        if (tid == 0) fetched();
     }
 }
 
-// Exclusive scan of (binned packets, items) per key: a cell with at least
-// min_count packets is binned (its packets and ceil(n / kBinT) items count),
-// other cells count zero.  off[K] receives the totals.
-__device__ __forceinline__ int2 bin_pair(const int *count, int64_t k, int64_t K, int min_count) {
+// Exclusive scan of (binned packets, items) per key: a bin with at least
+// kBinMinCount packets counts its packets and ceil(n / kBinT) items, other bins
+// count zero.  off[K] receives the totals.
+__device__ __forceinline__ int2 bin_pair(const int *count, int64_t k, int64_t K) {
     if (k >= K) return make_int2(0, 0);
     const int n = count[k];
-    return n >= min_count ? make_int2(n, (n + kBinT - 1) / kBinT) : make_int2(0, 0);
+    return n >= kBinMinCount ? make_int2(n, (n + kBinT - 1) / kBinT) : make_int2(0, 0);
 }
 
 __device__ __forceinline__ int2 block_exclusive_scan(int2 v, int2 *total) {
@@ -523,11 +715,11 @@ __device__ __forceinline__ int2 block_exclusive_scan(int2 v, int2 *total) {
     return make_int2(before.x + x.x - v.x, before.y + x.y - v.y);
 }
 
-__global__ void __launch_bounds__(1024) bin_scan1_kernel(const int *__restrict__ count, int64_t K, int min_count,
+__global__ void __launch_bounds__(1024) bin_scan1_kernel(const int *__restrict__ count, int64_t K,
                                                          int2 *__restrict__ off, int2 *__restrict__ bsum) {
     const int64_t k = blockIdx.x * (int64_t)1024 + threadIdx.x;
     int2 tot;
-    const int2 e = block_exclusive_scan(bin_pair(count, k, K, min_count), &tot);
+    const int2 e = block_exclusive_scan(bin_pair(count, k, K), &tot);
     if (k < K) off[k] = e;
     if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
 }
@@ -559,8 +751,8 @@ __global__ void __launch_bounds__(1024) bin_scan3_kernel(int2 *__restrict__ off,
     off[k] = v;
 }
 
-// The binned scatter of d >= 2 (FP32): binning, items, then the binned
-// kernel and the per-packet kernel over the loose list, all on stream st.
+// The binned scatter (FP32): binning, records and items, then the binned kernel
+// and the per-packet kernel over the loose list, all on stream st.
 template <int D, int N1>
 fgr_status launch_binned_d(const BinLaunch &L, cudaStream_t st, const PacketsDev &pk, const Params32 &P, void *W,
                            uint8_t *flags, StageMarks *marks) {
@@ -568,26 +760,31 @@ fgr_status launch_binned_d(const BinLaunch &L, cudaStream_t st, const PacketsDev
     const BinBuffers &b = L.buf;
     FGR_CUDA_TRY(cudaMemsetAsync(b.count, 0, sizeof(int) * (size_t)K, st));
     FGR_CUDA_TRY(cudaMemsetAsync(b.ctr, 0, sizeof(int) * 4, st));
-    const unsigned pblocks = (unsigned)((m + 255) / 256);
-    bin_key_kernel<D><<<pblocks, 256, 0, st>>>(pk.q, pk.p, pk.a, m, P.c, L.box, b.key, b.count);
-    if (L.clear_rows > 0) {  // the caller cleared the row flags, not W
-        bin_mark_rows_kernel<D><<<(unsigned)((K + 255) / 256), 256, 0, st>>>(b.count, P.c, L.box, flags);
-        clear_flagged_rows_kernel<<<(unsigned)(L.num_sms * 8), 256, 0, st>>>((float4 *)W, flags, L.clear_rows,
-                                                                          L.row_cells / 2);
-    }
+    if (D == 3) FGR_CUDA_TRY(cudaMemsetAsync(b.kbox, 0x7f, sizeof(int4) * (size_t)K, st));
+    const unsigned pblocks = (unsigned)((m + 255) / 256), kblocks = (unsigned)((K + 255) / 256);
+    bin_key_kernel<D><<<pblocks, 256, 0, st>>>(pk.q, pk.p, pk.a, m, P.c, L.box, b.key, b.rank, b.count);
+    bin_mark_rows_kernel<D><<<kblocks, 256, 0, st>>>(b.count, P.c, L.box, flags);
+    // about 64 warps per SM: few long rows (d = 2: 5,796 of 37 KB) are cut into
+    // parts (139 us with one warp per 32 rows, 19 us so), many short ones not
+    const int64_t warps = (L.rows + 31) / 32, row_f4 = L.row_cells / 2;
+    const int64_t parts = std::max<int64_t>(1, std::min<int64_t>((int64_t)L.num_sms * 64 / warps, (row_f4 + 31) / 32));
+    const dim3 cgrid((unsigned)std::min<int64_t>((warps + 7) / 8, (int64_t)L.num_sms * 8),
+                     (unsigned)std::min<int64_t>(parts, 65535));
+    clear_flagged_rows_kernel<<<cgrid, 256, 0, st>>>((float4 *)W, flags, L.rows, row_f4);
     const int64_t nblk = (K + 1023) / 1024;
-    bin_scan1_kernel<<<(unsigned)nblk, 1024, 0, st>>>(b.count, K, L.min_count, b.off, b.bsum);
+    bin_scan1_kernel<<<(unsigned)nblk, 1024, 0, st>>>(b.count, K, b.off, b.bsum);
     bin_scan2_kernel<<<1, 1024, 0, st>>>(b.bsum, nblk, b.off, K);
     bin_scan3_kernel<<<(unsigned)nblk, 1024, 0, st>>>(b.off, K, b.bsum);
-    bin_place_kernel<<<pblocks, 256, 0, st>>>(b.key, m, b.off, b.count, b.sorted, b.loose, b.ctr);
-    bin_items_kernel<<<(unsigned)((K + 255) / 256), 256, 0, st>>>(b.off, K, b.items);
+    bin_place_kernel<D><<<pblocks, 256, 0, st>>>(pk.q, pk.p, pk.s, pk.a, m, P.c, L.split, b.key, b.rank, b.off, b.rec,
+                                                 b.kbox, b.loose, b.ctr);
+    bin_items_kernel<D><<<kblocks, 256, 0, st>>>(b.off, b.kbox, P.c, L.box, b.items);
     FGR_CUDA_TRY(cudaGetLastError());
     if (marks) marks->binned();
     constexpr int smem = binned_smem_bytes<D, N1>();
     FGR_CUDA_TRY(cudaFuncSetAttribute(binned_scatter_kernel<D, N1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       smem));
-    binned_scatter_kernel<D, N1><<<(unsigned)(L.num_sms * kBinCtasPerSm), kBinT, smem, st>>>(
-        pk.q, pk.p, pk.s, pk.a, m, P, L.box, b.sorted, b.items, b.off + K, b.ctr + 1, (float2 *)W, flags);
+    binned_scatter_kernel<D, N1><<<(unsigned)(L.num_sms * bin_ctas_per_sm<D>()), kBinT, smem, st>>>(
+        P, L.box, b.rec, b.items, b.off + K, b.ctr + 1, (float2 *)W);
     constexpr int T = coeff_threads<false, N1>();
     coeff_scatter_list_kernel<D, false, N1><<<(unsigned)(L.num_sms * 4), T, 0, st>>>(
         pk.q, pk.p, pk.s, pk.a, m, P, W, flags, b.loose, b.ctr);

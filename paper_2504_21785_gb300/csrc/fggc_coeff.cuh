@@ -138,16 +138,16 @@ __device__ __forceinline__ void packet_weight32(const Common &c, double s, doubl
 
 // Parity part (PX, PY) of a surrogate polynomial over X^PX Y^PY, in powers of
 // xx = X^2 and yy = Y^2 (Horner; the terms of total degree surrogate_total).
+// One multiply-add per coefficient, which it reads from the constant bank; the
+// packed form (real and imaginary part at once) needs them in registers.
 template <int N1, int PX, int PY>
 __device__ __forceinline__ float parity_part(const float *C, float xx, float yy) {
     constexpr int T = surrogate_total<N1>();
     float r = 0.f;
 #pragma unroll
     for (int i = kPow - 1; i >= 0; --i) {
-        constexpr int none = -1;
-        const int left = T - 2 * i - PX - PY;
-        const int jtop = left < 0 ? none : (left / 2 < kPow - 1 ? left / 2 : kPow - 1);
-        float u = jtop >= 0 ? C[i * kPow + jtop] : 0.f;
+        const int jtop = (T - 2 * i - PX - PY) / 2 < kPow - 1 ? (T - 2 * i - PX - PY) / 2 : kPow - 1;
+        float u = C[i * kPow + jtop];
 #pragma unroll
         for (int j = kPow - 1; j >= 0; --j)
             if (j < jtop) u = fmaf(u, yy, C[i * kPow + j]);
@@ -156,29 +156,22 @@ __device__ __forceinline__ float parity_part(const float *C, float xx, float yy)
     return r;
 }
 
-// The coefficients e of one orbit's four neighbours (orbit order, Lsa::order).
+// f(X, Y), f(X, -Y), f(-X, Y), f(-X, -Y) of one orbit's polynomial: its four
+// coefficients up to the conjugation of the middle two.
 template <int N1>
-__device__ __forceinline__ void orbit_coeffs(const float *C, float X, float Y, float *er, float *ei) {
+__device__ __forceinline__ void orbit_values(const float *C, float X, float Y, float2 *f) {
+    static_assert(surrogate_total<N1>() >= 2 * kPow, "every power of X^2 has a term");
     constexpr int kPart = kPow * kPow;
     const float xx = X * X, yy = Y * Y, xy = X * Y;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {  // real, imaginary part of f
+    for (int h = 0; h < 2; ++h) {  // real, imaginary part
         const float *H = C + h * 4 * kPart;
         const float ee = parity_part<N1, 0, 0>(H, xx, yy), oe = X * parity_part<N1, 1, 0>(H + kPart, xx, yy);
         const float eo = parity_part<N1, 0, 1>(H + 2 * kPart, xx, yy), oo = parity_part<N1, 1, 1>(H + 3 * kPart, xx, yy);
         const float p = fmaf(xy, oo, ee), n = fmaf(-xy, oo, ee), m = fmaf(Y, eo, oe), o = fmaf(-Y, eo, oe);
-        // f(X, Y), f(X, -Y), f(-X, Y), f(-X, -Y); the middle two conjugated
-        if (h == 0) {
-            er[0] = p + m;
-            er[1] = n + o;
-            er[2] = n - o;
-            er[3] = p - m;
-        } else {
-            ei[0] = p + m;
-            ei[1] = -n - o;
-            ei[2] = o - n;
-            ei[3] = p - m;
-        }
+        const float v[4] = {p + m, n + o, n - o, p - m};
+#pragma unroll
+        for (int g = 0; g < 4; ++g) (h == 0 ? f[g].x : f[g].y) = v[g];
     }
 }
 
@@ -194,16 +187,25 @@ __device__ __forceinline__ void orbit_phase(const Common &c, int o, float zr, fl
     }
 }
 
-// All coefficients of one dimension, times the phases that depend on the neighbour.
-template <int N1, class PT>
-__device__ __forceinline__ void coeff_dim32(const PT &P, float X, float Y, float zr, float zi, float *cr, float *ci) {
+// All coefficients of one dimension, times the phases that depend on the
+// neighbour and a factor (yr, yi): out(k, re, im).
+template <int N1, class PT, class Out>
+__device__ __forceinline__ void coeff_dim32(const PT &P, float X, float Y, float zr, float zi, float yr, float yi,
+                                            Out out) {
 #pragma unroll
     for (int o = 0; o < N1 / 4; ++o) {
-        float er[4], ei[4], vr, vi;
-        orbit_coeffs<N1>(P.poly + o * kOrbitTable, X, Y, er, ei);
+        float2 f[4];
+        float vr, vi, hr[2], hi[2];
+        orbit_values<N1>(P.poly + o * kOrbitTable, X, Y, f);
         orbit_phase<N1>(P.c, o, zr, zi, vr, vi);
+        cmul(yr, yi, vr, vi, hr[0], hi[0]);
+        cmul(yr, yi, vr, -vi, hr[1], hi[1]);
 #pragma unroll
-        for (int g = 0; g < 4; ++g) cmul(er[g], ei[g], vr, (g & 1) ? -vi : vi, cr[4 * o + g], ci[4 * o + g]);
+        for (int g = 0; g < 4; ++g) {
+            float re, im;
+            cmul(f[g].x, g == 1 || g == 2 ? -f[g].y : f[g].y, hr[g & 1], hi[g & 1], re, im);
+            out(4 * o + g, re, im);
+        }
     }
 }
 
@@ -264,7 +266,10 @@ __device__ __forceinline__ void coeff_scatter_body(const double *__restrict__ q,
         } else {
             float X, Y, zr, zi;
             dim_setup32(c, q[l * m + j], p[l * m + j], a0[l], b0[l], X, Y, zr, zi, rB, xy);
-            coeff_dim32<N1>(P, X, Y, zr, zi, cr, ci);
+            coeff_dim32<N1>(P, X, Y, zr, zi, 1.f, 0.f, [&](int k, float re, float im) {
+                cr[k] = re;
+                ci[k] = im;
+            });
         }
         if (l < D - 1) {
 #pragma unroll

@@ -48,53 +48,86 @@ struct FggcBuffers {
     uint8_t *flags = nullptr;
     int2 *brange = nullptr;
     void *tables = nullptr;  // per-pass tables (node windows, point phases, tile bands)
-    void *bin = nullptr;     // binning buffers of the 3-D FP32 scatter (NULL: per-packet scatter)
-    int64_t bin_m = 0;       // packets the binning buffers hold
+    void *bin = nullptr;     // binning buffers of the FP32 scatter, d >= 2 (NULL: per-packet scatter)
+    size_t bin_bytes = 0;    // bytes of the binning buffers
     unsigned long long *terms = nullptr;  // node-point terms of the passes (timed calls only)
     void *fft = nullptr;      // DFT lines of the commensurate grid stage (box.fft_elems complex)
     void *twiddle = nullptr;  // e^{2 pi i j / N}, j < N / 2 <= 4096 (complex)
 };
 
-// Binning of the 3-D scatter (fggc_bin.cuh): key box of the outer anchor
-// cells (a0, b0) of dimensions 0..d-2 whose neighbours can reach the node box,
-// key = row-major index over (a0_0, b0_0, a0_1, b0_1).
+// Binning of the FP32 scatter (fggc_bin.cuh).  A packet's key is the row-major
+// index over its outer anchor (a0, b0) of dimensions 0..d-2, restricted to the
+// anchors whose neighbours can reach the node box, and the kBinTileA x kBinTileB
+// tile of its inner anchor (dimension d-1; d = 3: one tile).
 struct BinBox {
-    int ka_lo[2] = {}, KA[2] = {1, 1}, kb_lo[2] = {}, KB[2] = {1, 1};
+    int ka_lo[3] = {}, KA[3] = {1, 1, 1}, kb_lo[3] = {}, KB[3] = {1, 1, 1};  // anchors per dimension
+    int tiles_a = 1, tiles_b = 1;
     int dqmin = 0, dqmax = 0, dpmin = 0, dpmax = 0;  // neighbour shift ranges
     int64_t K = 0;                                   // keys
+};
+
+// Constants of a packet's record as unevaluated FP32 sums (see split_double).
+struct SplitConst {
+    float inv_dq[2], inv_dp[2], cc[2], half_cc[2], inv_2pi_eps[2], pref[2];
+};
+
+// A binned packet: per dimension the offsets (sx, ty) from its cell centre, the
+// weight with the neighbour-independent phase, e^{i cq cp A / 2} of the inner
+// dimension and the inner anchor relative to the node box.
+struct BinRecord {
+    float4 x;  // sx, ty of dimension 0, then of the last
+    float4 w;  // weight, z of the last dimension
+    float4 y;  // inner anchor (two ints), then sx, ty of dimension 1 (d = 3)
+};
+
+// Up to kBinT packets of one key: first record, packets, the inner target box
+// [ta0, ta1] x [tb0, tb1] in the node box, and z of the outer dimensions.
+struct BinItem {
+    int4 at;   // key, first record, packets, 0
+    int4 box;  // ta0, ta1, tb0, tb1
+    float4 z;  // dimension 0, dimension 1
 };
 
 // Device buffers of the binning (m packets, K keys).
 struct BinBuffers {
     int *key = nullptr;     // [m] key of each packet (-1: adds nothing)
-    int *count = nullptr;   // [K] packets per key, then the placement cursor
-    int2 *off = nullptr;    // [K + 1] (first sorted packet, first item) per key; totals at K
-    int2 *bsum = nullptr;   // [ceil(K / 1024)] block totals of the scan
-    int *sorted = nullptr;  // [m] binned packets by key
+    int *rank = nullptr;    // [m] place of the packet within its key
     int *loose = nullptr;   // [m] packets of small cells
-    int4 *items = nullptr;  // [max items] (key, first sorted packet, packets)
+    BinRecord *rec = nullptr;  // [m] records of the binned packets, by key
+    int *count = nullptr;   // [K] packets per key
+    int4 *kbox = nullptr;   // [K] min a, min -a, min b, min -b of the inner anchors per key
+    int2 *off = nullptr;    // [K + 1] (first record, first item) per key; totals at K
+    int2 *bsum = nullptr;   // [ceil(K / 1024)] block totals of the scan
+    BinItem *items = nullptr;  // [max items]
     int *ctr = nullptr;     // [4] loose count, work counter
 };
 
 struct BinLaunch {
     BinBox box;
     BinBuffers buf;
-    int min_count = 8;   // smallest binned cell (kBinMinCount)
+    SplitConst split;
     int num_sms = 1;
-    // rows of W (each row_cells cells) to clear before the scatter: only the
-    // rows the binned packets reach are marked and zeroed (0: W is cleared by
-    // the caller)
-    int64_t clear_rows = 0;
+    // rows of W (each row_cells cells): only the rows that binned packets reach
+    // are marked and zeroed
+    int64_t rows = 0;
     int64_t row_cells = 0;
 };
 
 // Largest key box of the binned scatter; larger boxes use the per-packet kernel.
 constexpr int64_t kMaxBinKeys = int64_t(1) << 26;
-// Smallest binned cell (packets); smaller cells take the per-packet kernel.
+// Smallest bin (packets); smaller ones take the per-packet kernel.
 constexpr int kBinMinCount = 8;
+// d = 2: inner anchors per tile.  Larger tiles repeat fewer target cells at their
+// edges, smaller ones give items that one CTA takes whole; at the flow's density
+// of one packet per cell 24 x 16, 20 x 12 and 32 x 16 measured the same (2-D
+// workload 1.37 ms), 16 x 12 1.43, 12 x 12 1.48 and 8 x 8 1.77 ms.
+constexpr int kBinTileA = 24, kBinTileB = 16;
+// d = 2: the fewest packets.  The binning's launches take about 40 us, the
+// per-packet kernel 0.25 us per 1024 packets and the binned one half of that.
+constexpr int64_t kBinMinPackets2d = 1 << 17;
 
-// Key box of a node box (false when the binned scatter does not apply).
-bool make_bin_box(const FggcBox &box, int d, BinBox *bb);
+// Key box of a node box and m packets (false when the binned scatter does not apply).
+bool make_bin_box(const FggcBox &box, int d, int64_t m, BinBox *bb);
 // Bytes of the binning buffers for m packets and key box bb.
 size_t bin_buffer_bytes(int64_t m, const BinBox &bb);
 // Carves the binning buffers out of one device block of bin_buffer_bytes.
@@ -176,12 +209,12 @@ fgr_status launch_coeff_scatter_d2(int n1, cudaStream_t st, const PacketsDev &pk
                                    const Params32 *p32, void *W, uint8_t *flags);
 fgr_status launch_coeff_scatter_d3(int n1, cudaStream_t st, const PacketsDev &pk, const Params64 *p64,
                                    const Params32 *p32, void *W, uint8_t *flags);
-// The binned scatter (FP32, d = 3, n1 = 4 or 8): binning kernels, then the
-// binned kernel and the per-packet kernel over the loose list.  (In 2-D a
-// packet has only 64 contributions and an outer cell reaches 8 rows: the
-// per-packet kernel is faster there, measured on the 2-D workload.)
+// The binned scatter (FP32, d = 2 or 3, n1 = 4 or 8): binning kernels, then the
+// binned kernel and the per-packet kernel over the loose list.
 fgr_status launch_binned_scatter(int d, int n1, const BinLaunch &L, cudaStream_t st, const PacketsDev &pk,
                                  const Params32 &P, void *W, uint8_t *flags, StageMarks *marks);
+fgr_status launch_binned_d2(int n1, const BinLaunch &L, cudaStream_t st, const PacketsDev &pk, const Params32 &P,
+                            void *W, uint8_t *flags, StageMarks *marks);
 fgr_status launch_binned_d3(int n1, const BinLaunch &L, cudaStream_t st, const PacketsDev &pk, const Params32 &P,
                             void *W, uint8_t *flags, StageMarks *marks);
 

@@ -160,3 +160,56 @@ def test_every_cell_at_the_smallest_binned_size():
     cells = [((a, b), (a2, 3)) for a in range(-5, 5) for b in range(-6, 6) for a2 in range(-2, 3)]
     pk, mesh = clustered(11, 3, eps, cells, [8] * len(cells), (-0.6, 0.6), (-0.5, 0.5))
     _check(pk, mesh, _grid([33, 30, 27]), eps, npts=200)
+
+
+def lattice_2d(seed, n_a, n_b, per_dim_jitter, thin=1.0):
+    """One packet per dq x dp cell of a 4-D box (what the flow of a mesh
+    preserves), jittered, a share `thin` of them kept."""
+    eps = 1 / 64
+    mesh = mesh_for(2, eps)
+    rng = np.random.default_rng(seed)
+    idx = np.indices((n_a, n_b, n_a, n_b)).reshape(4, -1)
+    idx = idx[:, rng.random(idx.shape[1]) < thin]
+    j = rng.uniform(-per_dim_jitter, per_dim_jitter, idx.shape)
+    q = np.stack([(idx[0] - n_a // 2 + j[0]) * mesh.dq, (idx[2] - n_a // 2 + j[2]) * mesh.dq])
+    p = np.stack([(idx[1] - n_b // 2 + j[1]) * mesh.dp, (idx[3] - n_b // 2 + j[3]) * mesh.dp])
+    m = q.shape[1]
+    perm = rng.permutation(m)
+    a = rng.standard_normal((2, m)) * (rng.random(m) < 0.95)  # some exact zeros
+    return {"q": np.ascontiguousarray(q[:, perm]), "p": np.ascontiguousarray(p[:, perm]),
+            "s": rng.uniform(-3, 3, m), "a": np.ascontiguousarray(a)}, mesh, eps
+
+
+@pytest.mark.parametrize("n_a,n_b,thin", [(26, 17, 0.7), (20, 20, 0.9), (30, 40, 0.1)])
+@pytest.mark.parametrize("nq,np_", [(4, 2), (2, 2), (2, 4)])
+def test_binned_2d_tiles(n_a, n_b, thin, nq, np_):
+    """Packets in every tile of a 2-D set large enough to be binned (edges of the
+    24 x 16 tiles, bins of one, two and many items, small bins on the list), on a
+    grid that cuts part of them off: against the same call with Q and P halves
+    that are too few to be binned."""
+    pk, mesh, eps = lattice_2d(3, n_a, n_b, 0.45, thin)
+    m = pk["s"].size
+    assert m >= 1 << 17
+    grid = dict(d=2, n=[65, 44], lo=[-0.7, -0.5], hi=[1.1, 0.9])
+    opt = _gpu.options("fp32", nq=nq, np_=np_)
+    got = _gpu.reconstruct("fggc", pk, grid, eps, opt)
+    ref = np.zeros(got.shape, np.complex128)
+    step = (1 << 17) - 1  # each part stays on the per-packet kernel
+    for i in range(0, m, step):
+        part = {k: np.ascontiguousarray(pk[k][..., i:i + step]) for k in ("q", "p", "s", "a")}
+        ref += _gpu.reconstruct("fggc", part, grid, eps, opt)
+    # both sides round the same contributions and sums to FP32 (2e-7 each)
+    assert _gpu.rel_l2(got, ref) <= 2e-6
+
+
+def test_binned_2d_out_of_fp32_range_packets():
+    """Packets whose offsets or phases leave the FP32 form (far centres, large
+    actions, tiny amplitudes) inside a binned set."""
+    pk, mesh, eps = lattice_2d(4, 20, 20, 0.45)
+    m = pk["s"].size
+    pk["s"][::7] *= 1e6
+    pk["a"][:, ::11] *= 1e-35
+    grid = dict(d=2, n=[40, 36], lo=[-0.6, -0.6], hi=[0.6, 0.7])
+    got = _gpu.reconstruct("fggc", pk, grid, eps, _gpu.options("fp32"))
+    ref = _gpu.reconstruct("fggc", pk, grid, eps, _gpu.options("fp64", window_r=6.0))
+    assert _gpu.rel_l2(got, ref) <= 2e-6
