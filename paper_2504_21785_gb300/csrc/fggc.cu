@@ -324,7 +324,14 @@ __device__ __forceinline__ void grid_pass_body(const void *__restrict__ in_v, vo
         Real g[kPassPts][MAXBAND];
 #pragma unroll
         for (int r = 0; r < kPassPts; ++r) {
+            // FP32: offsets from the point's nearest node, so that they keep their
+            // relative accuracy however wide the tile is
             const double dx0 = xm[r] - (double)a_first * pp.dq;
+            float kc = 0.f, d0 = 0.f;
+            if constexpr (!FP64) {
+                kc = rintf((float)dx0 / dqf);
+                d0 = (float)fma(-(double)kc, pp.dq, dx0);
+            }
 #pragma unroll
             for (int i = 0; i < MAXBAND; ++i) {
                 g[r][i] = 0;
@@ -333,7 +340,7 @@ __device__ __forceinline__ void grid_pass_body(const void *__restrict__ in_v, vo
                         const double dx = xm[r] - (double)(a_first + i) * pp.dq;
                         g[r][i] = exp(dx * dx * pp.neg_half_inv_eps);
                     } else {
-                        const float dxf = (float)dx0 - (float)i * dqf;
+                        const float dxf = fmaf(kc - (float)i, dqf, d0);
                         g[r][i] = ex2_approx(dxf * dxf * cef);
                     }
                 }
@@ -425,6 +432,7 @@ __device__ __forceinline__ void grid_pass_body(const void *__restrict__ in_v, vo
 }
 
 #include "fggc_tma.cuh"
+#include "fggc_rows.cuh"
 
 template <bool FP64, int MAXBAND, int TP>
 __global__ void __launch_bounds__(TP) grid_pass_kernel(const void *__restrict__ in_v, void *__restrict__ out_v,
@@ -551,6 +559,41 @@ fgr_status launch_brange(const void *in, int64_t rows, int A, int B, const uint8
 // Entries of the pass tables for a pass over N points and A nodes (int2 /
 // float2 units): node windows, point phases and tile bands (at most N / 32 + 1).
 inline int64_t pass_table_entries(int64_t A, int64_t N) { return A + N + N / 32 + 1; }
+
+inline int row_halves(int B) { return (B + kRowHalf - 1) / kRowHalf; }
+
+// 8-byte entries of the row boxes and ranges of all passes of grid_rows_kernel:
+// a box per row of the first pass, then ranges per tile of contracted points and
+// outer node.
+inline int64_t row_box_entries(const Common &c, int D, const Grid &G) {
+    int64_t rows = 1;
+    for (int l = 0; l < D - 1; ++l) rows *= (int64_t)c.A[l] * c.B[l];
+    int64_t total = 2 * rows;
+    for (int l = D - 1; l > 0; --l) {
+        rows = rows / ((int64_t)c.A[l - 1] * c.B[l - 1]) * ((G.n[l] + kBoxPts - 1) / kBoxPts);
+        total += rows * row_halves(c.B[l - 1]);
+    }
+    return total;
+}
+
+// Pass tables (tiles of kRowPts points) of every dimension (blockIdx.y), and every
+// point's nearest node and offset from it.
+struct RowTables {
+    PassParams pp[kMaxDim];
+    PassTables tab[kMaxDim];
+    int64_t tiles[kMaxDim];
+    float2 *near[kMaxDim];
+};
+__global__ void row_tables_kernel(const __grid_constant__ RowTables T) {
+    const int l = blockIdx.y;
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const PassParams &pp = T.pp[l];
+    pass_tables_body(pp, kRowPts, T.tiles[l], T.tab[l], i);
+    if (i < pp.N) {
+        const double x = grid_x(pp.lo, pp.h, i), a = fmin(fmax(rint(x / pp.dq), -1e9), 1e9);
+        T.near[l][i] = make_float2((float)fma(-a, pp.dq, x), __int_as_float((int)a));
+    }
+}
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link
 // against the driver library); nullptr when unavailable.
@@ -875,7 +918,8 @@ fgr_status make_box(const fgr_ctx *ctx, const int *hb, int margin, FggcBox *box)
         x.maxbuf = std::max(x.maxbuf, prodN * pre);
     }
     if (D == 1) x.maxbuf = 0;
-    for (int l = 0; l < D; ++l) x.table_entries = std::max(x.table_entries, pass_table_entries(c.A[l], G.n[l]));
+    for (int l = 0; l < D; ++l) x.table_entries += pass_table_entries(c.A[l], G.n[l]) + (D > 1 ? G.n[l] : 0);
+    if (D > 1) x.max_lines = std::max(x.max_lines, row_box_entries(c, D, G));
     // DFT grid stage: one N-point line per (row, a) of each pass
     prodN = 1;
     for (int l = D - 1; l >= 0; --l) {
@@ -1072,8 +1116,11 @@ __global__ void __launch_bounds__(256) tables_batch_kernel(const __grid_constant
     pass_tables_body(B.pp[r], tp, mtiles, B.tab[r], (int64_t)(blockIdx.x - B.block0[r]) * 256 + threadIdx.x);
 }
 
+// (FP32: four CTAs of 128 per SM; left to itself the compiler packs the 64-node
+// form into 96 registers and the batch of 32 1-D requests takes 0.65 ms instead
+// of 0.30)
 template <bool FP64, int MAXBAND, int TP>
-__global__ void __launch_bounds__(TP) grid_pass_batch_kernel(const __grid_constant__ PassBatch B) {
+__global__ void __launch_bounds__(TP, !FP64 && TP == 128 ? 4 : 1) grid_pass_batch_kernel(const __grid_constant__ PassBatch B) {
     const int r = batch_request(B.block0, B.n);
     const int64_t local = blockIdx.x - B.block0[r];
     const int64_t row = local / B.tiles[r];
@@ -1119,6 +1166,133 @@ PassParams pass_params(const fgr_ctx *ctx, const Common &c, int l, int64_t prodN
     return pp;
 }
 
+// The grid stage of d >= 2 (FP32) by grid_rows_kernel.  boxes_known: the row
+// boxes of the first pass are in b.brange already (the binned scatter).
+template <int D>
+fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, bool boxes_known, void *u_dev,
+                        cudaStream_t st, StageTimer *timer, int64_t *launches) {
+    const Common &c = box.c;
+    const Grid &G = ctx->grid;
+    // tables of every dimension in one launch
+    RowTables T{};
+    PassParams pp[D];
+    {
+        int64_t prodN = 1, most = 0;
+        char *at = (char *)b.tables;
+        for (int l = D - 1; l >= 0; --l) {
+            pp[l] = pass_params(ctx, c, l, prodN);
+            prodN *= G.n[l];
+            T.pp[l] = pp[l];
+            T.tiles[l] = (G.n[l] + kRowPts - 1) / kRowPts;
+            T.tab[l].win = reinterpret_cast<int2 *>(at);
+            T.tab[l].ph = reinterpret_cast<float2 *>(T.tab[l].win + pp[l].A);
+            T.tab[l].band = reinterpret_cast<int2 *>(T.tab[l].ph + pp[l].N);
+            at += 8 * pass_table_entries(pp[l].A, pp[l].N);
+            T.near[l] = reinterpret_cast<float2 *>(at);
+            at += 8 * pp[l].N;
+            most = std::max<int64_t>(most, std::max<int64_t>(pp[l].A, pp[l].N));
+        }
+        row_tables_kernel<<<dim3((unsigned)((most + 255) / 256), D), 256, 0, st>>>(T);
+    }
+    // the rows' boxes and ranges of every pass
+    int4 *rbox = reinterpret_cast<int4 *>(b.brange);
+    if (!boxes_known)
+        row_scan_kernel<<<(unsigned)((box.rows0 + 7) / 8), 256, 0, st>>>((const float2 *)b.W, box.rows0, c.A[D - 1],
+                                                                       c.B[D - 1], b.flags, rbox);
+    int2 *range[D] = {};
+    {
+        int2 *at = reinterpret_cast<int2 *>(rbox + box.rows0);
+        int64_t rows = box.rows0;
+        for (int l = D - 1; l > 0; --l) {
+            const int members = c.A[l - 1] * c.B[l - 1], halves = row_halves(c.B[l - 1]);
+            const int64_t groups = rows / members, tiles = (G.n[l] + kBoxPts - 1) / kBoxPts;
+            range[l - 1] = at;
+            FGR_CUDA_TRY(cudaMemsetAsync(at, 0x7f, sizeof(int2) * (size_t)(tiles * groups * halves), st));
+            row_range_kernel<<<dim3((unsigned)groups, (unsigned)((members + 15) / 16)), 128, 0, st>>>(
+                l == D - 1 ? rbox : nullptr, range[l], row_halves(c.B[l]), members, c.B[l - 1], groups, T.tab[l].win,
+                halves, at);
+            rows = groups * tiles;
+            at += rows * halves;
+            ++*launches;
+        }
+    }
+    FGR_CUDA_TRY(cudaGetLastError());
+    if (timer) timer->mark(&ctx->timing.last.grid_ms);
+    const void *cur = b.W;
+    for (int l = D - 1; l >= 0; --l) {
+        void *dst = l == 0 ? u_dev : (cur == b.buf1 ? b.buf2 : b.buf1);
+        RowPass R{};
+        R.pp = pp[l];
+        R.lines = std::min(pass_band(kRowPts, pp[l].h, pp[l].rs, pp[l].dq), pp[l].A);
+        R.gl = l > 0 ? c.B[l - 1] : (int)G.n[D - 1];
+        const int64_t outer = pp[l].rows / R.gl;
+        // rows per CTA: up to kRowMax, fewer when that leaves SMs idle
+        int rpc = kRowMax;
+        while (rpc > kRowWarps && outer * ((R.gl + rpc - 1) / rpc) * T.tiles[l] < 3 * (int64_t)ctx->num_sms) rpc /= 2;
+        R.parts = (R.gl + rpc - 1) / rpc;
+        R.rpc = (R.gl + R.parts - 1) / R.parts;
+        R.chunks = (c.B[l] + kRowB - 1) / kRowB;
+        R.near = T.near[l];
+        // which nodes: the first pass by row, the others by the tiles of the row's points
+        const int64_t tiles2 = D == 3 ? (G.n[D - 1] + kBoxPts - 1) / kBoxPts : 1;
+        R.range = range[l];
+        R.d1 = INT64_MAX;
+        if (l == D - 1) {
+            R.box = rbox;
+        } else if (l > 0) {  // d = 3, second pass: rows (m_2, a_0, b_0)
+            R.d1 = R.stride = (int64_t)c.A[0] * c.B[0];
+            R.s1 = kBoxLog;
+        } else if (D == 3) {  // rows (m_1, m_2)
+            R.d1 = G.n[D - 1];
+            R.stride = tiles2;
+            R.s1 = R.s0 = kBoxLog;
+        } else {  // rows m_1
+            R.s0 = kBoxLog;
+        }
+        if (l > 0) {
+            R.next = range[l - 1];
+            R.next_lines = c.A[l - 1];
+            R.next_halves = row_halves(c.B[l - 1]);
+            R.next_shift = l < D - 1 ? kBoxLog : 0;
+            R.next_groups = l == 2 ? (int64_t)c.A[0] * c.B[0] : tiles2;
+        }
+        CUtensorMap map, map_half;
+        if (!pass_tensor_map(cur, pp[l], kRowLines, &map) || !pass_tensor_map(cur, pp[l], kRowLines / 2, &map_half)) {
+            set_error("fggc: no tensor map for a grid pass");
+            return FGR_E_INTERNAL;
+        }
+        FGR_CUDA_TRY(cudaFuncSetAttribute(grid_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)kRowSmemMax));
+        const dim3 grid((unsigned)(outer * R.parts), (unsigned)T.tiles[l]);
+        grid_rows_kernel<<<grid, kRowWarps * 32, row_pass_smem(R.lines, R.rpc, R.chunks), st>>>(map, map_half, (float2 *)dst, R,
+                                                                                   T.tab[l], ctx->dev_err);
+        FGR_CUDA_TRY(cudaGetLastError());
+        ++*launches;
+        if (timer) timer->mark(&ctx->timing.last.pass_ms);
+        cur = dst;
+    }
+    return FGR_OK;
+}
+
+// Whether grid_rows_kernel serves the box: every pass's factor table, staged rows
+// and work list fit the shared memory, the tensor maps' rules hold (16-byte
+// bases, even b extents: make_box) and the grids fit a launch.
+bool rows_apply(const fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, int D) {
+    if (ctx->opt.precision != FGR_FP32 || D < 2 || b.terms || ctx->tune.pass_tile == 128 || !tensor_map_encoder())
+        return false;
+    const Grid &G = ctx->grid;
+    int64_t prodN = 1;
+    for (int l = D - 1; l >= 0; --l) {
+        if (ctx->fft_logn[l] > 0) return false;
+        const PassParams pp = pass_params(ctx, box.c, l, prodN);
+        prodN *= G.n[l];
+        const int lines = std::min(pass_band(kRowPts, pp.h, pp.rs, pp.dq), pp.A);
+        if (row_pass_smem(lines, kRowMax, (pp.B + kRowB - 1) / kRowB) > kRowSmemMax || pp.rows >= INT_MAX || pp.rows * (int64_t)pp.A >= INT_MAX - 64 || pp.N > INT_MAX / 2 || pp.B < 2)
+            return false;
+    }
+    return G.n[D - 1] <= INT_MAX && (((uintptr_t)b.W | (uintptr_t)b.buf1 | (uintptr_t)b.buf2) & 15) == 0;
+}
+
 // Clears the node box and runs the coefficient scatter and the grid passes
 // into u_dev (all stream-ordered: no allocation, no host synchronisation).
 template <int D>
@@ -1159,6 +1333,7 @@ fgr_status enqueue_fggc(fgr_ctx *ctx, const PacketsDev &pk, const FggcBox &box, 
             bl.num_sms = ctx->num_sms;
             bl.rows = box.rows0;
             bl.row_cells = box.cells / box.rows0;
+            bl.row_box = reinterpret_cast<int4 *>(b.brange);
             StageMarks marks{timer, &ctx->timing.last.coeff_ms};
             r = launch_binned_scatter(D, L.n1, bl, st, pk, P, b.W, b.flags, &marks);
             *launches += 8;  // key, 3 scan, place, items, binned, loose
@@ -1170,6 +1345,11 @@ fgr_status enqueue_fggc(fgr_ctx *ctx, const PacketsDev &pk, const FggcBox &box, 
     ++*launches;
     if (timer) timer->mark(&ctx->timing.last.scatter_ms);
 
+    if constexpr (D > 1) {
+        if (rows_apply(ctx, box, b, D)) {
+            return enqueue_rows<D>(ctx, box, b, binned, u_dev, st, timer, launches);
+        }
+    }
     // separable passes, last dimension first
     const void *cur = b.W;
     int64_t prodN_after = 1;  // product of N of contracted dimensions

@@ -220,21 +220,23 @@ __global__ void __launch_bounds__(256) bin_place_kernel(const double *__restrict
     const double sv = s[j], ar = a[j], ai = a[m + j];
     if (k < 0) return;
     const int2 o = off[k], o1 = off[k + 1];
+    int a0, b0;
     if (o1.x == o.x) {
         loose[aggregated_add(nloose, 0)] = (int)j;
-        return;
+        a0 = floor_div_int(qv[D - 1], c.dqv, c.inv_dq) - c.amin[D - 1];
+        b0 = floor_div_int(pv[D - 1], c.dpv, c.inv_dp) - c.bmin[D - 1];
+    } else {
+        float sx[D], ty[D];
+        float2 w, z;
+        packet_record<D>(c, sc, qv, pv, sv, ar, ai, sx, ty, a0, b0, w, z);
+        a0 -= c.amin[D - 1];
+        b0 -= c.bmin[D - 1];
+        BinRecord r;
+        r.x = make_float4(sx[0], ty[0], sx[D - 1], ty[D - 1]);
+        r.w = make_float4(w.x, w.y, z.x, z.y);
+        r.y = make_float4(__int_as_float(a0), __int_as_float(b0), sx[D / 2], ty[D / 2]);
+        rec[o.x + rank[j]] = r;
     }
-    float sx[D], ty[D];
-    int a0, b0;
-    float2 w, z;
-    packet_record<D>(c, sc, qv, pv, sv, ar, ai, sx, ty, a0, b0, w, z);
-    a0 -= c.amin[D - 1];
-    b0 -= c.bmin[D - 1];
-    BinRecord r;
-    r.x = make_float4(sx[0], ty[0], sx[D - 1], ty[D - 1]);
-    r.w = make_float4(w.x, w.y, z.x, z.y);
-    r.y = make_float4(__int_as_float(a0), __int_as_float(b0), sx[D / 2], ty[D / 2]);
-    rec[o.x + rank[j]] = r;
     if constexpr (D == 3) {
         // most packets find their key's box wide enough already (a stale read
         // only costs an atomic)
@@ -267,6 +269,29 @@ __device__ __forceinline__ void key_anchors(const BinBox &bb, unsigned k, int *o
     }
 }
 
+// Inner target box (ta0, ta1, tb0, tb1) of a key's packets in the node box;
+// false if their neighbours reach past the node box.
+template <int D>
+__device__ __forceinline__ bool key_box(const Common &c, const BinBox &bb, const int4 *kbox, int64_t k, int ta, int tb,
+                                        int4 &box) {
+    int4 an;  // inner anchors: first and last a, first and last b (relative to the node box)
+    if constexpr (D == 3) {
+        const int4 b = kbox[k];
+        an = make_int4(b.x, -b.y, b.z, -b.w);
+    } else {
+        an.x = bb.ka_lo[1] - c.amin[1] + ta * kBinTileA;
+        an.y = bb.ka_lo[1] - c.amin[1] + min(bb.KA[1], (ta + 1) * kBinTileA) - 1;
+        an.z = bb.kb_lo[1] - c.bmin[1] + tb * kBinTileB;
+        an.w = bb.kb_lo[1] - c.bmin[1] + min(bb.KB[1], (tb + 1) * kBinTileB) - 1;
+    }
+    an.x += bb.dqmin;
+    an.y += bb.dqmax;
+    an.z += bb.dpmin;
+    an.w += bb.dpmax;
+    box = make_int4(max(0, an.x), min(c.A[D - 1] - 1, an.y), max(0, an.z), min(c.B[D - 1] - 1, an.w));
+    return an.x >= 0 && an.y < c.A[D - 1] && an.z >= 0 && an.w < c.B[D - 1];
+}
+
 // One item per kBinT packets of every bin.
 template <int D>
 __global__ void bin_items_kernel(const int2 *__restrict__ off, const int4 *__restrict__ kbox, const Common c,
@@ -278,21 +303,8 @@ __global__ void bin_items_kernel(const int2 *__restrict__ off, const int4 *__res
     if (n == 0) return;
     int oa[D - 1], ob[D - 1], ta, tb;
     key_anchors<D>(bb, (unsigned)k, oa, ob, ta, tb);
-    int4 an;  // inner anchors: first and last a, first and last b (relative to the node box)
-    if constexpr (D == 3) {
-        const int4 b = kbox[k];
-        an = make_int4(b.x, -b.y, b.z, -b.w);
-    } else {
-        an.x = bb.ka_lo[1] - c.amin[1] + ta * kBinTileA;
-        an.y = bb.ka_lo[1] - c.amin[1] + min(bb.KA[1], (ta + 1) * kBinTileA) - 1;
-        an.z = bb.kb_lo[1] - c.bmin[1] + tb * kBinTileB;
-        an.w = bb.kb_lo[1] - c.bmin[1] + min(bb.KB[1], (tb + 1) * kBinTileB) - 1;
-    }
     BinItem it;
-    const bool inside = an.x + bb.dqmin >= 0 && an.y + bb.dqmax < c.A[D - 1] && an.z + bb.dpmin >= 0 &&
-                        an.w + bb.dpmax < c.B[D - 1];
-    it.box = make_int4(max(0, an.x + bb.dqmin), min(c.A[D - 1] - 1, an.y + bb.dqmax), max(0, an.z + bb.dpmin),
-                       min(c.B[D - 1] - 1, an.w + bb.dpmax));
+    const bool inside = key_box<D>(c, bb, kbox, k, ta, tb, it.box);
     float z[4] = {1.f, 0.f, 1.f, 0.f};
 #pragma unroll
     for (int l = 0; l < D - 1; ++l) {
@@ -309,26 +321,41 @@ __global__ void bin_items_kernel(const int2 *__restrict__ off, const int4 *__res
 
 // Before the scatter: marks every row of W that the packets of an occupied key
 // will reach (the n1^(d-1) outer neighbours of its anchor cell that lie in the
-// node box), one thread per key.  The binned and per-packet kernels reach
-// exactly these rows, so only they need clearing.
+// node box) and widens the rows' boxes (min a, min -a, min b, min -b of the inner
+// nodes) by the key's, one thread per key.  The binned and per-packet kernels
+// reach exactly these rows, so only they need clearing.
 template <int D>
-__global__ void bin_mark_rows_kernel(const int *__restrict__ count, const Common c, const BinBox bb,
-                                     uint8_t *__restrict__ row_flag) {
+__global__ void bin_mark_rows_kernel(const int *__restrict__ count, const int4 *__restrict__ kbox, const Common c,
+                                     const BinBox bb, uint8_t *__restrict__ row_flag, int4 *row_box) {
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k >= bb.K || count[k] == 0) return;
     int oa[D - 1], ob[D - 1], ta, tb;
     key_anchors<D>(bb, (unsigned)k, oa, ob, ta, tb);
+    int4 box;
+    key_box<D>(c, bb, kbox, k, ta, tb, box);
+    const bool lands = box.x <= box.y && box.z <= box.w;
+    auto mark = [&](int64_t row) {
+        row_flag[row] = 1;
+        if (!lands) return;
+        // (a stale read only costs an atomic)
+        const int4 v = __ldcg(row_box + row);
+        int *b = reinterpret_cast<int *>(row_box + row);
+        if (box.x < v.x) atomicMin(b, box.x);
+        if (-box.y < v.y) atomicMin(b + 1, -box.y);
+        if (box.z < v.z) atomicMin(b + 2, box.z);
+        if (-box.w < v.w) atomicMin(b + 3, -box.w);
+    };
     for (int k0 = 0; k0 < c.n1; ++k0) {
         const int ia0 = oa[0] + c.dq[k0] - c.amin[0], ib0 = ob[0] + c.dp[k0] - c.bmin[0];
         if ((unsigned)ia0 >= (unsigned)c.A[0] || (unsigned)ib0 >= (unsigned)c.B[0]) continue;
         const int64_t row0 = (int64_t)ia0 * c.ra[0] + (int64_t)ib0 * c.rb[0];
         if constexpr (D == 2) {
-            row_flag[row0] = 1;
+            mark(row0);
         } else {
             for (int k1 = 0; k1 < c.n1; ++k1) {
                 const int ia1 = oa[1] + c.dq[k1] - c.amin[1], ib1 = ob[1] + c.dp[k1] - c.bmin[1];
                 if ((unsigned)ia1 >= (unsigned)c.A[1] || (unsigned)ib1 >= (unsigned)c.B[1]) continue;
-                row_flag[row0 + (int64_t)ia1 * c.ra[1] + (int64_t)ib1 * c.rb[1]] = 1;
+                mark(row0 + (int64_t)ia1 * c.ra[1] + (int64_t)ib1 * c.rb[1]);
             }
         }
     }
@@ -763,7 +790,15 @@ fgr_status launch_binned_d(const BinLaunch &L, cudaStream_t st, const PacketsDev
     if (D == 3) FGR_CUDA_TRY(cudaMemsetAsync(b.kbox, 0x7f, sizeof(int4) * (size_t)K, st));
     const unsigned pblocks = (unsigned)((m + 255) / 256), kblocks = (unsigned)((K + 255) / 256);
     bin_key_kernel<D><<<pblocks, 256, 0, st>>>(pk.q, pk.p, pk.a, m, P.c, L.box, b.key, b.rank, b.count);
-    bin_mark_rows_kernel<D><<<kblocks, 256, 0, st>>>(b.count, P.c, L.box, flags);
+    const int64_t nblk = (K + 1023) / 1024;
+    bin_scan1_kernel<<<(unsigned)nblk, 1024, 0, st>>>(b.count, K, b.off, b.bsum);
+    bin_scan2_kernel<<<1, 1024, 0, st>>>(b.bsum, nblk, b.off, K);
+    bin_scan3_kernel<<<(unsigned)nblk, 1024, 0, st>>>(b.off, K, b.bsum);
+    bin_place_kernel<D><<<pblocks, 256, 0, st>>>(pk.q, pk.p, pk.s, pk.a, m, P.c, L.split, b.key, b.rank, b.off, b.rec,
+                                                 b.kbox, b.loose, b.ctr);
+    // the rows and their boxes, and the clearing of those rows
+    FGR_CUDA_TRY(cudaMemsetAsync(L.row_box, 0x7f, sizeof(int4) * (size_t)L.rows, st));
+    bin_mark_rows_kernel<D><<<kblocks, 256, 0, st>>>(b.count, b.kbox, P.c, L.box, flags, L.row_box);
     // about 64 warps per SM: few long rows (d = 2: 5,796 of 37 KB) are cut into
     // parts (139 us with one warp per 32 rows, 19 us so), many short ones not
     const int64_t warps = (L.rows + 31) / 32, row_f4 = L.row_cells / 2;
@@ -771,12 +806,6 @@ fgr_status launch_binned_d(const BinLaunch &L, cudaStream_t st, const PacketsDev
     const dim3 cgrid((unsigned)std::min<int64_t>((warps + 7) / 8, (int64_t)L.num_sms * 8),
                      (unsigned)std::min<int64_t>(parts, 65535));
     clear_flagged_rows_kernel<<<cgrid, 256, 0, st>>>((float4 *)W, flags, L.rows, row_f4);
-    const int64_t nblk = (K + 1023) / 1024;
-    bin_scan1_kernel<<<(unsigned)nblk, 1024, 0, st>>>(b.count, K, b.off, b.bsum);
-    bin_scan2_kernel<<<1, 1024, 0, st>>>(b.bsum, nblk, b.off, K);
-    bin_scan3_kernel<<<(unsigned)nblk, 1024, 0, st>>>(b.off, K, b.bsum);
-    bin_place_kernel<D><<<pblocks, 256, 0, st>>>(pk.q, pk.p, pk.s, pk.a, m, P.c, L.split, b.key, b.rank, b.off, b.rec,
-                                                 b.kbox, b.loose, b.ctr);
     bin_items_kernel<D><<<kblocks, 256, 0, st>>>(b.off, b.kbox, P.c, L.box, b.items);
     FGR_CUDA_TRY(cudaGetLastError());
     if (marks) marks->binned();

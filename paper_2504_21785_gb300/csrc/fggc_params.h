@@ -37,8 +37,8 @@ struct FggcBox {
     int64_t cells = 0;      // node cells
     int64_t rows0 = 0;      // rows of the first grid pass
     int64_t maxbuf = 0;     // elements of each pass buffer (d > 1)
-    int64_t max_lines = 0;  // (row, a) lines of the b-range scan
-    int64_t table_entries = 0;  // 8-byte entries of the largest pass table
+    int64_t max_lines = 0;  // 8-byte entries of the b-ranges ((row, a) lines) or row boxes (two each)
+    int64_t table_entries = 0;  // 8-byte entries of the pass tables of all dimensions
     int64_t fft_elems = 0;      // complex elements of the DFT lines of the largest pass (0: no DFT stage)
     bool empty = true;      // no packet reaches the grid
 };
@@ -46,7 +46,7 @@ struct FggcBox {
 struct FggcBuffers {
     void *W = nullptr, *buf1 = nullptr, *buf2 = nullptr;
     uint8_t *flags = nullptr;
-    int2 *brange = nullptr;
+    int2 *brange = nullptr;  // b-range per (row, a) line, or row boxes (int4)
     void *tables = nullptr;  // per-pass tables (node windows, point phases, tile bands)
     void *bin = nullptr;     // binning buffers of the FP32 scatter, d >= 2 (NULL: per-packet scatter)
     size_t bin_bytes = 0;    // bytes of the binning buffers
@@ -111,6 +111,7 @@ struct BinLaunch {
     // are marked and zeroed
     int64_t rows = 0;
     int64_t row_cells = 0;
+    int4 *row_box = nullptr;  // [rows] receives the box of every row's inner nodes
 };
 
 // Largest key box of the binned scatter; larger boxes use the per-packet kernel.

@@ -192,6 +192,7 @@ __global__ void __launch_bounds__(32, 32) grid_pass_tma_kernel(const __grid_cons
             const int a_first = a_lo + ac * MAXBAND;
             nb = min(MAXBAND, nb_total - ac * MAXBAND);
             const double dx0 = xm - (double)a_first * pp.dq;
+            const float kc = rintf((float)dx0 / dqf), d0 = (float)fma(-(double)kc, pp.dq, dx0);  // nearest node
             // node windows: one coalesced load, then broadcast by shuffles
             const int2 wl = lane < nb ? tab.win[a_first - pp.amin + lane] : make_int2(1, 0);
 #pragma unroll
@@ -199,7 +200,7 @@ __global__ void __launch_bounds__(32, 32) grid_pass_tma_kernel(const __grid_cons
                 const int wx = __shfl_sync(0xffffffffu, wl.x, i), wy = __shfl_sync(0xffffffffu, wl.y, i);
                 g[i] = 0.f;
                 if (i < nb && valid && m >= wx && m <= wy) {
-                    const float dxf = (float)dx0 - (float)i * dqf;
+                    const float dxf = fmaf(kc - (float)i, dqf, d0);
                     g[i] = ex2_approx(dxf * dxf * cef);
                 }
             }

@@ -213,3 +213,36 @@ def test_binned_2d_out_of_fp32_range_packets():
     got = _gpu.reconstruct("fggc", pk, grid, eps, _gpu.options("fp32"))
     ref = _gpu.reconstruct("fggc", pk, grid, eps, _gpu.options("fp64", window_r=6.0))
     assert _gpu.rel_l2(got, ref) <= 2e-6
+
+
+@pytest.mark.parametrize("n", [(1, 70), (65, 8), (128, 63), (200, 129)])
+@pytest.mark.parametrize("spread", [0.05, 1.3])
+def test_grid_rows_2d_edges(n, spread):
+    """The row-wise grid passes at the edges of their 64-point tiles and of the
+    ranges they read: one point, one more than a tile, windows that leave points
+    without any node, few and many lines; against FP64."""
+    eps = 1 / 64
+    rng = np.random.default_rng(8)
+    m = 400
+    q, p = rng.uniform(-spread, spread, (2, m)), rng.uniform(-1.5, 1.5, (2, m))
+    p[0] -= 2 * q[0]  # position and momentum correlated: ranges narrower than boxes
+    pk = {"q": q, "p": p, "s": rng.uniform(-1, 1, m), "a": rng.standard_normal((2, m))}
+    grid = dict(d=2, n=list(n), lo=[-1.6, -2.0], hi=[1.1, 1.7])
+    got = _gpu.reconstruct("fggc", pk, grid, eps, _gpu.options("fp32"))
+    ref = _gpu.reconstruct("fggc", pk, grid, eps, _gpu.options("fp64", window_r=6.0))
+    # coefficients, two phases and Gaussians per dimension in FP32: below 2e-6
+    assert _gpu.rel_l2(got, ref) <= 2e-6
+
+
+@pytest.mark.parametrize("n", [(20, 65, 9), (66, 1, 130)])
+def test_grid_rows_3d_edges(n):
+    eps = 1 / 64
+    rng = np.random.default_rng(9)
+    m = 900
+    q, p = rng.uniform(-0.4, 0.4, (3, m)), rng.uniform(-0.5, 0.5, (3, m))
+    p += 1.5 * q
+    pk = {"q": q, "p": p, "s": rng.uniform(-1, 1, m), "a": rng.standard_normal((2, m))}
+    grid = dict(d=3, n=list(n), lo=[-1.0, -1.2, -0.9], hi=[1.1, 0.8, 1.3])
+    got = _gpu.reconstruct("fggc", pk, grid, eps, _gpu.options("fp32"))
+    ref = _gpu.reconstruct("fggc", pk, grid, eps, _gpu.options("fp64", window_r=6.0))
+    assert _gpu.rel_l2(got, ref) <= 2e-6
