@@ -174,6 +174,7 @@ struct PassParams {
 };
 
 constexpr int kCB = 32;
+constexpr int kSlice = 8;  // b values per unit of a b-slice (see launch_pass)
 
 // One grid point per thread keeps the Gaussian factors of the band (MAXBAND
 // registers) small enough for several CTAs per SM.  A CTA covers TP = 128 or
@@ -275,10 +276,10 @@ __device__ __forceinline__ void grid_pass_body(const void *__restrict__ in_v, vo
         ulo = s_blo;
         uhi = s_bhi;
     }
-    // b-slice of this CTA: part zs of nz of [ulo, uhi], whole chunks
-    const int nchunk = uhi >= ulo ? (uhi - ulo + kCB) / kCB : 0;
-    const int per = (nchunk + nz - 1) / nz;
-    const int bs = ulo + zs * per * kCB, be = min(uhi + 1, bs + per * kCB);
+    // b-slice of this CTA: part zs of nz of [ulo, uhi], in units of kSlice values
+    const int nunit = uhi >= ulo ? (uhi - ulo + kSlice) / kSlice : 0;
+    const int per = (nunit + nz - 1) / nz;
+    const int bs = ulo + zs * per * kSlice, be = min(uhi + 1, bs + per * kSlice);
     if ((flags && !flags[row]) || bs >= be || nb_total <= 0) {
         if (!split) {
 #pragma unroll
@@ -562,6 +563,14 @@ inline int64_t pass_table_entries(int64_t A, int64_t N) { return A + N + N / 32 
 
 inline int row_halves(int B) { return (B + kRowHalf - 1) / kRowHalf; }
 
+// Whether the FP64 phase tables of every dimension stay small (64 MB each).
+constexpr int64_t kRowPhaseMax = int64_t(1) << 22;
+inline bool row_phases_fit(const Common &c, int D, const Grid &G) {
+    for (int l = 0; l < D; ++l)
+        if (G.n[l] * (1 + (int64_t)row_halves(c.B[l])) > kRowPhaseMax || row_halves(c.B[l]) >= 65535) return false;
+    return true;
+}
+
 // 8-byte entries of the row boxes and ranges of all passes of grid_rows_kernel:
 // a box per row of the first pass, then ranges per tile of contracted points and
 // outer node.
@@ -576,20 +585,37 @@ inline int64_t row_box_entries(const Common &c, int D, const Grid &G) {
     return total;
 }
 
-// Pass tables (tiles of kRowPts points) of every dimension (blockIdx.y), and every
-// point's nearest node and offset from it.
+// 8-byte entries of a dimension's tables for grid_rows_kernel: the pass tables and
+// every point's nearest node (FP32) or the phases (FP64).
+inline int64_t row_table_entries(bool fp64, int64_t A, int64_t N, int B) {
+    const int64_t t = (pass_table_entries(A, N) + 1) & ~int64_t(1);
+    return t + (fp64 ? 2 * N * (1 + row_halves(B)) : (N + 1) & ~int64_t(1));
+}
+
+// Tables of every dimension (blockIdx.y): the pass tables (tiles of row_pts points)
+// and, FP32, every point's nearest node and offset from it; FP64, the rotation
+// e^{i dp x / eps} and the phases of the middle b of every kRowHalf values
+// (blockIdx.z: 0, and 1 + the index of the four).
 struct RowTables {
     PassParams pp[kMaxDim];
     PassTables tab[kMaxDim];
     int64_t tiles[kMaxDim];
     float2 *near[kMaxDim];
+    double2 *phase[kMaxDim];
 };
+template <bool FP64>
 __global__ void row_tables_kernel(const __grid_constant__ RowTables T) {
     const int l = blockIdx.y;
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const PassParams &pp = T.pp[l];
-    pass_tables_body(pp, kRowPts, T.tiles[l], T.tab[l], i);
-    if (i < pp.N) {
+    if (blockIdx.z == 0) pass_tables_body(pp, row_pts<FP64>(), T.tiles[l], T.tab[l], i);
+    if (FP64 && i < pp.N && (int)blockIdx.z <= (pp.B + kRowHalf - 1) / kRowHalf) {
+        const double b = blockIdx.z == 0 ? 1.0 : (double)(pp.bmin + ((int)blockIdx.z - 1) * kRowHalf + 3);
+        double sn, cs;
+        sincos(b * (pp.dp_over_eps * grid_x(pp.lo, pp.h, i)), &sn, &cs);
+        T.phase[l][blockIdx.z * pp.N + i] = make_double2(cs, sn);
+    }
+    if (!FP64 && i < pp.N) {
         const double x = grid_x(pp.lo, pp.h, i), a = fmin(fmax(rint(x / pp.dq), -1e9), 1e9);
         T.near[l][i] = make_float2((float)fma(-a, pp.dq, x), __int_as_float((int)a));
     }
@@ -612,16 +638,16 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
     return fn;
 }
 
-// Tensor map of a pass input (complex64) as lines x B cells, box kTB cells x
-// band lines.  False when the input does not meet the copy engine's rules
+// Tensor map of a pass input as lines x B cells, box kTB cells x band lines
+// (complex64 cells as 8-byte elements, complex128 as two).  False when the input does not meet the copy engine's rules
 // (16-byte aligned base, 16-byte multiple line stride) or encoding fails.
-bool pass_tensor_map(const void *in, const PassParams &pp, int band_lines, CUtensorMap *map) {
+bool pass_tensor_map(const void *in, const PassParams &pp, int band_lines, CUtensorMap *map, int parts = 1) {
     PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
     const int64_t lines = pp.rows * (int64_t)pp.A;
     if (!enc || ((uintptr_t)in & 15) || (pp.B & 1) || lines >= INT_MAX - 64 || pp.B < 2) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)pp.B, (cuuint64_t)lines};
-    const cuuint64_t strides[1] = {(cuuint64_t)pp.B * 8};
-    const cuuint32_t box[2] = {(cuuint32_t)kTB, (cuuint32_t)band_lines};
+    const cuuint64_t dims[2] = {(cuuint64_t)pp.B * parts, (cuuint64_t)lines};
+    const cuuint64_t strides[1] = {(cuuint64_t)pp.B * 8 * parts};
+    const cuuint32_t box[2] = {(cuuint32_t)(kTB * parts), (cuuint32_t)band_lines};
     const cuuint32_t estr[2] = {1, 1};
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, const_cast<void *>(in), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -640,18 +666,25 @@ fgr_status launch_pass(const void *in, void *out, const PassParams &pp, const ui
     // narrow tiles where they cut the band (the work per grid point) by more
     // than a quarter, unless the autotuner or the caller fixed the tile
     const int band128 = pass_band(128, pp.h, pp.rs, pp.dq), band32 = pass_band(32, pp.h, pp.rs, pp.dq);
-    const int tp = tile_pref == 32 || tile_pref == 128 ? tile_pref : (4 * band32 < 3 * band128 ? 32 : 128);
+    // (FP64 also where the 128-point tiles are fewer than the SMs: the FP64 pipe binds
+    // and every SM has its own)
+    const bool few = FP64 && pp.rows * ((pp.N + 127) / 128) < 148;
+    const int tp = tile_pref == 32 || tile_pref == 128 ? tile_pref : (few || 4 * band32 < 3 * band128 ? 32 : 128);
     const int band = tp == 32 ? band32 : band128;
     const int64_t mtiles = (pp.N + tp - 1) / tp;
     if (mtiles > 65535) {
         set_error("fggc: %lld points per grid dimension; at most %d supported", (long long)pp.N, 65535 * tp);
         return FGR_E_INVALID;
     }
-    // split the b-range when rows x tiles alone cannot fill the device
+    // split the b-range when rows x tiles alone cannot fill the device: FP32 into
+    // whole chunks (a CTA's Gaussian factors cost as much as about 8 b values), FP64
+    // down to kSlice values, whose phases (a sine and cosine each) outweigh them
+    // (1024 points x 110 b values: 189 us in 32-value slices of 128-point tiles, 133
+    // in 16-value and 84 in 8-value slices of 32-point tiles)
     const int64_t target = target_ctas;
-    const int nchunk = (pp.B + kCB - 1) / kCB;
+    const int unit = FP64 ? kSlice : kCB, nunit = (pp.B + unit - 1) / unit;
     int splits = (int)std::min<int64_t>(std::max<int64_t>(1, (target + pp.rows * mtiles - 1) / (pp.rows * mtiles)),
-                                        std::max(1, std::min(nchunk, 64)));
+                                        std::max(1, std::min(nunit, 64)));
     if (splits > 1) {
         FGR_CUDA_TRY(cudaMemsetAsync(out, 0, (FP64 ? 16 : 8) * (size_t)pp.rows * (size_t)pp.N, st));
     }
@@ -785,12 +818,11 @@ Common base_common(const fgr_ctx *ctx) {
     const Lsa &L = ctx->lsa;
     Common c{};
     c.n1 = L.n1;
-    const bool fp32 = ctx->opt.precision == FGR_FP32;
     for (int k = 0; k < L.n1; ++k) {
-        const int kk = fp32 ? L.order[k] : k;
-        c.dq[k] = L.dq[kk];
-        c.dp[k] = L.dp[kk];
+        c.dq[k] = L.dq[L.order[k]];
+        c.dp[k] = L.dp[L.order[k]];
     }
+    c.u3 = L.u3;
     c.v3 = L.v3;
     c.dqv = M.dq;
     c.dpv = M.dp;
@@ -798,7 +830,7 @@ Common base_common(const fgr_ctx *ctx) {
     c.inv_dp = 1.0 / M.dp;
     c.cq2_4 = M.cq * M.cq / 4;
     c.cp2_4 = M.cp * M.cp / 4;
-    c.half_cqcp = M.cqcp / 2;
+    c.cqcp_4 = M.cqcp / 4;
     c.cc = M.cqcp / (2 * M_PI);
     c.inv_2pi_eps = 1.0 / (2 * M_PI * M.eps);
     c.pref = M.pref;
@@ -918,7 +950,10 @@ fgr_status make_box(const fgr_ctx *ctx, const int *hb, int margin, FggcBox *box)
         x.maxbuf = std::max(x.maxbuf, prodN * pre);
     }
     if (D == 1) x.maxbuf = 0;
-    for (int l = 0; l < D; ++l) x.table_entries += pass_table_entries(c.A[l], G.n[l]) + (D > 1 ? G.n[l] : 0);
+    // (FP64 phase tables beyond kRowPhaseMax points x b ranges: the other pass kernels)
+    const bool fp64 = ctx->opt.precision == FGR_FP64, rows64 = D > 1 && row_phases_fit(c, D, G);
+    for (int l = 0; l < D; ++l) x.table_entries += D == 1 ? pass_table_entries(c.A[l], G.n[l])
+                                 : row_table_entries(fp64 && rows64, c.A[l], G.n[l], c.B[l]);
     if (D > 1) x.max_lines = std::max(x.max_lines, row_box_entries(c, D, G));
     // DFT grid stage: one N-point line per (row, a) of each pass
     prodN = 1;
@@ -1166,11 +1201,13 @@ PassParams pass_params(const fgr_ctx *ctx, const Common &c, int l, int64_t prodN
     return pp;
 }
 
-// The grid stage of d >= 2 (FP32) by grid_rows_kernel.  boxes_known: the row
+// The grid stage of d >= 2 by grid_rows_kernel.  boxes_known: the row
 // boxes of the first pass are in b.brange already (the binned scatter).
-template <int D>
+template <int D, bool FP64>
 fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, bool boxes_known, void *u_dev,
                         cudaStream_t st, StageTimer *timer, int64_t *launches) {
+    using C2 = typename std::conditional<FP64, double2, float2>::type;
+    constexpr int kRowPts = row_pts<FP64>();
     const Common &c = box.c;
     const Grid &G = ctx->grid;
     // tables of every dimension in one launch
@@ -1178,6 +1215,7 @@ fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, 
     PassParams pp[D];
     {
         int64_t prodN = 1, most = 0;
+        int halves = 0;
         char *at = (char *)b.tables;
         for (int l = D - 1; l >= 0; --l) {
             pp[l] = pass_params(ctx, c, l, prodN);
@@ -1187,18 +1225,21 @@ fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, 
             T.tab[l].win = reinterpret_cast<int2 *>(at);
             T.tab[l].ph = reinterpret_cast<float2 *>(T.tab[l].win + pp[l].A);
             T.tab[l].band = reinterpret_cast<int2 *>(T.tab[l].ph + pp[l].N);
-            at += 8 * pass_table_entries(pp[l].A, pp[l].N);
-            T.near[l] = reinterpret_cast<float2 *>(at);
-            at += 8 * pp[l].N;
+            // (16-byte alignment: an even number of entries)
+            char *more = at + 8 * ((pass_table_entries(pp[l].A, pp[l].N) + 1) & ~int64_t(1));
+            T.near[l] = reinterpret_cast<float2 *>(more);
+            T.phase[l] = reinterpret_cast<double2 *>(more);
+            at += 8 * row_table_entries(FP64, pp[l].A, pp[l].N, pp[l].B);
+            halves = std::max(halves, row_halves(pp[l].B));
             most = std::max<int64_t>(most, std::max<int64_t>(pp[l].A, pp[l].N));
         }
-        row_tables_kernel<<<dim3((unsigned)((most + 255) / 256), D), 256, 0, st>>>(T);
+        row_tables_kernel<FP64><<<dim3((unsigned)((most + 255) / 256), D, FP64 ? 1 + halves : 1), 256, 0, st>>>(T);
     }
     // the rows' boxes and ranges of every pass
     int4 *rbox = reinterpret_cast<int4 *>(b.brange);
     if (!boxes_known)
-        row_scan_kernel<<<(unsigned)((box.rows0 + 7) / 8), 256, 0, st>>>((const float2 *)b.W, box.rows0, c.A[D - 1],
-                                                                       c.B[D - 1], b.flags, rbox);
+        row_scan_kernel<C2><<<(unsigned)((box.rows0 + 7) / 8), 256, 0, st>>>((const C2 *)b.W, box.rows0, c.A[D - 1],
+                                                                           c.B[D - 1], b.flags, rbox);
     int2 *range[D] = {};
     {
         int2 *at = reinterpret_cast<int2 *>(rbox + box.rows0);
@@ -1233,6 +1274,7 @@ fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, 
         R.rpc = (R.gl + R.parts - 1) / R.parts;
         R.chunks = (c.B[l] + kRowB - 1) / kRowB;
         R.near = T.near[l];
+        R.phase = T.phase[l];
         // which nodes: the first pass by row, the others by the tiles of the row's points
         const int64_t tiles2 = D == 3 ? (G.n[D - 1] + kBoxPts - 1) / kBoxPts : 1;
         R.range = range[l];
@@ -1257,15 +1299,16 @@ fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, 
             R.next_groups = l == 2 ? (int64_t)c.A[0] * c.B[0] : tiles2;
         }
         CUtensorMap map, map_half;
-        if (!pass_tensor_map(cur, pp[l], kRowLines, &map) || !pass_tensor_map(cur, pp[l], kRowLines / 2, &map_half)) {
+        if (!pass_tensor_map(cur, pp[l], kRowLines, &map, FP64 ? 2 : 1) ||
+            !pass_tensor_map(cur, pp[l], kRowLines / 2, &map_half, FP64 ? 2 : 1)) {
             set_error("fggc: no tensor map for a grid pass");
             return FGR_E_INTERNAL;
         }
-        FGR_CUDA_TRY(cudaFuncSetAttribute(grid_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        FGR_CUDA_TRY(cudaFuncSetAttribute(grid_rows_kernel<FP64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)kRowSmemMax));
         const dim3 grid((unsigned)(outer * R.parts), (unsigned)T.tiles[l]);
-        grid_rows_kernel<<<grid, kRowWarps * 32, row_pass_smem(R.lines, R.rpc, R.chunks), st>>>(map, map_half, (float2 *)dst, R,
-                                                                                   T.tab[l], ctx->dev_err);
+        grid_rows_kernel<FP64><<<grid, kRowWarps * 32, row_pass_smem<FP64>(R.lines, R.rpc, R.chunks), st>>>(
+            map, map_half, (C2 *)dst, R, T.tab[l], ctx->dev_err);
         FGR_CUDA_TRY(cudaGetLastError());
         ++*launches;
         if (timer) timer->mark(&ctx->timing.last.pass_ms);
@@ -1278,16 +1321,20 @@ fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, 
 // and work list fit the shared memory, the tensor maps' rules hold (16-byte
 // bases, even b extents: make_box) and the grids fit a launch.
 bool rows_apply(const fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, int D) {
-    if (ctx->opt.precision != FGR_FP32 || D < 2 || b.terms || ctx->tune.pass_tile == 128 || !tensor_map_encoder())
-        return false;
+    if (D < 2 || b.terms || ctx->tune.pass_tile == 128 || !tensor_map_encoder()) return false;
     const Grid &G = ctx->grid;
+    const bool fp64 = ctx->opt.precision == FGR_FP64;
+    if (fp64 && !row_phases_fit(box.c, D, G)) return false;
     int64_t prodN = 1;
     for (int l = D - 1; l >= 0; --l) {
         if (ctx->fft_logn[l] > 0) return false;
         const PassParams pp = pass_params(ctx, box.c, l, prodN);
         prodN *= G.n[l];
-        const int lines = std::min(pass_band(kRowPts, pp.h, pp.rs, pp.dq), pp.A);
-        if (row_pass_smem(lines, kRowMax, (pp.B + kRowB - 1) / kRowB) > kRowSmemMax || pp.rows >= INT_MAX || pp.rows * (int64_t)pp.A >= INT_MAX - 64 || pp.N > INT_MAX / 2 || pp.B < 2)
+        const int lines = std::min(pass_band(fp64 ? row_pts<true>() : row_pts<false>(), pp.h, pp.rs, pp.dq), pp.A);
+        const int chunks = (pp.B + kRowB - 1) / kRowB;
+        if ((fp64 ? row_pass_smem<true>(lines, kRowMax, chunks) : row_pass_smem<false>(lines, kRowMax, chunks)) >
+                kRowSmemMax ||
+            pp.rows >= INT_MAX || pp.rows * (int64_t)pp.A >= INT_MAX - 64 || pp.N > INT_MAX / 2 || pp.B < 2)
             return false;
     }
     return G.n[D - 1] <= INT_MAX && (((uintptr_t)b.W | (uintptr_t)b.buf1 | (uintptr_t)b.buf2) & 15) == 0;
@@ -1317,9 +1364,7 @@ fgr_status enqueue_fggc(fgr_ctx *ctx, const PacketsDev &pk, const FggcBox &box, 
     if (fp64) {
         Params64 P{};
         P.c = c;
-        memcpy(P.vr, L.vr, sizeof(P.vr));
-        memcpy(P.vi, L.vi, sizeof(P.vi));
-        memcpy(P.inv_lam, L.inv_lam, sizeof(P.inv_lam));
+        P.f = factors64(L);
         fgr_status r = launch_coeff_scatter(D, L.n1, st, pk, &P, nullptr, b.W, b.flags);
         if (r != FGR_OK) return r;
     } else {
@@ -1347,7 +1392,8 @@ fgr_status enqueue_fggc(fgr_ctx *ctx, const PacketsDev &pk, const FggcBox &box, 
 
     if constexpr (D > 1) {
         if (rows_apply(ctx, box, b, D)) {
-            return enqueue_rows<D>(ctx, box, b, binned, u_dev, st, timer, launches);
+            return fp64 ? enqueue_rows<D, true>(ctx, box, b, binned, u_dev, st, timer, launches)
+                        : enqueue_rows<D, false>(ctx, box, b, binned, u_dev, st, timer, launches);
         }
     }
     // separable passes, last dimension first
@@ -1576,9 +1622,7 @@ fgr_status enqueue_fggc_batch(int n, const FggcRequest *req, cudaStream_t st) {
         std::unique_ptr<ScatterBatch32> b32;
         if (fp64) {
             b64.reset(new ScatterBatch64());
-            memcpy(b64->vr, L.vr, sizeof(b64->vr));
-            memcpy(b64->vi, L.vi, sizeof(b64->vi));
-            memcpy(b64->inv_lam, L.inv_lam, sizeof(b64->inv_lam));
+            b64->f = factors64(L);
             base = b64.get();
         } else {
             b32.reset(new ScatterBatch32());
@@ -1874,12 +1918,11 @@ extern "C" fgr_status fgr_reconstruct_fggc_noalloc(fgr_ctx *ctx, const fgr_packe
 
     Common c{};
     c.n1 = L.n1;
-    const bool fp32 = ctx->opt.precision == FGR_FP32;
     for (int k = 0; k < L.n1; ++k) {
-        const int kk = fp32 ? L.order[k] : k;
-        c.dq[k] = L.dq[kk];
-        c.dp[k] = L.dp[kk];
+        c.dq[k] = L.dq[L.order[k]];
+        c.dp[k] = L.dp[L.order[k]];
     }
+    c.u3 = L.u3;
     c.v3 = L.v3;
     c.dqv = M.dq;
     c.dpv = M.dp;
@@ -1887,7 +1930,7 @@ extern "C" fgr_status fgr_reconstruct_fggc_noalloc(fgr_ctx *ctx, const fgr_packe
     c.inv_dp = 1.0 / M.dp;
     c.cq2_4 = M.cq * M.cq / 4;
     c.cp2_4 = M.cp * M.cp / 4;
-    c.half_cqcp = M.cqcp / 2;
+    c.cqcp_4 = M.cqcp / 4;
     c.cc = M.cqcp / (2 * M_PI);
     c.inv_2pi_eps = 1.0 / (2 * M_PI * M.eps);
     c.pref = M.pref;
@@ -1945,9 +1988,7 @@ extern "C" fgr_status fgr_reconstruct_fggc_noalloc(fgr_ctx *ctx, const fgr_packe
     if (fp64) {
         Params64 P{};
         P.c = c;
-        memcpy(P.vr, L.vr, sizeof(P.vr));
-        memcpy(P.vi, L.vi, sizeof(P.vi));
-        memcpy(P.inv_lam, L.inv_lam, sizeof(P.inv_lam));
+        P.f = factors64(L);
         rc = launch_coeff_scatter(1, L.n1, st, PacketsDev{m, pk->q, pk->p, pk->s, pk->a}, &P, nullptr, W, flags);
         if (rc != FGR_OK) return rc;
     } else {

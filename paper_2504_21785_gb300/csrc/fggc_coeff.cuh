@@ -26,68 +26,138 @@ __device__ __forceinline__ void cmul(float ar, float ai, float br, float bi, flo
 // with the least-squares tables shared by the batch (same strategy).
 struct Params64View {
     const Common &c;
-    const double *vr, *vi, *inv_lam;
+    const Factors64 &f;
 };
 struct Params32View {
     const Common &c;
     const float *poly;
 };
 
-// FP64: per-dimension coefficients through the eigen factors (PT: Params64
-// or Params64View).
+// FP64: the coefficients of one dimension through the eigen factors (PT: Params64
+// or Params64View), in the symmetric form of build_lsa: with (sx, ty) the offset
+// from the cell centre, the right-hand side of neighbour (u, v) is
+//   e^{-cq^2 (u - sx)^2 / 4} e^{i cq cp u ty / 2} e^{-cp^2 (v - ty)^2 / 4} e^{-i cq cp v sx / 2},
+// one exponential per u and per v and a sine and cosine per |u| and per |v| for all
+// neighbours; sums and differences of mirror images bring it to the sectors' real
+// bases.  The phases are those of dim_setup32: z = e^{i cq cp A / 2}, and T takes
+// the packet's share in turns.  The FP64 pipe binds (16 clocks of an SM per warp
+// instruction): against an exponential, two sines and cosines and two complex
+// matrix rows per neighbour (N1 = 8: about 1360 instructions, now 570; N1 = 4: 590,
+// now 340) 705,600 2-D Q2P2 packets take 1.74 -> 0.98 ms.
 template <int N, class PT>
-__device__ __forceinline__ void coeff_dim64(const PT &P, double Q, double Pm, int &a0, int &b0,
+__device__ __forceinline__ void coeff_dim64(const PT &P, double Q, double Pm, int &a0, int &b0, double &T,
                                             double *cr, double *ci) {
     const Common &c = P.c;
     const double r = __ddiv_rn(Q, c.dqv), rp = __ddiv_rn(Pm, c.dpv);
     const double fa = floor(r), fb = floor(rp);
-    const double s = r - fa, t = rp - fb;
+    const double sx = (r - fa) - 0.5, ty = (rp - fb) - 0.5;
     a0 = (int)fmin(fmax(fa, -1e9), 1e9);
     b0 = (int)fmin(fmax(fb, -1e9), 1e9);
-    constexpr int n = N;
-    double fr[N], fi[N];
-#pragma unroll
-    for (int j = 0; j < n; ++j) {  // eq. 3.23
-        const double u = c.dq[j] - s, v = c.dp[j] - t;
-        const double mag = exp(-c.cq2_4 * u * u - c.cp2_4 * v * v);
-        double sn, cs;
-        sincos(c.half_cqcp * (s - c.dq[j]) * (c.dp[j] + t), &sn, &cs);
-        fr[j] = mag * cs;
-        fi[j] = mag * sn;
+    {
+        double t = c.cc * (r * (fb + 0.5));
+        t -= rint(t);
+        T -= t + 0.5 * c.cc * (sx * ty);
     }
-    double yr[N], yi[N];
-#pragma unroll
-    for (int i = 0; i < n; ++i) {  // y = diag(1/lam) V^H f
-        double sr = 0, si = 0;
-#pragma unroll
-        for (int j = 0; j < n; ++j) {
-            const double vr = P.vr[j * kMaxN1 + i], vi = P.vi[j * kMaxN1 + i];
-            sr += vr * fr[j] + vi * fi[j];
-            si += vr * fi[j] - vi * fr[j];
-        }
-        yr[i] = sr * P.inv_lam[i];
-        yi[i] = si * P.inv_lam[i];
+    double zr, zi;
+    {
+        double t = 0.5 * c.cc * (fa + 0.5);
+        t -= rint(t);
+        sincospi(2.0 * t, &zi, &zr);
     }
-    // node phase base (turns): -cc * r * b0 and -cc * a0
-    double t0 = -c.cc * (r * fb);
-    t0 -= rint(t0);
-    double t1 = -c.cc * fa;
-    t1 -= rint(t1);
+    // Gaussian and phase factors of u, v = -1/2, 1/2 and (where the strategy has
+    // them) -3/2, 3/2
+    double ur[2][2], ui[2][2], vr2[2][2], vi2[2][2];
 #pragma unroll
-    for (int k = 0; k < n; ++k) {  // c~ = conj(V y), times the node phase
-        double sr = 0, si = 0;
-#pragma unroll
-        for (int i = 0; i < n; ++i) {
-            const double vr = P.vr[k * kMaxN1 + i], vi = P.vi[k * kMaxN1 + i];
-            sr += vr * yr[i] - vi * yi[i];
-            si += vr * yi[i] + vi * yr[i];
+    for (int t = 0; t < (N >= 8 ? 2 : 1); ++t) {
+        const double h = t + 0.5;
+        if (t == 0 || c.u3) {
+            double sn, cs;
+            sincos(2.0 * h * c.cqcp_4 * ty, &sn, &cs);
+            const double lo = exp(-c.cq2_4 * ((h + sx) * (h + sx))), hi = exp(-c.cq2_4 * ((h - sx) * (h - sx)));
+            ur[t][0] = lo * cs;
+            ui[t][0] = -lo * sn;
+            ur[t][1] = hi * cs;
+            ui[t][1] = hi * sn;
         }
-        si = -si;
-        double tk = t0 + c.dp[k] * t1 - c.cc * (double)(c.dq[k] * c.dp[k]);
-        tk -= rint(tk);
-        double sn, cs;
-        sincospi(2.0 * tk, &sn, &cs);
-        cmul(sr, si, cs, sn, cr[k], ci[k]);
+        if (t == 0 || c.v3) {
+            double sn, cs;
+            sincos(2.0 * h * c.cqcp_4 * sx, &sn, &cs);
+            const double lo = exp(-c.cp2_4 * ((h + ty) * (h + ty))), hi = exp(-c.cp2_4 * ((h - ty) * (h - ty)));
+            vr2[t][0] = lo * cs;
+            vi2[t][0] = lo * sn;
+            vr2[t][1] = hi * cs;
+            vi2[t][1] = -hi * sn;
+        }
+    }
+    double gr[2][N / 2], gi[2][N / 2];
+#pragma unroll
+    for (int o = 0; o < N / 4; ++o) {
+        const bool u3 = N >= 8 && ((c.u3 >> o) & 1), v3 = N >= 8 && ((c.v3 >> o) & 1);
+        double br[4], bi[4];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            const int a = g >> 1, b = g & 1;
+            cmul(u3 ? ur[N >= 8 ? 1 : 0][a] : ur[0][a], u3 ? ui[N >= 8 ? 1 : 0][a] : ui[0][a],
+                 v3 ? vr2[N >= 8 ? 1 : 0][b] : vr2[0][b], v3 ? vi2[N >= 8 ? 1 : 0][b] : vi2[0][b], br[g], bi[g]);
+        }
+        const double pr = br[0] + br[3], pi = bi[0] + bi[3], qr = br[1] + br[2], qi = bi[1] + bi[2];
+        gr[0][2 * o] = pr + qr;
+        gi[0][2 * o] = pi + qi;
+        gr[0][2 * o + 1] = pi - qi;
+        gi[0][2 * o + 1] = qr - pr;
+        const double mr = br[0] - br[3], mi = bi[0] - bi[3], nr = br[1] - br[2], ni = bi[1] - bi[2];
+        gr[1][2 * o] = mr + nr;
+        gi[1][2 * o] = mi + ni;
+        gr[1][2 * o + 1] = mi - ni;
+        gi[1][2 * o + 1] = nr - mr;
+    }
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        double wr[N / 2], wi[N / 2];
+#pragma unroll
+        for (int i = 0; i < N / 2; ++i) {
+            double tr = 0, ti = 0;
+#pragma unroll
+            for (int a = 0; a < N / 2; ++a) {
+                tr = fma(P.f.sec[s][a * kMaxHalf + i], gr[s][a], tr);
+                ti = fma(P.f.sec[s][a * kMaxHalf + i], gi[s][a], ti);
+            }
+            wr[i] = tr * P.f.inv[s][i];
+            wi[i] = ti * P.f.inv[s][i];
+        }
+#pragma unroll
+        for (int a = 0; a < N / 2; ++a) {
+            double tr = 0, ti = 0;
+#pragma unroll
+            for (int i = 0; i < N / 2; ++i) {
+                tr = fma(P.f.sec[s][a * kMaxHalf + i], wr[i], tr);
+                ti = fma(P.f.sec[s][a * kMaxHalf + i], wi[i], ti);
+            }
+            gr[s][a] = tr;
+            gi[s][a] = ti;
+        }
+    }
+#pragma unroll
+    for (int o = 0; o < N / 4; ++o) {
+        // x1 + i x2 and x1 - i x2 of the even half, y1 + i y2 and y1 - i y2 of the odd
+        const double er = gr[0][2 * o] - gi[0][2 * o + 1], ei = gi[0][2 * o] + gr[0][2 * o + 1];
+        const double fr = gr[0][2 * o] + gi[0][2 * o + 1], fi = gi[0][2 * o] - gr[0][2 * o + 1];
+        const double hr = gr[1][2 * o] - gi[1][2 * o + 1], hi = gi[1][2 * o] + gr[1][2 * o + 1];
+        const double lr = gr[1][2 * o] + gi[1][2 * o + 1], li = gi[1][2 * o] - gr[1][2 * o + 1];
+        double vr = zr, vi = zi;
+        if (N >= 8 && ((c.v3 >> o) & 1)) {
+            double r2, i2;
+            cmul(zr, zi, zr, zi, r2, i2);
+            cmul(r2, i2, zr, zi, vr, vi);
+        }
+        // e^{-i cq cp v (A + u / 2)} of u < 0 and of u > 0, for v < 0
+        double p0r, p0i, p1r, p1i;
+        cmul(vr, vi, P.f.kap_r[o], -P.f.kap_i[o], p0r, p0i);
+        cmul(vr, vi, P.f.kap_r[o], P.f.kap_i[o], p1r, p1i);
+        cmul(er + hr, ei + hi, p0r, p0i, cr[4 * o], ci[4 * o]);
+        cmul(fr + lr, fi + li, p0r, -p0i, cr[4 * o + 1], ci[4 * o + 1]);
+        cmul(fr - lr, fi - li, p1r, p1i, cr[4 * o + 2], ci[4 * o + 2]);
+        cmul(er - hr, ei - hi, p1r, -p1i, cr[4 * o + 3], ci[4 * o + 3]);
     }
 }
 
@@ -252,9 +322,9 @@ __device__ __forceinline__ void coeff_scatter_body(const double *__restrict__ q,
     // others go to this thread's column of shared memory (read back only by
     // this thread, so no barrier is needed)
     Real cl_r[N1], cl_i[N1];
-    Real wr, wi;  // weight pref * A * e^{i S/eps} (FP32: and the packet's gauge phase)
+    Real wr, wi;  // weight pref * A * e^{i S/eps} and the packet's gauge phase
     int a0[D], b0[D];
-    double rB = 0.0;
+    double rB = 0.0;  // (FP64: that phase, in turns)
     float xy = 0.f;
     // one dimension at a time (for d = 3 not unrolled: three unrolled copies
     // of the coefficient evaluation do not fit the register file)
@@ -262,7 +332,7 @@ __device__ __forceinline__ void coeff_scatter_body(const double *__restrict__ q,
     for (int l = 0; l < D; ++l) {
         Real cr[N1], ci[N1];
         if constexpr (FP64) {
-            coeff_dim64<N1>(P, q[l * m + j], p[l * m + j], a0[l], b0[l], cr, ci);
+            coeff_dim64<N1>(P, q[l * m + j], p[l * m + j], a0[l], b0[l], rB, cr, ci);
         } else {
             float X, Y, zr, zi;
             dim_setup32(c, q[l * m + j], p[l * m + j], a0[l], b0[l], X, Y, zr, zi, rB, xy);
@@ -291,7 +361,7 @@ __device__ __forceinline__ void coeff_scatter_body(const double *__restrict__ q,
         double ts = s[j] * c.inv_2pi_eps;
         ts -= rint(ts);
         double sn, cs;
-        sincospi(2.0 * ts, &sn, &cs);
+        sincospi(2.0 * (ts + rB), &sn, &cs);
         cmul(ar * c.pref, ai * c.pref, cs, sn, wr, wi);
     } else {
         packet_weight32(c, s[j], ar, ai, rB, xy, wr, wi);
@@ -341,7 +411,7 @@ __global__ void __launch_bounds__(coeff_threads<FP64, N1>()) coeff_scatter_kerne
     const double *__restrict__ q, const double *__restrict__ p, const double *__restrict__ s,
     const double *__restrict__ a, int64_t m, const __grid_constant__ ParamsT<FP64> P, void *__restrict__ W_v,
     uint8_t *__restrict__ row_flag) {
-    const int64_t j = blockIdx.x * (int64_t)coeff_threads<FP64, N1>() + threadIdx.x;
+    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (j < m) coeff_scatter_body<D, FP64, N1>(q, p, s, a, m, j, P, W_v, row_flag);
 }
 
@@ -350,7 +420,7 @@ __global__ void __launch_bounds__(coeff_threads<FP64, N1>(), 4) coeff_scatter3_k
     const double *__restrict__ q, const double *__restrict__ p, const double *__restrict__ s,
     const double *__restrict__ a, int64_t m, const __grid_constant__ ParamsT<FP64> P, void *__restrict__ W_v,
     uint8_t *__restrict__ row_flag) {
-    const int64_t j = blockIdx.x * (int64_t)coeff_threads<FP64, N1>() + threadIdx.x;
+    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (j < m) coeff_scatter_body<D, FP64, N1>(q, p, s, a, m, j, P, W_v, row_flag);
 }
 
@@ -376,7 +446,7 @@ __global__ void __launch_bounds__(coeff_threads<FP64, N1>(), D == 3 ? 4 : 1) coe
     const int64_t j = (int64_t)(blockIdx.x - B.block0[r]) * coeff_threads<FP64, N1>() + threadIdx.x;
     if (j >= B.m[r]) return;
     if constexpr (FP64) {
-        const Params64View v{B.c[r], B.vr, B.vi, B.inv_lam};
+        const Params64View v{B.c[r], B.f};
         coeff_scatter_body<D, FP64, N1>(B.q[r], B.p[r], B.s[r], B.a[r], B.m[r], j, v, B.W[r], B.flags[r]);
     } else {
         const Params32View v{B.c[r], B.poly};
@@ -405,9 +475,12 @@ fgr_status launch_scatter_batch_dim(int n1, cudaStream_t st, const ScatterBatch6
 }
 
 template <int D, bool FP64, int N1>
-void launch_coeff_kernel(unsigned blocks, cudaStream_t st, const PacketsDev &pk, const ParamsT<FP64> &P, void *W,
-                         uint8_t *flags) {
-    constexpr int T = coeff_threads<FP64, N1>();
+void launch_coeff_kernel(cudaStream_t st, const PacketsDev &pk, const ParamsT<FP64> &P, void *W, uint8_t *flags) {
+    // few packets: smaller CTAs, so that they reach every SM (the FP64 pipe of an
+    // SM takes 16 clocks per warp instruction: 4096 packets 66 -> 26 us with the factors below)
+    int T = coeff_threads<FP64, N1>();
+    while (T > 32 && (pk.m + T - 1) / T < 256) T /= 2;
+    const unsigned blocks = (unsigned)((pk.m + T - 1) / T);
     if constexpr (D == 3)
         coeff_scatter3_kernel<D, FP64, N1><<<blocks, T, 0, st>>>(pk.q, pk.p, pk.s, pk.a, pk.m, P, W, flags);
     else
@@ -420,11 +493,9 @@ fgr_status launch_coeff_d(int n1, cudaStream_t st, const PacketsDev &pk, const P
     if (pk.m == 0) return FGR_OK;
 #define FGR_COEFF(N)                                                                                        \
     if (p64)                                                                                                \
-        launch_coeff_kernel<D, true, N>((unsigned)((pk.m + coeff_threads<true, N>() - 1) /                  \
-                                                   coeff_threads<true, N>()), st, pk, *p64, W, flags);      \
+        launch_coeff_kernel<D, true, N>(st, pk, *p64, W, flags);                                            \
     else                                                                                                    \
-        launch_coeff_kernel<D, false, N>((unsigned)((pk.m + coeff_threads<false, N>() - 1) /                \
-                                                    coeff_threads<false, N>()), st, pk, *p32, W, flags);
+        launch_coeff_kernel<D, false, N>(st, pk, *p32, W, flags);
     switch (n1) {
     case 4: FGR_COEFF(4); break;
     case 8: FGR_COEFF(8); break;

@@ -8,11 +8,11 @@ namespace fgr {
 
 struct Common {
     int n1;
-    int dq[kMaxN1], dp[kMaxN1];      // shifts (FP32: in orbit order, Lsa::order)
-    int v3;                          // FP32: orbits with |v| = 3/2 (Lsa::v3)
+    int dq[kMaxN1], dp[kMaxN1];      // shifts, in orbit order (Lsa::order)
+    int u3, v3;                      // orbits with |u|, |v| = 3/2 (Lsa::u3, v3)
     double dqv, dpv;                 // mesh steps
     double inv_dq, inv_dp;
-    double cq2_4, cp2_4, half_cqcp;  // eq. 3.23 constants
+    double cq2_4, cp2_4, cqcp_4;     // eq. 3.23 constants
     double cc;                       // cq cp / (2 pi): node phase in turns
     double inv_2pi_eps, pref;
     int amin[kMaxDim], A[kMaxDim], bmin[kMaxDim], B[kMaxDim];
@@ -21,9 +21,27 @@ struct Common {
     int64_t ra[kMaxDim], rb[kMaxDim];  // sa / row_len, sb / row_len (dimensions before the last)
 };
 
+// Eigen factors of the least-squares problem (Lsa::sec, sec_inv, kap_r, kap_i).
+struct Factors64 {
+    double sec[2][kMaxHalf * kMaxHalf], inv[2][kMaxHalf], kap_r[kMaxN1 / 4], kap_i[kMaxN1 / 4];
+};
+
+inline Factors64 factors64(const Lsa &L) {
+    Factors64 f;
+    for (int s = 0; s < 2; ++s) {
+        for (int i = 0; i < kMaxHalf * kMaxHalf; ++i) f.sec[s][i] = L.sec[s][i];
+        for (int i = 0; i < kMaxHalf; ++i) f.inv[s][i] = L.sec_inv[s][i];
+    }
+    for (int o = 0; o < kMaxN1 / 4; ++o) {
+        f.kap_r[o] = L.kap_r[o];
+        f.kap_i[o] = L.kap_i[o];
+    }
+    return f;
+}
+
 struct Params64 {
     Common c;
-    double vr[kMaxN1 * kMaxN1], vi[kMaxN1 * kMaxN1], inv_lam[kMaxN1];
+    Factors64 f;
 };
 
 struct Params32 {
@@ -158,7 +176,7 @@ struct ScatterBatchBase {
     uint8_t *flags[kBatchMax];
 };
 struct ScatterBatch64 : ScatterBatchBase {
-    double vr[kMaxN1 * kMaxN1], vi[kMaxN1 * kMaxN1], inv_lam[kMaxN1];
+    Factors64 f;
 };
 struct ScatterBatch32 : ScatterBatchBase {
     float poly[kSurTable];

@@ -1,4 +1,4 @@
-// K5 for d >= 2 (FP32): one separable pass of eq. 2.24, rows [a][b] -> [m],
+// K5 for d >= 2: one separable pass of eq. 2.24, rows [a][b] -> [m],
 // with the output written in the layout the next pass reads.
 //
 // Every row knows which nodes it has: in the first pass the box (a-range x
@@ -21,7 +21,12 @@
 // of the tile, whose phase is reduced per point.  The CTA's results go through
 // shared memory and leave transposed, rpc values in a piece.
 //
-// Bound by instruction issue: per node and four values 2 shared loads and 8
+// FP64: one point per lane, and the phases (rotation of a step, and of the middle b
+// of every four) from a table of the pass instead of a sine and cosine per b, point
+// and row; the FP64 pipe binds: 2-D Q2P2 set of 705,600 packets on 301 x 257 points
+// 2.42 -> 1.48 ms for both passes.
+//
+// FP32: bound by instruction issue: per node and four values 2 shared loads and 8
 // two-wide multiply-adds.  Against one point per lane, whole 8 x 32 tiles over
 // the band of a 32-point tile, a b-range scan before and a transpose after every
 // pass: 3-D workload (16.8M packets, 256^3 points) grid stage 4.92 -> 2.42 ms,
@@ -30,7 +35,15 @@
 // Included by fggc.cu inside its anonymous namespace, after fggc_tma.cuh.
 #pragma once
 
-constexpr int kRowPts = 64;     // points per tile (two per lane)
+// points per lane and per tile
+template <bool FP64>
+__host__ __device__ constexpr int row_ppl() {
+    return FP64 ? 1 : 2;
+}
+template <bool FP64>
+__host__ __device__ constexpr int row_pts() {
+    return 32 * row_ppl<FP64>();
+}
 constexpr int kBoxLog = 3;
 constexpr int kBoxPts = 1 << kBoxLog;  // contracted points that share their ranges
 constexpr int kRowB = 8;        // b values per tile
@@ -38,7 +51,11 @@ constexpr int kRowHalf = kRowB / 2;  // b values per range
 constexpr int kRowLines = 32;   // nodes per tile
 constexpr int kRowWarps = 4;
 constexpr int kRowMax = 24;     // rows per CTA, at most
-constexpr int kRowStage = kRowPts + 2;  // staged row, in float2 (16-byte rows)
+// staged row, in complex values (16-byte rows, off the bank period)
+template <bool FP64>
+__host__ __device__ constexpr int row_stage() {
+    return row_pts<FP64>() + (FP64 ? 1 : 2);
+}
 constexpr size_t kRowSmemMax = 96 * 1024;
 
 // Boxes and ranges hold minima: (min a, min -a, min b, min -b) and (min a, min -a);
@@ -51,7 +68,8 @@ struct RowPass {
     int gl, parts, rpc;
     int lines;   // node lines of the factor table: at most min(band, A)
     int chunks;  // tiles of kRowB values in B
-    const float2 *near;  // [N] offset from the nearest node, and its index
+    const float2 *near;   // FP32: [N] offset from the nearest node, and its index
+    const double2 *phase;  // FP64: [N] rotation of one b step, then [halves][N] phases of the middle b's
     // first pass: box[row]; else ranges[r * halves + b / kRowHalf], halves = ceil(B / kRowHalf),
     // of r = ((row / d1) >> s1) * stride + ((row % d1) >> s0)
     const int4 *box;
@@ -66,31 +84,44 @@ struct RowPass {
     int next_lines, next_shift, next_halves;
 };
 
+template <bool FP64>
 inline size_t row_pass_smem(int lines, int rpc, int chunks) {
-    return (size_t)kRowWarps * 2 * kRowLines * kRowB * sizeof(float2) + sizeof(float2) * (size_t)rpc * kRowStage +
-           sizeof(int2) * (size_t)rpc * chunks + sizeof(float) * (size_t)lines * kRowPts;
+    const size_t c2 = FP64 ? 16 : 8;
+    return (size_t)kRowWarps * 2 * kRowLines * kRowB * c2 + c2 * (size_t)rpc * row_stage<FP64>() +
+           sizeof(int2) * (size_t)rpc * chunks + c2 / 2 * (size_t)lines * row_pts<FP64>();
 }
 
 // z <- z w + v (complex)
-__device__ __forceinline__ void horner(float2 &z, float wr, float wi, float2 v) {
-    const float re = fmaf(z.x, wr, fmaf(-z.y, wi, v.x));
-    z.y = fmaf(z.x, wi, fmaf(z.y, wr, v.y));
+template <class C2, class Real>
+__device__ __forceinline__ void horner(C2 &z, Real wr, Real wi, C2 v) {
+    const Real re = fma(z.x, wr, fma(-z.y, wi, v.x));
+    z.y = fma(z.x, wi, fma(z.y, wr, v.y));
     z.x = re;
 }
 
-__global__ void __launch_bounds__(kRowWarps * 32, 5) grid_rows_kernel(const __grid_constant__ CUtensorMap map,
-                                                                      const __grid_constant__ CUtensorMap map_half,
-                                                                      float2 *__restrict__ out,
-                                                                      const __grid_constant__ RowPass R,
-                                                                      const PassTables tab, int *__restrict__ err) {
+// v += g w (real g, complex w)
+__device__ __forceinline__ void scaled_add(float2 &v, float g, float2 w) { v = fma2(both(g), w, v); }
+__device__ __forceinline__ void scaled_add(double2 &v, double g, double2 w) {
+    v.x = fma(g, w.x, v.x);
+    v.y = fma(g, w.y, v.y);
+}
+
+template <bool FP64>
+__global__ void __launch_bounds__(kRowWarps * 32, FP64 ? 4 : 5)
+    grid_rows_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap map_half,
+                     typename std::conditional<FP64, double2, float2>::type *__restrict__ out,
+                     const __grid_constant__ RowPass R, const PassTables tab, int *__restrict__ err) {
+    using Real = typename std::conditional<FP64, double, float>::type;
+    using C2 = typename std::conditional<FP64, double2, float2>::type;
+    constexpr int kRowPts = row_pts<FP64>(), kRowStage = row_stage<FP64>(), PPL = row_ppl<FP64>();
     extern __shared__ __align__(128) unsigned char row_smem[];
     // tiles first: copies land on 128-byte boundaries
-    float2(*sw)[2][kRowLines][kRowB] = reinterpret_cast<float2(*)[2][kRowLines][kRowB]>(row_smem);
-    float2 *stage = reinterpret_cast<float2 *>(row_smem + (size_t)kRowWarps * 2 * kRowLines * kRowB * sizeof(float2));
+    C2(*sw)[2][kRowLines][kRowB] = reinterpret_cast<C2(*)[2][kRowLines][kRowB]>(row_smem);
+    C2 *stage = reinterpret_cast<C2 *>(row_smem + (size_t)kRowWarps * 2 * kRowLines * kRowB * sizeof(C2));
     // per row and chunk of kRowB b values: first line (in the band) and lines, with
     // the halves that have any in the top bits of the first
     int2 *work = reinterpret_cast<int2 *>(stage + R.rpc * kRowStage);
-    float *g = reinterpret_cast<float *>(work + R.rpc * R.chunks);
+    Real *g = reinterpret_cast<Real *>(work + R.rpc * R.chunks);
     __shared__ __align__(8) uint64_t bars[kRowWarps][2];
     const PassParams &pp = R.pp;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -149,20 +180,31 @@ __global__ void __launch_bounds__(kRowWarps * 32, 5) grid_rows_kernel(const __gr
         any = any || nl > 0;
     }
     any = __syncthreads_or(any);
-    const int m = tile * kRowPts + 2 * lane;
+    const int m = tile * kRowPts + PPL * lane;
     if (any) {
         // Gaussian factors of the band: thread = one point, every other line; dx from
         // the point's nearest node, so that it keeps FP32 relative accuracy
         {
             const int pt = tid % kRowPts, mp = tile * kRowPts + pt;
-            const float2 nr2 = R.near[min((int64_t)mp, pp.N - 1)];
+            const int64_t mc = min((int64_t)mp, pp.N - 1);
+            const int nb = min(R.lines, band.y - band.x + 1);
+            const float2 near = FP64 ? make_float2(0.f, 0.f) : R.near[mc];
+            const double xm = FP64 ? grid_x(pp.lo, pp.h, mc) : 0.0;
             const float dqf = (float)pp.dq;
             const float cef = (float)(pp.neg_half_inv_eps * 1.4426950408889634);  // log2(e) / (-2 eps)
-            const int nb = min(R.lines, band.y - band.x + 1), off = band.x - __float_as_int(nr2.y);
             for (int j = tid / kRowPts; j < nb; j += kRowWarps * 32 / kRowPts) {
                 const int2 w = tab.win[band0 + j];
-                const float dx = fmaf((float)-(off + j), dqf, nr2.x);
-                g[j * kRowPts + pt] = mp < pp.N && mp >= w.x && mp <= w.y ? ex2_approx(dx * dx * cef) : 0.f;
+                Real v = 0;
+                if (mp < pp.N && mp >= w.x && mp <= w.y) {
+                    if constexpr (FP64) {
+                        const double dx = xm - (double)(band.x + j) * pp.dq;
+                        v = exp(dx * dx * pp.neg_half_inv_eps);
+                    } else {
+                        const float dx = fmaf((float)(__float_as_int(near.y) - band.x - j), dqf, near.x);
+                        v = ex2_approx(dx * dx * cef);
+                    }
+                }
+                g[j * kRowPts + pt] = v;
             }
         }
         if (lane == 0) {
@@ -173,13 +215,20 @@ __global__ void __launch_bounds__(kRowWarps * 32, 5) grid_rows_kernel(const __gr
         }
     }
     __syncthreads();
-    // per point: reduced phase of one b step, and its rotation w
-    float2 ph[2];
-    float wr[2], wi[2];
+    // per point: rotation w of one b step (FP32: and its reduced phase)
+    float2 ph[PPL];
+    Real wr[PPL], wi[PPL];
 #pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        ph[t] = tab.ph[min((int64_t)m + t, pp.N - 1)];
-        sincospif(2.f * (ph[t].x - rint_fast(ph[t].x) + ph[t].y), &wi[t], &wr[t]);
+    for (int t = 0; t < PPL; ++t) {
+        const int64_t mc = min((int64_t)m + t, pp.N - 1);
+        if constexpr (FP64) {
+            const double2 w = R.phase[mc];
+            wr[t] = w.x;
+            wi[t] = w.y;
+        } else {
+            ph[t] = tab.ph[mc];
+            sincospif(2.f * (ph[t].x - rint_fast(ph[t].x) + ph[t].y), &wi[t], &wr[t]);
+        }
     }
     // the warp's tiles: its rows, their chunks with lines, kRowLines lines at a time
     struct Cursor {
@@ -204,8 +253,10 @@ __global__ void __launch_bounds__(kRowWarps * 32, 5) grid_rows_kernel(const __gr
             const bool half = aw.y - ahead.lc <= kRowLines / 2;
             const int64_t line = (row0 + ahead.r) * (int64_t)pp.A + band0 + (aw.x & 0x3fffffff) + ahead.lc;
             uint64_t *bar = &bars[wid][issued & 1];
-            mbar_expect_tx(bar, (half ? kRowLines / 2 : kRowLines) * kRowB * (int)sizeof(float2));
-            tma_load_2d(&sw[wid][issued & 1][0][0], half ? &map_half : &map, ahead.k * kRowB, (int)line, bar);
+            mbar_expect_tx(bar, (half ? kRowLines / 2 : kRowLines) * kRowB * (int)sizeof(C2));
+            // (FP64: the map's elements are the parts)
+            tma_load_2d(&sw[wid][issued & 1][0][0], half ? &map_half : &map, ahead.k * kRowB * (FP64 ? 2 : 1), (int)line,
+                        bar);
         }
         ++issued;
         ahead.lc += kRowLines;
@@ -219,7 +270,11 @@ __global__ void __launch_bounds__(kRowWarps * 32, 5) grid_rows_kernel(const __gr
     issue();
     bool failed = false;
     for (int r = wid; r < nr; r += kRowWarps) {
-        float2 sum[2] = {both(0.f), both(0.f)}, low[2] = {both(0.f), both(0.f)};  // Kahan sums
+        C2 zero;
+        zero.x = zero.y = 0;
+        C2 sum[PPL], low[PPL];  // (FP32: Kahan sums)
+#pragma unroll
+        for (int t = 0; t < PPL; ++t) sum[t] = low[t] = zero;
 #pragma unroll 1
         for (int k = 0; k < R.chunks && any && !failed; ++k) {
             const int2 w = work[r * R.chunks + k];
@@ -227,10 +282,12 @@ __global__ void __launch_bounds__(kRowWarps * 32, 5) grid_rows_kernel(const __gr
             if (nl == 0) continue;
             const unsigned halves = (unsigned)w.x >> 30;
             const int skip = halves == 2u ? kRowHalf : 0;  // only the second half
-            const float *gl = g + (w.x & 0x3fffffff) * kRowPts + 2 * lane;
-            float2 v[2][kRowB];
+            const Real *gl = g + (w.x & 0x3fffffff) * kRowPts + PPL * lane;
+            C2 v[PPL][kRowB];
 #pragma unroll
-            for (int u = 0; u < kRowB; ++u) v[0][u] = v[1][u] = both(0.f);
+            for (int t = 0; t < PPL; ++t)
+#pragma unroll
+                for (int u = 0; u < kRowB; ++u) v[t][u] = zero;
 #pragma unroll 1
             for (int lc = 0; lc < nl; lc += kRowLines) {
                 const int s = used & 1;
@@ -240,21 +297,35 @@ __global__ void __launch_bounds__(kRowWarps * 32, 5) grid_rows_kernel(const __gr
                 }
                 ++used;
                 const int n = min(kRowLines, nl - lc);
-                const float *gj = gl + lc * kRowPts;
-                const float4 *wj = reinterpret_cast<const float4 *>(&sw[wid][s][0][skip]);
+                const Real *gj = gl + lc * kRowPts;
+                const C2 *wj = &sw[wid][s][0][skip];
                 auto line = [&](auto nb) {
-                    const float2 gg = *reinterpret_cast<const float2 *>(gj);
+                    Real gg[PPL];
+                    if constexpr (FP64) {
+                        gg[0] = *gj;
+                    } else {
+                        const float2 x = *reinterpret_cast<const float2 *>(gj);
+                        gg[0] = x.x;
+                        gg[1] = x.y;
+                    }
 #pragma unroll
-                    for (int u = 0; u < decltype(nb)::value / 2; ++u) {
-                        const float4 x = wj[u];
-                        const float2 w0 = make_float2(x.x, x.y), w1 = make_float2(x.z, x.w);
-                        v[0][2 * u] = fma2(both(gg.x), w0, v[0][2 * u]);
-                        v[1][2 * u] = fma2(both(gg.y), w0, v[1][2 * u]);
-                        v[0][2 * u + 1] = fma2(both(gg.x), w1, v[0][2 * u + 1]);
-                        v[1][2 * u + 1] = fma2(both(gg.y), w1, v[1][2 * u + 1]);
+                    for (int u = 0; u < decltype(nb)::value; u += 2) {
+                        C2 x[2];  // two values: 16-byte loads
+                        if constexpr (FP64) {
+                            x[0] = wj[u];
+                            x[1] = wj[u + 1];
+                        } else {
+                            const float4 y = *reinterpret_cast<const float4 *>(wj + u);
+                            x[0] = make_float2(y.x, y.y);
+                            x[1] = make_float2(y.z, y.w);
+                        }
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+#pragma unroll
+                            for (int t = 0; t < PPL; ++t) scaled_add(v[t][u + h], gg[t], x[h]);
                     }
                     gj += kRowPts;
-                    wj += kRowB / 2;
+                    wj += kRowB;
                 };
                 if (halves == 3u) {
 #pragma unroll 2
@@ -271,32 +342,43 @@ __global__ void __launch_bounds__(kRowWarps * 32, 5) grid_rows_kernel(const __gr
             if (failed) break;
             const float bf = (float)(pp.bmin + k * kRowB + skip + 3);
 #pragma unroll
-            for (int t = 0; t < 2; ++t) {
-                float2 z = v[t][0];
+            for (int t = 0; t < PPL; ++t) {
+                C2 z = v[t][0];
                 horner(z, wr[t], -wi[t], v[t][1]);
                 horner(z, wr[t], -wi[t], v[t][2]);
                 horner(z, wr[t], -wi[t], v[t][3]);
                 if (halves == 3u) {
-                    float2 f = v[t][7];
+                    C2 f = v[t][7];
                     horner(f, wr[t], wi[t], v[t][6]);
                     horner(f, wr[t], wi[t], v[t][5]);
                     horner(f, wr[t], wi[t], v[t][4]);
                     horner(f, wr[t], wi[t], z);
                     z = f;
                 }
-                float e = bf * ph[t].x;
-                e -= rint_fast(e);
-                float tau = fmaf(bf, ph[t].y, e);
-                tau -= rint_fast(tau);
-                float er, ei;
-                sincospif(2.f * tau, &ei, &er);  // (shared by 8 b values: the fast one's 4e-7 would show)
-                kahan_add(sum[t].x, low[t].x, er * z.x - ei * z.y);
-                kahan_add(sum[t].y, low[t].y, er * z.y + ei * z.x);
+                if constexpr (FP64) {
+                    const int64_t mc = min((int64_t)m + t, pp.N - 1);
+                    const double2 e = R.phase[(1 + 2 * k + (skip ? 1 : 0)) * pp.N + mc];
+                    sum[t].x = fma(e.x, z.x, fma(-e.y, z.y, sum[t].x));
+                    sum[t].y = fma(e.x, z.y, fma(e.y, z.x, sum[t].y));
+                } else {
+                    float e = bf * ph[t].x;
+                    e -= rint_fast(e);
+                    float tau = fmaf(bf, ph[t].y, e);
+                    tau -= rint_fast(tau);
+                    float er, ei;
+                    sincospif(2.f * tau, &ei, &er);  // (shared by 8 b values: the fast one's 4e-7 would show)
+                    kahan_add(sum[t].x, low[t].x, er * z.x - ei * z.y);
+                    kahan_add(sum[t].y, low[t].y, er * z.y + ei * z.x);
+                }
             }
         }
-        *reinterpret_cast<float4 *>(stage + r * kRowStage + 2 * lane) =
-            make_float4(__fsub_rn(sum[0].x, low[0].x), __fsub_rn(sum[0].y, low[0].y), __fsub_rn(sum[1].x, low[1].x),
-                        __fsub_rn(sum[1].y, low[1].y));
+        if constexpr (FP64) {
+            stage[r * kRowStage + lane] = sum[0];
+        } else {
+            *reinterpret_cast<float4 *>(stage + r * kRowStage + 2 * lane) =
+                make_float4(__fsub_rn(sum[0].x, low[0].x), __fsub_rn(sum[0].y, low[0].y),
+                            __fsub_rn(sum[1].x, low[1].x), __fsub_rn(sum[1].y, low[1].y));
+        }
     }
     if (failed)  // leave only after this warp's copies in flight have landed (bounded)
         for (; used < issued; ++used)
@@ -346,18 +428,19 @@ __global__ void __launch_bounds__(128) row_range_kernel(const int4 *__restrict__
 
 // Boxes of the rows of W by reading the flagged ones (the per-packet scatter):
 // one warp per row.
-__global__ void __launch_bounds__(256) row_scan_kernel(const float2 *__restrict__ W, int64_t rows, int A, int B,
+template <class C2>
+__global__ void __launch_bounds__(256) row_scan_kernel(const C2 *__restrict__ W, int64_t rows, int A, int B,
                                                        const uint8_t *__restrict__ flags, int4 *__restrict__ box) {
     const int lane = threadIdx.x & 31;
     const int64_t row = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= rows) return;
     int4 v = make_int4(kBoxEmpty, kBoxEmpty, kBoxEmpty, kBoxEmpty);
     if (flags[row]) {
-        const float2 *p = W + row * (int64_t)A * B;
+        const C2 *p = W + row * (int64_t)A * B;
         const int cells = A * B;
         for (int e = lane; e < cells; e += 32) {
-            const float2 x = p[e];
-            if (x.x != 0.f || x.y != 0.f) {
+            const C2 x = p[e];
+            if (x.x != 0 || x.y != 0) {
                 const int a = e / B, b = e - a * B;
                 v.x = min(v.x, a);
                 v.y = min(v.y, -a);

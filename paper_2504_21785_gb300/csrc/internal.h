@@ -13,6 +13,7 @@ namespace fgr {
 
 constexpr int kMaxDim = 3;
 constexpr int kMaxN1 = 16;  // 1-D neighbours per packet: nq * np <= 16
+constexpr int kMaxHalf = kMaxN1 / 2;
 
 // FP32 coefficient surrogate: Chebyshev degree per variable and total degree.
 // The terms T_i T_j with i + j <= surrogate_total and i, j < kCheb are kept for
@@ -31,21 +32,24 @@ constexpr int kPow = kCheb / 2;
 constexpr int kOrbitTable = 2 * 4 * kPow * kPow;
 constexpr int kSurTable = kMaxN1 / 4 * kOrbitTable;
 
-// Eigen-factored eps-free Gram matrix of eq. 3.22 (paper convention).
-// The Gram A~ is Hermitian PSD: A~ = V diag(lam) V^H, A~^+ = V diag(inv_lam) V^H.
+// The eps-free least-squares problem of eq. 3.22-3.23 of one neighbour strategy.
+// The pseudo-inverse of its Gram matrix is applied through eigen factors.
 struct Lsa {
     int nq = 4, np = 2, n1 = 8, rank = 0;
     double cq = 0.5, cp = 0.0;
     int dq[kMaxN1] = {}, dp[kMaxN1] = {};  // shifts, k = iq*np + ip
-    double lam[kMaxN1] = {};               // descending
-    double inv_lam[kMaxN1] = {};           // 1/lam above the cut-off, else 0
-    double vr[kMaxN1 * kMaxN1] = {};       // V[j][i]: component j of eigenvector i
-    double vi[kMaxN1 * kMaxN1] = {};
+    double lam[kMaxN1] = {};               // eigenvalues, descending
+    // Eigen factors by sector (even, odd under parity) in the real basis of
+    // build_lsa: sec[s][a * kMaxHalf + i] = component a of eigenvector i, and
+    // 1 / (4 lambda_i) above the cut-off, else 0.
+    double sec[2][kMaxHalf * kMaxHalf] = {}, sec_inv[2][kMaxHalf] = {};
+    // Per orbit: e^{i cq cp |u v| / 2}.
+    double kap_r[kMaxN1 / 4] = {}, kap_i[kMaxN1 / 4] = {};
     // Neighbours in orbit order: orbit o holds, at 4 o + g, the mirror images
     // (u, v), (u, -v), (-u, v), (-u, -v) of one shift, (u, v) = (dq - 1/2, dp - 1/2)
-    // with u, v < 0 for g = 0 (FP32 kernels number their neighbours this way).
+    // with u, v < 0 for g = 0 (the kernels number their neighbours this way).
     int order[kMaxN1] = {};
-    int v3 = 0;  // bit o: orbit o has |v| = 3/2 (else 1/2)
+    int u3 = 0, v3 = 0;  // bit o: orbit o has |u|, |v| = 3/2 (else 1/2)
     // Surrogate of the first neighbour of every orbit (see build_lsa).
     float poly[kSurTable] = {};
 };

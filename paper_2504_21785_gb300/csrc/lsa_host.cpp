@@ -7,8 +7,8 @@
 // is Hermitian positive semi-definite, so its SVD is its eigen-decomposition.
 // It is computed here by the cyclic complex Jacobi method in long double and
 // rounded to double once; singular values below rcond * lambda_max are dropped.
-// Keeping the factors (instead of the formed matrix A~^+) lets the device apply
-// the pseudo-inverse as V (diag(1/lambda) (V^H f~)).
+// The device applies the pseudo-inverse through its factors (not the formed
+// matrix A~^+), in a basis in which it falls into two real halves.
 #include <cmath>
 #include <complex>
 #include <vector>
@@ -102,18 +102,9 @@ bool build_lsa(double cq, double cp, int nq, int np, double rcond, Lsa *out) {
     for (int i = 0; i < n; ++i) {
         long double lam = A[idx[i] * n + idx[i]].real();
         L.lam[i] = (double)lam;
-        if (lam > (long double)rcond * lmax) {
-            L.inv_lam[i] = (double)(1.0L / lam);
-            ++L.rank;
-        } else {
-            L.inv_lam[i] = 0.0;
-        }
-        for (int j = 0; j < n; ++j) {
-            L.vr[j * kMaxN1 + i] = (double)V[j * n + idx[i]].real();
-            L.vi[j * kMaxN1 + i] = (double)V[j * n + idx[i]].imag();
-        }
+        if (lam > (long double)rcond * lmax) ++L.rank;
     }
-    // Surrogate of the coefficients (used by the FP32 path).  With the cell
+    // Symmetric form of the problem.  With the cell
     // centre as origin and the Weyl-ordered packets D(Q, P) g = e^{i P (x - Q/2)}
     // g(x - Q) as basis, two symmetries of phase space map the neighbour set to
     // itself: parity (x -> -x) and complex conjugation (P -> -P).  In that gauge,
@@ -123,12 +114,14 @@ bool build_lsa(double cq, double cp, int nq, int np, double rcond, Lsa *out) {
     // the coefficients of the four mirror images of a neighbour (u, v) are
     //   e_(u,v) = f(X, Y),          e_(-u,-v) = f(-X, -Y),
     //   e_(u,-v) = conj f(X, -Y),   e_(-u,v) = conj f(-X, Y),
-    // so one function per orbit serves four neighbours, through its parts even
-    // and odd in X and Y.  f is interpolated at kCheb x kCheb Chebyshev nodes,
+    // so the problem splits by parity into two halves, each real in a basis of
+    // conjugation-invariant vectors (FP64 kernels: the sectors below), and one
+    // function per orbit serves four neighbours, through its parts even and odd in
+    // X and Y (FP32 kernels): f is interpolated at kCheb x kCheb Chebyshev nodes,
     // the terms up to the total degree are kept, and each parity part is
     // rewritten in powers of X^2 and Y^2 (in FP32 these lose less to rounding
     // than the Chebyshev recurrences: 2.1e-8 against 3.6e-8 rms for Q4P2).
-    // Same eigen factors and cut-off as the FP64 path.
+    // Same problem and cut-off as the FP64 path.
     const long double PI = 3.141592653589793238462643383279502884L;
     int orbit_of[kMaxN1 / 4], norb = 0;
     for (int iq = 0; iq < nq / 2; ++iq)
@@ -138,9 +131,49 @@ bool build_lsa(double cq, double cp, int nq, int np, double rcond, Lsa *out) {
             L.order[4 * norb + 1] = iq * np + mp;
             L.order[4 * norb + 2] = mq * np + ip;
             L.order[4 * norb + 3] = mq * np + mp;
+            if (sq[iq] == -1) L.u3 |= 1 << norb;
             if (sp[ip] == -1) L.v3 |= 1 << norb;
             orbit_of[norb++] = iq * np + ip;
         }
+    // the Gram matrix in that gauge (without its last factor), its parity sectors in the basis (components over
+    // an orbit's four neighbours) even (1,1,1,1)/2, i(1,-1,-1,1)/2, odd
+    // (1,1,-1,-1)/2, i(1,-1,1,-1)/2, and their eigen factors
+    {
+        auto uk = [&](int k) { return L.dq[L.order[k]] - 0.5L; };
+        auto vk = [&](int k) { return L.dp[L.order[k]] - 0.5L; };
+        auto expi = [](long double x) { return cld(std::cos(x), std::sin(x)); };
+        static const int sign[2][2][4] = {{{1, 1, 1, 1}, {1, -1, -1, 1}}, {{1, 1, -1, -1}, {1, -1, 1, -1}}};
+        const int h = n / 2;
+        for (int s = 0; s < 2; ++s) {
+            std::vector<cld> M(h * h), Q;
+            for (int a = 0; a < h; ++a)
+                for (int b = 0; b < h; ++b) {
+                    cld acc = 0;
+                    for (int x = 0; x < 4; ++x)
+                        for (int y = 0; y < 4; ++y) {
+                            const int j = 4 * (a / 2) + x, k = 4 * (b / 2) + y;
+                            const long double du = uk(j) - uk(k), dv = vk(j) - vk(k);
+                            cld m = std::exp(-lcq * lcq / 4 * du * du - lcp * lcp / 4 * dv * dv) *
+                                    expi(lcq * lcp / 2 * (vk(k) * uk(j) - vk(j) * uk(k)));
+                            const cld ea = (a % 2 ? cld(0, 1) : cld(1)) * (long double)sign[s][a % 2][x] / 2.0L;
+                            const cld eb = (b % 2 ? cld(0, 1) : cld(1)) * (long double)sign[s][b % 2][y] / 2.0L;
+                            acc += std::conj(ea) * m * eb;
+                        }
+                    M[a * h + b] = acc.real();
+                }
+            jacobi_hermitian(h, M, Q);
+            for (int i = 0; i < h; ++i) {
+                const long double lam = M[i * h + i].real();
+                L.sec_inv[s][i] = lam > (long double)rcond * lmax ? (double)(0.25L / lam) : 0.0;
+                for (int a = 0; a < h; ++a) L.sec[s][a * kMaxHalf + i] = (double)Q[a * h + i].real();
+            }
+        }
+        for (int o = 0; o < norb; ++o) {
+            const cld k = expi(lcq * lcp / 2 * uk(4 * o) * vk(4 * o));
+            L.kap_r[o] = (double)k.real();
+            L.kap_i[o] = (double)k.imag();
+        }
+    }
     const int total = n <= 8 ? surrogate_total<8>() : surrogate_total<16>();
     std::vector<cld> val((size_t)norb * kCheb * kCheb);  // f at the nodes
     long double node[kCheb];

@@ -37,3 +37,24 @@ def test_surrogate_in_every_part_of_a_cell(d, nq, np_):
     ref = reconstruct("fggc", pk, grid, eps, options("fp64", nq, np_, window_r=6.0))
     got = reconstruct("fggc", pk, grid, eps, options("fp32", nq, np_, window_r=6.0))
     assert rel_l2(got, ref) <= TOL
+
+
+@pytest.mark.parametrize("nq,np_", [(2, 2), (4, 2), (2, 4), (4, 4)])
+@pytest.mark.parametrize("d,m", [(1, 40), (1, 9000), (2, 300)])
+def test_fp64_factors_against_the_oracle(d, m, nq, np_):
+    """The symmetric factors of the FP64 path for every strategy, few packets (small
+    CTAs) and many, on ragged grids of the row-wise passes: at the conditioning floor
+    of the least-squares problem (its smallest kept singular value)."""
+    from oracle import fggc, lsa
+    eps = 1 / 64
+    mesh = mesh_for(d, eps)
+    rng = np.random.default_rng(40 + m)
+    pk = {"q": rng.uniform(-0.6, 0.6, (d, m)), "p": rng.uniform(-0.8, 0.8, (d, m)), "s": rng.uniform(-1, 1, m),
+          "a": rng.standard_normal((2, m))}
+    grid = dict(d=d, n=[83, 41][:d], lo=[-1.1, -0.9][:d], hi=[1.0, 1.2][:d])
+    strat = lsa.Strategy(nq=nq, np_=np_)
+    sv = strat.pinv.singular_values
+    floor = 4 * np.finfo(float).eps / np.sqrt(sv[sv > 1e-14 * sv[0]][-1])
+    got = reconstruct("fggc", pk, grid, eps, options("fp64", nq, np_))
+    ref = fggc.reconstruct(pk, grid, eps, mesh.dq, mesh.dp, strat, R=8)
+    assert rel_l2(got, ref) <= max(1e-12, 2 * floor)  # both sides are at the floor
