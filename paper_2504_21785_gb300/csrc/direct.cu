@@ -615,6 +615,16 @@ __device__ __forceinline__ void direct_tile(const void *__restrict__ recs_v, con
     }
 }
 
+// Compensated summation (Kahan): s += x, the negated rounding error kept in c; the
+// sum is s - c.
+__device__ __forceinline__ void kahan_sum(float &s, float &c, float x) {
+    const float y = __fsub_rn(x, c), t = __fadd_rn(s, y);
+    c = __fsub_rn(__fsub_rn(t, s), y);
+    s = t;
+}
+
+#include "direct_1d.cuh"
+
 template <int D, bool FP64>
 __global__ void __launch_bounds__(kThreads) direct_kernel(const void *__restrict__ recs_v,
                                                           const int64_t *__restrict__ off,
@@ -1004,6 +1014,26 @@ fgr_status launch_tc(fgr_ctx *ctx, const Prepared &pr, void *u_dev, cudaStream_t
     return FGR_OK;
 }
 
+// The 1-D FP32 sum on grids that resolve the Gaussian: slices of every tile's list
+// into partial sums, then their sum.  Four slices of 128 threads for the one of 256
+// of direct_kernel even out the tiles' lists (the whole call on the 1-D workload: two 389, four 370, six 364 us).
+fgr_status launch_1d(fgr_ctx *ctx, const Prepared &pr, void *u_dev, cudaStream_t st, Scratch &scratch,
+                     StageTimer &timer) {
+    const int slices = 4 * pr.P.splits;
+    const int64_t stride = (int64_t)pr.ntiles * tileT<1>(0);
+    auto *part = (float2 *)scratch.get(sizeof(float2) * (size_t)(slices * stride));
+    if (!part) return FGR_E_NOMEM;
+    direct1_kernel<<<dim3((unsigned)pr.ntiles, (unsigned)slices), kD1Threads, 0, st>>>(
+        reinterpret_cast<const RecF<1> *>(pr.recs), pr.off, pr.P, part);
+    direct1_sum_kernel<<<(unsigned)((ctx->grid.n[0] + 127) / 128), 128, 0, st>>>(part, slices, stride, ctx->grid.n[0],
+                                                                              reinterpret_cast<float2 *>(u_dev));
+    FGR_CUDA_TRY(cudaGetLastError());
+    timer.mark(&ctx->timing.last.direct_ms);
+    ctx->timing.last.launches = 5;
+    timer.finish();
+    return FGR_OK;
+}
+
 template <int D>
 fgr_status launch(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStream_t st, Scratch &scratch) {
     const bool fp64 = ctx->opt.precision == FGR_FP64;
@@ -1021,6 +1051,8 @@ fgr_status launch(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStream_t 
         dim3 grid((unsigned)pr.ntiles, (unsigned)pr.P.splits);
         if (fp64)
             direct_kernel<D, true><<<grid, kThreads, 0, st>>>(pr.recs, pr.off, pr.P, u_dev);
+        else if (4.0 * ctx->grid.h[0] <= std::sqrt(ctx->mesh.eps))  // see direct_1d.cuh
+            return launch_1d(ctx, pr, u_dev, st, scratch, timer);
         else
             direct_kernel<D, false><<<grid, kThreads, 0, st>>>(pr.recs, pr.off, pr.P, u_dev);
         FGR_CUDA_TRY(cudaGetLastError());
