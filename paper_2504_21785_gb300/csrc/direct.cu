@@ -542,10 +542,11 @@ __device__ __forceinline__ void direct_tile(const void *__restrict__ recs_v, con
                     accd[r][1] += Rd.ar * gi + Rd.ai * gr;
                 }
             } else {
-                // the first point evaluated in full, the next kTpt - 1 along
-                // the last dimension by the exact recurrences of the Gaussian
-                // (ratio rho, itself multiplied by e^{-h^2/eps} per step) and of
-                // the phase (rotation by e^{2 pi i nu})
+                // the thread's first point inside the window (one before it can
+                // underflow on grids coarser than the Gaussian) evaluated in full,
+                // the next along the last dimension by the exact recurrences of the
+                // Gaussian (ratio rho, itself multiplied by e^{-h^2/eps} per step)
+                // and of the phase (rotation by e^{2 pi i nu})
                 const RecF<D> &Rf = reinterpret_cast<const RecF<D> &>(R);
                 float kk[D];
                 bool in = true;
@@ -558,6 +559,8 @@ __device__ __forceinline__ void direct_tile(const void *__restrict__ recs_v, con
                 const float wl = Rf.wlen[D - 1];
                 in = in && kk[D - 1] > -(float)kTpt && kk[D - 1] < wl;
                 if (!in) continue;
+                const float skip = fmaxf(-kk[D - 1], 0.f);  // points before the window
+                kk[D - 1] += skip;
                 float e = 0.f, tau = Rf.tau0, dxl = 0.f;
 #pragma unroll
                 for (int l = 0; l < D; ++l) {
@@ -579,8 +582,8 @@ __device__ __forceinline__ void direct_tile(const void *__restrict__ recs_v, con
                 float wr = rho * rot.x, wi = rho * rot.y;
 #pragma unroll
                 for (int r = 0; r < kTpt; ++r) {
-                    const float k = kk[D - 1] + (float)r;
-                    if (k >= 0.f && k < wl) {
+                    if ((float)r < skip) continue;
+                    if (kk[D - 1] + ((float)r - skip) < wl) {
                         accf[r][0] += vr;
                         accf[r][1] += vi;
                     }
@@ -1017,12 +1020,18 @@ fgr_status launch_tc(fgr_ctx *ctx, const Prepared &pr, void *u_dev, cudaStream_t
 // The 1-D FP32 sum on grids that resolve the Gaussian: slices of every tile's list
 // into partial sums, then their sum.  Four slices of 128 threads for the one of 256
 // of direct_kernel even out the tiles' lists (the whole call on the 1-D workload: two 389, four 370, six 364 us).
-fgr_status launch_1d(fgr_ctx *ctx, const Prepared &pr, void *u_dev, cudaStream_t st, Scratch &scratch,
+constexpr int kD1Slices = 4;
+// Partial sums (40 MB at most); null, without an error, where the memory is short:
+// direct_kernel needs none.
+float2 *partials_1d(const Prepared &pr, Scratch &scratch) {
+    auto *part = (float2 *)scratch.get(sizeof(float2) * (size_t)kD1Slices * pr.P.splits * pr.ntiles * tileT<1>(0));
+    if (!part) clear_error();
+    return part;
+}
+fgr_status launch_1d(fgr_ctx *ctx, const Prepared &pr, float2 *part, void *u_dev, cudaStream_t st,
                      StageTimer &timer) {
-    const int slices = 4 * pr.P.splits;
+    const int slices = kD1Slices * pr.P.splits;
     const int64_t stride = (int64_t)pr.ntiles * tileT<1>(0);
-    auto *part = (float2 *)scratch.get(sizeof(float2) * (size_t)(slices * stride));
-    if (!part) return FGR_E_NOMEM;
     direct1_kernel<<<dim3((unsigned)pr.ntiles, (unsigned)slices), kD1Threads, 0, st>>>(
         reinterpret_cast<const RecF<1> *>(pr.recs), pr.off, pr.P, part);
     direct1_sum_kernel<<<(unsigned)((ctx->grid.n[0] + 127) / 128), 128, 0, st>>>(part, slices, stride, ctx->grid.n[0],
@@ -1051,8 +1060,8 @@ fgr_status launch(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStream_t 
         dim3 grid((unsigned)pr.ntiles, (unsigned)pr.P.splits);
         if (fp64)
             direct_kernel<D, true><<<grid, kThreads, 0, st>>>(pr.recs, pr.off, pr.P, u_dev);
-        else if (4.0 * ctx->grid.h[0] <= std::sqrt(ctx->mesh.eps))  // see direct_1d.cuh
-            return launch_1d(ctx, pr, u_dev, st, scratch, timer);
+        else if (float2 *part = 4.0 * ctx->grid.h[0] <= std::sqrt(ctx->mesh.eps) ? partials_1d(pr, scratch) : nullptr)
+            return launch_1d(ctx, pr, part, u_dev, st, timer);  // see direct_1d.cuh
         else
             direct_kernel<D, false><<<grid, kThreads, 0, st>>>(pr.recs, pr.off, pr.P, u_dev);
         FGR_CUDA_TRY(cudaGetLastError());
