@@ -1095,7 +1095,11 @@ fgr_status fgr_fggc_plan_create(fgr_ctx *ctx, const fgr_packets *pk, int32_t mar
             BinBox bb;
             if (e == cudaSuccess && ctx->opt.precision == FGR_FP32 && make_bin_box(b, ctx->d, pk->m, &bb)) {
                 pl->buf.bin_bytes = bin_buffer_bytes(pk->m, bb);
-                e = palloc(&pl->buf.bin, pl->buf.bin_bytes);
+                if (palloc(&pl->buf.bin, pl->buf.bin_bytes) != cudaSuccess) {  // the per-packet scatter needs none
+                    cudaGetLastError();
+                    pl->buf.bin = nullptr;
+                    pl->buf.bin_bytes = 0;
+                }
             }
             if (e != cudaSuccess) return fail(e);
         }

@@ -173,6 +173,13 @@ struct PassParams {
     double dp_over_eps;
 };
 
+// v += g w (real g, complex w)
+__device__ __forceinline__ void scaled_add(float2 &v, float g, float2 w) { v = fma2(both(g), w, v); }
+__device__ __forceinline__ void scaled_add(double2 &v, double g, double2 w) {
+    v.x = fma(g, w.x, v.x);
+    v.y = fma(g, w.y, v.y);
+}
+
 constexpr int kCB = 32;
 constexpr int kSlice = 8;  // b values per unit of a b-slice (see launch_pass)
 
@@ -356,9 +363,9 @@ __device__ __forceinline__ void grid_pass_body(const void *__restrict__ in_v, vo
             }
             __syncthreads();
             for (int bb = 0; bb < nbb; bb += 2) {  // b pairs; the padding column is zero
-                Real vr[kPassPts][2], vi[kPassPts][2];
+                C2 v[kPassPts][2];
 #pragma unroll
-                for (int r = 0; r < kPassPts; ++r) vr[r][0] = vr[r][1] = vi[r][0] = vi[r][1] = 0;
+                for (int r = 0; r < kPassPts; ++r) v[r][0] = v[r][1] = zero;
 #pragma unroll
                 for (int i = 0; i < MAXBAND; ++i) {
                     if (i < nb) {
@@ -368,17 +375,13 @@ __device__ __forceinline__ void grid_pass_body(const void *__restrict__ in_v, vo
                             w1 = sw[i][bb + 1];
                         } else {  // one 16-byte shared load for the pair
                             const float4 w = *reinterpret_cast<const float4 *>(&sw[i][bb]);
-                            w0.x = w.x;
-                            w0.y = w.y;
-                            w1.x = w.z;
-                            w1.y = w.w;
+                            w0 = make_float2(w.x, w.y);
+                            w1 = make_float2(w.z, w.w);
                         }
 #pragma unroll
                         for (int r = 0; r < kPassPts; ++r) {
-                            vr[r][0] += g[r][i] * w0.x;
-                            vi[r][0] += g[r][i] * w0.y;
-                            vr[r][1] += g[r][i] * w1.x;
-                            vi[r][1] += g[r][i] * w1.y;
+                            scaled_add(v[r][0], g[r][i], w0);
+                            scaled_add(v[r][1], g[r][i], w1);
                         }
                     }
                 }
@@ -404,8 +407,8 @@ __device__ __forceinline__ void grid_pass_body(const void *__restrict__ in_v, vo
                             er = cs;
                             ei = sn;
                         }
-                        accr[r] += er * vr[r][u] - ei * vi[r][u];
-                        acci[r] += er * vi[r][u] + ei * vr[r][u];
+                        accr[r] += er * v[r][u].x - ei * v[r][u].y;
+                        acci[r] += er * v[r][u].y + ei * v[r][u].x;
                     }
                 }
             }
@@ -1505,7 +1508,10 @@ fgr_status launch(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStream_t 
     if (ctx->opt.precision == FGR_FP32 && make_bin_box(box, D, pk.m, &bb)) {
         b.bin_bytes = bin_buffer_bytes(pk.m, bb);
         b.bin = scratch.get(b.bin_bytes);
-        if (!b.bin) return FGR_E_NOMEM;
+        if (!b.bin) {  // the per-packet scatter needs none
+            clear_error();
+            b.bin_bytes = 0;
+        }
     }
     if (ctx->timing.enabled && ctx->timing.count_terms) {
         b.terms = (unsigned long long *)scratch.get(sizeof(unsigned long long));

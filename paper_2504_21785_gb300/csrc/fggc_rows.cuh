@@ -99,13 +99,6 @@ __device__ __forceinline__ void horner(C2 &z, Real wr, Real wi, C2 v) {
     z.x = re;
 }
 
-// v += g w (real g, complex w)
-__device__ __forceinline__ void scaled_add(float2 &v, float g, float2 w) { v = fma2(both(g), w, v); }
-__device__ __forceinline__ void scaled_add(double2 &v, double g, double2 w) {
-    v.x = fma(g, w.x, v.x);
-    v.y = fma(g, w.y, v.y);
-}
-
 template <bool FP64>
 __global__ void __launch_bounds__(kRowWarps * 32, FP64 ? 4 : 5)
     grid_rows_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap map_half,
