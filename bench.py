@@ -345,18 +345,25 @@ def reconstruction_roofline(d, M, nodes, kern, ms_step):
     per-stage CUDA events of the timed steps (kern: mean per stage).
 
     Scatter (K3+K4): unit = one contribution A e^{iS/eps} c_k of a packet to a
-    node (eq. 2.25), an 8-byte reduction in L2 as the method states it, M 8^d
-    per launch (Q4P2), against the best rate at which this GB300's L2 absorbs
-    8-byte reductions (a warp on 32 consecutive cells, probed); the binned 3-D
-    kernel sums a cell's contributions in registers first, so it issues fewer
-    reductions than contributions.  Grid passes (K5): unit = one node-point
+    node (eq. 2.25), M 8^d per launch (Q4P2).  The binned kernel (d >= 2) sums a
+    cell's contributions in registers: a complex multiply-add (8 FLOPs) each,
+    against the measured FP32 FMA rate.  The per-packet kernel (d = 1) issues an
+    8-byte reduction in L2 each, against the best rate at which this GB300's L2
+    absorbs them (a warp on 32 consecutive cells, probed).  Grid passes (K5): unit = one node-point
     term W[a, b] g(x_m - a dq) (a real x complex multiply-add, 4 FLOPs), counted
     on the device per launch (occupied b-range x window points over every
     (row, a) line), against the measured FP32 FMA rate."""
     contrib = M * 8 ** d
     scatter_ms, pass_ms = kern["scatter_ms"], kern["pass_ms"]
     if scatter_ms >= pass_ms:
-        out = {"kernel": "coefficient + scatter (K3+K4: binned_scatter_kernel in 3-D)", "bound": "l2",
+        out = {"kernel": "coefficient + scatter (K3+K4: binned_scatter_kernel)", "bound": "alu",
+               "achieved": 8.0 * contrib / (scatter_ms * 1e-3) / 1e12, "peak": FP32_PEAK_TFLOPS,
+               "unit": "TFLOP/s", "traffic": SCATTER_TRAFFIC_BYTES.get((d, M)),
+               "launch_ms": scatter_ms, "units_per_launch": contrib,
+               "unit_def": "one contribution of a packet to a node (eq. 2.25): a complex multiply-add (8 FLOPs); "
+                           "M 8^d per launch",
+               "peak_source": "FFMA probe on this GB300 (74.6 TFLOP/s; nominal 80.5 at 2.07 GHz)"} if d >= 2 else {
+               "kernel": "coefficient + scatter (K3+K4)", "bound": "l2",
                "achieved": contrib / (scatter_ms * 1e-3) / 1e9, "peak": L2_RED_COALESCED_GPS,
                "unit": "G contributions/s", "traffic": SCATTER_TRAFFIC_BYTES.get((d, M)),
                "launch_ms": scatter_ms, "units_per_launch": contrib,
