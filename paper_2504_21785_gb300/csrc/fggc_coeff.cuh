@@ -309,7 +309,8 @@ template <int D, bool FP64, int N1, class PT>
 __device__ __forceinline__ void coeff_scatter_body(const double *__restrict__ q, const double *__restrict__ p,
                                                    const double *__restrict__ s, const double *__restrict__ a,
                                                    int64_t m, int64_t j, const PT &P,
-                                                   void *__restrict__ W_v, uint8_t *__restrict__ row_flag) {
+                                                   void *__restrict__ W_v, uint8_t *__restrict__ row_flag,
+                                                   int k_first = 0, int k_end = N1) {
     using Real = typename std::conditional<FP64, double, float>::type;
     using C2 = typename std::conditional<FP64, double2, float2>::type;
     constexpr int kT = coeff_threads<FP64, N1>();
@@ -375,7 +376,7 @@ __device__ __forceinline__ void coeff_scatter_body(const double *__restrict__ q,
         emit_row<D - 1, N1>(W, c, a0[D - 1], b0[D - 1], cl_r, cl_i, 0, wr, wi);
     } else {
 #pragma unroll 1
-        for (int k0 = 0; k0 < N1; ++k0) {
+        for (int k0 = k_first; k0 < k_end; ++k0) {  // neighbours of dimension 0
             const int ia0 = a0[0] + c.dq[k0] - c.amin[0], ib0 = b0[0] + c.dp[k0] - c.bmin[0];
             const bool in0 = (unsigned)ia0 < (unsigned)c.A[0] && (unsigned)ib0 < (unsigned)c.B[0];
             if (!in0) continue;
@@ -424,7 +425,9 @@ __global__ void __launch_bounds__(coeff_threads<FP64, N1>(), 4) coeff_scatter3_k
     if (j < m) coeff_scatter_body<D, FP64, N1>(q, p, s, a, m, j, P, W_v, row_flag);
 }
 
-// The same over the packets list[0 .. *count) (device count), grid-stride.
+// The same over the packets list[0 .. *count) (device count), grid-stride.  A short
+// list takes N1 threads per packet, one neighbour of dimension 0 each (a packet's 512
+// reductions one after the other took 46 us of a small 3-D call, 17 us so).
 template <int D, bool FP64, int N1>
 __global__ void __launch_bounds__(coeff_threads<FP64, N1>(), D == 3 ? 4 : 1) coeff_scatter_list_kernel(
     const double *__restrict__ q, const double *__restrict__ p, const double *__restrict__ s,
@@ -432,8 +435,12 @@ __global__ void __launch_bounds__(coeff_threads<FP64, N1>(), D == 3 ? 4 : 1) coe
     uint8_t *__restrict__ row_flag, const int *__restrict__ list, const int *__restrict__ count) {
     constexpr int kT = coeff_threads<FP64, N1>();
     const int n = *count;
-    for (int64_t t = blockIdx.x * (int64_t)kT + threadIdx.x; t < n; t += (int64_t)gridDim.x * kT)
-        coeff_scatter_body<D, FP64, N1>(q, p, s, a, m, list[t], P, W_v, row_flag);
+    const int per = (int64_t)n * N1 <= (int64_t)gridDim.x * kT ? N1 : 1;
+    for (int64_t t = blockIdx.x * (int64_t)kT + threadIdx.x; t < (int64_t)n * per; t += (int64_t)gridDim.x * kT) {
+        const int k = per == 1 ? 0 : (int)(t % N1);
+        coeff_scatter_body<D, FP64, N1>(q, p, s, a, m, list[per == 1 ? t : t / N1], P, W_v, row_flag, k,
+                                        per == 1 ? N1 : k + 1);
+    }
 }
 
 // Batched form: the CTAs of every request of a launch (same dimension,
