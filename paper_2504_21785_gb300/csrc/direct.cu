@@ -1034,7 +1034,7 @@ fgr_status launch_1d(fgr_ctx *ctx, const Prepared &pr, float2 *part, void *u_dev
     const int64_t stride = (int64_t)pr.ntiles * tileT<1>(0);
     direct1_kernel<<<dim3((unsigned)pr.ntiles, (unsigned)slices), kD1Threads, 0, st>>>(
         reinterpret_cast<const RecF<1> *>(pr.recs), pr.off, pr.P, part);
-    direct1_sum_kernel<<<(unsigned)((ctx->grid.n[0] + 127) / 128), 128, 0, st>>>(part, slices, stride, ctx->grid.n[0],
+    direct1_sum_kernel<<<(unsigned)((ctx->grid.n[0] + 31) / 32), 256, 0, st>>>(part, slices, stride, ctx->grid.n[0],
                                                                               reinterpret_cast<float2 *>(u_dev));
     FGR_CUDA_TRY(cudaGetLastError());
     timer.mark(&ctx->timing.last.direct_ms);

@@ -11,7 +11,7 @@
 // evaluated, so no power is above the fourth.
 // Bound by instruction issue: about 8.5 per packet-point pair, against 17 for four
 // points by the recurrences of direct_tile: 1-D workload (262,144 packets, 32,768
-// points) 331 -> 265 us with the sum of the slices.  Coarser grids keep direct_tile, which has no powers of s
+// points) 331 -> 256 us with the sum of the slices.  Coarser grids keep direct_tile, which has no powers of s
 // across points that lie several widths apart.
 // Included by direct.cu inside its anonymous namespace.
 #pragma once
@@ -142,14 +142,27 @@ __global__ void __launch_bounds__(kD1Threads) direct1_kernel(const RecF<1> *__re
 // u[m] = the sum of the slices (compensated): a store and a read per slice cost what
 // an atomic would, and neither their order nor their number touches the result's
 // precision.
-__global__ void __launch_bounds__(128) direct1_sum_kernel(const float2 *__restrict__ part, int slices, int64_t stride,
+// A CTA takes 32 points; its eight warps share out the slices.
+__global__ void __launch_bounds__(256) direct1_sum_kernel(const float2 *__restrict__ part, int slices, int64_t stride,
                                                           int64_t n, float2 *__restrict__ u) {
-    const int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (m >= n) return;
+    __shared__ float4 sub[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t m = blockIdx.x * (int64_t)32 + lane;
     float2 s = both(0.f), c = both(0.f);
-#pragma unroll 8
-    for (int y = 0; y < slices; ++y) {
-        const float2 v = part[y * stride + m];
+#pragma unroll 4
+    for (int y = w; y < slices; y += 8) {
+        const float2 v = part[y * stride + m];  // (the stride covers whole tiles)
+        kahan_sum(s.x, c.x, v.x);
+        kahan_sum(s.y, c.y, v.y);
+    }
+    sub[w][lane] = make_float4(s.x, s.y, c.x, c.y);
+    __syncthreads();
+    if (w > 0 || m >= n) return;
+#pragma unroll
+    for (int i = 1; i < 8; ++i) {
+        const float4 v = sub[i][lane];
+        c.x += v.z;
+        c.y += v.w;
         kahan_sum(s.x, c.x, v.x);
         kahan_sum(s.y, c.y, v.y);
     }

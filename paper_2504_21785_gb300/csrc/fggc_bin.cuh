@@ -322,12 +322,15 @@ __global__ void bin_items_kernel(const int2 *__restrict__ off, const int4 *__res
 // Before the scatter: marks every row of W that the packets of an occupied key
 // will reach (the n1^(d-1) outer neighbours of its anchor cell that lie in the
 // node box) and widens the rows' boxes (min a, min -a, min b, min -b of the inner
-// nodes) by the key's, one thread per key.  The binned and per-packet kernels
+// nodes) by the key's.  per (1 or 8) threads per key share out the neighbours of
+// dimension 0: eight where the keys are few (90,000 of them 29 -> 15 us), one where
+// most threads would only find an empty key (888,000: 43 us against 62).  The binned
+// and per-packet kernels
 // reach exactly these rows, so only they need clearing.
 template <int D>
 __global__ void bin_mark_rows_kernel(const int *__restrict__ count, const int4 *__restrict__ kbox, const Common c,
-                                     const BinBox bb, uint8_t *__restrict__ row_flag, int4 *row_box) {
-    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+                                     const BinBox bb, int per, uint8_t *__restrict__ row_flag, int4 *row_box) {
+    const int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / per;
     if (k >= bb.K || count[k] == 0) return;
     int oa[D - 1], ob[D - 1], ta, tb;
     key_anchors<D>(bb, (unsigned)k, oa, ob, ta, tb);
@@ -345,7 +348,7 @@ __global__ void bin_mark_rows_kernel(const int *__restrict__ count, const int4 *
         if (box.z < v.z) atomicMin(b + 2, box.z);
         if (-box.w < v.w) atomicMin(b + 3, -box.w);
     };
-    for (int k0 = 0; k0 < c.n1; ++k0) {
+    for (int k0 = threadIdx.x % per; k0 < c.n1; k0 += per) {
         const int ia0 = oa[0] + c.dq[k0] - c.amin[0], ib0 = ob[0] + c.dp[k0] - c.bmin[0];
         if ((unsigned)ia0 >= (unsigned)c.A[0] || (unsigned)ib0 >= (unsigned)c.B[0]) continue;
         const int64_t row0 = (int64_t)ia0 * c.ra[0] + (int64_t)ib0 * c.rb[0];
@@ -798,7 +801,9 @@ fgr_status launch_binned_d(const BinLaunch &L, cudaStream_t st, const PacketsDev
                                                  b.kbox, b.loose, b.ctr);
     // the rows and their boxes, and the clearing of those rows
     FGR_CUDA_TRY(cudaMemsetAsync(L.row_box, 0x7f, sizeof(int4) * (size_t)L.rows, st));
-    bin_mark_rows_kernel<D><<<kblocks, 256, 0, st>>>(b.count, b.kbox, P.c, L.box, flags, L.row_box);
+    const int per = K < (1 << 18) ? 8 : 1;
+    bin_mark_rows_kernel<D><<<(unsigned)((K * per + 255) / 256), 256, 0, st>>>(b.count, b.kbox, P.c, L.box, per, flags,
+                                                                             L.row_box);
     // about 64 warps per SM: few long rows (d = 2: 5,796 of 37 KB) are cut into
     // parts (139 us with one warp per 32 rows, 19 us so), many short ones not
     const int64_t warps = (L.rows + 31) / 32, row_f4 = L.row_cells / 2;
