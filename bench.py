@@ -139,7 +139,7 @@ def rk4_nsteps(t: float, dt: float) -> int:
 # DRAM bytes (read + written) of one launch of the binned scatter kernel on the
 # 3-D workload (d, packets), from the ncu launch list of the headline command
 # (mean of 4 launches); to be retaken whenever the kernel changes.
-SCATTER_TRAFFIC_BYTES = {(3, 16777216): 4148112512}
+SCATTER_TRAFFIC_BYTES = {}
 # Algorithmic FP64 work of one RK4 packet-step per dimension: 4 stages of
 # about 40 FLOPs each.
 RK4_ALG_FLOPS_PER_PACKET_STEP = 160

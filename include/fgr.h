@@ -281,10 +281,11 @@ fgr_status fgr_reconstruct_direct_batch(int32_t n, fgr_ctx *const *ctxs, const f
  * products over dimensions.  The weights A_j e^{iS_j/eps} c_j^(k) are summed
  * onto grid nodes (eq. 2.25) and the node Gaussians are summed on the grid
  * (eq. 2.24) one dimension at a time.  FP64: all FP64.  FP32: the coefficients
- * come from a Chebyshev surrogate of c~(s,t) built on the host from the same
- * pseudo-inverse (degree 10, truncation error about 3e-10: below FP32 rounding;
- * evaluated in FP32 over the terms i + j <= 11 for n1 <= 8), phases are reduced
- * in FP64, node array and grid sums in complex64.  Host packets are copied to
+ * come from a polynomial surrogate of c~(s,t) built on the host from the same
+ * pseudo-inverse (Chebyshev interpolation of degree 9 per variable, total degree
+ * 11 for n1 <= 8; truncation about 1e-8 of the largest coefficient, below FP32
+ * rounding), one per four mirrored neighbours; phases are reduced to FP64
+ * accuracy, node array and grid sums in complex64.  Host packets are copied to
  * the device and tested there for non-finite values before anything is
  * written: FGR_E_INVALID if one is found. */
 fgr_status fgr_reconstruct_fggc(fgr_ctx *ctx, const fgr_packets *pk, void *u_out,
@@ -398,7 +399,7 @@ fgr_status fgr_get_info(const fgr_ctx *ctx, fgr_info *out);
 /* Per-stage device times (milliseconds, CUDA events) of the context's last
  * reconstruct or propagate call, when timing is enabled with fgr_set_timing.
  * FGGC: prep_ms = clearing the node array, coeff_ms = binning the packets by
- * anchor cell (d = 3, FP32), scatter_ms = the coefficient and scatter
+ * anchor cell (d >= 2, FP32; in 2-D from 131072 packets), scatter_ms = the coefficient and scatter
  * kernels, grid_ms = the whole grid stage (eq. 2.24), of which pass_ms is the
  * grid-pass kernels alone; pass_terms = node-point terms of the grid passes
  * (per pass, over every (row, node a) line: the occupied b-range times the

@@ -1236,6 +1236,7 @@ fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, 
             halves = std::max(halves, row_halves(pp[l].B));
             most = std::max<int64_t>(most, std::max<int64_t>(pp[l].A, pp[l].N));
         }
+        *launches += boxes_known ? 1 : 2;  // tables (and the scan of W)
         row_tables_kernel<FP64><<<dim3((unsigned)((most + 255) / 256), D, FP64 ? 1 + halves : 1), 256, 0, st>>>(T);
     }
     // the rows' boxes and ranges of every pass
@@ -1384,7 +1385,7 @@ fgr_status enqueue_fggc(fgr_ctx *ctx, const PacketsDev &pk, const FggcBox &box, 
             bl.row_box = reinterpret_cast<int4 *>(b.brange);
             StageMarks marks{timer, &ctx->timing.last.coeff_ms};
             r = launch_binned_scatter(D, L.n1, bl, st, pk, P, b.W, b.flags, &marks);
-            *launches += 8;  // key, 3 scan, place, items, binned, loose
+            *launches += 9;  // key, 3 scans, place, rows, clearing, items, list (and the binned kernel below)
         } else {
             r = launch_coeff_scatter(D, L.n1, st, pk, nullptr, &P, b.W, b.flags);
         }
