@@ -1021,10 +1021,28 @@ fgr_status launch_tc(fgr_ctx *ctx, const Prepared &pr, void *u_dev, cudaStream_t
 // into partial sums, then their sum.  Four slices of 128 threads for the one of 256
 // of direct_kernel even out the tiles' lists (the whole call on the 1-D workload: two 389, four 370, six 364 us).
 constexpr int kD1Slices = 4;
-// Partial sums (40 MB at most); null, without an error, where the memory is short:
-// direct_kernel needs none.
+// Where direct1_kernel runs.  Its partial sums cost a store and a read per slice and
+// point whatever the packets are, so it needs pairs enough to pay for them.  Whole
+// calls, direct_kernel -> direct1_kernel, us: 4096 packets at 192 pairs per point
+// 2^10 points 72 -> 52, 2^17 109 -> 82, 2^22 923 -> 651, 2^23 1132 -> 1153; at 48 pairs
+// per point 2^13 75 -> 55, 2^22 545 -> 394; 64 packets at 0.75 and 3 pairs per point 2^15
+// 44 -> 52, 2^20 47 -> 85, 2^23 86 -> 363.  So: 4096 packets, 48 pairs per point and
+// at most kD1MaxBytes of partial sums (those of 2^22 points, one split).
+// kD1Pts points have to lie within a few widths of each other (direct_1d.cuh).
+constexpr int64_t kD1MinPackets = 4096;
+constexpr double kD1MinPairsPerPoint = 48.0;
+constexpr size_t kD1MaxBytes = (size_t)1 << 27;
+inline size_t partial_bytes_1d(const Prepared &pr) {
+    return sizeof(float2) * (size_t)kD1Slices * pr.P.splits * pr.ntiles * tileT<1>(0);
+}
+inline bool use_direct1(const fgr_ctx *ctx, const Prepared &pr, int64_t m) {
+    const double n = (double)ctx->grid.n[0], h = ctx->grid.h[0];
+    return 4.0 * h <= std::sqrt(ctx->mesh.eps) && m >= kD1MinPackets && partial_bytes_1d(pr) <= kD1MaxBytes &&
+           (double)m * std::min(2.0 * ctx->mesh.rs / h, n) >= kD1MinPairsPerPoint * n;
+}
+// Null, without an error, where the memory is short: direct_kernel needs none.
 float2 *partials_1d(const Prepared &pr, Scratch &scratch) {
-    auto *part = (float2 *)scratch.get(sizeof(float2) * (size_t)kD1Slices * pr.P.splits * pr.ntiles * tileT<1>(0));
+    auto *part = (float2 *)scratch.get(partial_bytes_1d(pr));
     if (!part) clear_error();
     return part;
 }
@@ -1060,8 +1078,8 @@ fgr_status launch(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStream_t 
         dim3 grid((unsigned)pr.ntiles, (unsigned)pr.P.splits);
         if (fp64)
             direct_kernel<D, true><<<grid, kThreads, 0, st>>>(pr.recs, pr.off, pr.P, u_dev);
-        else if (float2 *part = 4.0 * ctx->grid.h[0] <= std::sqrt(ctx->mesh.eps) ? partials_1d(pr, scratch) : nullptr)
-            return launch_1d(ctx, pr, part, u_dev, st, timer);  // see direct_1d.cuh
+        else if (float2 *part = use_direct1(ctx, pr, pk.m) ? partials_1d(pr, scratch) : nullptr)
+            return launch_1d(ctx, pr, part, u_dev, st, timer);
         else
             direct_kernel<D, false><<<grid, kThreads, 0, st>>>(pr.recs, pr.off, pr.P, u_dev);
         FGR_CUDA_TRY(cudaGetLastError());
