@@ -361,7 +361,7 @@ __device__ __forceinline__ void separable_chunk(const int *__restrict__ srec, co
 
 // One (output tile, packet slice) work item of the direct sum, executed by the
 // whole CTA; shared by the one-request kernel and the batched persistent kernel.
-template <int D, bool FP64>
+template <int D, bool FP64, bool COARSE = true>
 __device__ __forceinline__ void direct_tile(const void *__restrict__ recs_v, const int64_t *__restrict__ off,
                                             const DirectParams &P, void *__restrict__ u_v, const int tile,
                                             const int split, const int nsplit) {
@@ -559,7 +559,11 @@ __device__ __forceinline__ void direct_tile(const void *__restrict__ recs_v, con
                 const float wl = Rf.wlen[D - 1];
                 in = in && kk[D - 1] > -(float)kTpt && kk[D - 1] < wl;
                 if (!in) continue;
-                const float skip = fmaxf(-kk[D - 1], 0.f);  // points before the window
+                // points before the window; where 4 h <= sqrt(eps) the four points lie within
+                // a width of each other, nothing is lost from the first one on, and the
+                // checks below are left out (!COARSE: 64 packets on 2^15 points 48 -> 44 us,
+                // 4096 on 2^23 points 1377 -> 1130 us)
+                const float skip = COARSE ? fmaxf(-kk[D - 1], 0.f) : 0.f;
                 kk[D - 1] += skip;
                 float e = 0.f, tau = Rf.tau0, dxl = 0.f;
 #pragma unroll
@@ -582,8 +586,9 @@ __device__ __forceinline__ void direct_tile(const void *__restrict__ recs_v, con
                 float wr = rho * rot.x, wi = rho * rot.y;
 #pragma unroll
                 for (int r = 0; r < kTpt; ++r) {
-                    if ((float)r < skip) continue;
-                    if (kk[D - 1] + ((float)r - skip) < wl) {
+                    if (COARSE && (float)r < skip) continue;
+                    const float k = kk[D - 1] + ((float)r - skip);
+                    if ((COARSE || k >= 0.f) && k < wl) {
                         accf[r][0] += vr;
                         accf[r][1] += vi;
                     }
@@ -628,11 +633,11 @@ __device__ __forceinline__ void kahan_sum(float &s, float &c, float x) {
 
 #include "direct_1d.cuh"
 
-template <int D, bool FP64>
+template <int D, bool FP64, bool COARSE = true>
 __global__ void __launch_bounds__(kThreads) direct_kernel(const void *__restrict__ recs_v,
                                                           const int64_t *__restrict__ off,
                                                           DirectParams P, void *__restrict__ u_v) {
-    direct_tile<D, FP64>(recs_v, off, P, u_v, blockIdx.x, blockIdx.y, P.splits);
+    direct_tile<D, FP64, COARSE>(recs_v, off, P, u_v, blockIdx.x, blockIdx.y, P.splits);
 }
 
 // Records in the list of every tile (the home-tile box of direct_tile).
@@ -1076,10 +1081,13 @@ fgr_status launch(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStream_t 
     if (D == 1) {
         // 1-D: a few long tiles of similar load; one CTA per (tile, slice)
         dim3 grid((unsigned)pr.ntiles, (unsigned)pr.P.splits);
+        const bool fine = 4.0 * ctx->grid.h[0] <= std::sqrt(ctx->mesh.eps);
         if (fp64)
             direct_kernel<D, true><<<grid, kThreads, 0, st>>>(pr.recs, pr.off, pr.P, u_dev);
         else if (float2 *part = use_direct1(ctx, pr, pk.m) ? partials_1d(pr, scratch) : nullptr)
             return launch_1d(ctx, pr, part, u_dev, st, timer);
+        else if (fine)
+            direct_kernel<D, false, false><<<grid, kThreads, 0, st>>>(pr.recs, pr.off, pr.P, u_dev);
         else
             direct_kernel<D, false><<<grid, kThreads, 0, st>>>(pr.recs, pr.off, pr.P, u_dev);
         FGR_CUDA_TRY(cudaGetLastError());
