@@ -136,9 +136,9 @@ def rk4_nsteps(t: float, dt: float) -> int:
     return int(n) if abs(r - n) <= 1e-9 * max(n, 1.0) else int(math.ceil(r))
 
 
-# DRAM bytes (read + written) of one launch of the binned scatter kernel on the
-# 3-D workload (d, packets), from the ncu launch list of the headline command
-# (mean of 4 launches); to be retaken whenever the kernel changes.
+# DRAM bytes (read + written) of one launch of the binned scatter kernel by
+# (d, packets), where ncu counted them for the kernel as it is; none so far (the
+# block then reports traffic null).
 SCATTER_TRAFFIC_BYTES = {}
 # Algorithmic FP64 work of one RK4 packet-step per dimension: 4 stages of
 # about 40 FLOPs each.
