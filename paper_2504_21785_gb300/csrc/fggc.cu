@@ -1253,9 +1253,11 @@ fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, 
             const int64_t groups = rows / members, tiles = (G.n[l] + kBoxPts - 1) / kBoxPts;
             range[l - 1] = at;
             FGR_CUDA_TRY(cudaMemsetAsync(at, 0x7f, sizeof(int2) * (size_t)(tiles * groups * halves), st));
-            row_range_kernel<<<dim3((unsigned)groups, (unsigned)((members + 15) / 16)), 128, 0, st>>>(
-                l == D - 1 ? rbox : nullptr, range[l], row_halves(c.B[l]), members, c.B[l - 1], groups, T.tab[l].win,
-                halves, at);
+            // (every extent in x: a plane of nodes may have more than 65535 x 16 members)
+            const int64_t parts = (members + 15) / 16;
+            row_range_kernel<<<(unsigned)(groups * parts), 128, 0, st>>>(
+                l == D - 1 ? rbox : nullptr, range[l], row_halves(c.B[l]), members, (int)parts, c.B[l - 1], groups,
+                T.tab[l].win, halves, at);
             rows = groups * tiles;
             at += rows * halves;
             ++*launches;
@@ -1336,9 +1338,13 @@ bool rows_apply(const fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, in
         prodN *= G.n[l];
         const int lines = std::min(pass_band(fp64 ? row_pts<true>() : row_pts<false>(), pp.h, pp.rs, pp.dq), pp.A);
         const int chunks = (pp.B + kRowB - 1) / kRowB;
+        const int pts = fp64 ? row_pts<true>() : row_pts<false>();
+        // (rows bounds the launch of row_range_kernel and, with it, the nodes A x B of
+        // the other planes; A x B of a row is an int of row_scan_kernel)
         if ((fp64 ? row_pass_smem<true>(lines, kRowMax, chunks) : row_pass_smem<false>(lines, kRowMax, chunks)) >
                 kRowSmemMax ||
-            pp.rows >= INT_MAX || pp.rows * (int64_t)pp.A >= INT_MAX - 64 || pp.N > INT_MAX / 2 || pp.B < 2)
+            pp.rows >= INT_MAX || pp.rows * (int64_t)pp.A >= INT_MAX - 64 || pp.B < 2 ||
+            (int64_t)pp.A * pp.B >= INT_MAX || (pp.N + pts - 1) / pts > 65535)
             return false;
     }
     return G.n[D - 1] <= INT_MAX && (((uintptr_t)b.W | (uintptr_t)b.buf1 | (uintptr_t)b.buf2) & 15) == 0;

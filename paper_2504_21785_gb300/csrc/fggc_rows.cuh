@@ -389,12 +389,13 @@ __global__ void __launch_bounds__(kRowWarps * 32, FP64 ? 4 : 5)
 // reach the points of tile t through their windows (win: first and last point of
 // every node) widen out[(t * groups + g) * halves + b / kRowHalf] by a.  A
 // member's nodes: box[g * members + i], or range[(g * members + i) * in_halves ...].
-// Eight lanes per member share out its tiles.
+// Eight lanes per member share out its tiles; CTA p of the parts of a group has members
+// 16 p to 16 p + 15.
 __global__ void __launch_bounds__(128) row_range_kernel(const int4 *__restrict__ box, const int2 *__restrict__ range,
-                                                        int in_halves, int members, int B, int64_t groups,
+                                                        int in_halves, int members, int parts, int B, int64_t groups,
                                                         const int2 *__restrict__ win, int halves, int2 *out) {
-    const int64_t g = blockIdx.x;
-    const int i = blockIdx.y * (blockDim.x / 8) + threadIdx.x / 8;
+    const int64_t g = blockIdx.x / (unsigned)parts;
+    const int i = (int)(blockIdx.x % (unsigned)parts) * (blockDim.x / 8) + threadIdx.x / 8;
     if (i >= members) return;
     int lo = kBoxEmpty, hi = kBoxEmpty;
     if (box) {
