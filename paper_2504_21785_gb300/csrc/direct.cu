@@ -813,7 +813,7 @@ struct BatchParams {
 // kernel parameters may take up to 32764 bytes (sm_70 and later, CUDA 12.1+)
 static_assert(sizeof(BatchParams) <= 32000, "batch parameters exceed the kernel parameter space");
 
-template <int D, bool FP64>
+template <int D, bool FP64, bool COARSE = true>
 __global__ void __launch_bounds__(kThreads) direct_batch_kernel(const __grid_constant__ BatchParams B,
                                                                 unsigned long long *__restrict__ counter) {
     __shared__ long long s_item;
@@ -832,7 +832,7 @@ __global__ void __launch_bounds__(kThreads) direct_batch_kernel(const __grid_con
         }
         const BatchReq &R = B.req[lo];
         const long long j = item - B.item_start[lo];
-        direct_tile<D, FP64>(R.recs, R.off, R.P, R.u, (int)(j / R.P.splits), (int)(j % R.P.splits), R.P.splits);
+        direct_tile<D, FP64, COARSE>(R.recs, R.off, R.P, R.u, (int)(j / R.P.splits), (int)(j % R.P.splits), R.P.splits);
     }
 }
 
@@ -1212,10 +1212,14 @@ fgr_status launch_batch(int n, fgr_ctx *const *ctxs, const PacketsDev *pks, void
         return FGR_OK;
     }
     const int64_t ctas = std::min<int64_t>(total, (int64_t)ctxs[0]->num_sms * 8);
-    if (fp64)
-        direct_batch_kernel<D, true><<<(unsigned)ctas, kThreads, 0, st>>>(B, counter);
-    else
-        direct_batch_kernel<D, false><<<(unsigned)ctas, kThreads, 0, st>>>(B, counter);
+    // (the checks that coarse grids need cost fine ones 8 to 16 %: 8 requests of 262,144
+    // packets on 32,768 points 3.24 -> 3.76 ms)
+    bool fine = true;
+    for (int r = 0; r < n; ++r) fine = fine && 4.0 * ctxs[r]->grid.h[0] <= std::sqrt(ctxs[r]->mesh.eps);
+    auto *kernel = fp64   ? direct_batch_kernel<D, true>
+                   : fine ? direct_batch_kernel<D, false, false>
+                          : direct_batch_kernel<D, false>;
+    kernel<<<(unsigned)ctas, kThreads, 0, st>>>(B, counter);
     FGR_CUDA_TRY(cudaGetLastError());
     return FGR_OK;
 }
