@@ -219,10 +219,29 @@ struct DirectParams {
     float q_last;        // e^{-h^2 / eps} of the last dimension (Gaussian ratio step)
     float q_dim[3];      // e^{-h_l^2 / eps} per dimension (factor tables, d >= 2)
     float q8[3];         // e^{-64 h_l^2 / eps}: Gaussian ratio step over 8 grid lines (tensor-core path)
+    int coarse;          // bit l: coarse_step of dimension l
+    int alone;           // coarse grids, 1-D: every point by itself
     double inv_eps;      // FP64 path
     double neg_half_inv_eps;
     int splits;
 };
+
+// Coarse grids.  The recurrences over a run of four points start at most three steps
+// before the window (R widths sqrt(eps) to a side): from 13 widths on the start
+// underflows, every later point of the run is lost with it, and the ratio may overflow
+// (0 x inf).  Up to one width per step what is lost lies beyond ten widths (e^-50);
+// wider steps keep the recurrences while the start stays within 13 widths.  Other grids
+// start at the first point inside the window, which holds for windows of up to
+// kRunWidths (start above e^-41, e^{-h^2/eps} above e^-81 where three points of a run
+// lie in the window), or evaluate every point by itself (wider windows, and the factor
+// tables of d >= 2, which this does not bound).  With the recurrences 7 points at
+// h = 4.6 sqrt(eps), R = 6, were off by 0.16 to 0.48, or NaN.
+constexpr double kRunWidths = 9.0;
+constexpr int kFine = 0, kCoarse = 1, kAlone = 2, kMixed = 3;
+inline bool coarse_step(const Mesh &M, double h) {
+    const double step = h / M.sigma;
+    return step > 1.0 && M.R + 3.0 * step > 13.0;
+}
 
 // FP32, d >= 2: the term of a packet factorises over dimensions,
 //   pref A e^{i S/eps} prod_l exp(-(x_l - Q_l)^2 / (2 eps) + i P_l (x_l - Q_l) / eps),
@@ -259,7 +278,27 @@ __device__ __forceinline__ void separable_local(int tid, int *loc) {
     }
 }
 
+// The factor of dimension l at line k of a record's window: Gaussian and phase in full
+// (dx: the line's offset from the centre).
 template <int D>
+__device__ __forceinline__ float2 full_factor(const RecF<D> &R, const DirectParams &P, int l, float k, float &dx) {
+    dx = fmaf(k, P.hf[l], R.delta[l]);
+    float ex = dx * dx * P.ce;
+    float fr = k * R.nuhi[l];
+    fr -= rint_fast(fr);
+    float tau = fmaf(k, R.nulo[l], fr);
+    if (l == 0) {
+        ex += R.la;
+        tau += R.tau0;
+    }
+    tau -= rint_fast(tau);
+    float sn, cs;
+    __sincosf(6.283185307179586f * tau, &sn, &cs);
+    const float ga = ex2_approx(ex);
+    return make_float2(ga * cs, ga * sn);
+}
+
+template <int D, int MODE>
 __device__ __forceinline__ void separable_chunk(const int *__restrict__ srec, const int nrec, const DirectParams &P,
                                                 const int *t, float2 *__restrict__ sfac, float (*accf)[2]) {
     constexpr int kWords = sizeof(RecF<D>) / 4;
@@ -276,7 +315,23 @@ __device__ __forceinline__ void separable_chunk(const int *__restrict__ srec, co
         // a thread fills 4 consecutive grid lines of one record and dimension
         // (tile extents are multiples of 4), the first by ex2 and one sincos,
         // the next three by the exact recurrences of the Gaussian ratio
-        // (rho_{k+1} = rho_k e^{-h^2/eps}) and the phase rotation e^{2 pi i nu}
+        // (rho_{k+1} = rho_k e^{-h^2/eps}) and the phase rotation e^{2 pi i nu};
+        // on coarse grids a thread fills single lines (coarse_step)
+        if (MODE == kCoarse || (MODE == kMixed && P.coarse)) {
+            for (int e = threadIdx.x; e < ns * kT; e += kThreads) {
+                int k = e % kT, l = 0;
+#pragma unroll
+                for (int j = 0; j < D - 1; ++j)
+                    if (l == j && k >= tileT<D>(j)) {
+                        k -= tileT<D>(j);
+                        l = j + 1;
+                    }
+                const RecF<D> &R = *reinterpret_cast<const RecF<D> *>(&srec[(s0 + e / kT) * kWords]);
+                const float kf = (float)(t[l] * tileT<D>(l) + k) - R.mlo[l];
+                float dx;
+                sfac[e] = kf >= 0.f && kf < R.wlen[l] ? full_factor<D>(R, P, l, kf, dx) : make_float2(0.f, 0.f);
+            }
+        } else
         for (int e4 = threadIdx.x; e4 < ns * (kT / 4); e4 += kThreads) {
             const int e = 4 * e4;
             const int jr = s0 + e / kT;
@@ -292,20 +347,9 @@ __device__ __forceinline__ void separable_chunk(const int *__restrict__ srec, co
             const float wl = R.wlen[l];
             float4 out01 = make_float4(0.f, 0.f, 0.f, 0.f), out23 = out01;
             if (kf + 3.f >= 0.f && kf < wl) {  // some of the four lines lie in the window
-                const float dx = fmaf(kf, P.hf[l], R.delta[l]);
-                float ex = dx * dx * P.ce;
-                float fr = kf * R.nuhi[l];
-                fr -= rint_fast(fr);
-                float tau = fmaf(kf, R.nulo[l], fr);
-                if (l == 0) {
-                    ex += R.la;
-                    tau += R.tau0;
-                }
-                tau -= rint_fast(tau);
-                float sn, cs;
-                __sincosf(6.283185307179586f * tau, &sn, &cs);
-                const float ga = ex2_approx(ex);
-                float fr0 = ga * cs, fi0 = ga * sn;
+                float dx;
+                const float2 f0 = full_factor<D>(R, P, l, kf, dx);
+                float fr0 = f0.x, fi0 = f0.y;
                 float rs_, rc_;
                 __sincosf(6.283185307179586f * (R.nuhi[l] + R.nulo[l]), &rs_, &rc_);
                 float rho = ex2_approx(P.ce * P.hf[l] * fmaf(2.f, dx, P.hf[l]));
@@ -361,7 +405,11 @@ __device__ __forceinline__ void separable_chunk(const int *__restrict__ srec, co
 
 // One (output tile, packet slice) work item of the direct sum, executed by the
 // whole CTA; shared by the one-request kernel and the batched persistent kernel.
-template <int D, bool FP64, bool COARSE = true>
+// MODE (FP32): a grid without or with a coarse dimension (DirectParams::coarse, and
+// alone), or any of them, as a batch may have: a test of the two at run time, outside
+// the loops, costs the plain kernels 3 to 15 % (1-D, 65,536 packets on 4096 points:
+// 47.6 -> 55 us, 2-D CUDA-core sum 1840 -> 1900 us).
+template <int D, bool FP64, int MODE>
 __device__ __forceinline__ void direct_tile(const void *__restrict__ recs_v, const int64_t *__restrict__ off,
                                             const DirectParams &P, void *__restrict__ u_v, const int tile,
                                             const int split, const int nsplit) {
@@ -512,12 +560,83 @@ __device__ __forceinline__ void direct_tile(const void *__restrict__ recs_v, con
         const int64_t left = L - c * kThreads;
         const int nrec = left < kThreads ? (int)left : kThreads;
         if constexpr (!FP64 && D >= 2)
-            separable_chunk<D>(srec, nrec, P, t, sfac, accf);
-        else
-        for (int jr = 0; jr < nrec; ++jr) {
-            const Rec &R = *reinterpret_cast<const Rec *>(&srec[jr * kWords]);
-            if (FP64) {
-                const RecD<D> &Rd = reinterpret_cast<const RecD<D> &>(R);
+            separable_chunk<D, MODE>(srec, nrec, P, t, sfac, accf);
+        else if constexpr (!FP64) {
+            // a record's first point of the thread evaluated in full, the next by the
+            // exact recurrences of the Gaussian (ratio rho, itself multiplied by
+            // e^{-h^2/eps} per step) and of the phase (rotation by e^{2 pi i nu}); on
+            // coarse grids from the first point inside the window or every point by
+            // itself (coarse_step)
+            if (MODE == kCoarse || MODE == kAlone || (MODE == kMixed && P.coarse)) {
+                for (int jr = 0; jr < nrec; ++jr) {
+                    const RecF<1> &R = *reinterpret_cast<const RecF<1> *>(&srec[jr * kWords]);
+                    const float k0 = mf[0] - R.mlo[0], wl = R.wlen[0];
+                    if (!(k0 > -(float)kTpt && k0 < wl)) continue;
+                    float dx;
+                    if (MODE == kAlone || (MODE == kMixed && P.alone)) {
+#pragma unroll
+                        for (int r = 0; r < kTpt; ++r) {
+                            const float k = k0 + (float)r;
+                            if (!(k >= 0.f && k < wl)) continue;
+                            const float2 v = full_factor<1>(R, P, 0, k, dx);
+                            accf[r][0] += v.x;
+                            accf[r][1] += v.y;
+                        }
+                        continue;
+                    }
+                    const float skip = fmaxf(-k0, 0.f), k1 = k0 + skip;  // points before the window
+                    const float2 v1 = full_factor<1>(R, P, 0, k1, dx);
+                    float vr = v1.x, vi = v1.y;
+                    const float rho = ex2_approx(P.ce_h * fmaf(2.f, dx, P.hf[0]));
+                    const float2 rot = srot[jr];
+                    float wr = rho * rot.x, wi = rho * rot.y;
+#pragma unroll
+                    for (int r = 0; r < kTpt; ++r) {
+                        if ((float)r < skip) continue;
+                        if (k1 + ((float)r - skip) < wl) {
+                            accf[r][0] += vr;
+                            accf[r][1] += vi;
+                        }
+                        if (r + 1 < kTpt) {
+                            const float nr = vr * wr - vi * wi;
+                            vi = vr * wi + vi * wr;
+                            vr = nr;
+                            wr *= P.q_last;
+                            wi *= P.q_last;
+                        }
+                    }
+                }
+            } else {
+                for (int jr = 0; jr < nrec; ++jr) {
+                    const RecF<1> &R = *reinterpret_cast<const RecF<1> *>(&srec[jr * kWords]);
+                    const float k0 = mf[0] - R.mlo[0], wl = R.wlen[0];
+                    if (!(k0 > -(float)kTpt && k0 < wl)) continue;
+                    float dx;
+                    const float2 v0 = full_factor<1>(R, P, 0, k0, dx);
+                    float vr = v0.x, vi = v0.y;
+                    const float rho = ex2_approx(P.ce_h * fmaf(2.f, dx, P.hf[0]));
+                    const float2 rot = srot[jr];
+                    float wr = rho * rot.x, wi = rho * rot.y;
+#pragma unroll
+                    for (int r = 0; r < kTpt; ++r) {
+                        const float k = k0 + (float)r;
+                        if (k >= 0.f && k < wl) {
+                            accf[r][0] += vr;
+                            accf[r][1] += vi;
+                        }
+                        if (r + 1 < kTpt) {
+                            const float nr = vr * wr - vi * wi;
+                            vi = vr * wi + vi * wr;
+                            vr = nr;
+                            wr *= P.q_last;
+                            wi *= P.q_last;
+                        }
+                    }
+                }
+            }
+        } else {
+            for (int jr = 0; jr < nrec; ++jr) {
+                const RecD<D> &Rd = *reinterpret_cast<const RecD<D> *>(&srec[jr * kWords]);
 #pragma unroll
                 for (int r = 0; r < kTpt; ++r) {
                     bool in = valid[r];
@@ -540,65 +659,6 @@ __device__ __forceinline__ void direct_tile(const void *__restrict__ recs_v, con
                     const double gr = ga * cs, gi = ga * sn;
                     accd[r][0] += Rd.ar * gr - Rd.ai * gi;
                     accd[r][1] += Rd.ar * gi + Rd.ai * gr;
-                }
-            } else {
-                // the thread's first point inside the window (one before it can
-                // underflow on grids coarser than the Gaussian) evaluated in full,
-                // the next along the last dimension by the exact recurrences of the
-                // Gaussian (ratio rho, itself multiplied by e^{-h^2/eps} per step)
-                // and of the phase (rotation by e^{2 pi i nu})
-                const RecF<D> &Rf = reinterpret_cast<const RecF<D> &>(R);
-                float kk[D];
-                bool in = true;
-#pragma unroll
-                for (int l = 0; l < D - 1; ++l) {
-                    kk[l] = mf[l] - Rf.mlo[l];
-                    in = in && kk[l] >= 0.f && kk[l] < Rf.wlen[l];
-                }
-                kk[D - 1] = mf[D - 1] - Rf.mlo[D - 1];
-                const float wl = Rf.wlen[D - 1];
-                in = in && kk[D - 1] > -(float)kTpt && kk[D - 1] < wl;
-                if (!in) continue;
-                // points before the window; where 4 h <= sqrt(eps) the four points lie within
-                // a width of each other, nothing is lost from the first one on, and the
-                // checks below are left out (!COARSE: 64 packets on 2^15 points 48 -> 44 us,
-                // 4096 on 2^23 points 1377 -> 1130 us)
-                const float skip = COARSE ? fmaxf(-kk[D - 1], 0.f) : 0.f;
-                kk[D - 1] += skip;
-                float e = 0.f, tau = Rf.tau0, dxl = 0.f;
-#pragma unroll
-                for (int l = 0; l < D; ++l) {
-                    const float kf = kk[l];
-                    const float dx = fmaf(kf, P.hf[l], Rf.delta[l]);
-                    e = fmaf(dx, dx, e);
-                    float f = kf * Rf.nuhi[l];
-                    f -= rint_fast(f);
-                    tau += fmaf(kf, Rf.nulo[l], f);
-                    dxl = dx;
-                }
-                tau -= rint_fast(tau);
-                float sn, cs;
-                __sincosf(6.283185307179586f * tau, &sn, &cs);
-                const float ga = ex2_approx(fmaf(e, P.ce, Rf.la));
-                float vr = ga * cs, vi = ga * sn;
-                const float rho = ex2_approx(P.ce_h * fmaf(2.f, dxl, P.hf[D - 1]));
-                const float2 rot = srot[jr];
-                float wr = rho * rot.x, wi = rho * rot.y;
-#pragma unroll
-                for (int r = 0; r < kTpt; ++r) {
-                    if (COARSE && (float)r < skip) continue;
-                    const float k = kk[D - 1] + ((float)r - skip);
-                    if ((COARSE || k >= 0.f) && k < wl) {
-                        accf[r][0] += vr;
-                        accf[r][1] += vi;
-                    }
-                    if (r + 1 < kTpt) {
-                        const float nr = vr * wr - vi * wi;
-                        vi = vr * wi + vi * wr;
-                        vr = nr;
-                        wr *= P.q_last;
-                        wi *= P.q_last;
-                    }
                 }
             }
         }
@@ -633,11 +693,11 @@ __device__ __forceinline__ void kahan_sum(float &s, float &c, float x) {
 
 #include "direct_1d.cuh"
 
-template <int D, bool FP64, bool COARSE = true>
+template <int D, bool FP64, int MODE>
 __global__ void __launch_bounds__(kThreads) direct_kernel(const void *__restrict__ recs_v,
                                                           const int64_t *__restrict__ off,
                                                           DirectParams P, void *__restrict__ u_v) {
-    direct_tile<D, FP64, COARSE>(recs_v, off, P, u_v, blockIdx.x, blockIdx.y, P.splits);
+    direct_tile<D, FP64, MODE>(recs_v, off, P, u_v, blockIdx.x, blockIdx.y, P.splits);
 }
 
 // Records in the list of every tile (the home-tile box of direct_tile).
@@ -766,7 +826,7 @@ inline size_t plan_items_capacity(int ntiles, int target) {
 // Balanced direct sum: persistent CTAs pull the planned items in order.  With
 // a yield word, the CTAs from index keep on stop before pulling another item
 // while the word is > 0; the remaining CTAs finish every item.
-template <int D, bool FP64>
+template <int D, bool FP64, int MODE>
 __global__ void __launch_bounds__(kThreads) direct_items_kernel(const void *__restrict__ recs_v,
                                                                 const int64_t *__restrict__ off, DirectParams P,
                                                                 void *__restrict__ u_v,
@@ -786,7 +846,7 @@ __global__ void __launch_bounds__(kThreads) direct_items_kernel(const void *__re
         const long long item = s_item;
         if (item >= total) break;
         const int2 it = items[item];
-        direct_tile<D, FP64>(recs_v, off, P, u_v, it.x, it.y & 0xff, it.y >> 8);
+        direct_tile<D, FP64, MODE>(recs_v, off, P, u_v, it.x, it.y & 0xff, it.y >> 8);
     }
 }
 
@@ -813,7 +873,7 @@ struct BatchParams {
 // kernel parameters may take up to 32764 bytes (sm_70 and later, CUDA 12.1+)
 static_assert(sizeof(BatchParams) <= 32000, "batch parameters exceed the kernel parameter space");
 
-template <int D, bool FP64, bool COARSE = true>
+template <int D, bool FP64, int MODE>
 __global__ void __launch_bounds__(kThreads) direct_batch_kernel(const __grid_constant__ BatchParams B,
                                                                 unsigned long long *__restrict__ counter) {
     __shared__ long long s_item;
@@ -832,7 +892,7 @@ __global__ void __launch_bounds__(kThreads) direct_batch_kernel(const __grid_con
         }
         const BatchReq &R = B.req[lo];
         const long long j = item - B.item_start[lo];
-        direct_tile<D, FP64, COARSE>(R.recs, R.off, R.P, R.u, (int)(j / R.P.splits), (int)(j % R.P.splits), R.P.splits);
+        direct_tile<D, FP64, MODE>(R.recs, R.off, R.P, R.u, (int)(j / R.P.splits), (int)(j % R.P.splits), R.P.splits);
     }
 }
 
@@ -850,7 +910,7 @@ __global__ void batch_item_start_kernel(const int *__restrict__ nitems, int n, i
     }
 }
 
-template <int D, bool FP64>
+template <int D, bool FP64, int MODE>
 __global__ void __launch_bounds__(kThreads) direct_batch_items_kernel(const __grid_constant__ BatchParams B,
                                                                       const int *__restrict__ start,
                                                                       unsigned long long *__restrict__ counter) {
@@ -873,7 +933,7 @@ __global__ void __launch_bounds__(kThreads) direct_batch_items_kernel(const __gr
         }
         const BatchReq &R = B.req[lo];
         const int2 it = R.items[item - s_start[lo]];
-        direct_tile<D, FP64>(R.recs, R.off, R.P, R.u, it.x, it.y & 0xff, it.y >> 8);
+        direct_tile<D, FP64, MODE>(R.recs, R.off, R.P, R.u, it.x, it.y & 0xff, it.y >> 8);
     }
 }
 
@@ -955,6 +1015,8 @@ fgr_status prepare(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStream_t
     P.q_last = (float)std::exp(-g.h[D - 1] * g.h[D - 1] / M.eps);
     for (int l = 0; l < D; ++l) P.q_dim[l] = (float)std::exp(-g.h[l] * g.h[l] / M.eps);
     for (int l = 0; l < D; ++l) P.q8[l] = (float)std::exp(-64.0 * g.h[l] * g.h[l] / M.eps);
+    for (int l = 0; l < D; ++l) P.coarse |= coarse_step(M, g.h[l]) ? 1 << l : 0;
+    P.alone = M.R > kRunWidths;
     P.inv_eps = 1.0 / M.eps;
     P.neg_half_inv_eps = -0.5 / M.eps;
     const int target = ctx->num_sms * ctx->tune.direct_ctas_per_sm;
@@ -1081,15 +1143,16 @@ fgr_status launch(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStream_t 
     if (D == 1) {
         // 1-D: a few long tiles of similar load; one CTA per (tile, slice)
         dim3 grid((unsigned)pr.ntiles, (unsigned)pr.P.splits);
-        const bool fine = 4.0 * ctx->grid.h[0] <= std::sqrt(ctx->mesh.eps);
         if (fp64)
-            direct_kernel<D, true><<<grid, kThreads, 0, st>>>(pr.recs, pr.off, pr.P, u_dev);
+            direct_kernel<D, true, kFine><<<grid, kThreads, 0, st>>>(pr.recs, pr.off, pr.P, u_dev);
         else if (float2 *part = use_direct1(ctx, pr, pk.m) ? partials_1d(pr, scratch) : nullptr)
             return launch_1d(ctx, pr, part, u_dev, st, timer);
-        else if (fine)
-            direct_kernel<D, false, false><<<grid, kThreads, 0, st>>>(pr.recs, pr.off, pr.P, u_dev);
+        else if (pr.P.coarse && pr.P.alone)
+            direct_kernel<D, false, kAlone><<<grid, kThreads, 0, st>>>(pr.recs, pr.off, pr.P, u_dev);
+        else if (pr.P.coarse)
+            direct_kernel<D, false, kCoarse><<<grid, kThreads, 0, st>>>(pr.recs, pr.off, pr.P, u_dev);
         else
-            direct_kernel<D, false><<<grid, kThreads, 0, st>>>(pr.recs, pr.off, pr.P, u_dev);
+            direct_kernel<D, false, kFine><<<grid, kThreads, 0, st>>>(pr.recs, pr.off, pr.P, u_dev);
         FGR_CUDA_TRY(cudaGetLastError());
         timer.mark(&ctx->timing.last.direct_ms);
         ctx->timing.last.launches = 4;
@@ -1119,20 +1182,14 @@ fgr_status launch(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStream_t 
     plan_items_kernel<<<1, kPlanThreads, 0, st>>>(load, ntiles, target, rank, rank + ntiles, items,
                                                   reinterpret_cast<int *>(cnt + 1));
     int per_sm = 1;
-    if (fp64)
-        FGR_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, direct_items_kernel<D, true>, kThreads, 0));
-    else
-        FGR_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, direct_items_kernel<D, false>, kThreads, 0));
+    auto *kernel = fp64          ? direct_items_kernel<D, true, kFine>
+                   : pr.P.coarse ? direct_items_kernel<D, false, kCoarse>
+                                 : direct_items_kernel<D, false, kFine>;
+    FGR_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, 0));
     const unsigned ctas = (unsigned)(ctx->num_sms * std::max(1, per_sm));
     const int keep = std::max(ctx->num_sms, (int)ctas - ctx->num_sms);  // one slot per SM can be given up
-    if (fp64)
-        direct_items_kernel<D, true><<<ctas, kThreads, 0, st>>>(pr.recs, pr.off, pr.P, u_dev, items,
-                                                                reinterpret_cast<int *>(cnt + 1), cnt,
-                                                                ctx->yield_flag, keep);
-    else
-        direct_items_kernel<D, false><<<ctas, kThreads, 0, st>>>(pr.recs, pr.off, pr.P, u_dev, items,
-                                                                 reinterpret_cast<int *>(cnt + 1), cnt,
-                                                                 ctx->yield_flag, keep);
+    kernel<<<ctas, kThreads, 0, st>>>(pr.recs, pr.off, pr.P, u_dev, items, reinterpret_cast<int *>(cnt + 1), cnt,
+                                      ctx->yield_flag, keep);
     FGR_CUDA_TRY(cudaGetLastError());
     timer.mark(&ctx->timing.last.direct_ms);
     ctx->timing.last.launches = 6;
@@ -1193,32 +1250,25 @@ fgr_status launch_batch(int n, fgr_ctx *const *ctxs, const PacketsDev *pks, void
     auto *counter = (unsigned long long *)shared.get(sizeof(unsigned long long));
     if (!counter) return FGR_E_NOMEM;
     FGR_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), st));
+    int coarse = 0;
+    for (int r = 0; r < B.n; ++r) coarse |= B.req[r].P.coarse;
     if (D >= 2) {
         int *start = nitems + kBatchMax;
         batch_item_start_kernel<<<1, 32, 0, st>>>(nitems, B.n, start);
         int per_sm = 1;
-        if (fp64)
-            FGR_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, direct_batch_items_kernel<D, true>,
-                                                                       kThreads, 0));
-        else
-            FGR_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, direct_batch_items_kernel<D, false>,
-                                                                       kThreads, 0));
+        auto *kernel = fp64     ? direct_batch_items_kernel<D, true, kFine>
+                       : coarse ? direct_batch_items_kernel<D, false, kMixed>
+                                : direct_batch_items_kernel<D, false, kFine>;
+        FGR_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, 0));
         const unsigned ctas = (unsigned)(ctxs[0]->num_sms * std::max(1, per_sm));
-        if (fp64)
-            direct_batch_items_kernel<D, true><<<ctas, kThreads, 0, st>>>(B, start, counter);
-        else
-            direct_batch_items_kernel<D, false><<<ctas, kThreads, 0, st>>>(B, start, counter);
+        kernel<<<ctas, kThreads, 0, st>>>(B, start, counter);
         FGR_CUDA_TRY(cudaGetLastError());
         return FGR_OK;
     }
     const int64_t ctas = std::min<int64_t>(total, (int64_t)ctxs[0]->num_sms * 8);
-    // (the checks that coarse grids need cost fine ones 8 to 16 %: 8 requests of 262,144
-    // packets on 32,768 points 3.24 -> 3.76 ms)
-    bool fine = true;
-    for (int r = 0; r < n; ++r) fine = fine && 4.0 * ctxs[r]->grid.h[0] <= std::sqrt(ctxs[r]->mesh.eps);
-    auto *kernel = fp64   ? direct_batch_kernel<D, true>
-                   : fine ? direct_batch_kernel<D, false, false>
-                          : direct_batch_kernel<D, false>;
+    auto *kernel = fp64     ? direct_batch_kernel<D, true, kFine>
+                   : coarse ? direct_batch_kernel<D, false, kMixed>
+                            : direct_batch_kernel<D, false, kFine>;
     kernel<<<(unsigned)ctas, kThreads, 0, st>>>(B, counter);
     FGR_CUDA_TRY(cudaGetLastError());
     return FGR_OK;

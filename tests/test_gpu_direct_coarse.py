@@ -8,7 +8,7 @@ import paper_2504_21785_gb300 as fgr
 from oracle import fga
 from workloads.wkb import mesh_for
 
-from ._gpu import options, rel_l2, to_device
+from ._gpu import options, reconstruct, rel_l2, to_device
 
 pytestmark = pytest.mark.gpu
 
@@ -32,7 +32,19 @@ def _case(d, steps, seed, m=300):
     return pk, dict(d=d, n=n, lo=lo, hi=hi), eps
 
 
-@pytest.mark.parametrize("d", [1])
+@pytest.mark.parametrize("steps", [(1.1,), (2.3,), (2.4,), (4.6,), (2.6, 0.3), (0.2, 4.6), (7.0, 7.0), (2.3, 2.4), (4.6, 0.3, 2.6), (0.9, 1.1, 0.9)])
+@pytest.mark.parametrize("window_r", [6.0, 20.0])
+def test_coarse_grids_and_wide_windows(steps, window_r):
+    d = len(steps)
+    pk, grid, eps = _case(d, steps, 7)
+    mesh = mesh_for(d, eps)
+    got = reconstruct("direct", pk, grid, eps, options("fp32", window_r=window_r, flags=fgr.FGR_FLAG_DIRECT_FMA))
+    ref = fga.direct_sum(pk, grid, eps, mesh.dq, mesh.dp, R=window_r)
+    assert np.all(np.isfinite(got))
+    assert rel_l2(got, ref) <= TOL
+
+
+@pytest.mark.parametrize("d", [1, 2])
 @pytest.mark.parametrize("steps", [(0.2, 0.1, 0.25), (0.2, 1.5, 4.6, 0.9)])
 def test_batched_direct_on_fine_and_coarse_grids(d, steps):
     """A batch of fine grids, and one with grids on either side of the rule."""
