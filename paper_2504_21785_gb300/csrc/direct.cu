@@ -1044,6 +1044,18 @@ bool tc_fits(const GridDev &g, int64_t *nst_out) {
     return runs <= tc::kSegMax && nst <= ((int64_t)1 << 30);
 }
 
+// Whether the tensor-core kernel's runs of up to eight lines, eight steps apart, keep
+// every term: a run that starts where the Gaussian underflows (13 widths from the
+// centre) is lost from there on.  Windows of up to kRunWidths never reach that far;
+// wider ones do on grids whose runs (56 h) span more than 7 widths (e^-19 at what is
+// lost), where the CUDA-core kernel's runs of four neighbouring points are right (2-D,
+// h = sqrt(eps) / 2: off by 2.6e-3 with a window of 13 widths, NaN with 40).
+inline bool tc_runs_hold(const Mesh &M, const GridDev &g, int d) {
+    for (int l = 0; l < d; ++l)
+        if (M.R > kRunWidths && 64.0 * g.h[l] * g.h[l] > M.eps) return false;
+    return true;
+}
+
 // Tensor-core direct sum (FP32, d = 2, 3): loads of the super tiles, items
 // heaviest first, one persistent CTA per SM.
 template <int D>
@@ -1159,7 +1171,8 @@ fgr_status launch(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStream_t 
         timer.finish();
         return FGR_OK;
     }
-    if (D >= 2 && !fp64 && !(ctx->opt.flags & FGR_FLAG_DIRECT_FMA) && tc_fits<D == 3 ? 3 : 2>(pr.P.g, nullptr)) {
+    if (D >= 2 && !fp64 && !(ctx->opt.flags & FGR_FLAG_DIRECT_FMA) && tc_runs_hold(ctx->mesh, pr.P.g, D) &&
+        tc_fits<D == 3 ? 3 : 2>(pr.P.g, nullptr)) {
         fgr_status rt = launch_tc<D == 3 ? 3 : 2>(ctx, pr, u_dev, st, scratch);
         if (rt != FGR_OK) return rt;
         timer.mark(&ctx->timing.last.direct_ms);

@@ -32,15 +32,27 @@ def _case(d, steps, seed, m=300):
     return pk, dict(d=d, n=n, lo=lo, hi=hi), eps
 
 
+@pytest.mark.parametrize("flags", [0, fgr.FGR_FLAG_DIRECT_FMA])
 @pytest.mark.parametrize("steps", [(1.1,), (2.3,), (2.4,), (4.6,), (2.6, 0.3), (0.2, 4.6), (7.0, 7.0), (2.3, 2.4), (4.6, 0.3, 2.6), (0.9, 1.1, 0.9)])
 @pytest.mark.parametrize("window_r", [6.0, 20.0])
-def test_coarse_grids_and_wide_windows(steps, window_r):
+def test_coarse_grids_and_wide_windows(steps, window_r, flags):
     d = len(steps)
     pk, grid, eps = _case(d, steps, 7)
     mesh = mesh_for(d, eps)
-    got = reconstruct("direct", pk, grid, eps, options("fp32", window_r=window_r, flags=fgr.FGR_FLAG_DIRECT_FMA))
+    got = reconstruct("direct", pk, grid, eps, options("fp32", window_r=window_r, flags=flags))
     ref = fga.direct_sum(pk, grid, eps, mesh.dq, mesh.dp, R=window_r)
     assert np.all(np.isfinite(got))
+    assert rel_l2(got, ref) <= TOL
+
+
+@pytest.mark.parametrize("window_r", [9.0, 9.5, 13.0, 40.0])
+@pytest.mark.parametrize("step", [0.12, 0.13, 0.5])
+def test_wide_windows_on_fine_grids(step, window_r):
+    """Both sides of the tensor-core rule on windows and steps (h = sqrt(eps) / 8)."""
+    pk, grid, eps = _case(2, (step, step), 8)
+    mesh = mesh_for(2, eps)
+    got = reconstruct("direct", pk, grid, eps, options("fp32", window_r=window_r))
+    ref = fga.direct_sum(pk, grid, eps, mesh.dq, mesh.dp, R=window_r)
     assert rel_l2(got, ref) <= TOL
 
 
