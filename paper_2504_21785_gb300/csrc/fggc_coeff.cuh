@@ -33,17 +33,59 @@ struct Params32View {
     const float *poly;
 };
 
+// e^x - 1 for -1/4 <= x <= 0 (about an ulp): the Taylor series to x^13, whose next term
+// is below 2^-62 of the first.
+__device__ __forceinline__ double expm1_near(double x) {
+    double p = 1.0 / 6227020800.0;
+    p = fma(p, x, 1.0 / 479001600.0);
+    p = fma(p, x, 1.0 / 39916800.0);
+    p = fma(p, x, 1.0 / 3628800.0);
+    p = fma(p, x, 1.0 / 362880.0);
+    p = fma(p, x, 1.0 / 40320.0);
+    p = fma(p, x, 1.0 / 5040.0);
+    p = fma(p, x, 1.0 / 720.0);
+    p = fma(p, x, 1.0 / 120.0);
+    p = fma(p, x, 1.0 / 24.0);
+    p = fma(p, x, 1.0 / 6.0);
+    p = fma(p, x, 0.5);
+    return fma(p * x, x, x);
+}
+
+// Sine and cosine for |x| <= 3/32 (about an ulp): Taylor to x^9 and x^8, whose next
+// terms are below 2^-59 and 2^-55.
+__device__ __forceinline__ void sincos_near(double x, double &sn, double &cs) {
+    const double z = x * x;
+    double p = fma(1.0 / 362880.0, z, -1.0 / 5040.0), q = fma(1.0 / 40320.0, z, -1.0 / 720.0);
+    p = fma(p, z, 1.0 / 120.0);
+    q = fma(q, z, 1.0 / 24.0);
+    p = fma(p, z, -1.0 / 6.0);
+    q = fma(q, z, -0.5);
+    sn = fma(p * z, x, x);
+    cs = fma(q, z, 1.0);
+}
+
+// e^{x + i y} - 1 from e = e^x - 1 and the sine and cosine of y / 2.
+__device__ __forceinline__ void exp_minus_one(double e, double sn_half, double cs_half, double &re, double &im) {
+    const double q = 2.0 * sn_half * sn_half;  // 1 - cos y
+    re = fma(-(1.0 + e), q, e);
+    im = (1.0 + e) * (2.0 * sn_half * cs_half);
+}
+
 // FP64: the coefficients of one dimension through the eigen factors (PT: Params64
 // or Params64View), in the symmetric form of build_lsa: with (sx, ty) the offset
 // from the cell centre, the right-hand side of neighbour (u, v) is
 //   e^{-cq^2 (u - sx)^2 / 4} e^{i cq cp u ty / 2} e^{-cp^2 (v - ty)^2 / 4} e^{-i cq cp v sx / 2},
 // one exponential per u and per v and a sine and cosine per |u| and per |v| for all
 // neighbours; sums and differences of mirror images bring it to the sectors' real
-// bases.  The phases are those of dim_setup32: z = e^{i cq cp A / 2}, and T takes
-// the packet's share in turns.  The FP64 pipe binds (16 clocks of an SM per warp
-// instruction): against an exponential, two sines and cosines and two complex
-// matrix rows per neighbour (N1 = 8: about 1360 instructions, now 570; N1 = 4: 590,
-// now 340) 705,600 2-D Q2P2 packets take 1.74 -> 0.98 ms.
+// bases.  All of it is carried as f - 1: the problem's small eigenvalues divide the
+// rounding of f by up to their square root (2.6e-5 for Q4P2), f lies near one, and the
+// ones' share of every eigenvector is exact (Lsa::sec_one).  Relative to the result,
+// random packets: 3.2e-12 for Q4P2 with products of exponentials (4.7e-12 with one
+// exponential and phase per neighbour), 3.2e-13 so.  The phases are those of
+// dim_setup32: z = e^{i cq cp A / 2}, and T takes the packet's share in turns.  The
+// FP64 pipe binds (16 clocks of an SM per warp instruction): against an exponential,
+// two sines and cosines and two complex matrix rows per neighbour, 705,600 2-D Q2P2
+// packets take 1.73 -> 0.95 ms (1-D, 4096 Q4P2: 66 -> 27 us).
 template <int N, class PT>
 __device__ __forceinline__ void coeff_dim64(const PT &P, double Q, double Pm, int &a0, int &b0, double &T,
                                             double *cr, double *ci) {
@@ -65,30 +107,29 @@ __device__ __forceinline__ void coeff_dim64(const PT &P, double Q, double Pm, in
         sincospi(2.0 * t, &zi, &zr);
     }
     // Gaussian and phase factors of u, v = -1/2, 1/2 and (where the strategy has
-    // them) -3/2, 3/2
+    // them) -3/2, 3/2, less one
     double ur[2][2], ui[2][2], vr2[2][2], vi2[2][2];
+    auto factors = [&](auto expm1_of, auto sincos_of) {
 #pragma unroll
-    for (int t = 0; t < (N >= 8 ? 2 : 1); ++t) {
-        const double h = t + 0.5;
-        if (t == 0 || c.u3) {
+        for (int t = 0; t < (N >= 8 ? 2 : 1); ++t) {
+            const double h = t + 0.5;
             double sn, cs;
-            sincos(2.0 * h * c.cqcp_4 * ty, &sn, &cs);
-            const double lo = exp(-c.cq2_4 * ((h + sx) * (h + sx))), hi = exp(-c.cq2_4 * ((h - sx) * (h - sx)));
-            ur[t][0] = lo * cs;
-            ui[t][0] = -lo * sn;
-            ur[t][1] = hi * cs;
-            ui[t][1] = hi * sn;
+            if (t == 0 || c.u3) {
+                sincos_of(h * c.cqcp_4 * ty, sn, cs);
+                exp_minus_one(expm1_of(-c.cq2_4 * ((h + sx) * (h + sx))), -sn, cs, ur[t][0], ui[t][0]);
+                exp_minus_one(expm1_of(-c.cq2_4 * ((h - sx) * (h - sx))), sn, cs, ur[t][1], ui[t][1]);
+            }
+            if (t == 0 || c.v3) {
+                sincos_of(h * c.cqcp_4 * sx, sn, cs);
+                exp_minus_one(expm1_of(-c.cp2_4 * ((h + ty) * (h + ty))), sn, cs, vr2[t][0], vi2[t][0]);
+                exp_minus_one(expm1_of(-c.cp2_4 * ((h - ty) * (h - ty))), -sn, cs, vr2[t][1], vi2[t][1]);
+            }
         }
-        if (t == 0 || c.v3) {
-            double sn, cs;
-            sincos(2.0 * h * c.cqcp_4 * sx, &sn, &cs);
-            const double lo = exp(-c.cp2_4 * ((h + ty) * (h + ty))), hi = exp(-c.cp2_4 * ((h - ty) * (h - ty)));
-            vr2[t][0] = lo * cs;
-            vi2[t][0] = lo * sn;
-            vr2[t][1] = hi * cs;
-            vi2[t][1] = -hi * sn;
-        }
-    }
+    };
+    if (P.f.near)
+        factors([](double x) { return expm1_near(x); }, [](double x, double &s, double &c) { sincos_near(x, s, c); });
+    else
+        factors([](double x) { return expm1(x); }, [](double x, double &s, double &c) { sincos(x, &s, &c); });
     double gr[2][N / 2], gi[2][N / 2];
 #pragma unroll
     for (int o = 0; o < N / 4; ++o) {
@@ -97,8 +138,11 @@ __device__ __forceinline__ void coeff_dim64(const PT &P, double Q, double Pm, in
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
             const int a = g >> 1, b = g & 1;
-            cmul(u3 ? ur[N >= 8 ? 1 : 0][a] : ur[0][a], u3 ? ui[N >= 8 ? 1 : 0][a] : ui[0][a],
-                 v3 ? vr2[N >= 8 ? 1 : 0][b] : vr2[0][b], v3 ? vi2[N >= 8 ? 1 : 0][b] : vi2[0][b], br[g], bi[g]);
+            const double pr = u3 ? ur[N >= 8 ? 1 : 0][a] : ur[0][a], pi = u3 ? ui[N >= 8 ? 1 : 0][a] : ui[0][a];
+            const double qr = v3 ? vr2[N >= 8 ? 1 : 0][b] : vr2[0][b], qi = v3 ? vi2[N >= 8 ? 1 : 0][b] : vi2[0][b];
+            // (1 + p) (1 + q) - 1
+            br[g] = fma(-pi, qi, fma(pr, qr, pr + qr));
+            bi[g] = fma(pr, qi, fma(pi, qr, pi + qi));
         }
         const double pr = br[0] + br[3], pi = bi[0] + bi[3], qr = br[1] + br[2], qi = bi[1] + bi[2];
         gr[0][2 * o] = pr + qr;
@@ -116,7 +160,7 @@ __device__ __forceinline__ void coeff_dim64(const PT &P, double Q, double Pm, in
         double wr[N / 2], wi[N / 2];
 #pragma unroll
         for (int i = 0; i < N / 2; ++i) {
-            double tr = 0, ti = 0;
+            double tr = s == 0 ? P.f.one[i] : 0.0, ti = 0;
 #pragma unroll
             for (int a = 0; a < N / 2; ++a) {
                 tr = fma(P.f.sec[s][a * kMaxHalf + i], gr[s][a], tr);

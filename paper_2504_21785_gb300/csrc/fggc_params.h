@@ -2,6 +2,8 @@
 // code (fggc.cu) and the coefficient + scatter kernels (fggc_coeff*.cu).
 #pragma once
 
+#include <algorithm>
+
 #include "internal.h"
 
 namespace fgr {
@@ -21,17 +23,21 @@ struct Common {
     int64_t ra[kMaxDim], rb[kMaxDim];  // sa / row_len, sb / row_len (dimensions before the last)
 };
 
-// Eigen factors of the least-squares problem (Lsa::sec, sec_inv, kap_r, kap_i).
+// Eigen factors of the least-squares problem (Lsa::sec, sec_inv, sec_one, kap_r, kap_i).
 struct Factors64 {
-    double sec[2][kMaxHalf * kMaxHalf], inv[2][kMaxHalf], kap_r[kMaxN1 / 4], kap_i[kMaxN1 / 4];
+    double sec[2][kMaxHalf * kMaxHalf], inv[2][kMaxHalf], one[kMaxHalf], kap_r[kMaxN1 / 4], kap_i[kMaxN1 / 4];
+    int near;  // every Gaussian exponent of the right-hand side lies in [-1/4, 0], every half phase in [-3/32, 3/32]
 };
 
 inline Factors64 factors64(const Lsa &L) {
     Factors64 f;
+    const double q = 0.5 * L.cq * (L.u3 ? 2.0 : 1.0), p = 0.5 * L.cp * (L.v3 ? 2.0 : 1.0);
+    f.near = std::max(q, p) <= 0.5;
     for (int s = 0; s < 2; ++s) {
         for (int i = 0; i < kMaxHalf * kMaxHalf; ++i) f.sec[s][i] = L.sec[s][i];
         for (int i = 0; i < kMaxHalf; ++i) f.inv[s][i] = L.sec_inv[s][i];
     }
+    for (int i = 0; i < kMaxHalf; ++i) f.one[i] = L.sec_one[i];
     for (int o = 0; o < kMaxN1 / 4; ++o) {
         f.kap_r[o] = L.kap_r[o];
         f.kap_i[o] = L.kap_i[o];

@@ -43,6 +43,8 @@ struct Lsa {
     // build_lsa: sec[s][a * kMaxHalf + i] = component a of eigenvector i, and
     // 1 / (4 lambda_i) above the cut-off, else 0.
     double sec[2][kMaxHalf * kMaxHalf] = {}, sec_inv[2][kMaxHalf] = {};
+    // The even eigenvectors' products with a right-hand side of ones (coeff_dim64).
+    double sec_one[kMaxHalf] = {};
     // Per orbit: e^{i cq cp |u v| / 2}.
     double kap_r[kMaxN1 / 4] = {}, kap_i[kMaxN1 / 4] = {};
     // Neighbours in orbit order: orbit o holds, at 4 o + g, the mirror images

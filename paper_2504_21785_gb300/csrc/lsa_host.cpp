@@ -166,6 +166,11 @@ bool build_lsa(double cq, double cp, int nq, int np, double rcond, Lsa *out) {
                 const long double lam = M[i * h + i].real();
                 L.sec_inv[s][i] = lam > (long double)rcond * lmax ? (double)(0.25L / lam) : 0.0;
                 for (int a = 0; a < h; ++a) L.sec[s][a * kMaxHalf + i] = (double)Q[a * h + i].real();
+                if (s == 0) {  // (the sums over an orbit's ones: 4 in the first of its two components)
+                    long double one = 0;
+                    for (int a = 0; a < h; a += 2) one += 4 * Q[a * h + i].real();
+                    L.sec_one[i] = (double)one;
+                }
             }
         }
         for (int o = 0; o < norb; ++o) {
