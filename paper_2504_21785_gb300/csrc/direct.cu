@@ -949,6 +949,11 @@ struct Prepared {
     bool empty = true;
 };
 
+// Slices per tile for target CTAs in all.
+inline int tile_splits(int target, int64_t ntiles) {
+    return (int)std::max<int64_t>(1, std::min<int64_t>(64, (target + ntiles - 1) / ntiles));
+}
+
 template <int D>
 fgr_status prepare(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStream_t st, Scratch &scratch,
                    Prepared *pr) {
@@ -1019,8 +1024,7 @@ fgr_status prepare(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStream_t
     P.alone = M.R > kRunWidths;
     P.inv_eps = 1.0 / M.eps;
     P.neg_half_inv_eps = -0.5 / M.eps;
-    const int target = ctx->num_sms * ctx->tune.direct_ctas_per_sm;
-    P.splits = std::max(1, std::min(64, (target + ntiles - 1) / ntiles));
+    P.splits = tile_splits(ctx->num_sms * ctx->tune.direct_ctas_per_sm, ntiles);
     pr->recs = recs;
     pr->off = off;
     pr->ntiles = ntiles;
@@ -1111,17 +1115,18 @@ constexpr int kD1Slices = 4;
 constexpr int64_t kD1MinPackets = 4096;
 constexpr double kD1MinPairsPerPoint = 48.0;
 constexpr size_t kD1MaxBytes = (size_t)1 << 27;
-inline size_t partial_bytes_1d(const Prepared &pr) {
-    return sizeof(float2) * (size_t)kD1Slices * pr.P.splits * pr.ntiles * tileT<1>(0);
+inline size_t partial_bytes_1d(int splits, int64_t ntiles) {
+    return sizeof(float2) * (size_t)kD1Slices * splits * ntiles * tileT<1>(0);
 }
 inline bool use_direct1(const fgr_ctx *ctx, const Prepared &pr, int64_t m) {
     const double n = (double)ctx->grid.n[0], h = ctx->grid.h[0];
-    return 4.0 * h <= std::sqrt(ctx->mesh.eps) && m >= kD1MinPackets && partial_bytes_1d(pr) <= kD1MaxBytes &&
+    return 4.0 * h <= std::sqrt(ctx->mesh.eps) && m >= kD1MinPackets &&
+           partial_bytes_1d(pr.P.splits, pr.ntiles) <= std::min(kD1MaxBytes, ctx->spare_bytes) &&
            (double)m * std::min(2.0 * ctx->mesh.rs / h, n) >= kD1MinPairsPerPoint * n;
 }
 // Null, without an error, where the memory is short: direct_kernel needs none.
 float2 *partials_1d(const Prepared &pr, Scratch &scratch) {
-    auto *part = (float2 *)scratch.get(partial_bytes_1d(pr));
+    auto *part = (float2 *)scratch.get(partial_bytes_1d(pr.P.splits, pr.ntiles));
     if (!part) clear_error();
     return part;
 }
@@ -1288,6 +1293,12 @@ fgr_status launch_batch(int n, fgr_ctx *const *ctxs, const PacketsDev *pks, void
 }
 
 }  // namespace
+
+size_t direct1_spare_bytes(int64_t m, int64_t n, int target) {
+    const int64_t ntiles = (n + tileT<1>(0) - 1) / tileT<1>(0);
+    const size_t bytes = partial_bytes_1d(tile_splits(target, ntiles), ntiles);
+    return m >= kD1MinPackets && bytes <= kD1MaxBytes ? bytes : 0;
+}
 
 fgr_status run_direct_batch(int n, fgr_ctx *const *ctxs, const PacketsDev *pks, void *const *us, cudaStream_t st,
                             Scratch **scratch, Scratch &shared) {

@@ -1038,6 +1038,13 @@ size_t bin_buffer_bytes(int64_t m, const BinBox &bb) {
     return carve_bin_buffers(nullptr, m, bb, &b);
 }
 
+size_t fggc_spare_bytes(int d, int n1, int64_t m) {
+    if (d < 2 || (n1 != 4 && n1 != 8) || m >= INT_MAX || (d == 2 && m < kBinMinPackets2d)) return 0;
+    BinBox bb;
+    bb.K = m;  // (2-D: at most)
+    return bin_buffer_bytes(m, bb);
+}
+
 void bin_buffers_at(void *block, int64_t m, const BinBox &bb, BinBuffers *out) {
     carve_bin_buffers((char *)block, m, bb, out);
 }
@@ -1514,7 +1521,8 @@ fgr_status launch(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStream_t 
     BinBox bb;
     if (ctx->opt.precision == FGR_FP32 && make_bin_box(box, D, pk.m, &bb)) {
         b.bin_bytes = bin_buffer_bytes(pk.m, bb);
-        b.bin = scratch.get(b.bin_bytes);
+        // (3-D binning is part of what the method takes: its few keys hold most packets)
+        if (D > 2 || b.bin_bytes <= ctx->spare_bytes) b.bin = scratch.get(b.bin_bytes);
         if (!b.bin) {  // the per-packet scatter needs none
             clear_error();
             b.bin_bytes = 0;

@@ -105,6 +105,10 @@ struct fgr_ctx {
     // sum): while it is > 0 the persistent direct-sum CTAs past one per SM
     // stop between work items, so that waiting small requests get SM slots.
     const volatile int *yield_flag = nullptr;
+    // Bytes that a call may take for buffers it can do without (partial sums of the 1-D
+    // direct sum, binning of the 2-D FGGC scatter): the server's requests have what was
+    // reserved for them within the budget.
+    size_t spare_bytes = SIZE_MAX;
     int64_t *host_pinned = nullptr;  // small pinned buffer for device->host sizes
 };
 
@@ -173,6 +177,11 @@ fgr_status run_direct(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStrea
 // call returns FGR_E_INVALID, before writing anything, if one is not finite.
 fgr_status run_fggc(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStream_t st,
                     Scratch &scratch, bool check_finite = false);
+// Upper bounds of the buffers that a call can do without (fgr_ctx::spare_bytes) and of
+// the 3-D FGGC binning, for the server's account: FP32 1-D direct sums of n points
+// aiming at target CTAs, FP32 FGGC of m packets in d >= 2 dimensions.
+size_t direct1_spare_bytes(int64_t m, int64_t n, int target);
+size_t fggc_spare_bytes(int d, int n1, int64_t m);
 // Device bytes owned by an FGGC plan (api.cu).
 size_t plan_device_bytes(const fgr_fggc_plan *plan);
 

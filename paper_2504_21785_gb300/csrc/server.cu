@@ -60,7 +60,9 @@ enum class St { Queued, Running, Done };
 struct Job {
     uint64_t ticket = 0;
     fgr_request req{};
-    size_t footprint = 0;
+    size_t footprint = 0;  // bytes it needs
+    size_t spare = 0;      // bytes it runs faster with (fgr_ctx::spare_bytes)
+    size_t granted = 0;    // of these, reserved when it was admitted
     bool dev_out = false;
     bool large = false;  // a long direct sum (see kLargeMs)
     St st = St::Queued;
@@ -105,6 +107,7 @@ struct PlanEntry {
 
 struct fgr_server {
     int device = 0;
+    int num_sms = 1;
     size_t budget = 0;
     int max_inflight = 1;
     int max_batch = 16;
@@ -169,6 +172,17 @@ double est_direct_ms(const fgr_request &r, int64_t m) {
     double rate = r.d == 1 ? 1.2e12 : 8e12;
     if (r.opt.precision == FGR_FP64) rate *= 0.25;
     return pairs / rate * 1e3;
+}
+
+// Bytes of the buffers that a request can do without.
+size_t spare_bytes(const fgr_request &r, const PacketSet &ps, int num_sms) {
+    if (r.opt.precision != FGR_FP32) return 0;
+    if (r.method == 0) {  // (32 CTAs per SM: large requests, and most that the autotuner picks)
+        if (r.d > 1) return 0;
+        return std::max(fgr::direct1_spare_bytes(ps.m, r.grid.n[0], num_sms * fgr::Tuning().direct_ctas_per_sm),
+                        fgr::direct1_spare_bytes(ps.m, r.grid.n[0], num_sms * kLargeCtasPerSm));
+    }
+    return fgr::fggc_spare_bytes(r.d, (r.opt.nq ? r.opt.nq : 4) * (r.opt.np ? r.opt.np : 2), ps.m);
 }
 
 void publish_small(fgr_server *S) {
@@ -284,6 +298,7 @@ fgr_status enqueue_one(fgr_server *S, const Job &job, const PacketSet &ps, CtxCa
     fgr_ctx *ctx = nullptr;
     fgr_status st = cache.get(r, &ctx);
     if (st != FGR_OK) return st;
+    ctx->spare_bytes = job.granted;
     fgr_packets pk = packets_of(ps);
     if (r.method == 0) {
         if (!job.large || !S) return fgr_reconstruct_direct(ctx, &pk, r.u_out, stream);
@@ -313,6 +328,7 @@ fgr_status finish_one(fgr_server *S, const Job &job, const PacketSet &ps, CtxCac
         st = cache.get(job.req, &ctx);
         if (st == FGR_OK) {
             fgr_packets pk = packets_of(ps);
+            ctx->spare_bytes = job.granted;
             st = fgr_reconstruct_fggc(ctx, &pk, job.req.u_out, stream);
             if (cudaStreamSynchronize(stream) != cudaSuccess && st == FGR_OK) st = FGR_E_CUDA;
         }
@@ -345,6 +361,7 @@ void run_fggc_group(fgr_server *S, const Group &g, const std::vector<PacketSet> 
         fgr_ctx *ctx = nullptr;
         st[i] = cache.get(g[i]->req, &ctx);
         if (st[i] != FGR_OK) continue;
+        ctx->spare_bytes = g[i]->granted;
         bpk[i] = packets_of(ps[i]);
         planned[i] = acquire_plan(S, *g[i], ctx, bpk[i], stream);
         if (!planned[i]) {
@@ -448,7 +465,7 @@ void worker_main(fgr_server *S) {
                 job.res.status = st[i];
                 job.res.t_done_ms = t;
                 job.st = St::Done;
-                S->reserved -= job.footprint;
+                S->reserved -= job.footprint + job.granted;
                 S->sets[job.req.set_id].users -= 1;
                 job_finished(S, job);
             }
@@ -542,6 +559,7 @@ void scheduler_main(fgr_server *S) {
         // admit in arrival order (a small request may pass a large one, see
         // next_candidate) while slots and memory allow; a batchable request
         // takes the later compatible ones with it
+        Group alone;
         while (S->running < S->max_inflight) {
             c = next_candidate(S);
             if (c == S->queue.end() || !fits(S, **c)) break;
@@ -562,8 +580,16 @@ void scheduler_main(fgr_server *S) {
                 }
             S->running += 1;
             if (j->large) S->running_large += 1;
+            if (g.size() == 1) alone.push_back(j);
             S->admitted.push_back(std::move(g));
         }
+        // spare buffers where the budget has room for them beside every request that it
+        // admits (a batch has no use for them)
+        for (auto &j : alone)
+            if (S->resident + S->reserved + j->spare <= S->budget) {
+                j->granted = j->spare;
+                S->reserved += j->granted;
+            }
         S->cv_work.notify_all();
     }
 }
@@ -590,6 +616,7 @@ fgr_status fgr_server_create(size_t hbm_budget_bytes, int32_t max_inflight, fgr_
         delete S;
         return FGR_E_CUDA;
     }
+    if (cudaDeviceGetAttribute(&S->num_sms, cudaDevAttrMultiProcessorCount, S->device) != cudaSuccess) cudaGetLastError();
     S->budget = hbm_budget_bytes;
     S->max_inflight = max_inflight;
     int *word = nullptr;  // the yield word; without it large requests simply never yield
@@ -771,6 +798,7 @@ fgr_status fgr_submit(fgr_server *S, const fgr_request *req, uint64_t *ticket) {
     }
     j->footprint = footprint(j->req, it->second);
     j->large = j->req.method == 0 && est_direct_ms(j->req, it->second.m) > kLargeMs;
+    j->spare = spare_bytes(j->req, it->second, S->num_sms);
     // cached plans do not count: the scheduler frees them for requests that need their memory
     if (S->resident - S->plan_resident + j->footprint > S->budget) {
         set_error("submit: request needs %zu bytes; budget %zu with %zu resident in packet sets", j->footprint,
