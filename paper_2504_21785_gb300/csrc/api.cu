@@ -1094,8 +1094,11 @@ fgr_status fgr_fggc_plan_create(fgr_ctx *ctx, const fgr_packets *pk, int32_t mar
             if (e == cudaSuccess && b.fft_elems > 0) e = palloc(&pl->buf.twiddle, eb * 4096);
             BinBox bb;
             if (e == cudaSuccess && ctx->opt.precision == FGR_FP32 && make_bin_box(b, ctx->d, pk->m, &bb)) {
+                // (a plan that the server makes for a batch has no spare bytes: batches
+                // scatter per packet)
                 pl->buf.bin_bytes = bin_buffer_bytes(pk->m, bb);
-                if (palloc(&pl->buf.bin, pl->buf.bin_bytes) != cudaSuccess) {  // the per-packet scatter needs none
+                if ((ctx->d == 2 && pl->buf.bin_bytes > ctx->spare_bytes) ||
+                    palloc(&pl->buf.bin, pl->buf.bin_bytes) != cudaSuccess) {  // the per-packet scatter needs none
                     cudaGetLastError();
                     pl->buf.bin = nullptr;
                     pl->buf.bin_bytes = 0;

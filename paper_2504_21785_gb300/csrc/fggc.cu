@@ -1000,6 +1000,7 @@ bool make_bin_box(const FggcBox &box, int d, int64_t m, BinBox *bb) {
         if (K > kMaxBinKeys || K > m) return false;
     }
     x.K = K;
+    x.boxes = d == 3;
     *bb = x;
     return true;
 }
@@ -1024,7 +1025,7 @@ size_t carve_bin_buffers(char *p, int64_t m, const BinBox &bb, BinBuffers *out) 
     out->loose = (int *)take(sizeof(int) * M);
     out->rec = (BinRecord *)take(sizeof(BinRecord) * M);
     out->count = (int *)take(sizeof(int) * K);
-    out->kbox = (int4 *)take(sizeof(int4) * K);
+    out->kbox = bb.boxes ? (int4 *)take(sizeof(int4) * K) : nullptr;
     out->off = (int2 *)take(sizeof(int2) * (K + 1));
     out->bsum = (int2 *)take(sizeof(int2) * ((K + 1023) / 1024));
     out->items = (BinItem *)take(sizeof(BinItem) * (size_t)bin_max_items(m));
@@ -1042,6 +1043,7 @@ size_t fggc_spare_bytes(int d, int n1, int64_t m) {
     if (d < 2 || (n1 != 4 && n1 != 8) || m >= INT_MAX || (d == 2 && m < kBinMinPackets2d)) return 0;
     BinBox bb;
     bb.K = m;  // (2-D: at most)
+    bb.boxes = d == 3;
     return bin_buffer_bytes(m, bb);
 }
 

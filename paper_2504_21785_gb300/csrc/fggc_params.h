@@ -88,6 +88,7 @@ struct BinBox {
     int tiles_a = 1, tiles_b = 1;
     int dqmin = 0, dqmax = 0, dpmin = 0, dpmax = 0;  // neighbour shift ranges
     int64_t K = 0;                                   // keys
+    bool boxes = false;                              // every key keeps its inner anchors' box (d = 3)
 };
 
 // Constants of a packet's record as unevaluated FP32 sums (see split_double).
@@ -119,7 +120,7 @@ struct BinBuffers {
     int *loose = nullptr;   // [m] packets of small cells
     BinRecord *rec = nullptr;  // [m] records of the binned packets, by key
     int *count = nullptr;   // [K] packets per key
-    int4 *kbox = nullptr;   // [K] min a, min -a, min b, min -b of the inner anchors per key
+    int4 *kbox = nullptr;   // [K] min a, min -a, min b, min -b of the inner anchors per key (d = 3)
     int2 *off = nullptr;    // [K + 1] (first record, first item) per key; totals at K
     int2 *bsum = nullptr;   // [ceil(K / 1024)] block totals of the scan
     BinItem *items = nullptr;  // [max items]
