@@ -537,6 +537,15 @@ __global__ void pass_terms_kernel(const int2 *__restrict__ brange, int64_t lines
     if ((threadIdx.x & 31) == 0 && t) atomicAdd(out, t);
 }
 
+fgr_status launch_pass_terms(const int2 *brange, int64_t lines, int A, const int2 *win, int num_sms,
+                             unsigned long long *out, cudaStream_t st) {
+    const unsigned blocks =
+        (unsigned)std::max<int64_t>(1, std::min<int64_t>((lines + 255) / 256, (int64_t)num_sms * 8));
+    pass_terms_kernel<<<blocks, 256, 0, st>>>(brange, lines, A, win, out);
+    FGR_CUDA_TRY(cudaGetLastError());
+    return FGR_OK;
+}
+
 // flags: row flags of the first pass (lines of unmarked rows are empty), or null.
 template <bool FP64>
 fgr_status launch_brange(const void *in, int64_t rows, int A, int B, const uint8_t *flags, int2 *out,
@@ -1329,6 +1338,17 @@ fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, 
         if (timer) timer->mark(&ctx->timing.last.pass_ms);
         cur = dst;
     }
+    // (after the last mark: the inputs of the passes, cleared by the caller where a pass
+    // leaves them unwritten)
+    for (int l = D - 1; b.terms && l >= 0; --l) {
+        const void *in = l == D - 1 ? b.W : (l == D - 2 ? b.buf1 : b.buf2);
+        fgr_status r = launch_brange<FP64>(in, pp[l].rows, pp[l].A, pp[l].B, l == D - 1 ? b.flags : nullptr,
+                                           b.term_lines, st);
+        if (r == FGR_OK)
+            r = launch_pass_terms(b.term_lines, pp[l].rows * (int64_t)pp[l].A, pp[l].A, T.tab[l].win, ctx->num_sms,
+                                  b.terms, st);
+        if (r != FGR_OK) return r;
+    }
     return FGR_OK;
 }
 
@@ -1336,7 +1356,7 @@ fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, 
 // and work list fit the shared memory, the tensor maps' rules hold (16-byte
 // bases, even b extents: make_box) and the grids fit a launch.
 bool rows_apply(const fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, int D) {
-    if (D < 2 || b.terms || ctx->tune.pass_tile == 128 || !tensor_map_encoder()) return false;
+    if (D < 2 || ctx->tune.pass_tile == 128 || !tensor_map_encoder()) return false;
     const Grid &G = ctx->grid;
     const bool fp64 = ctx->opt.precision == FGR_FP64;
     if (fp64 && !row_phases_fit(box.c, D, G)) return false;
@@ -1446,11 +1466,9 @@ fgr_status enqueue_fggc(fgr_ctx *ctx, const PacketsDev &pk, const FggcBox &box, 
         if (timer) {
             timer->mark(&ctx->timing.last.pass_ms);
             if (b.terms) {
-                const int64_t lines = pp.rows * (int64_t)pp.A;
-                const unsigned blocks = (unsigned)std::max<int64_t>(
-                    1, std::min<int64_t>((lines + 255) / 256, (int64_t)ctx->num_sms * 8));
-                pass_terms_kernel<<<blocks, 256, 0, st>>>(b.brange, lines, pp.A, (const int2 *)b.tables, b.terms);
-                FGR_CUDA_TRY(cudaGetLastError());
+                r = launch_pass_terms(b.brange, pp.rows * (int64_t)pp.A, pp.A, (const int2 *)b.tables, ctx->num_sms,
+                                      b.terms, st);
+                if (r != FGR_OK) return r;
             }
         }
         if (D > 1) {
@@ -1534,6 +1552,14 @@ fgr_status launch(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStream_t 
         b.terms = (unsigned long long *)scratch.get(sizeof(unsigned long long));
         if (!b.terms) return FGR_E_NOMEM;
         FGR_CUDA_TRY(cudaMemsetAsync(b.terms, 0, sizeof(unsigned long long), st));
+        if (D > 1) {
+            b.term_lines = (int2 *)scratch.get(sizeof(int2) * (size_t)box.max_lines);
+            if (!b.term_lines) return FGR_E_NOMEM;
+            timer.mark(&ctx->timing.last.prep_ms);
+            FGR_CUDA_TRY(cudaMemsetAsync(b.buf1, 0, eb * (size_t)box.maxbuf, st));
+            FGR_CUDA_TRY(cudaMemsetAsync(b.buf2, 0, eb * (size_t)box.maxbuf, st));
+            timer.mark(nullptr);
+        }
     }
     r = enqueue_fggc<D>(ctx, pk, box, b, u_dev, st, &timer, &launches);
     if (r != FGR_OK) return r;

@@ -75,6 +75,7 @@ struct FggcBuffers {
     void *bin = nullptr;     // binning buffers of the FP32 scatter, d >= 2 (NULL: per-packet scatter)
     size_t bin_bytes = 0;    // bytes of the binning buffers
     unsigned long long *terms = nullptr;  // node-point terms of the passes (timed calls only)
+    int2 *term_lines = nullptr;  // b-range per line for counting them (d >= 2)
     void *fft = nullptr;      // DFT lines of the commensurate grid stage (box.fft_elems complex)
     void *twiddle = nullptr;  // e^{2 pi i j / N}, j < N / 2 <= 4096 (complex)
 };
