@@ -370,10 +370,11 @@ void fgr_fggc_plan_destroy(fgr_fggc_plan *plan);
  * 8, 16, 32; fgr_reconstruct_direct cuts each output tile's packet list into
  * slices in proportion to its length so that about that many items per SM
  * exist, heaviest first, and persistent CTAs pull them; the batched call gives
- * every tile of a request the same number of slices) and, for the FGGC grid passes (methods & 2), the tile width (128 or 32
- * grid points per CTA) with each CTA-per-SM target (4, 8, 16, 32, 64) on these
- * packets and this context's grid (u_out receives the last result), keeps the
- * fastest in the context and in a process-wide table keyed by (d, precision,
+ * every tile of a request the same number of slices) and, for the FGGC grid
+ * passes (methods & 2), the tile width (128 or 32 grid points per CTA) with each
+ * CTA-per-SM target (4, 8, 16, 32, 64; the row-wise passes of most calls in 2-D
+ * and 3-D have neither: both stay as they are) on these packets and this
+ * context's grid (u_out receives the last result), keeps the fastest in the context and in a process-wide table keyed by (d, precision,
  * packets and grid points rounded to powers of two) that seeds later contexts;
  * with FGR_TUNE_FILE set, the table is loaded from and appended to that file.
  * Waits for its own timing runs. */
@@ -381,8 +382,10 @@ fgr_status fgr_autotune(fgr_ctx *ctx, const fgr_packets *pk, void *u_out, int32_
                         void *cuda_stream);
 /* The context's launch shapes: work-item (direct sum) and CTA (grid passes)
  * targets per SM (1..256), and the grid-pass tile (32 or 128 grid points per
- * CTA; 0 = chosen from the node band width, the default).  FGR_E_INVALID for
- * values outside those ranges. */
+ * CTA; 0 = chosen from the node band width, the default).  A tile of 128 set here
+ * also selects the point-wise passes for 2-D and 3-D calls that the row-wise ones
+ * would serve; a tuned one does not.  FGR_E_INVALID for values outside those
+ * ranges. */
 fgr_status fgr_get_tuning(const fgr_ctx *ctx, int32_t *direct_ctas_per_sm, int32_t *pass_ctas_per_sm,
                           int32_t *pass_tile);
 fgr_status fgr_set_tuning(fgr_ctx *ctx, int32_t direct_ctas_per_sm, int32_t pass_ctas_per_sm,

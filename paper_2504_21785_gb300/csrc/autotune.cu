@@ -4,12 +4,13 @@
 // of (a) the number of CTAs per SM the direct sum aims for when it splits the
 // packet lists of its output tiles and (b) the grid passes' tile width (32 or
 // 128 grid points per CTA) together with the number of CTAs per SM they aim
-// for when they split the node range, on the caller's packets and grid.  The
-// fastest of each is kept in the context and in a process-wide table keyed by
-// the problem class (dimension, precision, packets and grid points rounded to
-// powers of two), from which new contexts of the same class start.  With
-// FGR_TUNE_FILE set, the table is read from and appended to that file (one
-// line per class: d precision log2(M) log2(points) direct pass tile).
+// for when they split the node range, on the caller's packets and grid.  Neither
+// of (b) shapes grid_rows_kernel: where it serves the call (most of d >= 2) they
+// keep their values.  The fastest of each is kept in the context and in a
+// process-wide table keyed by the problem class (dimension, precision, packets and
+// grid points rounded to powers of two), from which new contexts of the same class
+// start.  With FGR_TUNE_FILE set, the table is read from and appended to that file
+// (one line per class: d precision log2(M) log2(points) direct pass tile).
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -50,7 +51,7 @@ void load_file_locked() {
         int d, pr, lm, lg, a, b, t = 0;
         const int n = sscanf(line, "%d %d %d %d %d %d %d", &d, &pr, &lm, &lg, &a, &b, &t);
         if (n < 6 || a < 1 || a > 256 || b < 1 || b > 256 || (t != 0 && t != 32 && t != 128)) continue;
-        g_tuned[ClassKey(d, pr, lm, lg)] = Tuning{a, b, t};
+        g_tuned[ClassKey(d, pr, lm, lg)] = Tuning{a, b, t, false};
     }
     fclose(f);
 }
@@ -137,21 +138,25 @@ fgr_status fgr_autotune(fgr_ctx *ctx, const fgr_packets *pk, void *u_out, int32_
     }
     if (rc == FGR_OK && (methods & 2)) {
         float best_ms = 1e30f;
+        bool rows = false;
+        ctx->rows_probe = &rows;
+        ctx->tune.tile_fixed = best.tile_fixed = false;
         for (int tile : {128, 32}) {
             for (int c : {4, 8, 16, 32, 64}) {
                 ctx->tune.pass_tile = tile;
                 ctx->tune.pass_ctas_per_sm = c;
                 float ms;
                 rc = time_call(true, &ms);
-                if (rc != FGR_OK) break;
+                if (rc != FGR_OK || rows) break;
                 if (ms < best_ms) {
                     best_ms = ms;
                     best.pass_ctas_per_sm = c;
                     best.pass_tile = tile;
                 }
             }
-            if (rc != FGR_OK) break;
+            if (rc != FGR_OK || rows) break;
         }
+        ctx->rows_probe = nullptr;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -164,6 +169,7 @@ fgr_status fgr_autotune(fgr_ctx *ctx, const fgr_packets *pk, void *u_out, int32_
     load_file_locked();
     const ClassKey k = class_of(ctx, pk->m);
     g_tuned[k] = best;
+    g_tuned[k].tile_fixed = false;
     save_line(k, best);
     return FGR_OK;
 }
@@ -186,6 +192,7 @@ fgr_status fgr_set_tuning(fgr_ctx *ctx, int32_t direct_ctas_per_sm, int32_t pass
     ctx->tune.direct_ctas_per_sm = direct_ctas_per_sm;
     ctx->tune.pass_ctas_per_sm = pass_ctas_per_sm;
     ctx->tune.pass_tile = pass_tile;
+    ctx->tune.tile_fixed = pass_tile != 0;
     return FGR_OK;
 }
 

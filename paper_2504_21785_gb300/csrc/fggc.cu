@@ -1356,7 +1356,7 @@ fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, 
 // and work list fit the shared memory, the tensor maps' rules hold (16-byte
 // bases, even b extents: make_box) and the grids fit a launch.
 bool rows_apply(const fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, int D) {
-    if (D < 2 || ctx->tune.pass_tile == 128 || !tensor_map_encoder()) return false;
+    if (D < 2 || (ctx->tune.tile_fixed && ctx->tune.pass_tile == 128) || !tensor_map_encoder()) return false;
     const Grid &G = ctx->grid;
     const bool fp64 = ctx->opt.precision == FGR_FP64;
     if (fp64 && !row_phases_fit(box.c, D, G)) return false;
@@ -1431,6 +1431,7 @@ fgr_status enqueue_fggc(fgr_ctx *ctx, const PacketsDev &pk, const FggcBox &box, 
 
     if constexpr (D > 1) {
         if (rows_apply(ctx, box, b, D)) {
+            if (ctx->rows_probe) *ctx->rows_probe = true;
             return fp64 ? enqueue_rows<D, true>(ctx, box, b, binned, u_dev, st, timer, launches)
                         : enqueue_rows<D, false>(ctx, box, b, binned, u_dev, st, timer, launches);
         }

@@ -81,6 +81,9 @@ struct Tuning {
     int direct_ctas_per_sm = 8;  // direct sum: tiles x slices >= this x SMs
     int pass_ctas_per_sm = 16;   // grid passes: rows x tiles x b-slices >= this x SMs
     int pass_tile = 0;           // grid points per grid-pass CTA: 32, 128, or 0 (by the band width)
+    // pass_tile was set by the caller (fgr_set_tuning): 128 then also keeps d >= 2 calls off
+    // grid_rows_kernel; a tuned 128 only shapes the pass kernels where that one does not apply
+    bool tile_fixed = false;
 };
 
 // Seeds a new context's tuning from the process-wide table (autotune.cu).
@@ -109,6 +112,7 @@ struct fgr_ctx {
     // direct sum, binning of the 2-D FGGC scatter): the server's requests have what was
     // reserved for them within the budget.
     size_t spare_bytes = SIZE_MAX;
+    bool *rows_probe = nullptr;  // set by the autotuner: true when grid_rows_kernel served a call
     int64_t *host_pinned = nullptr;  // small pinned buffer for device->host sizes
 };
 
