@@ -181,7 +181,6 @@ __device__ __forceinline__ void scaled_add(double2 &v, double g, double2 w) {
 }
 
 constexpr int kCB = 32;
-constexpr int kSlice = 8;  // b values per unit of a b-slice (see launch_pass)
 
 // One grid point per thread keeps the Gaussian factors of the band (MAXBAND
 // registers) small enough for several CTAs per SM.  A CTA covers TP = 128 or
@@ -193,6 +192,13 @@ constexpr int kPassPts = 1;  // grid points per thread
 // node band of a tile of tp points (nodes whose window can reach it, + margin)
 inline int pass_band(int tp, double h, double rs, double dq) {
     return (int)std::ceil(((tp - 1) * h + 2 * rs) / dq) + 3;
+}
+
+// Tiles of tp points that a node of the box can reach.
+inline int64_t busy_tiles(const PassParams &pp, int tp) {
+    const double x0 = pp.amin * pp.dq - pp.rs, x1 = (pp.amin + pp.A - 1) * pp.dq + pp.rs;
+    const double m0 = std::max(0.0, (x0 - pp.lo) / pp.h), m1 = std::min((double)pp.N - 1, (x1 - pp.lo) / pp.h);
+    return m1 < m0 ? 0 : (int64_t)(m1 / tp) - (int64_t)(m0 / tp) + 1;
 }
 
 // Per-pass tables shared by all rows: the grid window of every node a (FP64
@@ -240,7 +246,7 @@ template <bool FP64, int MAXBAND, int TP>
 __device__ __forceinline__ void grid_pass_body(const void *__restrict__ in_v, void *__restrict__ out_v,
                                                const PassParams &pp, const uint8_t *__restrict__ flags,
                                                const int2 *__restrict__ brange, const PassTables &tab,
-                                               int64_t row, int tile, int zs, int nz) {
+                                               int64_t row, int tile, int zs, int nz, int unit) {
     using Real = typename std::conditional<FP64, double, float>::type;
     using C2 = typename std::conditional<FP64, double2, float2>::type;
     __shared__ __align__(16) C2 sw[MAXBAND][kCB];
@@ -283,10 +289,10 @@ __device__ __forceinline__ void grid_pass_body(const void *__restrict__ in_v, vo
         ulo = s_blo;
         uhi = s_bhi;
     }
-    // b-slice of this CTA: part zs of nz of [ulo, uhi], in units of kSlice values
-    const int nunit = uhi >= ulo ? (uhi - ulo + kSlice) / kSlice : 0;
+    // b-slice of this CTA: part zs of nz of [ulo, uhi], in units of unit values
+    const int nunit = uhi >= ulo ? (uhi - ulo + unit) / unit : 0;
     const int per = (nunit + nz - 1) / nz;
-    const int bs = ulo + zs * per * kSlice, be = min(uhi + 1, bs + per * kSlice);
+    const int bs = ulo + zs * per * unit, be = min(uhi + 1, bs + per * unit);
     if ((flags && !flags[row]) || bs >= be || nb_total <= 0) {
         if (!split) {
 #pragma unroll
@@ -441,9 +447,9 @@ __device__ __forceinline__ void grid_pass_body(const void *__restrict__ in_v, vo
 template <bool FP64, int MAXBAND, int TP>
 __global__ void __launch_bounds__(TP) grid_pass_kernel(const void *__restrict__ in_v, void *__restrict__ out_v,
                                                        PassParams pp, const uint8_t *__restrict__ flags,
-                                                       const int2 *__restrict__ brange, const PassTables tab) {
+                                                       const int2 *__restrict__ brange, const PassTables tab, int unit) {
     grid_pass_body<FP64, MAXBAND, TP>(in_v, out_v, pp, flags, brange, tab, blockIdx.x, blockIdx.y, blockIdx.z,
-                                      gridDim.z);
+                                      gridDim.z, unit);
 }
 
 template <class C2>
@@ -668,7 +674,7 @@ bool pass_tensor_map(const void *in, const PassParams &pp, int band_lines, CUten
 
 template <bool FP64>
 fgr_status launch_pass(const void *in, void *out, const PassParams &pp, const uint8_t *flags,
-                       const int2 *brange, int64_t target_ctas, int tile_pref, void *tables,
+                       const int2 *brange, int num_sms, int ctas_per_sm, int tile_pref, void *tables,
                        cudaStream_t st, StageMarks *before_pass = nullptr, int *err = nullptr) {
     if (pp.rows == 0 || pp.N == 0) return FGR_OK;
     if (pp.rows > INT_MAX) {
@@ -678,9 +684,10 @@ fgr_status launch_pass(const void *in, void *out, const PassParams &pp, const ui
     // narrow tiles where they cut the band (the work per grid point) by more
     // than a quarter, unless the autotuner or the caller fixed the tile
     const int band128 = pass_band(128, pp.h, pp.rs, pp.dq), band32 = pass_band(32, pp.h, pp.rs, pp.dq);
-    // (FP64 also where the 128-point tiles are fewer than the SMs: the FP64 pipe binds
-    // and every SM has its own)
-    const bool few = FP64 && pp.rows * ((pp.N + 127) / 128) < 148;
+    // (FP64: also where few 128-point tiles have nodes; the FP64 pipe binds and every SM
+    // has its own)
+    const int64_t busy = pp.rows * busy_tiles(pp, 128);
+    const bool few = FP64 && busy * 8 < num_sms;
     const int tp = tile_pref == 32 || tile_pref == 128 ? tile_pref : (few || 4 * band32 < 3 * band128 ? 32 : 128);
     const int band = tp == 32 ? band32 : band128;
     const int64_t mtiles = (pp.N + tp - 1) / tp;
@@ -688,15 +695,17 @@ fgr_status launch_pass(const void *in, void *out, const PassParams &pp, const ui
         set_error("fggc: %lld points per grid dimension; at most %d supported", (long long)pp.N, 65535 * tp);
         return FGR_E_INVALID;
     }
-    // split the b-range when rows x tiles alone cannot fill the device: FP32 into
-    // whole chunks (a CTA's Gaussian factors cost as much as about 8 b values), FP64
-    // down to kSlice values, whose phases (a sine and cosine each) outweigh them
-    // (1024 points x 110 b values: 189 us in 32-value slices of 128-point tiles, 133
-    // in 16-value and 84 in 8-value slices of 32-point tiles)
-    const int64_t target = target_ctas;
-    const int unit = FP64 ? kSlice : kCB, nunit = (pp.B + unit - 1) / unit;
-    int splits = (int)std::min<int64_t>(std::max<int64_t>(1, (target + pp.rows * mtiles - 1) / (pp.rows * mtiles)),
-                                        std::max(1, std::min(nunit, 64)));
+    // split the b-range when rows x tiles alone cannot fill the device, into whole chunks
+    // (a CTA repeats the Gaussian factors of its band: about 8 b values' work in FP32, 14 in
+    // FP64); FP64 where fewer tiles have nodes into 16 values, and 8 with the narrow tiles.
+    // 1-D calls, us, 128-point tiles in units of 8 / 16 / 32 values: 12,000 points, 21 busy
+    // tiles 280 / 314 / 413; 19,000, 33 busy 334 / 331 / 502; 5613, 44 busy 377 / 316 / 386;
+    // 8915, 70 busy 782 / 658 / 652; 22,464, 176 busy 642 / 621 / 507
+    const int64_t target = (int64_t)num_sms * ctas_per_sm;
+    const int unit = !FP64 || busy * 5 >= num_sms * 2 ? kCB : few ? kCB / 4 : kCB / 2;
+    const int nunit = (pp.B + unit - 1) / unit;
+    const int64_t ctas = FP64 ? std::max<int64_t>(1, pp.rows * busy_tiles(pp, tp)) : pp.rows * mtiles;
+    int splits = (int)std::min<int64_t>(std::max<int64_t>(1, (target + ctas - 1) / ctas), std::max(1, std::min(nunit, 64)));
     if (splits > 1) {
         FGR_CUDA_TRY(cudaMemsetAsync(out, 0, (FP64 ? 16 : 8) * (size_t)pp.rows * (size_t)pp.N, st));
     }
@@ -710,7 +719,7 @@ fgr_status launch_pass(const void *in, void *out, const PassParams &pp, const ui
     }
     if (before_pass) before_pass->binned();
     dim3 grid((unsigned)pp.rows, (unsigned)mtiles, (unsigned)splits);
-#define FGR_PASS(MB, TPV) grid_pass_kernel<FP64, MB, TPV><<<grid, TPV, 0, st>>>(in, out, pp, flags, brange, tab)
+#define FGR_PASS(MB, TPV) grid_pass_kernel<FP64, MB, TPV><<<grid, TPV, 0, st>>>(in, out, pp, flags, brange, tab, unit)
 #define FGR_PASS_TP(TPV)                                                                                    \
     if (band <= 16) FGR_PASS(16, TPV);                                                                      \
     else if (band <= 32) FGR_PASS(32, TPV);                                                                 \
@@ -1181,7 +1190,7 @@ __global__ void __launch_bounds__(TP, !FP64 && TP == 128 ? 4 : 1) grid_pass_batc
     const int64_t local = blockIdx.x - B.block0[r];
     const int64_t row = local / B.tiles[r];
     const int tile = (int)(local - row * B.tiles[r]);
-    grid_pass_body<FP64, MAXBAND, TP>(B.in[r], B.out[r], B.pp[r], B.flags[r], B.brange[r], B.tab[r], row, tile, 0, 1);
+    grid_pass_body<FP64, MAXBAND, TP>(B.in[r], B.out[r], B.pp[r], B.flags[r], B.brange[r], B.tab[r], row, tile, 0, 1, kCB);
 }
 
 template <class C2>
@@ -1448,7 +1457,6 @@ fgr_status enqueue_fggc(fgr_ctx *ctx, const PacketsDev &pk, const FggcBox &box, 
                             : launch_brange<false>(cur, pp.rows, pp.A, pp.B, fl, b.brange, st);
         if (r != FGR_OK) return r;
         ++*launches;
-        const int64_t target = (int64_t)ctx->num_sms * ctx->tune.pass_ctas_per_sm;
         StageMarks before{timer, &ctx->timing.last.grid_ms};  // the pass kernel is timed alone
         if (ctx->fft_logn[l] > 0 && b.fft) {
             r = fp64 ? launch_fft_pass<true>(cur, dst, pp, fl, b.brange, ctx->fft_logn[l], b.fft, b.twiddle,
@@ -1457,10 +1465,10 @@ fgr_status enqueue_fggc(fgr_ctx *ctx, const PacketsDev &pk, const FggcBox &box, 
                                               b.tables, st, &before);
             ++*launches;  // twiddles + DFT + contraction (tables and pass counted below)
         } else {
-            r = fp64 ? launch_pass<true>(cur, dst, pp, fl, b.brange, target, ctx->tune.pass_tile, b.tables, st,
-                                         &before, ctx->dev_err)
-                     : launch_pass<false>(cur, dst, pp, fl, b.brange, target, ctx->tune.pass_tile, b.tables, st,
-                                          &before, ctx->dev_err);
+            r = fp64 ? launch_pass<true>(cur, dst, pp, fl, b.brange, ctx->num_sms, ctx->tune.pass_ctas_per_sm,
+                                         ctx->tune.pass_tile, b.tables, st, &before, ctx->dev_err)
+                     : launch_pass<false>(cur, dst, pp, fl, b.brange, ctx->num_sms, ctx->tune.pass_ctas_per_sm,
+                                          ctx->tune.pass_tile, b.tables, st, &before, ctx->dev_err);
         }
         if (r != FGR_OK) return r;
         *launches += 2;  // tables + pass
@@ -2067,9 +2075,9 @@ extern "C" fgr_status fgr_reconstruct_fggc_noalloc(fgr_ctx *ctx, const fgr_packe
     while ((1 << lb) < bmax_abs + 1) ++lb;
     pp.two_pow_b = std::ldexp(1.0, std::max(1, 23 - lb));
     pp.inv_two_pow_b = 1.0 / pp.two_pow_b;
-    const int64_t target = (int64_t)ctx->num_sms * ctx->tune.pass_ctas_per_sm;
-    rc = fp64 ? launch_pass<true>(W, u_out, pp, flags, nullptr, target, ctx->tune.pass_tile, tables, st)
-              : launch_pass<false>(W, u_out, pp, flags, nullptr, target, ctx->tune.pass_tile, tables, st);
+    auto *pass = fp64 ? launch_pass<true> : launch_pass<false>;
+    rc = pass(W, u_out, pp, flags, nullptr, ctx->num_sms, ctx->tune.pass_ctas_per_sm, ctx->tune.pass_tile, tables, st,
+              nullptr, nullptr);
     if (rc != FGR_OK) return rc;
     if (!stream) FGR_CUDA_TRY(cudaStreamSynchronize(st));
     return FGR_OK;
