@@ -590,12 +590,12 @@ inline bool row_phases_fit(const Common &c, int D, const Grid &G) {
 }
 
 // 8-byte entries of the row boxes and ranges of all passes of grid_rows_kernel:
-// a box per row of the first pass, then ranges per tile of contracted points and
-// outer node.
+// ranges (or a box) per row of the first pass, then ranges per tile of contracted
+// points and outer node.
 inline int64_t row_box_entries(const Common &c, int D, const Grid &G) {
     int64_t rows = 1;
     for (int l = 0; l < D - 1; ++l) rows *= (int64_t)c.A[l] * c.B[l];
-    int64_t total = 2 * rows;
+    int64_t total = rows * std::max(2, row_halves(c.B[D - 1]));
     for (int l = D - 1; l > 0; --l) {
         rows = rows / ((int64_t)c.A[l - 1] * c.B[l - 1]) * ((G.n[l] + kBoxPts - 1) / kBoxPts);
         total += rows * row_halves(c.B[l - 1]);
@@ -1231,10 +1231,10 @@ PassParams pass_params(const fgr_ctx *ctx, const Common &c, int l, int64_t prodN
     return pp;
 }
 
-// The grid stage of d >= 2 by grid_rows_kernel.  boxes_known: the row
-// boxes of the first pass are in b.brange already (the binned scatter).
+// The grid stage of d >= 2 by grid_rows_kernel.  binned: the ranges (d = 3: boxes) of
+// the first pass's rows are in b.brange already (the binned scatter).
 template <int D, bool FP64>
-fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, bool boxes_known, void *u_dev,
+fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, bool binned, void *u_dev,
                         cudaStream_t st, StageTimer *timer, int64_t *launches) {
     using C2 = typename std::conditional<FP64, double2, float2>::type;
     constexpr int kRowPts = row_pts<FP64>();
@@ -1263,17 +1263,26 @@ fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, 
             halves = std::max(halves, row_halves(pp[l].B));
             most = std::max<int64_t>(most, std::max<int64_t>(pp[l].A, pp[l].N));
         }
-        *launches += boxes_known ? 1 : 2;  // tables (and the scan of W)
+        *launches += binned ? 1 : 2;  // tables (and the scan of W)
         row_tables_kernel<FP64><<<dim3((unsigned)((most + 255) / 256), D, FP64 ? 1 + halves : 1), 256, 0, st>>>(T);
     }
-    // the rows' boxes and ranges of every pass
-    int4 *rbox = reinterpret_cast<int4 *>(b.brange);
-    if (!boxes_known)
-        row_scan_kernel<C2><<<(unsigned)((box.rows0 + 7) / 8), 256, 0, st>>>((const C2 *)b.W, box.rows0, c.A[D - 1],
-                                                                           c.B[D - 1], b.flags, rbox);
+    // the rows' ranges (d = 3, binned: boxes) of the first pass, then of every other
+    int4 *rbox = D == 3 && binned ? reinterpret_cast<int4 *>(b.brange) : nullptr;
     int2 *range[D] = {};
+    const int halves0 = row_halves(c.B[D - 1]);
+    if (!rbox) range[D - 1] = reinterpret_cast<int2 *>(b.brange);
+    if (!binned) {
+        const int A = c.A[D - 1], B = c.B[D - 1], lanes = B <= 8 ? 8 : B <= 16 ? 16 : 32;
+        const int64_t chunks = (B + lanes - 1) / lanes, threads = box.rows0 * chunks * lanes;
+        const int64_t parts =
+            std::max<int64_t>(1, std::min<int64_t>((int64_t)ctx->num_sms * 2048 / threads, (A + 31) / 32));
+        if (parts > 1) FGR_CUDA_TRY(cudaMemsetAsync(range[D - 1], 0x7f, sizeof(int2) * (size_t)box.rows0 * halves0, st));
+        auto *scan = lanes == 8 ? row_scan_kernel<C2, 8> : lanes == 16 ? row_scan_kernel<C2, 16> : row_scan_kernel<C2, 32>;
+        scan<<<dim3((unsigned)((threads + 255) / 256), (unsigned)parts), 256, 0, st>>>(
+            (const C2 *)b.W, box.rows0, A, B, (int)chunks, halves0, b.flags, range[D - 1]);
+    }
     {
-        int2 *at = reinterpret_cast<int2 *>(rbox + box.rows0);
+        int2 *at = reinterpret_cast<int2 *>(b.brange) + box.rows0 * (rbox ? 2 : halves0);
         int64_t rows = box.rows0;
         for (int l = D - 1; l > 0; --l) {
             const int members = c.A[l - 1] * c.B[l - 1], halves = row_halves(c.B[l - 1]);
@@ -1281,10 +1290,11 @@ fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, 
             range[l - 1] = at;
             FGR_CUDA_TRY(cudaMemsetAsync(at, 0x7f, sizeof(int2) * (size_t)(tiles * groups * halves), st));
             // (every extent in x: a plane of nodes may have more than 65535 x 16 members)
-            const int64_t parts = (members + 15) / 16;
+            const int log_lanes = tiles >= 8 ? 3 : tiles >= 4 ? 2 : tiles >= 2 ? 1 : 0;
+            const int64_t parts = (((int64_t)members << log_lanes) + 127) / 128;
             row_range_kernel<<<(unsigned)(groups * parts), 128, 0, st>>>(
-                l == D - 1 ? rbox : nullptr, range[l], row_halves(c.B[l]), members, (int)parts, c.B[l - 1], groups,
-                T.tab[l].win, halves, at);
+                l == D - 1 ? rbox : nullptr, range[l], row_halves(c.B[l]), members, (int)parts, log_lanes,
+                c.B[l - 1], groups, T.tab[l].win, halves, at);
             rows = groups * tiles;
             at += rows * halves;
             ++*launches;
@@ -1306,14 +1316,23 @@ fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, 
         R.parts = (R.gl + rpc - 1) / rpc;
         R.rpc = (R.gl + R.parts - 1) / R.parts;
         R.chunks = (c.B[l] + kRowB - 1) / kRowB;
+        // slices of the b range: few rows and tiles of many chunks each (1000 packets over
+        // 515 x 980 outer nodes, 1021 x 5 points: second pass 430 -> 53 us)
+        const int64_t warps = pp[l].rows * T.tiles[l], target = (int64_t)ctx->num_sms * kRowSliceWarps;
+        R.slices = (int)std::max<int64_t>(1, std::min<int64_t>({target / warps, R.chunks / kRowSliceChunks, 65535}));
+        R.per = (R.chunks + R.slices - 1) / R.slices;
+        R.slices = (R.chunks + R.per - 1) / R.per;
+        if (R.slices > 1)
+            FGR_CUDA_TRY(cudaMemsetAsync(dst, 0, sizeof(C2) * (size_t)pp[l].rows * (size_t)pp[l].N, st));
         R.near = T.near[l];
         R.phase = T.phase[l];
         // which nodes: the first pass by row, the others by the tiles of the row's points
+        R.box = l == D - 1 ? rbox : nullptr;
         const int64_t tiles2 = D == 3 ? (G.n[D - 1] + kBoxPts - 1) / kBoxPts : 1;
         R.range = range[l];
         R.d1 = INT64_MAX;
         if (l == D - 1) {
-            R.box = rbox;
+            // range[row] as it is
         } else if (l > 0) {  // d = 3, second pass: rows (m_2, a_0, b_0)
             R.d1 = R.stride = (int64_t)c.A[0] * c.B[0];
             R.s1 = kBoxLog;
@@ -1339,7 +1358,7 @@ fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, 
         }
         FGR_CUDA_TRY(cudaFuncSetAttribute(grid_rows_kernel<FP64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)kRowSmemMax));
-        const dim3 grid((unsigned)(outer * R.parts), (unsigned)T.tiles[l]);
+        const dim3 grid((unsigned)(outer * R.parts), (unsigned)T.tiles[l], (unsigned)R.slices);
         grid_rows_kernel<FP64><<<grid, kRowWarps * 32, row_pass_smem<FP64>(R.lines, R.rpc, R.chunks), st>>>(
             map, map_half, (C2 *)dst, R, T.tab[l], ctx->dev_err);
         FGR_CUDA_TRY(cudaGetLastError());
@@ -1426,7 +1445,11 @@ fgr_status enqueue_fggc(fgr_ctx *ctx, const PacketsDev &pk, const FggcBox &box, 
             bl.num_sms = ctx->num_sms;
             bl.rows = box.rows0;
             bl.row_cells = box.cells / box.rows0;
-            bl.row_box = reinterpret_cast<int4 *>(b.brange);
+            if (D == 3)
+                bl.row_box = reinterpret_cast<int4 *>(b.brange);
+            else
+                bl.row_range = b.brange;
+            bl.halves = row_halves(c.B[D - 1]);
             StageMarks marks{timer, &ctx->timing.last.coeff_ms};
             r = launch_binned_scatter(D, L.n1, bl, st, pk, P, b.W, b.flags, &marks);
             *launches += 9;  // key, 3 scans, place, rows, clearing, items, list (and the binned kernel below)

@@ -322,14 +322,15 @@ __global__ void bin_items_kernel(const int2 *__restrict__ off, const int4 *__res
 // Before the scatter: marks every row of W that the packets of an occupied key
 // will reach (the n1^(d-1) outer neighbours of its anchor cell that lie in the
 // node box) and widens the rows' boxes (min a, min -a, min b, min -b of the inner
-// nodes) by the key's.  per (1 or 8) threads per key share out the neighbours of
+// nodes; d = 2: min a, min -a per four b values) by the key's.  per (1 or 8) threads per key share out the neighbours of
 // dimension 0: eight where the keys are few (90,000 of them 29 -> 15 us), one where
 // most threads would only find an empty key (888,000: 43 us against 62).  The binned
 // and per-packet kernels
 // reach exactly these rows, so only they need clearing.
 template <int D>
 __global__ void bin_mark_rows_kernel(const int *__restrict__ count, const int4 *__restrict__ kbox, const Common c,
-                                     const BinBox bb, int per, uint8_t *__restrict__ row_flag, int4 *row_box) {
+                                     const BinBox bb, int per, uint8_t *__restrict__ row_flag, int4 *row_box,
+                                     int2 *row_range, int halves) {
     const int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / per;
     if (k >= bb.K || count[k] == 0) return;
     int oa[D - 1], ob[D - 1], ta, tb;
@@ -341,6 +342,15 @@ __global__ void bin_mark_rows_kernel(const int *__restrict__ count, const int4 *
         row_flag[row] = 1;
         if (!lands) return;
         // (a stale read only costs an atomic)
+        if constexpr (D == 2) {
+            for (int h = box.z / kRowHalf; h <= box.w / kRowHalf; ++h) {
+                int2 *x = row_range + row * halves + h;
+                const int2 now = __ldcg(x);
+                if (box.x < now.x) atomicMin(&x->x, box.x);
+                if (-box.y < now.y) atomicMin(&x->y, -box.y);
+            }
+            return;
+        }
         const int4 v = __ldcg(row_box + row);
         int *b = reinterpret_cast<int *>(row_box + row);
         if (box.x < v.x) atomicMin(b, box.x);
@@ -800,10 +810,13 @@ fgr_status launch_binned_d(const BinLaunch &L, cudaStream_t st, const PacketsDev
     bin_place_kernel<D><<<pblocks, 256, 0, st>>>(pk.q, pk.p, pk.s, pk.a, m, P.c, L.split, b.key, b.rank, b.off, b.rec,
                                                  b.kbox, b.loose, b.ctr);
     // the rows and their boxes, and the clearing of those rows
-    FGR_CUDA_TRY(cudaMemsetAsync(L.row_box, 0x7f, sizeof(int4) * (size_t)L.rows, st));
+    if (D == 3)
+        FGR_CUDA_TRY(cudaMemsetAsync(L.row_box, 0x7f, sizeof(int4) * (size_t)L.rows, st));
+    else
+        FGR_CUDA_TRY(cudaMemsetAsync(L.row_range, 0x7f, sizeof(int2) * (size_t)L.rows * L.halves, st));
     const int per = K < (1 << 18) ? 8 : 1;
     bin_mark_rows_kernel<D><<<(unsigned)((K * per + 255) / 256), 256, 0, st>>>(b.count, b.kbox, P.c, L.box, per, flags,
-                                                                             L.row_box);
+                                                                             L.row_box, L.row_range, L.halves);
     // about 64 warps per SM: few long rows (d = 2: 5,796 of 37 KB) are cut into
     // parts (139 us with one warp per 32 rows, 19 us so), many short ones not
     const int64_t warps = (L.rows + 31) / 32, row_f4 = L.row_cells / 2;

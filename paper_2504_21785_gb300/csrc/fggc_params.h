@@ -70,7 +70,7 @@ struct FggcBox {
 struct FggcBuffers {
     void *W = nullptr, *buf1 = nullptr, *buf2 = nullptr;
     uint8_t *flags = nullptr;
-    int2 *brange = nullptr;  // b-range per (row, a) line, or row boxes (int4)
+    int2 *brange = nullptr;  // b-range per (row, a) line, or row boxes (int4) and ranges
     void *tables = nullptr;  // per-pass tables (node windows, point phases, tile bands)
     void *bin = nullptr;     // binning buffers of the FP32 scatter, d >= 2 (NULL: per-packet scatter)
     size_t bin_bytes = 0;    // bytes of the binning buffers
@@ -128,6 +128,9 @@ struct BinBuffers {
     int *ctr = nullptr;     // [4] loose count, work counter
 };
 
+// b values per range of a row's nodes (fggc_rows.cuh).
+constexpr int kRowHalf = 4;
+
 struct BinLaunch {
     BinBox box;
     BinBuffers buf;
@@ -137,7 +140,11 @@ struct BinLaunch {
     // are marked and zeroed
     int64_t rows = 0;
     int64_t row_cells = 0;
-    int4 *row_box = nullptr;  // [rows] receives the box of every row's inner nodes
+    // receive the inner nodes of every row: d = 3 its box, d = 2 the range of a per four b
+    // values (halves of them), as grid_rows_kernel reads them
+    int4 *row_box = nullptr;    // [rows]
+    int2 *row_range = nullptr;  // [rows][halves]
+    int halves = 0;
 };
 
 // Largest key box of the binned scatter; larger boxes use the per-packet kernel.

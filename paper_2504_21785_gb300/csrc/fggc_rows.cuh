@@ -1,12 +1,11 @@
 // K5 for d >= 2: one separable pass of eq. 2.24, rows [a][b] -> [m],
 // with the output written in the layout the next pass reads.
 //
-// Every row knows which nodes it has: in the first pass the box (a-range x
-// b-range) of its non-zero nodes, from the bins of the scatter (or a scan of W); in
-// the next ones, per four b values, the range of a, from the rows that feed them
-// and the node windows, for every kBoxPts points already contracted
-// (row_range_kernel; position and momentum are correlated, so that the box of a
-// row would be several times larger).  A pass reads and multiplies only those
+// Every row knows which nodes it has: per four b values the range of a (position and
+// momentum are correlated, so that the box of a row would be several times larger).  In
+// the first pass from a scan of W or, after the binned scatter, from the bins (d = 3: the
+// row's box); in the next ones from the rows that feed them and the node windows, for
+// every kBoxPts points already contracted (row_range_kernel).  A pass reads and multiplies only those
 // nodes, and writes only what the next pass reads, so the dead part of the node
 // array (3 rows of 4 on the 3-D workload) is neither read nor written.
 //
@@ -47,7 +46,7 @@ __host__ __device__ constexpr int row_pts() {
 constexpr int kBoxLog = 3;
 constexpr int kBoxPts = 1 << kBoxLog;  // contracted points that share their ranges
 constexpr int kRowB = 8;        // b values per tile
-constexpr int kRowHalf = kRowB / 2;  // b values per range
+static_assert(kRowB == 2 * kRowHalf, "a tile holds two ranges");
 constexpr int kRowLines = 32;   // nodes per tile
 constexpr int kRowWarps = 4;
 constexpr int kRowMax = 24;     // rows per CTA, at most
@@ -57,6 +56,8 @@ __host__ __device__ constexpr int row_stage() {
     return row_pts<FP64>() + (FP64 ? 1 : 2);
 }
 constexpr size_t kRowSmemMax = 96 * 1024;
+// Slices of a pass's b range: up to this many warps per SM, of at least this many chunks.
+constexpr int kRowSliceWarps = 16, kRowSliceChunks = 4;
 
 // Boxes and ranges hold minima: (min a, min -a, min b, min -b) and (min a, min -a);
 // kBoxEmpty where there is nothing.
@@ -66,12 +67,13 @@ struct RowPass {
     PassParams pp;
     // rows in groups of gl (consecutive b of a line of the next pass), parts CTAs per group
     int gl, parts, rpc;
+    int slices, per;  // CTAs (blockIdx.z) that share out a row's chunks, per chunks each, and add to the output
     int lines;   // node lines of the factor table: at most min(band, A)
     int chunks;  // tiles of kRowB values in B
     const float2 *near;   // FP32: [N] offset from the nearest node, and its index
     const double2 *phase;  // FP64: [N] rotation of one b step, then [halves][N] phases of the middle b's
-    // first pass: box[row]; else ranges[r * halves + b / kRowHalf], halves = ceil(B / kRowHalf),
-    // of r = ((row / d1) >> s1) * stride + ((row % d1) >> s0)
+    // ranges[r * halves + b / kRowHalf], halves = ceil(B / kRowHalf), of
+    // r = ((row / d1) >> s1) * stride + ((row % d1) >> s0); or box[row]
     const int4 *box;
     const int2 *range;
     int64_t d1, stride;
@@ -137,13 +139,16 @@ __global__ void __launch_bounds__(kRowWarps * 32, FP64 ? 4 : 5)
     const int64_t row0 = o * R.gl + r0;
     const int2 band = tab.band[tile];
     const int band0 = band.x - pp.amin;  // first node of the band
+    const int k_first = (int)blockIdx.z * R.per, k_end = k_first + R.per;
     bool any = false;
     for (int e = tid; e < nr * R.chunks; e += kRowWarps * 32) {
         const int r = e / R.chunks, k = e - r * R.chunks;
         const int64_t row = row0 + r;
         int lo = kBoxEmpty, hi = kBoxEmpty;  // min a, min -a
         unsigned halves = 0;
-        if (R.box) {
+        if (k < k_first || k >= k_end) {
+            // another slice's
+        } else if (R.box) {
             const int4 b = R.box[row];
             const int b0 = k * kRowB;
             if (b.x != kBoxEmpty && b.z < b0 + kRowB && -b.w >= b0) {
@@ -173,6 +178,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, FP64 ? 4 : 5)
         any = any || nl > 0;
     }
     any = __syncthreads_or(any);
+    if (!any && R.slices > 1) return;
     const int m = tile * kRowPts + PPL * lane;
     if (any) {
         // Gaussian factors of the band: thread = one point, every other line; dx from
@@ -380,7 +386,13 @@ __global__ void __launch_bounds__(kRowWarps * 32, FP64 ? 4 : 5)
     for (int e = tid; e < nr * kRowPts; e += kRowWarps * 32) {
         const int pt = e / nr, r = e - pt * nr;
         const int64_t mp = (int64_t)tile * kRowPts + pt;
-        if (mp < pp.N) out[mp * pp.rows + row0 + r] = stage[r * kRowStage + pt];
+        if (mp >= pp.N) continue;
+        C2 *to = out + (mp * pp.rows + row0 + r);
+        const C2 v = stage[r * kRowStage + pt];
+        if (R.slices > 1)
+            atomic_add_c(to, v.x, v.y);
+        else
+            *to = v;
     }
 }
 
@@ -389,13 +401,16 @@ __global__ void __launch_bounds__(kRowWarps * 32, FP64 ? 4 : 5)
 // reach the points of tile t through their windows (win: first and last point of
 // every node) widen out[(t * groups + g) * halves + b / kRowHalf] by a.  A
 // member's nodes: box[g * members + i], or range[(g * members + i) * in_halves ...].
-// Eight lanes per member share out its tiles; CTA p of the parts of a group has members
-// 16 p to 16 p + 15.
+// 1 << log_lanes lanes per member share out its tiles (one where there is a single tile:
+// 530,000 members 104 -> 35 us against eight); part p of a group has consecutive
+// members.
 __global__ void __launch_bounds__(128) row_range_kernel(const int4 *__restrict__ box, const int2 *__restrict__ range,
-                                                        int in_halves, int members, int parts, int B, int64_t groups,
-                                                        const int2 *__restrict__ win, int halves, int2 *out) {
+                                                        int in_halves, int members, int parts, int log_lanes, int B,
+                                                        int64_t groups, const int2 *__restrict__ win, int halves,
+                                                        int2 *out) {
     const int64_t g = blockIdx.x / (unsigned)parts;
-    const int i = (int)(blockIdx.x % (unsigned)parts) * (blockDim.x / 8) + threadIdx.x / 8;
+    const int i = (int)(((blockIdx.x % (unsigned)parts) * blockDim.x + threadIdx.x) >> log_lanes);
+    const int lanes = 1 << log_lanes;
     if (i >= members) return;
     int lo = kBoxEmpty, hi = kBoxEmpty;
     if (box) {
@@ -412,7 +427,7 @@ __global__ void __launch_bounds__(128) row_range_kernel(const int4 *__restrict__
     if (lo == kBoxEmpty) return;
     const int first = max(0, win[lo].x), last = win[-hi].y;  // windows ascend with the node
     const int a = i / B, h = (i - a * B) / kRowHalf;
-    for (int t = (first >> kBoxLog) + threadIdx.x % 8; t << kBoxLog <= last; t += 8) {
+    for (int t = (first >> kBoxLog) + (int)(threadIdx.x & (lanes - 1)); t << kBoxLog <= last; t += lanes) {
         int2 *x = out + (t * groups + g) * halves + h;
         const int2 now = __ldcg(x);  // (a stale read only costs an atomic)
         if (a < now.x) atomicMin(&x->x, a);
@@ -420,32 +435,42 @@ __global__ void __launch_bounds__(128) row_range_kernel(const int4 *__restrict__
     }
 }
 
-// Boxes of the rows of W by reading the flagged ones (the per-packet scatter):
-// one warp per row.
-template <class C2>
+// Ranges of a per row of W and four b values (see RowPass) by reading the flagged rows
+// (the per-packet scatter): LANES lanes take as many consecutive b values of a row, line
+// after line (few where B is small: 530,000 rows of 40 cells 126 -> 59 us), and
+// blockIdx.y of gridDim.y a part of the lines: rows too few to fill the device are cut,
+// and their ranges, empty before, take the parts' minima.
+template <class C2, int LANES>
 __global__ void __launch_bounds__(256) row_scan_kernel(const C2 *__restrict__ W, int64_t rows, int A, int B,
-                                                       const uint8_t *__restrict__ flags, int4 *__restrict__ box) {
-    const int lane = threadIdx.x & 31;
-    const int64_t row = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (row >= rows) return;
-    int4 v = make_int4(kBoxEmpty, kBoxEmpty, kBoxEmpty, kBoxEmpty);
-    if (flags[row]) {
-        const C2 *p = W + row * (int64_t)A * B;
-        const int cells = A * B;
-        for (int e = lane; e < cells; e += 32) {
-            const C2 x = p[e];
+                                                       int chunks, int halves, const uint8_t *__restrict__ flags,
+                                                       int2 *__restrict__ out) {
+    const int64_t i = blockIdx.x * (int64_t)(256 / LANES) + threadIdx.x / LANES;
+    const int64_t row = i / chunks;
+    const int b = (int)(i - row * chunks) * LANES + threadIdx.x % LANES;
+    int lo = kBoxEmpty, hi = kBoxEmpty;  // min a, min -a
+    if (row < rows && b < B && flags[row]) {
+        const int part = (A - 1) / (int)gridDim.y + 1, a0 = (int)blockIdx.y * part, a1 = min(A, a0 + part);
+        const C2 *p = W + (row * A + a0) * (int64_t)B + b;
+#pragma unroll 8
+        for (int a = a0; a < a1; ++a, p += B) {
+            const C2 x = *p;
             if (x.x != 0 || x.y != 0) {
-                const int a = e / B, b = e - a * B;
-                v.x = min(v.x, a);
-                v.y = min(v.y, -a);
-                v.z = min(v.z, b);
-                v.w = min(v.w, -b);
+                lo = min(lo, a);
+                hi = -a;
             }
         }
     }
-    v.x = __reduce_min_sync(0xffffffffu, v.x);
-    v.y = __reduce_min_sync(0xffffffffu, v.y);
-    v.z = __reduce_min_sync(0xffffffffu, v.z);
-    v.w = __reduce_min_sync(0xffffffffu, v.w);
-    if (lane == 0) box[row] = v;
+#pragma unroll
+    for (int o = 1; o < kRowHalf; o *= 2) {
+        lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = min(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+    if (threadIdx.x % kRowHalf > 0 || row >= rows || b >= B) return;
+    int2 *x = out + row * halves + b / kRowHalf;
+    if (gridDim.y == 1) {
+        *x = make_int2(lo, hi);
+    } else if (lo != kBoxEmpty) {
+        atomicMin(&x->x, lo);
+        atomicMin(&x->y, hi);
+    }
 }

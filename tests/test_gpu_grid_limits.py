@@ -43,3 +43,41 @@ def test_too_many_points_per_dimension_is_a_capacity_error():
     assert e.value.status == fgr.fgr.FGR_E_CAPACITY
     got = reconstruct("fggc", pk, dict(d=2, n=[40, 30], lo=[-1, -1], hi=[1, 1]), eps, options("fp32"))
     assert np.linalg.norm(got) > 0
+
+
+@pytest.mark.parametrize("prec,tol", [("fp32", 1e-5), ("fp64", 1e-10)])
+@pytest.mark.parametrize("b_nodes", [2, 7, 8, 9, 16, 17, 40])
+def test_rows_of_few_and_many_cells(b_nodes, prec, tol):
+    """The scan of the node array in groups of 8, 16 and 32 lanes."""
+    eps = 1 / 256
+    mesh = mesh_for(2, eps)
+    rng = np.random.default_rng(b_nodes)
+    m = 200
+    span = max(0.4, b_nodes - 2.4) * mesh.dp  # (anchors and the neighbour above them)
+    q = np.stack([rng.uniform(-0.3, 0.3, m), rng.uniform(-0.2, 0.2, m)])
+    p = np.stack([rng.uniform(-0.5, 0.5, m), 0.3 * mesh.dp + rng.uniform(0, span, m)])
+    pk = {"q": q, "p": p, "s": rng.uniform(-1, 1, m), "a": rng.standard_normal((2, m))}
+    grid = dict(d=2, n=[37, 66], lo=[-0.5, -0.6], hi=[0.6, 0.5])
+    R = 6.0 if prec == "fp32" else 8.0
+    got = reconstruct("fggc", pk, grid, eps, options(prec))
+    ref = fggc.reconstruct(pk, grid, eps, mesh.dq, mesh.dp, lsa.Strategy(nq=4, np_=2), R=R)
+    assert rel_l2(got, ref) <= tol
+
+
+@pytest.mark.parametrize("prec,tol", [("fp32", 1e-5), ("fp64", 1e-10)])
+def test_few_rows_of_a_wide_plane(prec, tol):
+    """Many nodes in dimension 1 and few in dimension 0: the scan's and the passes' parts
+    of a row."""
+    eps = 1 / 1024
+    mesh = mesh_for(2, eps)
+    rng = np.random.default_rng(4)
+    m = 60
+    q1, p1 = rng.uniform(-3, 3, m), rng.uniform(-4, 4, m)
+    q1[:2], p1[:2] = (-3, 3), (-4, 4)
+    pk = {"q": np.stack([rng.uniform(0.1, 0.9, m) * mesh.dq, q1]), "p": np.stack([rng.uniform(0.1, 0.9, m) * mesh.dp, p1]),
+          "s": rng.uniform(-1, 1, m), "a": rng.standard_normal((2, m))}
+    grid = dict(d=2, n=[5, 700], lo=[-0.03, -3.2], hi=[0.04, 3.2])
+    R = 6.0 if prec == "fp32" else 8.0
+    got = reconstruct("fggc", pk, grid, eps, options(prec))
+    ref = fggc.reconstruct(pk, grid, eps, mesh.dq, mesh.dp, lsa.Strategy(nq=4, np_=2), R=R)
+    assert rel_l2(got, ref) <= tol
