@@ -1310,9 +1310,12 @@ fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, 
         R.lines = std::min(pass_band(kRowPts, pp[l].h, pp[l].rs, pp[l].dq), pp[l].A);
         R.gl = l > 0 ? c.B[l - 1] : (int)G.n[D - 1];
         const int64_t outer = pp[l].rows / R.gl;
-        // rows per CTA: up to kRowMax, fewer when that leaves SMs idle
+        // rows per CTA: up to kRowMax, fewer where that gives few CTAs (a wave covers a part
+        // of the grid only, and the CTAs that meet it are the work: 2-D, 82,944 packets on
+        // 1024 x 993 points 236 us with 3 CTAs per SM asked for, 202 with 8, 185 with 16; 32
+        // cost small 3-D calls 8 %)
         int rpc = kRowMax;
-        while (rpc > kRowWarps && outer * ((R.gl + rpc - 1) / rpc) * T.tiles[l] < 3 * (int64_t)ctx->num_sms) rpc /= 2;
+        while (rpc > kRowWarps && outer * ((R.gl + rpc - 1) / rpc) * T.tiles[l] < 16 * (int64_t)ctx->num_sms) rpc /= 2;
         R.parts = (R.gl + rpc - 1) / rpc;
         R.rpc = (R.gl + R.parts - 1) / R.parts;
         R.chunks = (c.B[l] + kRowB - 1) / kRowB;
