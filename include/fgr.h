@@ -402,7 +402,7 @@ fgr_status fgr_get_info(const fgr_ctx *ctx, fgr_info *out);
 /* Per-stage device times (milliseconds, CUDA events) of the context's last
  * reconstruct or propagate call, when timing is enabled with fgr_set_timing.
  * FGGC: prep_ms = clearing the node array, coeff_ms = binning the packets by
- * anchor cell (d >= 2, FP32; in 2-D from 131072 packets), scatter_ms = the coefficient and scatter
+ * anchor cell (d >= 2, FP32; in 2-D from 262144 packets, Q4P2 and Q2P4), scatter_ms = the coefficient and scatter
  * kernels, grid_ms = the whole grid stage (eq. 2.24), of which pass_ms is the
  * grid-pass kernels alone; pass_terms = node-point terms of the grid passes
  * (per pass, over every (row, node a) line: the occupied b-range times the

@@ -989,7 +989,7 @@ fgr_status make_box(const fgr_ctx *ctx, const int *hb, int margin, FggcBox *box)
 
 bool make_bin_box(const FggcBox &box, int d, int64_t m, BinBox *bb) {
     if (d < 2 || box.empty || (box.c.n1 != 4 && box.c.n1 != 8) || m >= INT_MAX) return false;
-    if (d == 2 && m < kBinMinPackets2d) return false;
+    if (d == 2 && (m < kBinMinPackets2d || box.c.n1 != 8)) return false;
     const Common &c = box.c;
     BinBox x;
     x.dqmin = x.dpmin = INT_MAX;
@@ -1015,7 +1015,8 @@ bool make_bin_box(const FggcBox &box, int d, int64_t m, BinBox *bb) {
         x.tiles_a = (x.KA[1] + kBinTileA - 1) / kBinTileA;
         x.tiles_b = (x.KB[1] + kBinTileB - 1) / kBinTileB;
         K *= (int64_t)x.tiles_a * x.tiles_b;
-        if (K > kMaxBinKeys || K > m) return false;
+        const double filled = (double)x.KA[1] * x.KB[1] / ((double)x.tiles_a * x.tiles_b * kBinTileA * kBinTileB);
+        if (K > kMaxBinKeys || (double)m * filled < kBinMinMean2d * (double)K) return false;
     }
     x.K = K;
     x.boxes = d == 3;
@@ -1058,9 +1059,9 @@ size_t bin_buffer_bytes(int64_t m, const BinBox &bb) {
 }
 
 size_t fggc_spare_bytes(int d, int n1, int64_t m) {
-    if (d < 2 || (n1 != 4 && n1 != 8) || m >= INT_MAX || (d == 2 && m < kBinMinPackets2d)) return 0;
+    if (d < 2 || (n1 != 4 && n1 != 8) || m >= INT_MAX || (d == 2 && (m < kBinMinPackets2d || n1 != 8))) return 0;
     BinBox bb;
-    bb.K = m;  // (2-D: at most)
+    bb.K = d == 2 ? (int64_t)(m / kBinMinMean2d) : m;  // (2-D: at most)
     bb.boxes = d == 3;
     return bin_buffer_bytes(m, bb);
 }

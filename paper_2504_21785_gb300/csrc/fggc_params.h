@@ -156,9 +156,18 @@ constexpr int kBinMinCount = 8;
 // of one packet per cell 24 x 16, 20 x 12 and 32 x 16 measured the same (2-D
 // workload 1.37 ms), 16 x 12 1.43, 12 x 12 1.48 and 8 x 8 1.77 ms.
 constexpr int kBinTileA = 24, kBinTileB = 16;
-// d = 2: the fewest packets.  The binning's launches take about 40 us, the
-// per-packet kernel 0.25 us per 1024 packets and the binned one half of that.
-constexpr int64_t kBinMinPackets2d = 1 << 17;
+// Where the binned scatter runs in 2-D; each side was measured on sets in mesh order, whose
+// neighbouring threads' reductions meet in L2, and in random order.  n1 = 4: never (mesh
+// order, whole calls, binned / per packet: 147,456 packets 230 / 172 us, 1.0M 414 / 355,
+// 4.2M 907 / 874).  n1 = 8: from kBinMinPackets2d (mesh order 147,456: 247 / 197 us, 262,144:
+// 300 / 279, 419,904: 328 / 333, 1.6M: 626 / 808; random order, 262,144 on 50 x 45 cells per
+// plane 329 / 631), and where the mean bin, scaled by the part of a tile that the inner
+// plane fills, holds kBinMinMean2d packets: an item costs a CTA the same however few it
+// holds, and on small planes the reductions are cheap (5 x 6 cells, 4.2M packets, 8 per
+// bin: 4.6 / 3.2 ms; 24 per bin: 740 / 685 us; 48: 910 / 1196; whole tiles, 10 per bin:
+// 1.82 / 2.41 ms).
+constexpr int64_t kBinMinPackets2d = 1 << 18;
+constexpr double kBinMinMean2d = 8.0;
 
 // Key box of a node box and m packets (false when the binned scatter does not apply).
 bool make_bin_box(const FggcBox &box, int d, int64_t m, BinBox *bb);

@@ -1,0 +1,138 @@
+"""Paths that a call takes at the limits of the faster ones: packets outside the FP32
+form of the sorted records, memory too short for the binning or the partial sums, and
+the row-wise grid passes against the point-wise ones."""
+
+import os
+import subprocess
+import sys
+import textwrap
+
+import numpy as np
+import pytest
+
+import paper_2504_21785_gb300 as fgr
+
+from ._gpu import options, reconstruct, rel_l2
+from .test_gpu_binned import lattice_2d
+
+pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+def _binned(pk, grid, eps, opt):
+    """The call's result, and whether it binned its packets."""
+    with fgr.Context(grid["d"], grid, eps, opt) as ctx:
+        fgr.fgr_set_timing(ctx.handle, 1)
+        u = reconstruct("fggc", pk, grid, eps, opt, ctx=ctx)
+        return u, fgr.fgr_get_stats(ctx.handle).coeff_ms > 0
+
+
+def _in_parts(pk, grid, eps, opt):
+    """The sum of the results of parts that are too few to be binned."""
+    total, step = 0.0, (1 << 18) - 1
+    for i in range(0, pk["s"].size, step):
+        part = {k: np.ascontiguousarray(pk[k][..., i:i + step]) for k in ("q", "p", "s", "a")}
+        u, binned = _binned(part, grid, eps, opt)
+        assert not binned
+        total = total + u.astype(np.complex128)
+    return total
+
+
+@pytest.mark.parametrize("n_a,n_b,thin", [(26, 30, 0.7), (40, 22, 0.5), (23, 64, 0.15)])
+@pytest.mark.parametrize("nq,np_", [(4, 2), (2, 4)])
+def test_binned_2d_tiles_of_large_sets(n_a, n_b, thin, nq, np_):
+    """Edges of the 24 x 16 tiles, bins of one, two and many items and small bins, on a
+    grid that cuts part of the packets off."""
+    pk, mesh, eps = lattice_2d(3, n_a, n_b, 0.45, thin)
+    grid = dict(d=2, n=[65, 44], lo=[-0.7, -0.5], hi=[1.1, 0.9])
+    opt = options("fp32", nq=nq, np_=np_)
+    got, binned = _binned(pk, grid, eps, opt)
+    assert pk["s"].size >= 1 << 18 and binned
+    # both sides round the same contributions and sums to FP32 (2e-7 each)
+    assert rel_l2(got, _in_parts(pk, grid, eps, opt)) <= 2e-6
+
+
+@pytest.mark.parametrize("shift_a,shift_b,amp,act", [
+    (1 << 18, 0, 1.0, 1.0), (-(1 << 18), 0, 1.0, 1.0), (0, 1 << 18, 1.0, 1.0), ((1 << 18) - 10, 3, 1.0, 1.0),
+    (60, 40, 1.0, 3e4)])
+def test_records_at_the_limits_of_their_fp32_form(shift_a, shift_b, amp, act):
+    """Anchors of 2^18 cells and on both sides of it, and actions beyond 2^18 turns, in
+    every packet: the binned scatter against parts of the set that are too few to be
+    binned."""
+    pk, mesh, eps = lattice_2d(6, 26, 21, 0.45)
+    for l in range(2):
+        pk["q"][l] += shift_a * mesh.dq
+        pk["p"][l] += shift_b * mesh.dp
+    pk["a"] *= amp
+    pk["s"] *= act
+    lo = [shift_a * mesh.dq - 0.5, shift_a * mesh.dq - 0.6]
+    grid = dict(d=2, n=[40, 36], lo=lo, hi=[lo[0] + 1.1, lo[1] + 1.2])
+    got, binned = _binned(pk, grid, eps, options("fp32"))
+    assert binned
+    # both sides round the same contributions and sums to FP32 (2e-7 each)
+    assert rel_l2(got, _in_parts(pk, grid, eps, options("fp32"))) <= 2e-6
+
+
+@pytest.mark.parametrize("prec,tol", [("fp32", 2e-6), ("fp64", 1e-12)])
+@pytest.mark.parametrize("n", [(1, 70), (65, 8), (128, 63), (33, 64), (20, 65, 9), (66, 1, 130)])
+@pytest.mark.parametrize("spread", [0.05, 0.9])
+def test_row_wise_passes_against_point_wise_ones(n, spread, prec, tol):
+    """The edges of the row-wise passes' tiles and ranges, with the other pass kernels
+    (pass tile 128) on the same packets."""
+    d, eps = len(n), 1 / 64
+    rng = np.random.default_rng(8)
+    m = 400
+    q, p = rng.uniform(-spread, spread, (d, m)), rng.uniform(-0.8, 0.8, (d, m))
+    p[0] -= 2 * q[0]
+    pk = {"q": q, "p": p, "s": rng.uniform(-1, 1, m), "a": rng.standard_normal((2, m))}
+    # (a single point lies at lo)
+    lo = [-0.05 if k == 1 else x for k, x in zip(n, (-1.3, -1.1, -0.9))]
+    grid = dict(d=d, n=list(n), lo=lo, hi=[1.1, 1.2, 1.3][:d])
+    opt = options(prec)
+    out, launches = [], []
+    for tile in (0, 128):
+        with fgr.Context(d, grid, eps, opt) as ctx:
+            fgr.fgr_set_tuning(ctx.handle, 8, 16, tile)
+            fgr.fgr_set_timing(ctx.handle, 1)
+            out.append(reconstruct("fggc", pk, grid, eps, opt, ctx=ctx))
+            launches.append(fgr.fgr_get_stats(ctx.handle).launches)
+    assert launches[0] != launches[1]
+    # FP32: phases and Gaussians per dimension, below 2e-6; FP64: 1e-15 per term
+    assert rel_l2(out[0], out[1]) <= tol
+
+
+# The scratch allocation that a call can do without is the last of its own (8th of a 2-D
+# FGGC call, 5th of a 1-D direct sum): it fails once, the next call has it.
+@pytest.mark.parametrize("method,d,fail_at", [("fggc", 2, 8), ("direct", 1, 5)])
+def test_short_memory_takes_the_path_without_it(method, d, fail_at):
+    code = """
+        import sys
+        sys.path.insert(0, ".")
+        import numpy as np
+        import paper_2504_21785_gb300 as fgr
+        from tests._gpu import options, reconstruct, rel_l2
+        rng = np.random.default_rng(2)
+        d, m, eps = {d}, 1 << 18, 1 / 64
+        pk = {{"q": rng.uniform(-0.4, 0.4, (d, m)), "p": rng.uniform(-0.5, 0.5, (d, m)), "s": rng.uniform(-1, 1, m),
+              "a": rng.standard_normal((2, m))}}
+        grid = dict(d=d, n=[200, 30][:d], lo=[-0.6] * d, hi=[0.7] * d)
+        ctx = fgr.Context(d, grid, eps, options("fp32"))
+        fgr.fgr_set_timing(ctx.handle, 1)
+        out = []
+        for _ in range(2):
+            out.append(reconstruct("{method}", pk, grid, eps, options("fp32"), ctx=ctx))
+            s = fgr.fgr_get_stats(ctx.handle)
+            print("CALL", s.launches, int(s.coeff_ms > 0))
+        print("ERR", rel_l2(out[0], out[1]))
+    """
+    r = subprocess.run([sys.executable, "-c", textwrap.dedent(code.format(d=d, method=method))], cwd=ROOT,
+                       env=dict(os.environ, FGR_INJECT_ALLOC_FAILURE=str(fail_at), PYTHONPATH=ROOT),
+                       capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
+    lines = [line.split() for line in r.stdout.splitlines()]
+    short, whole = [x for x in lines if x[0] == "CALL"]
+    assert short[1] != whole[1]
+    if method == "fggc":
+        assert (short[2], whole[2]) == ("0", "1")
+    # the same FP32 terms in another order of summation
+    assert float([x for x in lines if x[0] == "ERR"][0][1]) <= 2e-6
