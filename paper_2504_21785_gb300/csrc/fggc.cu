@@ -1294,8 +1294,8 @@ fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, 
             const int log_lanes = tiles >= 8 ? 3 : tiles >= 4 ? 2 : tiles >= 2 ? 1 : 0;
             const int64_t parts = (((int64_t)members << log_lanes) + 127) / 128;
             row_range_kernel<<<(unsigned)(groups * parts), 128, 0, st>>>(
-                l == D - 1 ? rbox : nullptr, range[l], row_halves(c.B[l]), members, (int)parts, log_lanes,
-                c.B[l - 1], groups, T.tab[l].win, halves, at);
+                l == D - 1 ? rbox : nullptr, range[l], row_halves(c.B[l]), members, log_lanes, c.B[l - 1], groups,
+                T.tab[l].win, halves, at);
             rows = groups * tiles;
             at += rows * halves;
             ++*launches;
@@ -1323,10 +1323,10 @@ fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, 
         // slices of the b range: few rows and tiles of many chunks each (1000 packets over
         // 515 x 980 outer nodes, 1021 x 5 points: second pass 430 -> 53 us)
         const int64_t warps = pp[l].rows * T.tiles[l], target = (int64_t)ctx->num_sms * kRowSliceWarps;
-        R.slices = (int)std::max<int64_t>(1, std::min<int64_t>({target / warps, R.chunks / kRowSliceChunks, 65535}));
-        R.per = (R.chunks + R.slices - 1) / R.slices;
-        R.slices = (R.chunks + R.per - 1) / R.per;
-        if (R.slices > 1)
+        int slices = (int)std::max<int64_t>(1, std::min<int64_t>({target / warps, R.chunks / kRowSliceChunks, 65535}));
+        R.per = (R.chunks + slices - 1) / slices;
+        slices = (R.chunks + R.per - 1) / R.per;
+        if (slices > 1)
             FGR_CUDA_TRY(cudaMemsetAsync(dst, 0, sizeof(C2) * (size_t)pp[l].rows * (size_t)pp[l].N, st));
         R.near = T.near[l];
         R.phase = T.phase[l];
@@ -1360,11 +1360,11 @@ fgr_status enqueue_rows(fgr_ctx *ctx, const FggcBox &box, const FggcBuffers &b, 
             set_error("fggc: no tensor map for a grid pass");
             return FGR_E_INTERNAL;
         }
-        FGR_CUDA_TRY(cudaFuncSetAttribute(grid_rows_kernel<FP64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)kRowSmemMax));
-        const dim3 grid((unsigned)(outer * R.parts), (unsigned)T.tiles[l], (unsigned)R.slices);
-        grid_rows_kernel<FP64><<<grid, kRowWarps * 32, row_pass_smem<FP64>(R.lines, R.rpc, R.chunks), st>>>(
-            map, map_half, (C2 *)dst, R, T.tab[l], ctx->dev_err);
+        auto *kernel = slices > 1 ? grid_rows_kernel<FP64, true> : grid_rows_kernel<FP64, false>;
+        FGR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmemMax));
+        const dim3 grid((unsigned)(outer * R.parts), (unsigned)T.tiles[l], (unsigned)slices);
+        kernel<<<grid, kRowWarps * 32, row_pass_smem<FP64>(R.lines, R.rpc, R.chunks), st>>>(map, map_half, (C2 *)dst, R,
+                                                                                            T.tab[l], ctx->dev_err);
         FGR_CUDA_TRY(cudaGetLastError());
         ++*launches;
         if (timer) timer->mark(&ctx->timing.last.pass_ms);

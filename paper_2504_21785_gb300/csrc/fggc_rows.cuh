@@ -67,7 +67,7 @@ struct RowPass {
     PassParams pp;
     // rows in groups of gl (consecutive b of a line of the next pass), parts CTAs per group
     int gl, parts, rpc;
-    int slices, per;  // CTAs (blockIdx.z) that share out a row's chunks, per chunks each, and add to the output
+    int per;     // chunks per slice (blockIdx.z), where slices share out a row's chunks
     int lines;   // node lines of the factor table: at most min(band, A)
     int chunks;  // tiles of kRowB values in B
     const float2 *near;   // FP32: [N] offset from the nearest node, and its index
@@ -101,7 +101,8 @@ __device__ __forceinline__ void horner(C2 &z, Real wr, Real wi, C2 v) {
     z.x = re;
 }
 
-template <bool FP64>
+// SLICED: blockIdx.z takes R.per of the chunks and adds to the output (cleared before).
+template <bool FP64, bool SLICED>
 __global__ void __launch_bounds__(kRowWarps * 32, FP64 ? 4 : 5)
     grid_rows_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap map_half,
                      typename std::conditional<FP64, double2, float2>::type *__restrict__ out,
@@ -139,14 +140,14 @@ __global__ void __launch_bounds__(kRowWarps * 32, FP64 ? 4 : 5)
     const int64_t row0 = o * R.gl + r0;
     const int2 band = tab.band[tile];
     const int band0 = band.x - pp.amin;  // first node of the band
-    const int k_first = (int)blockIdx.z * R.per, k_end = k_first + R.per;
+    const int k_first = SLICED ? (int)blockIdx.z * R.per : 0, k_end = k_first + R.per;
     bool any = false;
     for (int e = tid; e < nr * R.chunks; e += kRowWarps * 32) {
         const int r = e / R.chunks, k = e - r * R.chunks;
         const int64_t row = row0 + r;
         int lo = kBoxEmpty, hi = kBoxEmpty;  // min a, min -a
         unsigned halves = 0;
-        if (k < k_first || k >= k_end) {
+        if (SLICED && (k < k_first || k >= k_end)) {
             // another slice's
         } else if (R.box) {
             const int4 b = R.box[row];
@@ -178,7 +179,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, FP64 ? 4 : 5)
         any = any || nl > 0;
     }
     any = __syncthreads_or(any);
-    if (!any && R.slices > 1) return;
+    if (SLICED && !any) return;
     const int m = tile * kRowPts + PPL * lane;
     if (any) {
         // Gaussian factors of the band: thread = one point, every other line; dx from
@@ -389,7 +390,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, FP64 ? 4 : 5)
         if (mp >= pp.N) continue;
         C2 *to = out + (mp * pp.rows + row0 + r);
         const C2 v = stage[r * kRowStage + pt];
-        if (R.slices > 1)
+        if (SLICED)
             atomic_add_c(to, v.x, v.y);
         else
             *to = v;
@@ -405,11 +406,12 @@ __global__ void __launch_bounds__(kRowWarps * 32, FP64 ? 4 : 5)
 // 530,000 members 104 -> 35 us against eight); part p of a group has consecutive
 // members.
 __global__ void __launch_bounds__(128) row_range_kernel(const int4 *__restrict__ box, const int2 *__restrict__ range,
-                                                        int in_halves, int members, int parts, int log_lanes, int B,
+                                                        int in_halves, int members, int log_lanes, int B,
                                                         int64_t groups, const int2 *__restrict__ win, int halves,
                                                         int2 *out) {
-    const int64_t g = blockIdx.x / (unsigned)parts;
-    const int i = (int)(((blockIdx.x % (unsigned)parts) * blockDim.x + threadIdx.x) >> log_lanes);
+    // (neighbouring CTAs of different groups, whose ranges are apart: 3-D workload 67 -> 28 us)
+    const int64_t g = blockIdx.x % (unsigned)groups;
+    const int i = (int)(((blockIdx.x / (unsigned)groups) * blockDim.x + threadIdx.x) >> log_lanes);
     const int lanes = 1 << log_lanes;
     if (i >= members) return;
     int lo = kBoxEmpty, hi = kBoxEmpty;
