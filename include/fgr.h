@@ -402,14 +402,16 @@ fgr_status fgr_get_info(const fgr_ctx *ctx, fgr_info *out);
 /* Per-stage device times (milliseconds, CUDA events) of the context's last
  * reconstruct or propagate call, when timing is enabled with fgr_set_timing.
  * FGGC: prep_ms = clearing the node array, coeff_ms = binning the packets by
- * anchor cell (d >= 2, FP32; in 2-D from 262144 packets, Q4P2 and Q2P4), scatter_ms = the coefficient and scatter
- * kernels, grid_ms = the whole grid stage (eq. 2.24), of which pass_ms is the
- * grid-pass kernels alone; pass_terms = node-point terms of the grid passes
+ * anchor cell (FP32; d = 3, and d = 2 where the set is large enough for it: from
+ * 131072 packets in random order, 262144 in mesh order, 1.6 million for Q2P2),
+ * scatter_ms = the coefficient and scatter kernels, grid_ms = the whole grid
+ * stage (eq. 2.24), of which pass_ms is the grid-pass kernels alone; pass_terms =
+ * node-point terms of the grid passes
  * (per pass, over every (row, node a) line: the occupied b-range times the
  * grid points in node a's window; counted on the device when timing is set to
  * 2, by a scan and a count per pass outside the stage times; total_ms then
- * includes the clearing of the pass buffers that the count needs).  fgr_set_timing: 0 off, 1 per-stage
- * events, 2 per-stage events and pass_terms. */
+ * includes the clearing of the pass buffers that the count needs).
+ * fgr_set_timing: 0 off, 1 per-stage events, 2 per-stage events and pass_terms. */
 typedef struct {
     double prep_ms, coeff_ms, scatter_ms, grid_ms, direct_ms, propagate_ms, total_ms;
     int64_t launches;       /* kernels launched by the last call */

@@ -1067,10 +1067,10 @@ fgr_status fgr_fggc_plan_create(fgr_ctx *ctx, const fgr_packets *pk, int32_t mar
             return e == cudaErrorMemoryAllocation ? FGR_E_NOMEM : FGR_E_CUDA;
         };
         auto palloc = [&](void **ptr, size_t bytes) { return cudaMallocFromPoolAsync(ptr, bytes, ctx->pool, st); };
-        cudaError_t e = palloc((void **)&pl->bnd, sizeof(int) * 12);
+        cudaError_t e = palloc((void **)&pl->bnd, sizeof(int) * 14);
         if (e == cudaSuccess) e = palloc((void **)&pl->overflow, sizeof(int));
         if (e != cudaSuccess) return fail(e);
-        int hb[12];
+        int hb[14];
         r = compute_node_bounds(ctx, dev, pl->bnd, hb, st);
         if (r != FGR_OK) {
             pl->release();

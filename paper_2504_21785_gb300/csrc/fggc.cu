@@ -144,13 +144,33 @@ __device__ __forceinline__ void bounds_body(const double *__restrict__ q, const 
     }
 }
 
+// Whether packets next to each other lie in cells next to each other: *order rises by one
+// per near pair and falls by one per other pair, over 32 consecutive packets per CTA.
+template <int D>
+__device__ __forceinline__ void order_probe(const double *__restrict__ q, const double *__restrict__ p, int64_t m,
+                                            const Common &c, int *order) {
+    if (threadIdx.x >= 32) return;
+    const int64_t j = min(m - 1, (int64_t)blockIdx.x * m / gridDim.x + threadIdx.x);
+    bool near = true;
+#pragma unroll
+    for (int l = 0; l < D; ++l) {
+        const unsigned a = (unsigned)floor_div_int(q[l * m + j], c.dqv, c.inv_dq);
+        const unsigned b = (unsigned)floor_div_int(p[l * m + j], c.dpv, c.inv_dp);
+        const unsigned da = __shfl_down_sync(0xffffffffu, a, 1) - a, db = __shfl_down_sync(0xffffffffu, b, 1) - b;
+        near = near && da + 2 <= 4 && db + 2 <= 4;
+    }
+    const unsigned pairs = __ballot_sync(0xffffffffu, near) & 0x7fffffffu;
+    if (threadIdx.x == 0) atomicAdd(order, 2 * __popc(pairs) - 31);
+}
+
 template <int D>
 __global__ void bounds_kernel(const double *__restrict__ q, const double *__restrict__ p,
                               const double *__restrict__ a, int64_t m, Common c, int aglo0, int aghi0,
                               int aglo1, int aghi1, int aglo2, int aghi2, int *__restrict__ out,
-                              const double *__restrict__ s) {
+                              const double *__restrict__ s, int *order) {
     const int aglo[3] = {aglo0, aglo1, aglo2}, aghi[3] = {aghi0, aghi1, aghi2};
     bounds_body<D>(q, p, a, m, c, aglo, aghi, out, blockIdx.x, gridDim.x, s);
+    if (D == 2 && order) order_probe<D>(q, p, m, c, order);
 }
 
 // CTAs of the bounds kernel: enough to fill the GPU, few enough that the
@@ -818,7 +838,7 @@ fgr_status launch_transpose(const void *in, void *out, int64_t R, int64_t Cc, cu
 // b[0..12) the empty bounds; b[12] (when present) the non-finite flag.
 __global__ void bounds_init_kernel(int *__restrict__ b, int n) {
     if (threadIdx.x < 12) b[threadIdx.x] = (threadIdx.x & 1) ? INT_MIN : INT_MAX;
-    if (threadIdx.x == 12 && n > 12) b[12] = 0;
+    if (threadIdx.x >= 12 && threadIdx.x < n) b[threadIdx.x] = 0;
 }
 
 // Sets *overflow when the packets' node bounds b[] leave the planned box.
@@ -890,25 +910,27 @@ void grid_node_range(const fgr_ctx *ctx, int *aglo, int *aghi) {
 }
 
 // Launches the node-bounds reduction of the packets into b[12] (device).
-// check_finite: also test every packet value (b holds 13 ints, b[12] the flag).
+// check_finite: also test every packet value (b[12] the flag).  order: b[13] > 0 where
+// neighbouring packets are near (2-D sets that may be binned); b then holds 14 ints.
 fgr_status launch_bounds_reduction(const fgr_ctx *ctx, const PacketsDev &pk, const Common &c, const int *aglo,
-                                   const int *aghi, int *b, cudaStream_t st, bool check_finite = false) {
-    bounds_init_kernel<<<1, 32, 0, st>>>(b, check_finite ? 13 : 12);
+                                   const int *aghi, int *b, cudaStream_t st, bool check_finite = false, bool order = false) {
+    bounds_init_kernel<<<1, 32, 0, st>>>(b, check_finite || order ? 14 : 12);
     const double *sv = check_finite ? pk.s : nullptr;
+    int *pr = order && ctx->opt.precision == FGR_FP32 && pk.m >= kBinMinPackets2d ? b + 13 : nullptr;
     if (pk.m > 0) {
         const unsigned blocks = bounds_blocks(ctx, pk.m);
         switch (ctx->d) {
         case 1:
             bounds_kernel<1><<<blocks, 256, 0, st>>>(pk.q, pk.p, pk.a, pk.m, c, aglo[0], aghi[0], aglo[1], aghi[1],
-                                                     aglo[2], aghi[2], b, sv);
+                                                     aglo[2], aghi[2], b, sv, pr);
             break;
         case 2:
             bounds_kernel<2><<<blocks, 256, 0, st>>>(pk.q, pk.p, pk.a, pk.m, c, aglo[0], aghi[0], aglo[1], aghi[1],
-                                                     aglo[2], aghi[2], b, sv);
+                                                     aglo[2], aghi[2], b, sv, pr);
             break;
         default:
             bounds_kernel<3><<<blocks, 256, 0, st>>>(pk.q, pk.p, pk.a, pk.m, c, aglo[0], aghi[0], aglo[1], aghi[1],
-                                                     aglo[2], aghi[2], b, sv);
+                                                     aglo[2], aghi[2], b, sv, pr);
         }
     }
     FGR_CUDA_TRY(cudaGetLastError());
@@ -917,7 +939,7 @@ fgr_status launch_bounds_reduction(const fgr_ctx *ctx, const PacketsDev &pk, con
 
 }  // namespace
 
-// Node box from the packets' bounds hb[12], widened by margin nodes on every
+// Node box from the packets' bounds hb[14], widened by margin nodes on every
 // side (a-ranges clipped to the grid-relevant range), and the sizes of the
 // buffers of one reconstruction.
 fgr_status make_box(const fgr_ctx *ctx, const int *hb, int margin, FggcBox *box) {
@@ -931,6 +953,7 @@ fgr_status make_box(const fgr_ctx *ctx, const int *hb, int margin, FggcBox *box)
     Common &c = x.c;
     x.empty = hb[0] == INT_MAX;
     if (x.empty) return FGR_OK;
+    x.apart = hb[13] <= 0;
     int64_t cells = 1;
     for (int l = 0; l < D; ++l) {
         const int alo = std::max(aglo[l], hb[l * 4 + 0] - margin), ahi = std::min(aghi[l], hb[l * 4 + 1] + margin);
@@ -989,7 +1012,7 @@ fgr_status make_box(const fgr_ctx *ctx, const int *hb, int margin, FggcBox *box)
 
 bool make_bin_box(const FggcBox &box, int d, int64_t m, BinBox *bb) {
     if (d < 2 || box.empty || (box.c.n1 != 4 && box.c.n1 != 8) || m >= INT_MAX) return false;
-    if (d == 2 && (m < kBinMinPackets2d || box.c.n1 != 8)) return false;
+    if (d == 2 && m < kBinMinPackets2d) return false;
     const Common &c = box.c;
     BinBox x;
     x.dqmin = x.dpmin = INT_MAX;
@@ -1016,7 +1039,10 @@ bool make_bin_box(const FggcBox &box, int d, int64_t m, BinBox *bb) {
         x.tiles_b = (x.KB[1] + kBinTileB - 1) / kBinTileB;
         K *= (int64_t)x.tiles_a * x.tiles_b;
         const double filled = (double)x.KA[1] * x.KB[1] / ((double)x.tiles_a * x.tiles_b * kBinTileA * kBinTileB);
-        if (K > kMaxBinKeys || (double)m * filled < kBinMinMean2d * (double)K) return false;
+        const double mean = (double)m * filled / (double)K;
+        if (K > kMaxBinKeys || mean < (box.apart ? kBinMinMean2d : kBinMinMeanNear)) return false;
+        const int64_t least = box.c.n1 == 8 ? kBinMinNear8 : mean < kBinDense ? kBinMinNear4 : kBinMinNear4 / 3;
+        if (!box.apart && m < least) return false;
     }
     x.K = K;
     x.boxes = d == 3;
@@ -1059,7 +1085,7 @@ size_t bin_buffer_bytes(int64_t m, const BinBox &bb) {
 }
 
 size_t fggc_spare_bytes(int d, int n1, int64_t m) {
-    if (d < 2 || (n1 != 4 && n1 != 8) || m >= INT_MAX || (d == 2 && (m < kBinMinPackets2d || n1 != 8))) return 0;
+    if (d < 2 || (n1 != 4 && n1 != 8) || m >= INT_MAX || (d == 2 && m < kBinMinPackets2d)) return 0;
     BinBox bb;
     bb.K = d == 2 ? (int64_t)(m / kBinMinMean2d) : m;  // (2-D: at most)
     bb.boxes = d == 3;
@@ -1530,12 +1556,12 @@ fgr_status launch(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStream_t 
     const Common c = base_common(ctx);
     int aglo[3], aghi[3];
     grid_node_range(ctx, aglo, aghi);
-    int *bnd = (int *)scratch.get(sizeof(int) * 13);
+    int *bnd = (int *)scratch.get(sizeof(int) * 14);
     if (!bnd) return FGR_E_NOMEM;
-    fgr_status r = launch_bounds_reduction(ctx, pk, c, aglo, aghi, bnd, st, check_finite);
+    fgr_status r = launch_bounds_reduction(ctx, pk, c, aglo, aghi, bnd, st, check_finite, true);
     if (r != FGR_OK) return r;
     launches += pk.m > 0 ? 2 : 1;
-    FGR_CUDA_TRY(cudaMemcpyAsync(ctx->host_pinned, bnd, sizeof(int) * 13, cudaMemcpyDeviceToHost, st));
+    FGR_CUDA_TRY(cudaMemcpyAsync(ctx->host_pinned, bnd, sizeof(int) * 14, cudaMemcpyDeviceToHost, st));
     int *herr = reinterpret_cast<int *>(ctx->host_pinned) + 16;
     FGR_CUDA_TRY(cudaMemcpyAsync(herr, ctx->dev_err, sizeof(int), cudaMemcpyDeviceToHost, st));
     FGR_CUDA_TRY(cudaStreamSynchronize(st));
@@ -1545,7 +1571,7 @@ fgr_status launch(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStream_t 
                   "or the tensor-core direct sum's pipeline); that call's output is incomplete");
         return FGR_E_TIMEOUT;
     }
-    int hb[13];
+    int hb[14];
     memcpy(hb, ctx->host_pinned, sizeof(hb));
     if (check_finite && hb[12]) {
         set_error("packets: a non-finite Q, P, S or A value");
@@ -1863,16 +1889,16 @@ fgr_status run_fggc(fgr_ctx *ctx, const PacketsDev &pk, void *u_dev, cudaStream_
 }
 
 // Node bounds of the packets (per dimension: a min, a max, b min, b max; a
-// clipped to the grid-relevant range) into hb on the host; waits for them.
+// clipped to the grid-relevant range) and order into hb[14] on the host; waits for them.
 fgr_status compute_node_bounds(fgr_ctx *ctx, const PacketsDev &pk, int *bnd_dev, int *hb, cudaStream_t st) {
     const Common c = base_common(ctx);
     int aglo[3], aghi[3];
     grid_node_range(ctx, aglo, aghi);
-    fgr_status r = launch_bounds_reduction(ctx, pk, c, aglo, aghi, bnd_dev, st);
+    fgr_status r = launch_bounds_reduction(ctx, pk, c, aglo, aghi, bnd_dev, st, false, true);
     if (r != FGR_OK) return r;
-    FGR_CUDA_TRY(cudaMemcpyAsync(ctx->host_pinned, bnd_dev, sizeof(int) * 12, cudaMemcpyDeviceToHost, st));
+    FGR_CUDA_TRY(cudaMemcpyAsync(ctx->host_pinned, bnd_dev, sizeof(int) * 14, cudaMemcpyDeviceToHost, st));
     FGR_CUDA_TRY(cudaStreamSynchronize(st));
-    memcpy(hb, ctx->host_pinned, sizeof(int) * 12);
+    memcpy(hb, ctx->host_pinned, sizeof(int) * 14);
     return FGR_OK;
 }
 
@@ -2036,7 +2062,7 @@ extern "C" fgr_status fgr_reconstruct_fggc_noalloc(fgr_ctx *ctx, const fgr_packe
     const int64_t m = pk->m;
     if (m > 0) {
         bounds_kernel<1><<<bounds_blocks(ctx, m), 256, 0, st>>>(pk->q, pk->p, pk->a, m, c, aglo, aghi,
-                                                                     0, -1, 0, -1, bnd, nullptr);
+                                                                     0, -1, 0, -1, bnd, nullptr, nullptr);
         FGR_CUDA_TRY(cudaGetLastError());
     }
     FGR_CUDA_TRY(cudaMemcpyAsync(ctx->host_pinned, bnd, sizeof(int) * 4, cudaMemcpyDeviceToHost, st));

@@ -65,6 +65,7 @@ struct FggcBox {
     int64_t table_entries = 0;  // 8-byte entries of the pass tables of all dimensions
     int64_t fft_elems = 0;      // complex elements of the DFT lines of the largest pass (0: no DFT stage)
     bool empty = true;      // no packet reaches the grid
+    bool apart = true;      // neighbouring packets mostly lie in cells more than two apart (d = 2)
 };
 
 struct FggcBuffers {
@@ -156,18 +157,22 @@ constexpr int kBinMinCount = 8;
 // of one packet per cell 24 x 16, 20 x 12 and 32 x 16 measured the same (2-D
 // workload 1.37 ms), 16 x 12 1.43, 12 x 12 1.48 and 8 x 8 1.77 ms.
 constexpr int kBinTileA = 24, kBinTileB = 16;
-// Where the binned scatter runs in 2-D; each side was measured on sets in mesh order, whose
-// neighbouring threads' reductions meet in L2, and in random order.  n1 = 4: never (mesh
-// order, whole calls, binned / per packet: 147,456 packets 230 / 172 us, 1.0M 414 / 355,
-// 4.2M 907 / 874).  n1 = 8: from kBinMinPackets2d (mesh order 147,456: 247 / 197 us, 262,144:
-// 300 / 279, 419,904: 328 / 333, 1.6M: 626 / 808; random order, 262,144 on 50 x 45 cells per
-// plane 329 / 631), and where the mean bin, scaled by the part of a tile that the inner
-// plane fills, holds kBinMinMean2d packets: an item costs a CTA the same however few it
-// holds, and on small planes the reductions are cheap (5 x 6 cells, 4.2M packets, 8 per
-// bin: 4.6 / 3.2 ms; 24 per bin: 740 / 685 us; 48: 910 / 1196; whole tiles, 10 per bin:
-// 1.82 / 2.41 ms).
-constexpr int64_t kBinMinPackets2d = 1 << 18;
-constexpr double kBinMinMean2d = 8.0;
+// Where the binned scatter runs in 2-D (whole calls, binned / per packet, in us).  The
+// per-packet kernel's reductions meet in L2 where packets that follow each other lie in
+// cells next to each other (mesh order), so the rule depends on the order, which the bounds
+// kernel samples (order_probe).
+// Apart: from kBinMinPackets2d (147,456 packets: n1 = 8 198 / 317, n1 = 4 185 / 197; 1.0M: 394
+// / 1909 and 324 / 925), where the mean bin holds kBinMinMean2d packets (2.0: 1086 / 1350).
+// Near, n1 = 8: from kBinMinNear8 (147,456: 183 / 150; 262,144: 300 / 279 and 221 / 192; 419,904:
+// 307 / 304; 1.6M: 590 / 762), mean kBinMinMeanNear.
+// Near, n1 = 4: from kBinMinNear4 (1.0M: 380 / 330; 1.6M: 478 / 467; 4.2M: 858 / 844 and 729 /
+// 805; 17M: 2319 / 3099), a third of that where bins hold kBinDense (1.0M: 191 / 291).
+// The mean bin is scaled by the part of a tile that the inner plane fills: an item costs a
+// CTA the same however few packets it holds, and on small planes the reductions are cheap
+// (5 x 6 cells, 4.2M packets, 8 per bin: 4.6 / 3.2 ms; 24 per bin: 740 / 685 us; 48: 910 /
+// 1196).
+constexpr int64_t kBinMinPackets2d = 1 << 17, kBinMinNear8 = 1 << 18, kBinMinNear4 = 3 << 19;
+constexpr double kBinMinMean2d = 2.0, kBinMinMeanNear = 8.0, kBinDense = 512.0;
 
 // Key box of a node box and m packets (false when the binned scatter does not apply).
 bool make_bin_box(const FggcBox &box, int d, int64_t m, BinBox *bb);
@@ -230,10 +235,11 @@ fgr_status launch_scatter_batch_d3(int n1, cudaStream_t st, const ScatterBatch64
 int scatter_threads(bool fp64, int n1);
 
 // Box from the packets' node bounds hb[12] (per dimension: a min, a max, b min,
-// b max), widened by margin nodes on every side.
+// b max), widened by margin nodes on every side, and their order hb[13] (of hb[14]).
 fgr_status make_box(const fgr_ctx *ctx, const int *hb, int margin, FggcBox *box);
 
-// Node bounds of the packets into hb[12] on the host (waits for them).
+// Node bounds and order of the packets into hb[14] on the host (waits for them);
+// bnd_dev: 14 device ints.
 fgr_status compute_node_bounds(fgr_ctx *ctx, const PacketsDev &pk, int *bnd_dev, int *hb, cudaStream_t st);
 
 // FGGC into u_dev with a planned box and buffers: stream-ordered only; sets

@@ -12,7 +12,7 @@ import pytest
 
 import paper_2504_21785_gb300 as fgr
 
-from ._gpu import options, reconstruct, rel_l2
+from ._gpu import options, reconstruct, rel_l2, to_device
 from .test_gpu_binned import lattice_2d
 
 pytestmark = pytest.mark.gpu
@@ -29,7 +29,7 @@ def _binned(pk, grid, eps, opt):
 
 def _in_parts(pk, grid, eps, opt):
     """The sum of the results of parts that are too few to be binned."""
-    total, step = 0.0, (1 << 18) - 1
+    total, step = 0.0, (1 << 17) - 1
     for i in range(0, pk["s"].size, step):
         part = {k: np.ascontiguousarray(pk[k][..., i:i + step]) for k in ("q", "p", "s", "a")}
         u, binned = _binned(part, grid, eps, opt)
@@ -50,6 +50,38 @@ def test_binned_2d_tiles_of_large_sets(n_a, n_b, thin, nq, np_):
     assert pk["s"].size >= 1 << 18 and binned
     # both sides round the same contributions and sums to FP32 (2e-7 each)
     assert rel_l2(got, _in_parts(pk, grid, eps, opt)) <= 2e-6
+
+
+@pytest.mark.parametrize("nq,np_", [(4, 2), (2, 2), (2, 4)])
+def test_packet_order_decides_on_2d_binning(nq, np_):
+    """The same packets out of order (binned) and in mesh order (too few of them, per
+    packet), in a call and through a plan."""
+    pk, mesh, eps = lattice_2d(5, 20, 19, 0.4)
+    m = pk["s"].size
+    assert 1 << 17 <= m < 1 << 18
+    cell = [np.floor(x[l] / dx) for l in range(2) for x, dx in ((pk["q"], mesh.dq), (pk["p"], mesh.dp))]
+    by_mesh = np.lexsort(cell[::-1])
+    grid = dict(d=2, n=[50, 61], lo=[-0.8, -0.7], hi=[0.9, 0.8])
+    opt = options("fp32", nq=nq, np_=np_)
+    torch = pytest.importorskip("torch")
+    out = []
+    for idx, want in ((np.arange(m), True), (by_mesh, False)):
+        x = {k: np.ascontiguousarray(pk[k][..., idx]) for k in ("q", "p", "s", "a")}
+        u, binned = _binned(x, grid, eps, opt)
+        assert binned == want
+        out.append(u)
+        arrays = to_device(x)
+        packets = fgr.make_packets(*arrays)
+        v = torch.zeros(tuple(grid["n"]), dtype=torch.complex64, device="cuda")
+        with fgr.Context(2, grid, eps, opt) as ctx:
+            plan = fgr.fgr_fggc_plan_create(ctx.handle, packets, 1)
+            fgr.fgr_reconstruct_fggc_planned(ctx.handle, plan, packets, v)
+            assert not fgr.fgr_fggc_plan_overflow(plan)
+            fgr.fgr_fggc_plan_destroy(plan)
+        out.append(v.cpu().numpy())
+    # both sides round the same contributions and sums to FP32 (2e-7 each)
+    for v in out[1:]:
+        assert rel_l2(v, out[0]) <= 2e-6
 
 
 @pytest.mark.parametrize("shift_a,shift_b,amp,act", [
