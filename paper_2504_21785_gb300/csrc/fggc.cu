@@ -1040,7 +1040,8 @@ bool make_bin_box(const FggcBox &box, int d, int64_t m, BinBox *bb) {
         K *= (int64_t)x.tiles_a * x.tiles_b;
         const double filled = (double)x.KA[1] * x.KB[1] / ((double)x.tiles_a * x.tiles_b * kBinTileA * kBinTileB);
         const double mean = (double)m * filled / (double)K;
-        if (K > kMaxBinKeys || mean < (box.apart ? kBinMinMean2d : kBinMinMeanNear)) return false;
+        const double far = box.cells > kBinL2Cells ? kBinMinMean2d / 2 : kBinMinMean2d;
+        if (K > kMaxBinKeys || mean < (box.apart ? far : kBinMinMeanNear)) return false;
         const int64_t least = box.c.n1 == 8 ? kBinMinNear8 : mean < kBinDense ? kBinMinNear4 : kBinMinNear4 / 3;
         if (!box.apart && m < least) return false;
     }
@@ -1087,7 +1088,7 @@ size_t bin_buffer_bytes(int64_t m, const BinBox &bb) {
 size_t fggc_spare_bytes(int d, int n1, int64_t m) {
     if (d < 2 || (n1 != 4 && n1 != 8) || m >= INT_MAX || (d == 2 && m < kBinMinPackets2d)) return 0;
     BinBox bb;
-    bb.K = d == 2 ? (int64_t)(m / kBinMinMean2d) : m;  // (2-D: at most)
+    bb.K = d == 2 ? (int64_t)(m * 2 / kBinMinMean2d) : m;  // (2-D: at most)
     bb.boxes = d == 3;
     return bin_buffer_bytes(m, bb);
 }

@@ -162,7 +162,9 @@ constexpr int kBinTileA = 24, kBinTileB = 16;
 // cells next to each other (mesh order), so the rule depends on the order, which the bounds
 // kernel samples (order_probe).
 // Apart: from kBinMinPackets2d (147,456 packets: n1 = 8 198 / 317, n1 = 4 185 / 197; 1.0M: 394
-// / 1909 and 324 / 925), where the mean bin holds kBinMinMean2d packets (2.0: 1086 / 1350).
+// / 1909 and 324 / 925), where the mean bin holds kBinMinMean2d packets (2.2: 656 / 448; 2.9:
+// 536 / 434; 4.3: 758 / 740; 5.8: 604 / 664), half of that where the node array is beyond L2
+// (kBinL2Cells; 2.0: 1086 / 1350).
 // Near, n1 = 8: from kBinMinNear8 (147,456: 183 / 150; 262,144: 300 / 279 and 221 / 192; 419,904:
 // 307 / 304; 1.6M: 590 / 762), mean kBinMinMeanNear.
 // Near, n1 = 4: from kBinMinNear4 (1.0M: 380 / 330; 1.6M: 478 / 467; 4.2M: 858 / 844 and 729 /
@@ -172,7 +174,8 @@ constexpr int kBinTileA = 24, kBinTileB = 16;
 // (5 x 6 cells, 4.2M packets, 8 per bin: 4.6 / 3.2 ms; 24 per bin: 740 / 685 us; 48: 910 /
 // 1196).
 constexpr int64_t kBinMinPackets2d = 1 << 17, kBinMinNear8 = 1 << 18, kBinMinNear4 = 3 << 19;
-constexpr double kBinMinMean2d = 2.0, kBinMinMeanNear = 8.0, kBinDense = 512.0;
+constexpr int64_t kBinL2Cells = 1 << 24;
+constexpr double kBinMinMean2d = 4.0, kBinMinMeanNear = 8.0, kBinDense = 512.0;
 
 // Key box of a node box and m packets (false when the binned scatter does not apply).
 bool make_bin_box(const FggcBox &box, int d, int64_t m, BinBox *bb);

@@ -84,6 +84,22 @@ def test_packet_order_decides_on_2d_binning(nq, np_):
         assert rel_l2(v, out[0]) <= 2e-6
 
 
+@pytest.mark.parametrize("wide,binned_whole", [(4.0, False), (1.5, True)])
+def test_small_bins_out_of_order_stay_per_packet(wide, binned_whole):
+    """Packets out of order over an inner plane of half a tile: binned where the
+    mean bin is worth it."""
+    rng = np.random.default_rng(9)
+    m, eps = 1 << 18, 1 / 64
+    q = np.stack([rng.uniform(-wide, wide, m), rng.uniform(-0.2, 0.2, m)])
+    p = np.stack([rng.uniform(-2 * wide, 2 * wide, m), rng.uniform(-0.2, 0.2, m)])
+    pk = {"q": q, "p": p, "s": rng.uniform(-1, 1, m), "a": rng.standard_normal((2, m))}
+    grid = dict(d=2, n=[200, 16], lo=[-4.5, -0.3], hi=[4.5, 0.3])
+    got, binned = _binned(pk, grid, eps, options("fp32"))
+    assert binned == binned_whole
+    # both sides round the same contributions and sums to FP32 (2e-7 each)
+    assert rel_l2(got, _in_parts(pk, grid, eps, options("fp32"))) <= 2e-6
+
+
 @pytest.mark.parametrize("shift_a,shift_b,amp,act", [
     (1 << 18, 0, 1.0, 1.0), (-(1 << 18), 0, 1.0, 1.0), (0, 1 << 18, 1.0, 1.0), ((1 << 18) - 10, 3, 1.0, 1.0),
     (60, 40, 1.0, 3e4)])
