@@ -1043,7 +1043,7 @@ bool make_bin_box(const FggcBox &box, int d, int64_t m, BinBox *bb) {
         const double far = box.cells > kBinL2Cells ? kBinMinMean2d / 2 : kBinMinMean2d;
         if (K > kMaxBinKeys || mean < (box.apart ? far : kBinMinMeanNear)) return false;
         const int64_t least = box.c.n1 == 8 ? kBinMinNear8 : mean < kBinDense ? kBinMinNear4 : kBinMinNear4 / 3;
-        if (!box.apart && m < least) return false;
+        if (!box.apart && (m < least || (box.c.n1 != 8 && (double)m < kBinMinFull * (double)K))) return false;
     }
     x.K = K;
     x.boxes = d == 3;

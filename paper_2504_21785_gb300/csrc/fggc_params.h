@@ -167,15 +167,16 @@ constexpr int kBinTileA = 24, kBinTileB = 16;
 // (kBinL2Cells; 2.0: 1086 / 1350).
 // Near, n1 = 8: from kBinMinNear8 (147,456: 183 / 150; 262,144: 300 / 279 and 221 / 192; 419,904:
 // 307 / 304; 1.6M: 590 / 762), mean kBinMinMeanNear.
-// Near, n1 = 4: from kBinMinNear4 (1.0M: 380 / 330; 1.6M: 478 / 467; 4.2M: 858 / 844 and 729 /
-// 805; 17M: 2319 / 3099), a third of that where bins hold kBinDense (1.0M: 191 / 291).
+// Near, n1 = 4: from kBinMinNear4 (1.0M: 380 / 330) where bins hold kBinMinFull packets (not
+// scaled; 4.2M on 1024^2 points, 35 per bin: 1079 / 960; 54: 859 / 815; 178: 729 / 805; 17M,
+// 173: 2319 / 3099), a third of that where the mean is kBinDense (1.0M: 191 / 291).
 // The mean bin is scaled by the part of a tile that the inner plane fills: an item costs a
 // CTA the same however few packets it holds, and on small planes the reductions are cheap
 // (5 x 6 cells, 4.2M packets, 8 per bin: 4.6 / 3.2 ms; 24 per bin: 740 / 685 us; 48: 910 /
 // 1196).
 constexpr int64_t kBinMinPackets2d = 1 << 17, kBinMinNear8 = 1 << 18, kBinMinNear4 = 3 << 19;
 constexpr int64_t kBinL2Cells = 1 << 24;
-constexpr double kBinMinMean2d = 4.0, kBinMinMeanNear = 8.0, kBinDense = 512.0;
+constexpr double kBinMinMean2d = 4.0, kBinMinMeanNear = 8.0, kBinMinFull = 96.0, kBinDense = 512.0;
 
 // Key box of a node box and m packets (false when the binned scatter does not apply).
 bool make_bin_box(const FggcBox &box, int d, int64_t m, BinBox *bb);

@@ -11,6 +11,7 @@ import numpy as np
 import pytest
 
 import paper_2504_21785_gb300 as fgr
+from workloads import mesh_for
 
 from ._gpu import options, reconstruct, rel_l2, to_device
 from .test_gpu_binned import lattice_2d
@@ -82,6 +83,25 @@ def test_packet_order_decides_on_2d_binning(nq, np_):
     # both sides round the same contributions and sums to FP32 (2e-7 each)
     for v in out[1:]:
         assert rel_l2(v, out[0]) <= 2e-6
+
+
+@pytest.mark.parametrize("shape,binned_whole", [((190, 175, 6, 8), False), ((95, 88, 16, 12), True)])
+def test_mesh_order_with_four_neighbours(shape, binned_whole):
+    """1.6 million packets in mesh order, Q2P2: binned where bins hold many of them."""
+    eps = 1 / 64
+    mesh = mesh_for(2, eps)
+    rng = np.random.default_rng(12)
+    idx = np.indices(shape).reshape(4, -1) + rng.uniform(0.1, 0.9, (4, int(np.prod(shape))))
+    idx -= np.array(shape)[:, None] // 2
+    m = idx.shape[1]
+    pk = {"q": idx[[0, 2]] * mesh.dq, "p": idx[[1, 3]] * mesh.dp, "s": rng.uniform(-1, 1, m),
+          "a": rng.standard_normal((2, m))}
+    grid = dict(d=2, n=[128, 24], lo=[-6.0, -0.6], hi=[6.0, 0.6])
+    opt = options("fp32", nq=2, np_=2)
+    got, binned = _binned(pk, grid, eps, opt)
+    assert binned == binned_whole
+    # both sides round the same contributions and sums to FP32 (2e-7 each)
+    assert rel_l2(got, _in_parts(pk, grid, eps, opt)) <= 2e-6
 
 
 @pytest.mark.parametrize("wide,binned_whole", [(4.0, False), (1.5, True)])
