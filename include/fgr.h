@@ -284,10 +284,11 @@ fgr_status fgr_reconstruct_direct_batch(int32_t n, fgr_ctx *const *ctxs, const f
  * come from a polynomial surrogate of c~(s,t) built on the host from the same
  * pseudo-inverse (Chebyshev interpolation of degree 9 per variable, total degree
  * 11 for n1 <= 8; truncation about 1e-8 of the largest coefficient, below FP32
- * rounding), one per four mirrored neighbours; phases are reduced to FP64
- * accuracy, node array and grid sums in complex64.  Host packets are copied to
- * the device and tested there for non-finite values before anything is
- * written: FGR_E_INVALID if one is found. */
+ * rounding), one per four mirrored neighbours; phases are reduced in FP64 or, where
+ * packets are binned, as sums of two FP32 numbers (2^-45 relative, for anchors and
+ * actions below 2^18 turns; FP64 beyond), node array and grid sums in complex64.
+ * Host packets are copied to the device and tested there for non-finite values
+ * before anything is written: FGR_E_INVALID if one is found. */
 fgr_status fgr_reconstruct_fggc(fgr_ctx *ctx, const fgr_packets *pk, void *u_out,
                                 void *cuda_stream);
 

@@ -11,7 +11,7 @@
 // evaluated, so no power is above the fourth.
 // Bound by instruction issue: about 8.5 per packet-point pair, against 17 for four
 // points by the recurrences of direct_tile: 1-D workload (262,144 packets, 32,768
-// points) 331 -> 256 us with the sum of the slices.  Coarser grids keep direct_tile,
+// points) 331 -> 259 us with the sum of the slices.  Coarser grids keep direct_tile,
 // which has no powers of s across points that lie several widths apart, and so do
 // calls with too few packet-point pairs for the partial sums (use_direct1).
 // Included by direct.cu inside its anonymous namespace.

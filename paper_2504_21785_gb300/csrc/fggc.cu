@@ -6,7 +6,8 @@
 // range whose Gaussians reach the grid (other nodes have empty windows); the
 // b-range spans the packets with non-zero amplitude (zero amplitudes add zeros).
 //
-// K3+K4 (one thread per packet).  Per dimension: r = Q/dq, a0 = floor(r),
+// K3+K4 (one thread per packet; FP32 sets in d = 2 and 3 that make_bin_box accepts are
+// sorted by cell and summed per cell, fggc_bin.cuh).  Per dimension: r = Q/dq, a0 = floor(r),
 // s = r - a0 and likewise b0, t for P (eq. 3.6-3.7, FP64).  The true LSA
 // coefficients c~_k(s,t) = conj(A~^+ f~(s,t))_k come from
 //   FP64: f~ of eq. 3.23 in FP64 and A~^+ applied through its eigen factors;
@@ -22,11 +23,14 @@
 //
 // K5 (separable grid stage).  u(x_m) = sum_{a,b} W'[a,b] prod_l g(x_{m_l} - a_l dq)
 // e^{i b_l dp x_{m_l}/eps} is contracted one dimension at a time: a pass maps
-// rows [a_l][b_l] to [m_l]; a transpose brings the next dimension innermost.
-// Each CTA owns 32 or 128 grid points of one row (one per thread): the band of
-// nodes a whose window covers them, g in registers, W staged through shared
+// rows [a_l][b_l] to [m_l].  Single and planned calls in d >= 2 run
+// grid_rows_kernel (fggc_rows.cuh; rows_apply has its limits), which writes the
+// next pass's layout.  The pass kernels below serve 1-D, batches, the DFT stage and
+// the rest: a CTA owns 32 or 128 grid points of one row (one per thread), the
+// band of nodes a whose window covers them, g in registers, W staged through shared
 // memory in chunks of b, and e^{i b dp x/eps} generated per (m, b) from a
-// phase reduced in FP64.
+// phase reduced in FP64; in d >= 2 a transpose brings the next dimension
+// innermost.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 

@@ -80,8 +80,8 @@ __device__ __forceinline__ void exp_minus_one(double e, double sn_half, double c
 // bases.  All of it is carried as f - 1: the problem's small eigenvalues divide the
 // rounding of f by up to their square root (2.6e-5 for Q4P2), f lies near one, and the
 // ones' share of every eigenvector is exact (Lsa::sec_one).  Relative to the result,
-// random packets: 3.2e-12 for Q4P2 with products of exponentials (4.7e-12 with one
-// exponential and phase per neighbour), 3.2e-13 so.  The phases are those of
+// random packets: 3.6e-12 for Q4P2 with products of exponentials (3.4e-12 with one
+// exponential and phase per neighbour), 3.4e-13 so.  The phases are those of
 // dim_setup32: z = e^{i cq cp A / 2}, and T takes the packet's share in turns.  The
 // FP64 pipe binds (16 clocks of an SM per warp instruction): against an exponential,
 // two sines and cosines and two complex matrix rows per neighbour, 705,600 2-D Q2P2

@@ -22,14 +22,15 @@
 //
 // FP64: one point per lane, and the phases (rotation of a step, and of the middle b
 // of every four) from a table of the pass instead of a sine and cosine per b, point
-// and row; the FP64 pipe binds: 2-D Q2P2 set of 705,600 packets on 301 x 257 points
-// 2.42 -> 1.48 ms for both passes.
+// and row; the FP64 pipe binds (94 %): 2-D Q2P2 set of 705,600 packets on 301 x 257
+// points 2.42 -> 0.84 ms for both passes (1.48 with up to 24 rows per CTA whatever the
+// wave covers).
 //
 // FP32: bound by instruction issue: per node and four values 2 shared loads and 8
 // two-wide multiply-adds.  Against one point per lane, whole 8 x 32 tiles over
 // the band of a 32-point tile, a b-range scan before and a transpose after every
-// pass: 3-D workload (16.8M packets, 256^3 points) grid stage 4.92 -> 2.42 ms,
-// 2-D (4.2M, 1024^2) 0.54 -> 0.44 ms.
+// pass: 3-D workload (16.8M packets, 256^3 points) grid stage 4.92 -> 2.50 ms,
+// 2-D (4.2M, 1024^2) 0.54 -> 0.41 ms.
 //
 // Included by fggc.cu inside its anonymous namespace, after fggc_tma.cuh.
 #pragma once

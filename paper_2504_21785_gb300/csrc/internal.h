@@ -72,7 +72,8 @@ struct Mesh {
 
 struct Timing {
     bool enabled = false;
-    bool count_terms = false;  // also count the grid passes' node-point terms (one kernel per pass)
+    bool count_terms = false;  // also count the grid passes' node-point terms (a scan and a count per pass,
+                               // after the last stage)
     fgr_stats last{};
 };
 
