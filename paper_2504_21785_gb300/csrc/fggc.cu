@@ -1213,11 +1213,12 @@ __global__ void __launch_bounds__(256) tables_batch_kernel(const __grid_constant
     pass_tables_body(B.pp[r], tp, mtiles, B.tab[r], (int64_t)(blockIdx.x - B.block0[r]) * 256 + threadIdx.x);
 }
 
-// (FP32: four CTAs of 128 per SM; left to itself the compiler packs the 64-node
-// form into 96 registers and the batch of 32 1-D requests takes 0.65 ms instead
-// of 0.30)
+// (FP32: three CTAs of 128 per SM.  Left to itself the compiler packs the 64-node form
+// into 96 registers and the batch of 32 1-D requests takes 0.65 ms instead of 0.30.  With
+// 146 registers instead of the 126 of four CTAs: 6 requests of 3000 to 11,000 packets
+// 202 -> 150 us, 32 of up to 65,536 346 -> 327)
 template <bool FP64, int MAXBAND, int TP>
-__global__ void __launch_bounds__(TP, !FP64 && TP == 128 ? 4 : 1) grid_pass_batch_kernel(const __grid_constant__ PassBatch B) {
+__global__ void __launch_bounds__(TP, !FP64 && TP == 128 ? 3 : 1) grid_pass_batch_kernel(const __grid_constant__ PassBatch B) {
     const int r = batch_request(B.block0, B.n);
     const int64_t local = blockIdx.x - B.block0[r];
     const int64_t row = local / B.tiles[r];
